@@ -26,6 +26,13 @@
 //     MMAs, one commit), and TX_GROUPS groups of four expander warps work on different pairs at
 //     the same time.
 //
+// What bounds it: on layers up to a few MB the chain launch -> set-up -> input -> MMAs -> epilogue -> cluster sum, twice per
+// forward.  A CTA with two expander groups therefore takes half of an SM's registers and of its shared memory, so that the next
+// launch's CTA starts, sets up and requests its first operands while this one works; it gets the tensor memory as soon as
+// this one has read its accumulators.  Graph replay, us per forward, before -> after: 4096 x 4096, k = 1664, l = 16: 9.31 -> 7.64;
+// 8192 x 8192, k = 3712: 15.2 -> 14.1; q/k/v of 4096 x 4096: 15.0 -> 13.4; 11008 x 4096 gate and up: 22.0 -> 20.0.  Layers so small
+// that every launch had idle SMs to start on gained nothing and pay the extra barriers (640 x 640: 5.8 -> 6.0).
+//
 // CTA = 128 sign rows x a slice of the reduction; the KS CTAs of a row block form a cluster and
 // reduce their partial outputs through distributed shared memory (deterministic, no atomics).
 // Column order inside a K block: MMA k index p is canonical column
@@ -41,11 +48,14 @@ namespace cg = cooperative_groups;
 namespace mdbf {
 
 // expander groups of 4 warps (template parameter G of the kernel; group g takes the pairs g, g + G, ...): 2 for
-// CTAs with few pairs (all latency, fewer warps start faster), 3 for long CTAs (+5 % on 70B-class layers; 4: worse)
+// CTAs with few pairs (all latency; two such CTAs fit on an SM), 3 for long CTAs (4: worse)
 constexpr int TX_ISSUERS = 4;                          // MMA issuer warps, one accumulator each (a thread issues ~1 MMA / 100+ clk here)
 constexpr int tx_threads(int groups) { return groups * 128 + TX_ISSUERS * 32 + 64; }   // + sign loader warp + V loader warp
+constexpr int tx_ctas(int groups) { return groups <= 2 ? 2 : 1; }      // CTAs per SM the registers are held to (72 a thread with two groups)
 constexpr int TX_MAX_SSTAGES = 16;                     // sign ring: 2 KB per stage (one pair of K blocks)
 constexpr int TX_MAX_ASTAGES = 7;                      // A / V stages: 64 TMEM columns + two V tiles each
+constexpr int TX_MAX_DYN = 220 * 1024;                 // dynamic shared memory
+constexpr int TX_LONG = 48;                            // pairs of K blocks per CTA from which on a CTA has three expander groups
 
 struct TxArgs {
     const uint2 *wk2;         // sign words, row-block major: [row block][kb_pad][128 rows], 64 bits each
@@ -75,6 +85,11 @@ struct TxMulti {
     int rb_start[TX_MAX_LAYERS + 1];   // first row block of each layer; rb_start[nlayers] = gridDim.x
     int nlayers;
 };
+
+// Cluster barrier in two halves.  The relaxed arrive orders no memory: it only says that this CTA runs.
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 
 // First test inline (the common case: the barrier has completed), bounded loop otherwise.
 __device__ __forceinline__ bool tx_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int32_t *status) {
@@ -128,6 +143,44 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
     }
     if (tid == 0) abort_flag_s = 0;
     fence_barrier_init();
+    cluster_arrive_relaxed();                                // awaited by every role once its own work is done, before the first store into another CTA
+    __syncthreads();
+
+    // What depends on no other launch is requested at once: the first fills of both rings and the rows of U.
+    const uint2 *sign_src = a.wk2 + ((size_t)rb * a.kb_pad + (size_t)pr0 * 2) * 128;
+    const uint16_t *v_src = a.vtile + (size_t)pr0 * 2 * NB * 64;
+    const int s_first = min(npr, nss), v_first = min(npr, nas);
+    if (warp == TX_W_ISSUER0 + TX_ISSUERS && lane == 0)
+        for (int pr = 0; pr < s_first; ++pr) {
+            mbar_arrive_expect_tx(s_full + 8 * pr, 2048u);
+            bulk_load(smem_base + off_s + (uint32_t)(pr * 2048), sign_src + (size_t)pr * 256, 2048u, s_full + 8 * pr);
+        }
+    if (warp == TX_W_ISSUER0 + TX_ISSUERS + 1 && lane == 0)
+        for (int pr = 0; pr < v_first; ++pr) {
+            mbar_arrive_expect_tx(v_full + 8 * pr, (uint32_t)VBYTES);
+            bulk_load(smem_base + (uint32_t)(pr * VBYTES), v_src + (size_t)pr * 2 * NB * 64, (uint32_t)VBYTES, v_full + 8 * pr);
+        }
+    const int row_l = (warp & 3) * 32 + lane;                // row of the tile = TMEM lane (expander warps)
+    uint32_t uw[(LP + 1) / 2];                               // U of this row, two modes per word (first expander group)
+#pragma unroll
+    for (int m = 0; m < (LP + 1) / 2; ++m) {
+        uw[m] = 0u;
+        if (warp < 4 && row0 + row_l < a.rows) {
+            const uint16_t *ur = reinterpret_cast<const uint16_t *>(a.U) + (size_t)(row0 + row_l) * a.l + 2 * m;
+            if (LP > 1 && a.l == LP) uw[m] = *reinterpret_cast<const uint32_t *>(ur);
+            else {
+                if (2 * m < a.l) uw[m] = ur[0];
+                if (2 * m + 1 < a.l) uw[m] |= (uint32_t)ur[1] << 16;
+            }
+        }
+    }
+
+    // Tensor memory.  Two CTAs fit on an SM but both want (nearly) all of its tensor memory, so the CTA of the next launch waits
+    // in the allocation while this one works, its launch latency, barrier set-up and first loads behind it (its warps
+    // sleep at the block barrier: polling ones cost the working CTA more than the early start gives).  Two rules keep that free
+    // of cycles: a CTA lets its dependents launch only when it holds its tensor memory (so no later launch can take it first), and
+    // while it holds it, it waits for earlier launches only, never for another CTA of its own (it frees it before it waits
+    // for the cluster).
     if (warp == TX_W_ISSUER0) {
         tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)a.tmem_cols);
         tmem_relinquish();
@@ -135,22 +188,17 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_launch_dependents();
     const uint32_t tmem = tmem_base_slot;
     const uint32_t tmem_a0 = tmem + (uint32_t)(TX_ISSUERS * NB);
 
-    pdl_launch_dependents();
-
-    const int row_l = (warp & 3) * 32 + lane;                // row of the tile = TMEM lane (expander warps)
     float outv = 0.f;
+    bool freed = false;
 
     if (warp < TX_W_ISSUER0) {
         // ============================ expanders, then epilogue ============================
         const int grp = warp >> 2;
         const int grow = row0 + row_l;
-        float u[LP];
-#pragma unroll
-        for (int t = 0; t < LP; ++t)
-            u[t] = (grp == 0 && grow < a.rows && t < a.l) ? env_load(a.U, (size_t)grow * a.l + t, a.env_dtype) : 0.f;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
 
         // stage the activation slice as bf16 pairs in MMA k order: pair `col` of a K block holds
@@ -197,7 +245,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
                                pack_bf16x2(lo[3], hi[3]));
             }
         }
-        asm volatile("bar.sync 2, %0;\n" ::"n"(TX_EXPANDERS) : "memory");
+        asm volatile("bar.sync 1, %0;\n" ::"n"(TX_EXPANDERS) : "memory");
 
         // One pair of K blocks per iteration: 2 x 64 sign bits of this row -> 64 TMEM columns.
         bool alive = true;
@@ -245,6 +293,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
         __syncwarp();
         if (alive && prev_as >= 0 && lane == 0) mbar_arrive(a_full + 8 * prev_as);
         if (grp != 0) alive = false;                         // only the first group runs the epilogue
+        cluster_wait();
         if (alive) alive = mbar_wait(acc_bar, 0u, abort_flag, a.status);
         tc_fence_after();
         if (alive) {
@@ -255,14 +304,14 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) sum[j] = 0.f;
 #pragma unroll
-                for (int a4 = 0; a4 < TX_ISSUERS; a4 += 4) {             // four accumulators per round of loads
-                    uint32_t d[4][16];
+                for (int a4 = 0; a4 < TX_ISSUERS; a4 += 2) {             // two accumulators per round of loads (registers)
+                    uint32_t d[2][16];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
+                    for (int q = 0; q < 2; ++q)
                         if (a4 + q < nacc) tmem_ld16(tmem + lane_base + (uint32_t)((a4 + q) * NB + cc * 16), d[q]);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
+                    for (int q = 0; q < 2; ++q)
                         if (a4 + q < nacc) {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) sum[j] += __uint_as_float(d[q][j]);
@@ -270,8 +319,15 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
                 }
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                    if (cc * 16 + j < LP) outv += u[(cc * 16 + j) % LP] * sum[j];
+                    if (cc * 16 + j < LP) {
+                        const uint32_t w = uw[(cc * 16 + j) % LP >> 1];
+                        outv += (a.env_dtype == MDBF_BF16 ? env16<true>((j & 1) ? w >> 16 : w & 0xFFFFu) : env16<false>((j & 1) ? w >> 16 : w & 0xFFFFu)) * sum[j];
+                    }
             }
+        }
+        if (grp == 0) {
+            tc_fence_before();
+            asm volatile("bar.arrive 2, 160;\n" ::: "memory");     // accumulators read: issuer warp 0 frees the tensor memory
         }
     }
     else if (warp < TX_W_ISSUER0 + TX_ISSUERS) {
@@ -314,40 +370,47 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
             else mbar_arrive(acc_bar);
         }
         __syncwarp();
+        cluster_wait();
+        if (w == 0) {
+            asm volatile("bar.sync 2, 160;\n" ::: "memory");
+            tc_fence_after();
+            freed = !*abort_flag;                            // no expired wait: every MMA has retired and every store was consumed
+            freed = __all_sync(0xffffffffu, freed);
+        }
     } else if (warp == TX_W_ISSUER0 + TX_ISSUERS) {
         // ============================== sign-word loader ================================
         if (lane == 0) {
             bool alive = true;
             int rs = 0;
-            uint32_t ph = 0;
-            const uint2 *src = a.wk2 + ((size_t)rb * a.kb_pad + (size_t)pr0 * 2) * 128;
-            for (int pr = 0; pr < npr; ++pr) {
+            uint32_t ph = 1;                                 // the first fill was requested above
+            for (int pr = nss; pr < npr; ++pr) {
                 alive = tx_wait(s_empty + 8 * rs, ph ^ 1u, abort_flag, a.status);
                 if (!alive) break;
                 mbar_arrive_expect_tx(s_full + 8 * rs, 2048u);
-                bulk_load(smem_base + off_s + (uint32_t)(rs * 2048), src + (size_t)pr * 256, 2048u, s_full + 8 * rs);
+                bulk_load(smem_base + off_s + (uint32_t)(rs * 2048), sign_src + (size_t)pr * 256, 2048u, s_full + 8 * rs);
                 if (++rs == nss) { rs = 0; ph ^= 1u; }
             }
             if (!alive) drain_delay();
         }
         __syncwarp();
-    } else {
+        cluster_wait();
+    } else if (warp == TX_W_ISSUER0 + TX_ISSUERS + 1) {
         // ================================ V-tile loader ==================================
         if (lane == 0) {
             bool alive = true;
             int vs = 0;
-            uint32_t ph = 0;
-            const uint16_t *src = a.vtile + (size_t)pr0 * 2 * NB * 64;
-            for (int pr = 0; pr < npr; ++pr) {
+            uint32_t ph = 1;
+            for (int pr = nas; pr < npr; ++pr) {
                 alive = tx_wait(a_empty + 8 * vs, ph ^ 1u, abort_flag, a.status);
                 if (!alive) break;
                 mbar_arrive_expect_tx(v_full + 8 * vs, (uint32_t)VBYTES);
-                bulk_load(smem_base + (uint32_t)(vs * VBYTES), src + (size_t)pr * 2 * NB * 64, (uint32_t)VBYTES, v_full + 8 * vs);
+                bulk_load(smem_base + (uint32_t)(vs * VBYTES), v_src + (size_t)pr * 2 * NB * 64, (uint32_t)VBYTES, v_full + 8 * vs);
                 if (++vs == nas) { vs = 0; ph ^= 1u; }
             }
             if (!alive) drain_delay();
         }
         __syncwarp();
+        cluster_wait();
     }
 
     // ------------------------------ cluster reduction and store ------------------------------
@@ -357,7 +420,9 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
     tc_fence_before();
     const unsigned crank = cluster.block_rank();
     if (warp < 4 && crank != 0) cluster.map_shared_rank(part, 0)[crank * 128 + row_l] = outv;
-    cluster.sync();
+    cluster_arrive();
+    if (freed) tmem_dealloc(tmem_base_slot, (uint32_t)a.tmem_cols);      // issuer warp 0, off the other ranks' critical path
+    cluster_wait();
     if (warp < 4 && crank == 0) {
         const unsigned nranks = cluster.num_blocks();
 #pragma unroll
@@ -372,25 +437,28 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
             else reinterpret_cast<float *>(a.out)[grow] = outv;
         }
     }
-    if (warp == TX_W_ISSUER0) tmem_dealloc(tmem, (uint32_t)a.tmem_cols);
+    if (warp == TX_W_ISSUER0 && !freed) {                        // a wait expired: only now is nothing in flight any more
+        tc_fence_after();
+        tmem_dealloc(tmem_base_slot, (uint32_t)a.tmem_cols);
+    }
 }
 
 // One layer per launch: the arguments are plain kernel parameters (fastest for the small layers).
 template <int LP, int G>
-__global__ void __launch_bounds__(tx_threads(G), 1) tmem_t1_kernel(const TxArgs a) {
+__global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_kernel(const TxArgs a) {
     tmem_t1_body<LP, G>(a, (int)blockIdx.x + a.rb0);
 }
 
 // The last term of a sum of layers (mode 4 of the epilogue), an instantiation of its own so that the plain kernel
 // carries no trace of it.
 template <int LP, int G>
-__global__ void __launch_bounds__(tx_threads(G), 1) tmem_t1_sumlast_kernel(const TxArgs a) {
+__global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_sumlast_kernel(const TxArgs a) {
     tmem_t1_body<LP, G, true>(a, (int)blockIdx.x + a.rb0);
 }
 
 // Several sibling layers per launch: each CTA picks its layer by its position in the grid.
 template <int LP, int G>
-__global__ void __launch_bounds__(tx_threads(G), 1) tmem_t1_multi_kernel(const __grid_constant__ TxMulti m) {
+__global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_multi_kernel(const __grid_constant__ TxMulti m) {
     int li = 0;
 #pragma unroll
     for (int i = 1; i < TX_MAX_LAYERS; ++i)
@@ -469,6 +537,18 @@ struct TxPlan {
 // 7B- and 70B-class shapes).
 static int fixed_cost() { return 48; }
 
+// Two CTAs of a launch that share an SM take turns at its tensor memory, which costs a launch twice its time.  CTAs that start while
+// the previous launch still holds the other SMs are put there by the hardware, two on every idle SM: a launch that follows one
+// whose CTAs leave no room beside them (three expander groups, the integer kernel) asks for more than half of an SM's
+// shared memory and gets an SM per CTA (8192 x 8192, k = 3712 with three groups in one stage and two in the other: 20.6 us without this).
+constexpr size_t TX_ALONE_DYN = 114 * 1024;
+
+// Two CTAs with two expander groups share an SM, so the split between L1 and shared memory is set to hold both (132 of 228 KB; the
+// plan keeps a CTA below half of that up to 40 pairs).  The integer kernel's stages get the same split, so an SM need
+// not drain to change it: with the largest split the 70B-class block lost 5 us to that, with none set launches of different
+// footprints did not share an SM (11008 x 4096: 20.2 instead of 13.2 us).
+constexpr int TX_CARVEOUT = 58;
+
 // One plan for all the layers of a launch.  Cluster size along the reduction: one CTA per SM (all of
 // TMEM), as few waves as possible, the per-CTA fixed part weighed against its share of the reduction.
 static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p) {
@@ -497,27 +577,30 @@ static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p
         max_per = max(max_per, p->pairs_per_cta[i]);
     }
     p->nastages = nas;
-    p->nsstages = max_per < TX_MAX_SSTAGES ? max_per : TX_MAX_SSTAGES;
+    p->nsstages = min(max_per, max_per >= TX_LONG ? TX_MAX_SSTAGES : 8);
     p->tmem_cols = 512;
     p->smem = 1024 + (size_t)nas * 2 * NB * 128 + (size_t)p->nsstages * 2048 + (size_t)max_per * 256 + 4096;
-    return nas >= 2 && p->smem <= 220 * 1024;
+    return nas >= 2 && p->smem <= TX_MAX_DYN;
 }
 
 static thread_local int g_t1_launches = 0;      // kernels the last one-token forward of this thread launched
 int last_t1_launch_count() { return g_t1_launches; }
 
 template <int LP, int G>
-static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, cudaStream_t st) {
+static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, bool alone, cudaStream_t st) {
     static PerDeviceOnce once;
     if (once.first()) {
-        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sumlast_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
+        if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
+        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
+        if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
+        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sumlast_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
+        if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sumlast_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m.rb_start[m.nlayers], p.ks, 1);
     cfg.blockDim = dim3(tx_threads(G));
-    cfg.dynamicSmemBytes = p.smem;
+    cfg.dynamicSmemBytes = alone && p.smem < TX_ALONE_DYN ? TX_ALONE_DYN : p.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -534,26 +617,29 @@ static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, cudaStream_t 
     ++g_t1_launches;
     return MDBF_OK;
 }
-// Two expander groups for CTAs with few pairs of K blocks, three from `long_cta` pairs per CTA on (16: the
-// 4096 x 4096 layers keep two groups, the 11008- and 70B-class layers get three).
+// Two expander groups, which leave room for the next launch's CTA, or three from TX_LONG pairs per CTA on, where the expanders' rate
+// counts and not the start: 28672 x 8192 pair of siblings, 64 pairs per CTA: 70.9 us with two groups, 55.4 with three; 14336 x 8192,
+// 32 pairs: 18.9 and 24.3.
+// `full`: in, whether the launch before this one leaves no room beside its CTAs; out, whether this one does.
 template <int LP>
-static mdbf_status_t launch_t1(const TxMulti &m, const TxPlan &p, cudaStream_t st) {
-    const int long_cta = 16;
+static mdbf_status_t launch_t1(const TxMulti &m, const TxPlan &p, bool *full, cudaStream_t st) {
     int max_per = 0;
     for (int i = 0; i < m.nlayers; ++i) max_per = max(max_per, p.pairs_per_cta[i]);
-    return max_per >= long_cta ? launch_t1g<LP, 3>(m, p, st) : launch_t1g<LP, 2>(m, p, st);
+    const bool alone = *full;
+    *full = max_per >= TX_LONG;
+    return *full ? launch_t1g<LP, 3>(m, p, false, st) : launch_t1g<LP, 2>(m, p, alone, st);
 }
 
 // One stage.  When the grid ends in a wave with only a few CTAs (448 row blocks on 148 SMs: the last 4 would
 // cost a whole wave), those row blocks go to a second, short launch that splits their reduction over a
 // cluster instead; both launches read the same input and write disjoint rows.
 template <int LP>
-static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const int *kb_pad, cudaStream_t st) {
+static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const int *kb_pad, bool *no_room, cudaStream_t st) {
     const int n = full.nlayers, R = full.rb_start[n];
     int max_per = 0;
     for (int i = 0; i < n; ++i) max_per = max(max_per, p.pairs_per_cta[i]);
     const int tail = R % 148;                                   // CTAs of the last wave (cluster size 1)
-    if (!(p.ks == 1 && R > 148 && tail > 0 && 4 * tail <= 148 && max_per >= 16)) return launch_t1<LP>(full, p, st);
+    if (!(p.ks == 1 && R > 148 && tail > 0 && 4 * tail <= 148 && max_per >= 16)) return launch_t1<LP>(full, p, no_room, st);
 
     TxMulti part[2] = {};
     int rows_tail[TX_MAX_LAYERS], kb_tail[TX_MAX_LAYERS], src_tail[TX_MAX_LAYERS];
@@ -573,16 +659,16 @@ static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const in
         }
     }
     TxPlan pt;
-    if (!plan_t1(part[1].nlayers, rows_tail, kb_tail, LP, &pt)) return launch_t1<LP>(full, p, st);
+    if (!plan_t1(part[1].nlayers, rows_tail, kb_tail, LP, &pt)) return launch_t1<LP>(full, p, no_room, st);
     for (int j = 0; j < part[1].nlayers; ++j) {
         TxArgs &t = part[1].layer[j];
         t.pairs_per_cta = pt.pairs_per_cta[j];
         t.nastages = pt.nastages; t.nsstages = pt.nsstages; t.tmem_cols = pt.tmem_cols;
         (void)src_tail[j];
     }
-    mdbf_status_t rc = launch_t1<LP>(part[0], p, st);
+    mdbf_status_t rc = launch_t1<LP>(part[0], p, no_room, st);
     if (rc) return rc;
-    return launch_t1<LP>(part[1], pt, st);
+    return launch_t1<LP>(part[1], pt, no_room, st);
 }
 
 // Both stages of n layers that read the same x (n = 1: a single layer): one launch per stage.
@@ -591,7 +677,7 @@ static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const in
 // terms add to it, the last one adds and rounds into sum_y.
 template <int LP>
 static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st,
-                            float *sum_acc = nullptr, void *sum_y = nullptr, int stages = 3) {
+                            float *sum_acc = nullptr, void *sum_y = nullptr, int stages = 3, bool no_room = false) {
     int rowsB[TX_MAX_LAYERS], kbB[TX_MAX_LAYERS], rowsA[TX_MAX_LAYERS], kbA[TX_MAX_LAYERS];
     for (int i = 0; i < n; ++i) {
         rowsB[i] = Ls[i]->d.k; kbB[i] = Ls[i]->kbpB;
@@ -623,10 +709,10 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
         s.nastages = pa.nastages; s.nsstages = pa.nsstages; s.tmem_cols = pa.tmem_cols; s.status = L.status;
         ma.rb_start[i + 1] = ma.rb_start[i] + ceil_div(d.d_out, 128);
     }
-    mdbf_status_t rc = (stages & 1) ? launch_stage<LP>(mb, pb, kbB, st) : MDBF_OK;     // stages: bit 0 = stage B, bit 1 = stage A
+    mdbf_status_t rc = (stages & 1) ? launch_stage<LP>(mb, pb, kbB, &no_room, st) : MDBF_OK;     // stages: bit 0 = stage B, bit 1 = stage A
     if (rc) return rc;
     if (!(stages & 2)) return MDBF_OK;
-    if (!sum_acc) return launch_stage<LP>(ma, pa, kbA, st);
+    if (!sum_acc) return launch_stage<LP>(ma, pa, kbA, &no_room, st);
     for (int i = 0; i < n; ++i) {
         TxMulti one = {};
         one.nlayers = 1;
@@ -643,21 +729,22 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
         s.stage_a = n == 1 ? 1 : i == 0 ? 2 : i == n - 1 ? 4 : 3;
         s.pairs_per_cta = p1.pairs_per_cta[0];
         s.nastages = p1.nastages; s.nsstages = p1.nsstages; s.tmem_cols = p1.tmem_cols;
-        rc = launch_stage<LP>(one, p1, &kbA[i], st);
+        rc = launch_stage<LP>(one, p1, &kbA[i], &no_room, st);
         if (rc) return rc;
     }
     return MDBF_OK;
 }
 
-// n <= TX_MAX_LAYERS layers with the same LP, all prepared for the one-token kernel.
-mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st, int stages) {
+// n <= TX_MAX_LAYERS layers with the same LP, all prepared for the one-token kernel.  no_room: the launch before this call leaves no
+// room beside its CTAs (see TX_ALONE_DYN).
+mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st, int stages, bool no_room) {
     switch (Ls[0]->LP) {
-        case 1: return run_t1<1>(Ls, n, x, ys, st, nullptr, nullptr, stages);
-        case 2: return run_t1<2>(Ls, n, x, ys, st, nullptr, nullptr, stages);
-        case 4: return run_t1<4>(Ls, n, x, ys, st, nullptr, nullptr, stages);
-        case 8: return run_t1<8>(Ls, n, x, ys, st, nullptr, nullptr, stages);
-        case 16: return run_t1<16>(Ls, n, x, ys, st, nullptr, nullptr, stages);
-        case 32: return run_t1<32>(Ls, n, x, ys, st, nullptr, nullptr, stages);
+        case 1: return run_t1<1>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 2: return run_t1<2>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 4: return run_t1<4>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 8: return run_t1<8>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 16: return run_t1<16>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 32: return run_t1<32>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
         default:
             set_error("mdbf_linear_forward: the one-token TMEM kernel handles l <= 32 (got %d)", Ls[0]->d.l);
             return MDBF_ERR_SHAPE;

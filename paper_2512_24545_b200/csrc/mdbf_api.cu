@@ -439,11 +439,17 @@ static mdbf_status_t forward_t1_auto(Layer *const *Ls, int n, const void *x, voi
     const void *xs[kMaxSiblings];
     for (int i = 0; i < n; ++i) xs[i] = x;
     int nl = 0;
-    for (int s = 0; s < 2; ++s) {
-        mdbf_status_t rc;
-        if (i8_stages >> s & 1) { rc = launch_forward_t1_group(Ls, n, xs, ys, st, 1 << s); nl += 2; }
-        else { rc = launch_forward_tmem_t1_multi(Ls, n, x, ys, st, 1 << s); nl += last_t1_launch_count(); }
+    if (i8_stages == 0) {
+        mdbf_status_t rc = launch_forward_tmem_t1_multi(Ls, n, x, ys, st, 3);
         if (rc) return rc;
+        nl = last_t1_launch_count();
+    } else {
+        for (int s = 0; s < 2; ++s) {
+            mdbf_status_t rc;
+            if (i8_stages >> s & 1) { rc = launch_forward_t1_group(Ls, n, xs, ys, st, 1 << s); nl += 2; }
+            else { rc = launch_forward_tmem_t1_multi(Ls, n, x, ys, st, 1 << s, s == 1); nl += last_t1_launch_count(); }      // s == 1: after the integer kernel
+            if (rc) return rc;
+        }
     }
     *launches = nl;
     *kernel_used = i8_stages == 3 ? MDBF_KERNEL_I8 : MDBF_KERNEL_TMEM;

@@ -95,3 +95,40 @@ def test_bounded_wait_times_out_and_the_context_survives():
         assert M.mdbf_poll_status(g.h) == 0                        # reading cleared it
         assert rel_err(g.forward(x), g.oracle_forward(x)) <= TOL["bf16"]       # still works
         assert M.mdbf_poll_status(g.h) == 0
+
+
+def test_layers_queued_back_to_back():
+    """Consecutive launches share SMs and hand tensor memory over: layers of different stage sizes (few and many pairs of K
+    blocks per CTA, clusters of 1 to 8, the integer kernel in between) queued without a wait give what each gives alone."""
+    shapes = [(256, 640, 12800, 16), (4096, 1024, 512, 16), (300, 6400, 12800, 4), (1000, 2100, 1300, 32), (20000, 256, 700, 1),
+              (640, 640, 256, 2)]
+    specs = [spec_of(do, di, k, l) for do, di, k, l in shapes]
+    layers = [GpuLayer(sp, 1) for sp in specs]
+    try:
+        xs = [torch.from_numpy(inputs.make_activations(sp, 1)).to(torch.bfloat16).cuda() for sp in specs]
+        alone = []
+        st = torch.cuda.current_stream().cuda_stream
+        for kernel in (M.KERNEL_TMEM, M.KERNEL_I8):
+            for g, x in zip(layers, xs):
+                if kernel == M.KERNEL_I8 and g.spec.l > 16:
+                    continue
+                y = torch.zeros((1, g.spec.d_out), dtype=torch.bfloat16, device="cuda")
+                M.mdbf_set_kernel(g.h, kernel)
+                M.mdbf_linear_forward(g.h, x.data_ptr(), y.data_ptr(), 1, M.BF16, st)
+                torch.cuda.synchronize()
+                alone.append((g, x, kernel, y))
+        rng = np.random.default_rng(5)
+        for _ in range(4):
+            order = rng.permutation(len(alone))
+            out = [torch.zeros_like(alone[i][3]) for i in order]
+            for i, y in zip(order, out):
+                g, x, kernel, _ = alone[i]
+                M.mdbf_set_kernel(g.h, kernel)
+                M.mdbf_linear_forward(g.h, x.data_ptr(), y.data_ptr(), 1, M.BF16, st)
+            torch.cuda.synchronize()
+            for i, y in zip(order, out):
+                assert M.mdbf_poll_status(alone[i][0].h) == 0
+                assert torch.equal(y, alone[i][3]), alone[i][0].spec
+    finally:
+        for g in layers:
+            g.close()
