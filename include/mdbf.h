@@ -171,12 +171,12 @@ mdbf_status_t mdbf_linear_forward(mdbf_handle_t h, const void *x, void *y, int32
  * the paper's (l, P) sweep uses the same sum with MDBF terms).  Every term is evaluated by the same
  * kernels as mdbf_linear_forward with an fp32 output: term 1 stores into `acc`, the others add to
  * it, and one pass rounds `acc` to y - so y carries a single rounding whatever P is.  With one
- * token, bf16 activations and at most four terms of one envelope-rank bucket, the first stage of
- * all terms shares a launch and the last term's epilogue does the final add and rounding
- * (P + 1 launches instead of 2P + 1, same result).
+ * token, bf16 activations and at most four terms of one envelope-rank bucket, each stage of all terms
+ * shares a launch, and the second adds the terms and rounds (two launches instead of 2P + 1, same result;
+ * `acc` is then left as it was).
  *   terms  P handles of equal d_out and d_in (k, l and env_dtype may differ), all distinct
  *   x, y   device, T x d_in read, T x d_out written, of act_dtype
- *   acc    device, T x d_out float32 scratch owned by the caller, overwritten
+ *   acc    device, T x d_out float32 scratch owned by the caller, overwritten where it is used
  * Asynchronous on `stream`, allocates nothing.  Errors: INVALID_ARG, SHAPE, DTYPE, CUDA. */
 mdbf_status_t mdbf_linear_forward_sum(const mdbf_handle_t *terms, int32_t P, const void *x, void *y, float *acc,
                                       int32_t T, int32_t act_dtype, void *stream);

@@ -67,12 +67,10 @@ struct TxArgs {
     int env_dtype, l;
     const void *in;           // stage B: bf16 x [cols]; stage A: fp32 z [cols]
     void *out;                // stage B: fp32 z [rows]; stage A: bf16 y [rows]
-    void *out_final;          // stage A, mode 4: bf16 y [rows] that receives round(out[] + this term)
     int npairs_total;         // pairs of K blocks along the reduction
     int pairs_per_cta;        // pairs per cluster rank
     int nastages, nsstages, tmem_cols;
-    int stage_a;              // 0: stage B (bf16 in, fp32 out); stage A (fp32 in): 1 bf16 out, 2 fp32 out, 3 added to fp32 out,
-                              // 4 last term of a sum: out_final = bf16(fp32 out + this term)
+    int stage_a;              // 0: stage B (bf16 in, fp32 out); stage A (fp32 in): 1 bf16 out, 2 fp32 out, 3 added to fp32 out
     int32_t *status;
 };
 
@@ -84,6 +82,7 @@ struct TxMulti {
     TxArgs layer[TX_MAX_LAYERS];
     int rb_start[TX_MAX_LAYERS + 1];   // first row block of each layer; rb_start[nlayers] = gridDim.x
     int nlayers;
+    int sum_ks;                        // > 0: the layers are terms of one sum, each with this many ranks in the cluster of a row block
 };
 
 // Cluster barrier in two halves.  The relaxed arrive orders no memory: it only says that this CTA runs.
@@ -100,10 +99,11 @@ __device__ __forceinline__ bool tx_wait(uint32_t bar, uint32_t parity, volatile 
 // Shared-memory plan (dynamic, 1024-byte aligned):
 //   vring [nastages][2 * NB * 128 B]   V tile images of a pair (B operand)
 //   sring [nsstages][2048 B]           packed sign words of a pair: [2][128 rows] uint2
-//   xp    [pairs_per_cta * 64] u32     activation pairs in MMA k order (bf16x2)
 //   part  [8][128] float               partial outputs pushed by the other cluster ranks (rank 0 only reads)
-template <int LP, int TX_GROUPS, bool SUM_LAST = false>
-__device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
+//   xp    [pairs_per_cta * 64] u32     activation pairs in MMA k order (bf16x2)
+// slice: which of its layer's shares of the reduction this CTA takes
+template <int LP, int TX_GROUPS>
+__device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, const int slice) {
     using namespace tm;
     constexpr int TX_EXPANDERS = TX_GROUPS * 128;
     constexpr int TX_W_ISSUER0 = TX_EXPANDERS / 32;
@@ -122,8 +122,8 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
     unsigned char *smem_gen = tx_smem_raw + (smem_base - smem_u32(tx_smem_raw));
     const int nas = a.nastages, nss = a.nsstages;
     const uint32_t off_s = (uint32_t)(nas * VBYTES);
-    const uint32_t off_x = off_s + (uint32_t)(nss * 2048);
-    const uint32_t off_p = off_x + (uint32_t)(a.pairs_per_cta * 256);
+    const uint32_t off_p = off_s + (uint32_t)(nss * 2048);   // before xp, whose size may differ between the ranks of a sum
+    const uint32_t off_x = off_p + 4096u;
     uint32_t *xp = reinterpret_cast<uint32_t *>(smem_gen + off_x);
     float *part = reinterpret_cast<float *>(smem_gen + off_p);
 
@@ -133,7 +133,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
                    a_full = smem_u32(&bars[NB2]), a_empty = smem_u32(&bars[NB3]), acc_bar = smem_u32(&bars[NB4]);
 
     const int row0 = rb * 128;
-    const int pr0 = blockIdx.y * a.pairs_per_cta;
+    const int pr0 = slice * a.pairs_per_cta;
     const int npr = max(0, min(a.pairs_per_cta, a.npairs_total - pr0));
 
     if (tid <= NB4) {       // s_full 1, s_empty 4, v_full 1, a_full 4, a_empty 1, acc_bar TX_ISSUERS
@@ -432,8 +432,6 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
         if (grow < a.rows && !*abort_flag && store_in_bounds((size_t)grow, (size_t)a.rows, a.status)) {
             if (a.stage_a == 1) reinterpret_cast<__nv_bfloat16 *>(a.out)[grow] = __float2bfloat16_rn(outv);
             else if (a.stage_a == 3) reinterpret_cast<float *>(a.out)[grow] += outv;      // a further term of a sum of layers
-            else if (SUM_LAST && a.stage_a == 4)                                           // its last term: one rounding of the whole sum
-                reinterpret_cast<__nv_bfloat16 *>(a.out_final)[grow] = __float2bfloat16_rn(reinterpret_cast<const float *>(a.out)[grow] + outv);
             else reinterpret_cast<float *>(a.out)[grow] = outv;
         }
     }
@@ -446,14 +444,17 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb) {
 // One layer per launch: the arguments are plain kernel parameters (fastest for the small layers).
 template <int LP, int G>
 __global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_kernel(const TxArgs a) {
-    tmem_t1_body<LP, G>(a, (int)blockIdx.x + a.rb0);
+    tmem_t1_body<LP, G>(a, (int)blockIdx.x + a.rb0, (int)blockIdx.y);
 }
 
-// The last term of a sum of layers (mode 4 of the epilogue), an instantiation of its own so that the plain kernel
-// carries no trace of it.
+// Stage A of the terms of a sum in one launch: the cluster of a row block holds the ranks of every term, and its reduction adds
+// them all, so y is rounded once and no fp32 sum goes through memory (two 4096 x 4096 terms, k = 896, l = 1, calls back to back:
+// one launch per term 15.5 us, this 12.1 us, most of both on the host).
 template <int LP, int G>
-__global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_sumlast_kernel(const TxArgs a) {
-    tmem_t1_body<LP, G, true>(a, (int)blockIdx.x + a.rb0);
+__global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_sum_kernel(const __grid_constant__ TxMulti m) {
+    const int term = (int)blockIdx.y / m.sum_ks;
+    const TxArgs a = m.layer[term];
+    tmem_t1_body<LP, G>(a, (int)blockIdx.x, (int)blockIdx.y - term * m.sum_ks);
 }
 
 // Several sibling layers per launch: each CTA picks its layer by its position in the grid.
@@ -464,7 +465,7 @@ __global__ void __launch_bounds__(tx_threads(G), tx_ctas(G)) tmem_t1_multi_kerne
     for (int i = 1; i < TX_MAX_LAYERS; ++i)
         if (i < m.nlayers && (int)blockIdx.x >= m.rb_start[i]) li = i;
     const TxArgs a = m.layer[li];                             // by value: one indexed read of the parameter block
-    tmem_t1_body<LP, G>(a, (int)blockIdx.x - m.rb_start[li] + a.rb0);
+    tmem_t1_body<LP, G>(a, (int)blockIdx.x - m.rb_start[li] + a.rb0, (int)blockIdx.y);
 }
 
 // ----------------------------------------------------------- pack-time private copies
@@ -551,17 +552,19 @@ constexpr int TX_CARVEOUT = 58;
 
 // One plan for all the layers of a launch.  Cluster size along the reduction: one CTA per SM (all of
 // TMEM), as few waves as possible, the per-CTA fixed part weighed against its share of the reduction.
-static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p) {
+// terms > 1: the n layers are the terms of a sum, whose ranks share the cluster of a row block (p->ks: all of them).
+static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p, int terms = 1) {
     const int NB = LP < 16 ? 16 : LP;
     int nas = (512 - TX_ISSUERS * NB) / 64;
     if (nas > TX_MAX_ASTAGES) nas = TX_MAX_ASTAGES;
-    const int max_ks = 8;                                     // portable cluster size
+    const int max_ks = 8 / terms;                             // portable cluster size
     int rb = 0, max_pairs = 0, min_pairs = 1 << 30;
     for (int i = 0; i < n; ++i) {
         rb += ceil_div(rows[i], 128);
         max_pairs = max(max_pairs, kb_pad[i] / 2);
         min_pairs = min(min_pairs, kb_pad[i] / 2);
     }
+    if (terms > 1) rb = ceil_div(rows[0], 128) * terms;
     long best_cost = -1;
     int best_ks = 1;
     for (int ks = 1; ks <= max_ks; ks *= 2) {
@@ -570,7 +573,7 @@ static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p
         const long cost = waves * (2 * ceil_div(max_pairs, ks) + fixed_cost());
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_ks = ks; }
     }
-    p->ks = best_ks;
+    p->ks = best_ks * terms;
     int max_per = 1;
     for (int i = 0; i < n; ++i) {
         p->pairs_per_cta[i] = ceil_div(kb_pad[i] / 2, best_ks);
@@ -594,8 +597,8 @@ static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, bool alone, c
         if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
         MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
         if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
-        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sumlast_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
-        if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sumlast_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
+        MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sum_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
+        if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_sum_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(m.rb_start[m.nlayers], p.ks, 1);
@@ -611,7 +614,7 @@ static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, bool alone, c
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    if (m.nlayers == 1 && m.layer[0].stage_a == 4) MDBF_CUDA(cudaLaunchKernelEx(&cfg, tmem_t1_sumlast_kernel<LP, G>, m.layer[0]));
+    if (m.sum_ks) MDBF_CUDA(cudaLaunchKernelEx(&cfg, tmem_t1_sum_kernel<LP, G>, m));
     else if (m.nlayers == 1) MDBF_CUDA(cudaLaunchKernelEx(&cfg, tmem_t1_kernel<LP, G>, m.layer[0]));
     else MDBF_CUDA(cudaLaunchKernelEx(&cfg, tmem_t1_multi_kernel<LP, G>, m));
     ++g_t1_launches;
@@ -672,12 +675,11 @@ static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const in
 }
 
 // Both stages of n layers that read the same x (n = 1: a single layer): one launch per stage.
-// sum != nullptr: the n layers are the terms of a sum; stage B of all terms shares one launch (they read the
-// same x), the stage-A launches follow one another: term 0 stores its fp32 output into sum_acc, the middle
-// terms add to it, the last one adds and rounds into sum_y.
+// sum_y != nullptr: the n layers are the terms of a sum; stage B of all terms shares one launch (they read the same x), stage A of
+// all terms another (tmem_t1_sum_kernel).
 template <int LP>
 static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st,
-                            float *sum_acc = nullptr, void *sum_y = nullptr, int stages = 3, bool no_room = false) {
+                            void *sum_y = nullptr, int stages = 3, bool no_room = false) {
     int rowsB[TX_MAX_LAYERS], kbB[TX_MAX_LAYERS], rowsA[TX_MAX_LAYERS], kbA[TX_MAX_LAYERS];
     for (int i = 0; i < n; ++i) {
         rowsB[i] = Ls[i]->d.k; kbB[i] = Ls[i]->kbpB;
@@ -704,7 +706,7 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
         TxArgs &s = ma.layer[i];
         s.wk2 = L.wk2A; s.kb_pad = L.kbpA; s.rows = d.d_out; s.cols = d.k;
         s.vtile = L.vxA; s.U = L.UA; s.env_dtype = d.env_dtype; s.l = d.l;
-        s.in = L.zsum; s.out = ys[i]; s.out_final = nullptr; s.stage_a = 1 + L.out_mode;
+        s.in = L.zsum; s.out = ys[i]; s.stage_a = 1 + L.out_mode;
         s.npairs_total = L.kbpA / 2; s.pairs_per_cta = pa.pairs_per_cta[i];
         s.nastages = pa.nastages; s.nsstages = pa.nsstages; s.tmem_cols = pa.tmem_cols; s.status = L.status;
         ma.rb_start[i + 1] = ma.rb_start[i] + ceil_div(d.d_out, 128);
@@ -712,39 +714,37 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
     mdbf_status_t rc = (stages & 1) ? launch_stage<LP>(mb, pb, kbB, &no_room, st) : MDBF_OK;     // stages: bit 0 = stage B, bit 1 = stage A
     if (rc) return rc;
     if (!(stages & 2)) return MDBF_OK;
-    if (!sum_acc) return launch_stage<LP>(ma, pa, kbA, &no_room, st);
-    for (int i = 0; i < n; ++i) {
-        TxMulti one = {};
-        one.nlayers = 1;
-        one.rb_start[1] = ceil_div(rowsA[i], 128);
-        TxPlan p1;
-        if (!plan_t1(1, &rowsA[i], &kbA[i], LP, &p1)) {
-            set_error("mdbf_linear_forward_sum: the one-token TMEM kernel does not fit this shape");
-            return MDBF_ERR_SHAPE;
-        }
-        TxArgs &s = one.layer[0];
-        s = ma.layer[i];
-        s.out = n == 1 ? sum_y : (void *)sum_acc;
-        s.out_final = sum_y;
-        s.stage_a = n == 1 ? 1 : i == 0 ? 2 : i == n - 1 ? 4 : 3;
-        s.pairs_per_cta = p1.pairs_per_cta[0];
-        s.nastages = p1.nastages; s.nsstages = p1.nsstages; s.tmem_cols = p1.tmem_cols;
-        rc = launch_stage<LP>(one, p1, &kbA[i], &no_room, st);
-        if (rc) return rc;
+    if (!sum_y) return launch_stage<LP>(ma, pa, kbA, &no_room, st);
+    // the terms of a sum: one launch, all of them rounded into y together
+    TxMulti sum = ma;
+    TxPlan ps;
+    if (!plan_t1(n, rowsA, kbA, LP, &ps, n)) {
+        set_error("mdbf_linear_forward_sum: the one-token TMEM kernel does not fit this shape");
+        return MDBF_ERR_SHAPE;
     }
-    return MDBF_OK;
+    sum.sum_ks = ps.ks / n;
+    sum.nlayers = n;
+    sum.rb_start[n] = ceil_div(rowsA[0], 128);
+    for (int i = 0; i < n; ++i) {
+        TxArgs &s = sum.layer[i];
+        s.out = sum_y;
+        s.stage_a = 1;
+        s.pairs_per_cta = ps.pairs_per_cta[i];
+        s.nastages = ps.nastages; s.nsstages = ps.nsstages; s.tmem_cols = ps.tmem_cols;
+    }
+    return launch_t1<LP>(sum, ps, &no_room, st);
 }
 
 // n <= TX_MAX_LAYERS layers with the same LP, all prepared for the one-token kernel.  no_room: the launch before this call leaves no
 // room beside its CTAs (see TX_ALONE_DYN).
 mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st, int stages, bool no_room) {
     switch (Ls[0]->LP) {
-        case 1: return run_t1<1>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
-        case 2: return run_t1<2>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
-        case 4: return run_t1<4>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
-        case 8: return run_t1<8>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
-        case 16: return run_t1<16>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
-        case 32: return run_t1<32>(Ls, n, x, ys, st, nullptr, nullptr, stages, no_room);
+        case 1: return run_t1<1>(Ls, n, x, ys, st, nullptr, stages, no_room);
+        case 2: return run_t1<2>(Ls, n, x, ys, st, nullptr, stages, no_room);
+        case 4: return run_t1<4>(Ls, n, x, ys, st, nullptr, stages, no_room);
+        case 8: return run_t1<8>(Ls, n, x, ys, st, nullptr, stages, no_room);
+        case 16: return run_t1<16>(Ls, n, x, ys, st, nullptr, stages, no_room);
+        case 32: return run_t1<32>(Ls, n, x, ys, st, nullptr, stages, no_room);
         default:
             set_error("mdbf_linear_forward: the one-token TMEM kernel handles l <= 32 (got %d)", Ls[0]->d.l);
             return MDBF_ERR_SHAPE;
@@ -752,15 +752,15 @@ mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *
 }
 
 // The terms of a sum of layers (same LP, at most TX_MAX_LAYERS) at one token: y = bf16(sum of the terms' outputs).
-mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, float *acc, void *y, cudaStream_t st) {
+mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, void *y, cudaStream_t st) {
     void *ys[TX_MAX_LAYERS] = {};
     switch (Ls[0]->LP) {
-        case 1: return run_t1<1>(Ls, n, x, ys, st, acc, y);
-        case 2: return run_t1<2>(Ls, n, x, ys, st, acc, y);
-        case 4: return run_t1<4>(Ls, n, x, ys, st, acc, y);
-        case 8: return run_t1<8>(Ls, n, x, ys, st, acc, y);
-        case 16: return run_t1<16>(Ls, n, x, ys, st, acc, y);
-        case 32: return run_t1<32>(Ls, n, x, ys, st, acc, y);
+        case 1: return run_t1<1>(Ls, n, x, ys, st, y);
+        case 2: return run_t1<2>(Ls, n, x, ys, st, y);
+        case 4: return run_t1<4>(Ls, n, x, ys, st, y);
+        case 8: return run_t1<8>(Ls, n, x, ys, st, y);
+        case 16: return run_t1<16>(Ls, n, x, ys, st, y);
+        case 32: return run_t1<32>(Ls, n, x, ys, st, y);
         default:
             set_error("mdbf_linear_forward_sum: the one-token TMEM kernel handles l <= 32 (got %d)", Ls[0]->d.l);
             return MDBF_ERR_SHAPE;

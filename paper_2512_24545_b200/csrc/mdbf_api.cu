@@ -549,8 +549,7 @@ mdbf_status_t mdbf_linear_forward_sum(const mdbf_handle_t *terms, int32_t P, con
     }
     cudaStream_t st = (cudaStream_t)stream;
     // One token, bf16, every term ready for the one-token kernel with the same envelope-rank bucket: stage B of
-    // all terms shares a launch, the last term's stage-A epilogue adds the fp32 sum of the others and rounds
-    // into y (P + 1 launches, no cast pass).
+    // all terms shares a launch, stage A of all terms another, which adds them and rounds into y (acc stays untouched).
     bool fused = T == 1 && act_dtype == MDBF_BF16 && P <= kMaxSiblings;
     for (int p = 0; p < P && fused; ++p) {
         const Layer &L = terms[p]->L;
@@ -566,7 +565,7 @@ mdbf_status_t mdbf_linear_forward_sum(const mdbf_handle_t *terms, int32_t P, con
             terms[p]->last_kernel = MDBF_KERNEL_TMEM;
             terms[p]->last_launches = 0;
         }
-        mdbf_status_t rc = launch_forward_tmem_t1_sum(Ls, P, x, acc, y, st);
+        mdbf_status_t rc = launch_forward_tmem_t1_sum(Ls, P, x, y, st);
         if (rc) return rc;
         terms[0]->last_launches = last_t1_launch_count();
         return MDBF_OK;

@@ -78,6 +78,16 @@ def test_terms_of_one_envelope_rank_at_one_token(P):
         np.testing.assert_array_equal(y, singles[0])
 
 
+@pytest.mark.parametrize("ks,l", [([2100, 130], 16), ([1100, 1400, 1025], 4), ([300, 1030, 64, 900], 1)])
+def test_terms_share_the_cluster_of_a_row_block(ks, l):
+    """One second-stage launch for all terms: clusters of several ranks per term, terms of different lengths."""
+    specs = term_specs(520, 384, ks, [l] * len(ks))
+    x = inputs.make_activations(specs[0], 1)
+    y, ref, _ = run_sum(specs, x)
+    assert np.all(np.isfinite(y))
+    assert rel_err(y, ref) <= TOL["bf16"]
+
+
 def test_fp32_terms_and_single_term():
     t = inputs.tiny()
     specs = [inputs.scaled(t, name="a", seed=1), inputs.scaled(t, name="b", seed=2, env_std=t.env_std * 0.5)]
