@@ -211,7 +211,8 @@ mdbf_status_t mdbf_prepare_host_staging(mdbf_handle_t h);
 
 /* Same computation with HOST buffers: copies x to the handle's device staging buffer, runs the
  * forward, copies y back, all on `stream`, and synchronises the stream before returning.  x_host /
- * y_host should be pinned for full copy bandwidth.  Needs mdbf_prepare_host_staging once per handle
+ * y_host should be pinned for full copy bandwidth (small pinned buffers are read and written by kernels, without the copy
+ * engine).  Needs mdbf_prepare_host_staging once per handle
  * (MDBF_ERR_INVALID_ARG otherwise). */
 mdbf_status_t mdbf_linear_forward_host(mdbf_handle_t h, const void *x_host, void *y_host, int32_t T,
                                        int32_t act_dtype, void *stream);
