@@ -28,6 +28,8 @@
 //              frees the TMEM slot, one the pair of activation tiles
 //   warp 18    one lane bulk-copies the envelope images (U once, V per pair, ring of 3 or 4)
 //   warp 19    one lane issues the mini-MMA of a pair (U image x V image, 128 columns, no swizzle)
+// Few row blocks and tokens leave SMs idle: then the reduction of a tile is split over a cluster of up to eight CTAs (SPLIT), each
+// running the same pipeline over its pairs, and the accumulators are added by token through distributed shared memory.
 // Shared memory holds only activation tiles (ring of 6 at 256 tokens per tile: the L2 latency of a
 // 32 KB tile is about one pair of MMA time, so the ring must run two pairs ahead) and the images.
 // TMEM: 256 accumulator + 128 envelope + 2 x 64 W_hat columns.
@@ -145,7 +147,7 @@ __device__ __forceinline__ bool mt_wait3(uint32_t bar_a, uint32_t par_a, uint32_
     return true;
 }
 
-template <bool STAGE_A>
+template <bool STAGE_A, bool SPLIT>
 __global__ void __launch_bounds__(MT_THREADS, 1)
 mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_out) {
     using namespace tm;
@@ -177,7 +179,11 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
     const int rb = blockIdx.x;
     const int row0 = rb * MT_BM;
     const int tau0 = blockIdx.y * a.bn;
-    const int nkb = (a.cols + MT_BK - 1) / MT_BK;
+    cg::cluster_group cluster = cg::this_cluster();
+    const unsigned crank = SPLIT ? cluster.block_rank() : 0u;
+    const int nkb_total = (a.cols + MT_BK - 1) / MT_BK;
+    const int kb0 = SPLIT ? (int)crank * 2 * a.ppc : 0;             // this rank's share of the reduction
+    const int nkb = SPLIT ? max(0, min(2 * a.ppc, nkb_total - kb0)) : nkb_total;
     const int npr = (nkb + 1) / 2;                                  // pairs of K blocks; the last one may hold one block
 
     if (tid == 0) {
@@ -217,7 +223,7 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
         const int arow = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const size_t wstride = 2 * MT_BM;                                  // 32-bit words from one K block to the next
-        const uint32_t *wp = reinterpret_cast<const uint32_t *>(a.wk2 + (size_t)rb * a.kb_pad * MT_BM + arow) + half;   // + kb * wstride
+        const uint32_t *wp = reinterpret_cast<const uint32_t *>(a.wk2 + ((size_t)rb * a.kb_pad + kb0) * MT_BM + arow) + half;   // + kb * wstride
         uint32_t w_next = grp < nkb ? __ldg(wp + (size_t)grp * wstride) : 0u;
         uint32_t w_next2 = grp + 2 < nkb ? __ldg(wp + (size_t)(grp + 2) * wstride) : 0u;
         bool alive = true;
@@ -265,7 +271,57 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
         // wait that expired in any thread has raised the abort flag before that thread arrived
         asm volatile("bar.sync %0, 128;\n" ::"r"(1 + (warp >> 2)) : "memory");
         alive = !*abort_flag;
-        if (alive && a.tma_out) {
+        if (SPLIT) {
+            // Partial sums reduce-scattered by token through distributed shared memory: rank r adds and stores the tokens
+            // [r tpr, (r + 1) tpr), tpr a multiple of 32.  The first barrier says that every rank's MMAs have retired, i.e. that the
+            // activation rings, which the sums go into, are idle; the second that the sums have arrived.  Both are passed on
+            // every path.
+            float *part = reinterpret_cast<float *>(smem_gen);           // [rank][tpr][128 rows]
+            cluster.sync();
+            if (alive) {
+                for (int ld = warp >> 2; ld * 32 < a.bn; ld += MT_XWARPS / 4) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem_d + lane_base + (uint32_t)(ld * 32), v);
+                    tmem_ld_wait();
+                    const int owner = ld * 32 / a.tpr;
+                    float *dst = cluster.map_shared_rank(part, owner) + ((int)crank * a.tpr + ld * 32 - owner * a.tpr) * MT_BM + arow;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) dst[j * MT_BM] = nkb > 0 ? __uint_as_float(v[j]) : 0.f;
+                }
+            }
+            tc_fence_before();
+            cluster.sync();
+            if (alive && !*abort_flag) {
+                // a warp per token, four rows per lane
+                const int nranks = (int)cluster.num_blocks();
+                const int r4 = row0 + 4 * lane, pitch = STAGE_A ? a.rows : a.zstride;
+                __nv_bfloat16 *out16 = STAGE_A ? a.y : a.zb;
+                const bool whole = (!STAGE_A || a.y_mode == 0) && r4 + 4 <= a.rows && (pitch & 3) == 0 && (reinterpret_cast<uintptr_t>(out16) & 7u) == 0;
+                for (int slot = warp; slot < a.tpr; slot += MT_XWARPS) {
+                    const int t = (int)crank * a.tpr + slot, tau = tau0 + t;
+                    if (t >= a.bn || tau >= a.T) break;
+                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int rk = 0; rk < nranks; ++rk) {
+                        const float4 q = *reinterpret_cast<const float4 *>(part + (rk * a.tpr + slot) * MT_BM + 4 * lane);
+                        sum.x += q.x; sum.y += q.y; sum.z += q.z; sum.w += q.w;
+                    }
+                    const size_t o = (size_t)tau * pitch + r4;
+                    if (whole) {
+                        if (store_in_bounds(o + 3, (size_t)a.T * pitch, a.status))
+                            *reinterpret_cast<uint2 *>(out16 + o) = make_uint2(pack_bf16x2(sum.x, sum.y), pack_bf16x2(sum.z, sum.w));
+                    } else {
+                        const float e4[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            if (r4 + e >= a.rows || !store_in_bounds(o + e, (size_t)a.T * pitch, a.status)) continue;
+                            if (!STAGE_A || a.y_mode == 0) out16[o + e] = __float2bfloat16_rn(e4[e]);
+                            else if (a.y_mode == 1) a.y32[o + e] = e4[e];
+                            else a.y32[o + e] += e4[e];
+                        }
+                    }
+                }
+            }
+        } else if (alive && a.tma_out) {
             // The four warps of group g = warp / 4 cover all 128 rows; they take tokens [64g, 64g + 64): accumulator ->
             // bf16 [token][128 rows] in the (now idle) activation ring -> one TMA store per group, which clips
             // rows and tokens outside the output.
@@ -330,7 +386,7 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
                 for (int h = 0; h < 2 && 2 * p + h < nkb; ++h) {
                     const int s = 2 * bp + h;
                     mbar_arrive_expect_tx(bfull_bar + 8 * s, b_bytes);
-                    tma_load_2d(smem_base + (uint32_t)s * b_bytes, &tmap_in, (2 * p + h) * MT_BK, tau0, bfull_bar + 8 * s);
+                    tma_load_2d(smem_base + (uint32_t)s * b_bytes, &tmap_in, (kb0 + 2 * p + h) * MT_BK, tau0, bfull_bar + 8 * s);
                 }
                 if (++bp == nbp) { bp = 0; ph ^= 1u; }
             }
@@ -349,7 +405,7 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
                 alive = mbar_wait(vempty_bar + 8 * vb, vph ^ 1u, abort_flag, a.status);
                 if (!alive) break;
                 mbar_arrive_expect_tx(vfull_bar + 8 * vb, img_bytes);
-                bulk_load(v_smem + (uint32_t)vb * img_bytes, a.vimg + (size_t)p * (img_bytes / 2), img_bytes, vfull_bar + 8 * vb);
+                bulk_load(v_smem + (uint32_t)vb * img_bytes, a.vimg + (size_t)(kb0 / 2 + p) * (img_bytes / 2), img_bytes, vfull_bar + 8 * vb);
                 if (++vb == nv) { vb = 0; vph ^= 1u; }
             }
             if (!alive) drain_delay();
@@ -411,6 +467,10 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
         __syncwarp();
     }
 
+    if (SPLIT && warp >= MT_W_TMA) {                    // the builder warps run these barriers inside their epilogue
+        cluster.sync();
+        cluster.sync();
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == MT_W_MMA) tmem_dealloc(tmem_d, MT_TMEM_COLS);
@@ -747,6 +807,66 @@ static int mt_ring(int kc, int nv, int bn, size_t part_bytes) {
 static size_t mt_smem_bytes(int kc, int nv, int bn, size_t part_bytes) {
     return (size_t)mt_ring(kc, nv, bn, part_bytes) * bn * MT_BK * 2 + (size_t)(1 + nv) * kc * 2048 + part_bytes + 1024;
 }
+// Tokens that a rank of a split large tile adds up (whole 32-column chunks), and whether the ranks' sums fit into the activation
+// ring they are pushed into: at 208 tokens, say, five ranks or more would run past it.
+static int mt_tpr(int bn, int ks) { return ceil_div(ceil_div(bn, ks), 32) * 32; }
+static bool mt_split_fits(int kc, int nv, int bn, int ks) {
+    return (size_t)ks * mt_tpr(bn, ks) * MT_BM * sizeof(float) <= (size_t)mt_ring(kc, nv, bn, 0) * bn * MT_BK * 2;
+}
+// CTAs of the split kernel that run at once in clusters of `ks` (one CTA per SM; the SMs of a graphics processing cluster that a cluster size does
+// not divide stay idle: 148 at one rank, 128 or fewer at eight).  Asked of the runtime once per device and size.
+static int mt_resident(int ks) {
+    static int known[64][9] = {};
+    int dev = 0;
+    if (ks == 1) return 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 128 / ks * ks;
+    if (!known[dev][ks]) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = ks;
+        cfg.gridDim = dim3(1, 1, ks);
+        cfg.blockDim = dim3(MT_THREADS);
+        cfg.dynamicSmemBytes = mt_smem_bytes(2, 4, MT_BN, 0);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(mat_stage_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mt_smem_bytes(4, 3, MT_BN, 0)) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, mat_stage_kernel<true, true>, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            n = 128 / ks;
+        }
+        known[dev][ks] = n * ks;
+    }
+    return known[dev][ks];
+}
+// Token tile and ranks along the reduction of one stage with more than 64 tokens: the least estimated time over waves of 148 CTAs.
+// A pair of K blocks costs 0.41 us + 0.16 us per 256 tokens (the issuing threads, then the tensor pipe), a CTA's set-up and
+// epilogue 4 us + 2 us per 256 tokens, a split another 2.4 us per 256 tokens and 0.3 us per rank (fitted to a sweep; in units of 10 ns).  Several
+// token tiles are multiples of 64 tokens, the boxes of the output's tensor map.
+// Measured, us per forward, unsplit 256-token tiles -> the plan's: 4096 x 4096, k = 1664, T = 777: 41.4 -> 32.5 (stage B: 52 CTAs of
+// 32 pairs -> 130 of 16); 1024 x 8192, k = 512, T = 2048: 53.5 -> 28.4; 8192 x 8192, k = 3712, T = 100: 65.4 -> 33.2;
+// 8192 x 8192, T = 2048 (232 CTAs) stays whole: 197, two ranks 215.
+static void plan_mat(int rows, int cols, int T, int kc, int nv, int *bn_out, int *ks_out) {
+    const int rb = ceil_div(rows, MT_BM), npr = ceil_div(ceil_div(cols, MT_BK), 2);
+    const int one = ceil_div(T, 16) * 16;
+    const int cand[4] = {T <= MT_BN ? one : 256, T <= MT_BN ? 0 : 192, 128, 0};
+    long best = -1;
+    *bn_out = cand[0]; *ks_out = 1;
+    if (T <= MS_BN) return;                                // the small-tile kernel plans its own split
+    for (int bn : cand) {
+        if (bn == 0 || (bn < T && bn % 64 != 0) || (bn == 128 && T <= 128 && one != 128)) continue;
+        for (int ks = 1; ks <= 8; ++ks) {
+            const int per = ceil_div(npr, ks);
+            if (ks > 1 && (per * (ks - 1) >= npr || !mt_split_fits(kc, nv, bn, ks))) continue;
+            const long waves = ceil_div(rb * ceil_div(T, bn) * ks, mt_resident(ks));
+            const long cost = waves * ((long)per * (41 + bn / 16) + 400 + bn * 25 / 32 + (ks > 1 ? bn * 15 / 16 + 30 * ks : 0));
+            if (best < 0 || cost < best) { best = cost; *bn_out = bn; *ks_out = ks; }
+        }
+    }
+}
 // Tensor map of a bf16 output [T][rows] with rows `pitch` elements apart: box of 128 rows x 64 tokens, no swizzle.
 static mdbf_status_t make_out_tensor_map(CUtensorMap *out, const void *base, int T, int rows, int pitch) {
     typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -778,11 +898,12 @@ static mdbf_status_t make_out_tensor_map(CUtensorMap *out, const void *base, int
 }
 
 template <bool STAGE_A>
-static mdbf_status_t launch_mat(const MatArgs &a0, const CUtensorMap &tm, const CUtensorMap &tmo, cudaStream_t st) {
+static mdbf_status_t launch_mat(const MatArgs &a0, int large_ks, const CUtensorMap &tm, const CUtensorMap &tmo, cudaStream_t st) {
     static PerDeviceOnce once;
     if (once.first()) {
         const int max_smem = (int)mt_smem_bytes(4, 3, MT_BN, 0);
-        MDBF_CUDA(cudaFuncSetAttribute(mat_stage_kernel<STAGE_A>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+        MDBF_CUDA(cudaFuncSetAttribute(mat_stage_kernel<STAGE_A, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+        MDBF_CUDA(cudaFuncSetAttribute(mat_stage_kernel<STAGE_A, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
         MDBF_CUDA(cudaFuncSetAttribute(mat_small_kernel<STAGE_A, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
         MDBF_CUDA(cudaFuncSetAttribute(mat_small_kernel<STAGE_A, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
     }
@@ -803,11 +924,15 @@ static mdbf_status_t launch_mat(const MatArgs &a0, const CUtensorMap &tm, const 
             if (best < 0 || cost < best) { best = cost; ks = c; }
         }
     }
+    if (!small) {
+        ks = large_ks;
+        if (ks > 1 && !mt_split_fits(a.kc, a.nv, a.bn, ks)) { set_error("materialised-envelope kernel: %d ranks do not fit tiles of %d tokens", ks, a.bn); return MDBF_ERR_SHAPE; }
+    }
     size_t part_bytes = 0;
     if (ks > 1) {
         a.ppc = ceil_div(npr, ks);
-        a.tpr = ceil_div(a.bn, ks);
-        part_bytes = (size_t)ks * a.tpr * MT_BM * sizeof(float);
+        a.tpr = small ? ceil_div(a.bn, ks) : mt_tpr(a.bn, ks);
+        if (small) part_bytes = (size_t)ks * a.tpr * MT_BM * sizeof(float);       // (the large tiles put them into the activation ring)
     }
     a.ns = mt_ring(a.kc, a.nv, a.bn, part_bytes);
     cudaLaunchConfig_t cfg = {};
@@ -824,7 +949,8 @@ static mdbf_status_t launch_mat(const MatArgs &a0, const CUtensorMap &tm, const 
     attr[1].val.clusterDim.z = ks;
     cfg.attrs = attr;
     cfg.numAttrs = ks > 1 ? 2 : 1;
-    if (!small) MDBF_CUDA(cudaLaunchKernelEx(&cfg, mat_stage_kernel<STAGE_A>, a, tm, tmo));
+    if (!small && ks > 1) MDBF_CUDA(cudaLaunchKernelEx(&cfg, mat_stage_kernel<STAGE_A, true>, a, tm, tmo));
+    else if (!small) MDBF_CUDA(cudaLaunchKernelEx(&cfg, mat_stage_kernel<STAGE_A, false>, a, tm, tmo));
     else if (ks > 1) MDBF_CUDA(cudaLaunchKernelEx(&cfg, mat_small_kernel<STAGE_A, true>, a, tm));
     else MDBF_CUDA(cudaLaunchKernelEx(&cfg, mat_small_kernel<STAGE_A, false>, a, tm));
     return MDBF_OK;
@@ -837,7 +963,10 @@ mdbf_status_t launch_forward_mat(Layer &L, const void *x, void *y, int T, cudaSt
                   "l <= 32, d_in a multiple of 8 and x aligned to 16 bytes");
         return MDBF_ERR_SHAPE;
     }
-    const int bn = T >= MT_BN ? MT_BN : ((T + 15) / 16) * 16;
+    int bnB, ksB, bnA, ksA;                               // token tile and ranks along the reduction of each stage
+    const int nv = L.kcm == 2 ? 4 : 3;
+    plan_mat(d.k, d.d_in, T, L.kcm, nv, &bnB, &ksB);
+    plan_mat(d.d_out, d.k, T, L.kcm, nv, &bnA, &ksA);
     // y goes out by TMA when its base and row pitch are 16-byte aligned and it is bf16; otherwise by plain stores.
     // Small tiles (T <= 64) always use plain stores and need no output maps.
     const bool small = T <= MS_BN;
@@ -848,9 +977,9 @@ mdbf_status_t launch_forward_mat(Layer &L, const void *x, void *y, int T, cudaSt
     mdbf_status_t rc;
     if (!(m.valid && m.x == x && m.T == T)) {
         m.valid = false;
-        rc = make_act_tensor_map(&m.tmx, x, (size_t)T, d.d_in, d.d_in, bn);
+        rc = make_act_tensor_map(&m.tmx, x, (size_t)T, d.d_in, d.d_in, bnB);
         if (rc) return rc;
-        rc = make_act_tensor_map(&m.tmz, L.zb, (size_t)T, d.k, L.padA, bn);
+        rc = make_act_tensor_map(&m.tmz, L.zb, (size_t)T, d.k, L.padA, bnA);
         if (rc) return rc;
         rc = make_out_tensor_map(&m.tmzo, L.zb, T, d.k, L.padA);
         if (rc) return rc;
@@ -866,19 +995,19 @@ mdbf_status_t launch_forward_mat(Layer &L, const void *x, void *y, int T, cudaSt
     MatArgs b = {};
     b.wk2 = L.wk2B; b.kb_pad = L.kbpB; b.rows = d.k; b.cols = d.d_in;
     b.uimg = L.uiB; b.vimg = L.viB; b.kc = L.kcm; b.env_fmt = d.env_dtype == MDBF_BF16 ? 1u : 0u;
-    b.nv = L.kcm == 2 ? 4 : 3;
-    b.T = T; b.bn = bn;  b.zb = L.zb; b.zstride = L.padA; b.status = L.status;
+    b.nv = nv;
+    b.T = T; b.bn = bnB; b.zb = L.zb; b.zstride = L.padA; b.status = L.status;
     b.tma_out = 1;
-    rc = launch_mat<false>(b, tmx, tmzo, st);
+    rc = launch_mat<false>(b, ksB, tmx, tmzo, st);
     if (rc) return rc;
 
     MatArgs a = {};
     a.wk2 = L.wk2A; a.kb_pad = L.kbpA; a.rows = d.d_out; a.cols = d.k;
     a.uimg = L.uiA; a.vimg = L.viA; a.kc = L.kcm; a.env_fmt = b.env_fmt; a.nv = b.nv;
-    a.T = T; a.bn = bn; 
+    a.T = T; a.bn = bnA;
     a.y = reinterpret_cast<__nv_bfloat16 *>(y); a.y32 = reinterpret_cast<float *>(y); a.y_mode = L.out_mode; a.status = L.status;
     a.tma_out = y_tma ? 1 : 0;
-    rc = launch_mat<true>(a, tmz, tmyo, st);
+    rc = launch_mat<true>(a, ksA, tmz, tmyo, st);
     if (rc) return rc;
     L.last_ksplit = -1;
     *launches = 2;

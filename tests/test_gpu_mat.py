@@ -155,3 +155,27 @@ def test_mat_kernels_seeded_random_shapes(shape):
         assert M.mdbf_poll_status(g.h) == 0
         assert np.all(np.isfinite(y))
         check_parity(g, x, y, averaging=k >= 32)                # few terms per output: the per-element bound alone
+
+
+@pytest.mark.parametrize("d_out,d_in,k,l,T", [
+    (256, 4096, 300, 16, 200),      # both stages split: two tiles of 128 tokens, several ranks
+    (130, 2056, 256, 32, 100),      # one tile of 112, wide modes
+    (260, 6400, 512, 4, 210),       # a tile of 224 or two of 128: the ranks' sums against the ring
+    (300, 12808, 128, 16, 777),     # eight ranks, tiles of 192 or 256, the last one ragged
+    (1000, 8192, 129, 1, 65), (70, 1288, 1100, 2, 513)])
+def test_large_tiles_split_over_a_cluster(d_out, d_in, k, l, T):
+    """More than 64 tokens with few row blocks: the reduction is split over a cluster, the sums are exchanged by token."""
+    spec = spec_of(d_out, d_in, k, l)
+    x = inputs.make_activations(spec, T)
+    with GpuLayer(spec, T) as g:
+        y = g.forward(x)
+        assert M.mdbf_last_kernel(g.h) == M.KERNEL_MAT
+        check_parity(g, x, y)
+        np.testing.assert_array_equal(y, g.forward(x))            # added in rank order
+        # fp32 outputs of a sum of one term: the split tiles' store mode
+        xd = torch.from_numpy(x).to(torch.bfloat16).cuda()
+        yd = torch.zeros((T, d_out), dtype=torch.bfloat16, device="cuda")
+        acc = torch.zeros((T, d_out), dtype=torch.float32, device="cuda")
+        M.mdbf_linear_forward_sum([g.h], xd.data_ptr(), yd.data_ptr(), acc.data_ptr(), T, M.BF16, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(yd.to(torch.float32).cpu().numpy(), y)
