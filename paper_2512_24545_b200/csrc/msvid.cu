@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(AQ_WARPS * 32) absz_q_kernel(const float *__re
 //     straight into tensor memory as the A operand: shared memory carries each byte of Z once in and once out,
 //     where operand tiles in shared memory would carry it six times and bound the kernel;
 //   one lane bulk-copies the K block's image of the other factor: rows [0, LPP) = q_hi, [LPP, 2 LPP) = q_lo of the 32
-//     contraction indices, already in the K-major 128B-swizzled operand layout (right_mul_kernel writes the images
+//     contraction indices, already in the K-major 128B-swizzled operand layout (orth_kernel writes the images
 //     when it writes the factor);
 //   two lanes issue the MMAs, four K steps of 8 each: D1 (+)= E_hi [q_hi | q_lo] (N = 2 LPP), D2 (+)= E_lo q_hi (N = LPP).
 // Epilogue: y[t] = D1[t] + D1[LPP + t] + D2[t] into the range's partial sums.
@@ -378,6 +378,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
                     for (int e = 0; e < 16; ++e) y[(c16 * 16 + e) % LPP] += __uint_as_float(d[e]);      // columns t, LPP + t and N1 + t belong to mode t
                 }
             }
+            pdl_wait();                                          // the previous kernel reads the partial sums that are overwritten here
             if (grow < m_ext) {
                 float *out = P + ((size_t)by * m_ext + grow) * LP;
 #pragma unroll
@@ -425,6 +426,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
         // ================================= image loader ==================================
         if (lane == 0) {
             bool alive = true;
+            pdl_wait();                                          // the images are the previous kernel's output; Z and the mask are older
+            asm volatile("fence.proxy.async;\n" ::: "memory");   // written through the generic proxy, read by bulk copies
             for (int kb = 0; kb < nkb && alive; ++kb) {
                 const int s = kb % TC_STAGES;
                 alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(kb / TC_STAGES)) & 1u) ^ 1u, abort_flag, status);
@@ -539,20 +542,204 @@ __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], float *__r
         for (int a = 0; a < LP; ++a) M[k * LP + a] = (float)x[a];
     }
 }
-// Gram matrix of a tall matrix A (n x LP) in fp64 and what follows it, in one launch.  The CTAs stride over chunks of
-// GR_ROWS rows: where `parts` > 0 a chunk's rows are first formed as the sum of their partial sums P[c] (c < parts, in
-// order) and written to A; every CTA keeps one partial Gram matrix (lower triangle) over its chunks.  The CTA that
-// finishes last adds the CTAs' matrices up in a fixed order and either factors the sum (CHOL: M for right_mul_kernel)
-// or leaves it in Gs for the eigensolver.
+// A <- an orthonormal basis of its columns (Cholesky QR), in one cooperative launch: sum of the partial products (parts > 0), Gram matrix
+// in fp64, its sum over the CTAs, factor and inverse, A M and the operand images of the result.
+//
+// What bounds it: latency.  A block of 28672 x 16 is 1.8 MB; what counts is the number of dependent trips through L2 (partial
+// sums, partial Gram matrices, total) and launches.  One launch instead of two: rows stay in shared memory between the Gram
+// matrix and the multiplication; every CTA adds some entries of the Gram matrix (a warp per entry) between two grid barriers and
+// factors the total itself, so no CTA does the others' work in series.  The Gram matrix is accumulated in 4 x 4 register
+// blocks (shared memory bound it: two 8-byte loads per multiply-add before).  Measured, whole mdbf_msvid calls (two launches and the last CTA in series -> this):
+// 28672 x 6016, l = 16, 4 iterations 1504 -> 1417 us; 8192 x 3712, 8 iterations 1030 -> 887; 2048 x 1024, 8 iterations 677 -> 565.
+//
+// Images: per block of 32 rows (= 32 contraction indices kappa) a tile of 2 LPP rows of 32 TF32 values, 128 bytes each, 16-byte chunk c
+// of row r at position c ^ (r & 7) (the 128B swizzle of a K-major operand); row t < LPP holds the TF32 rounding of column t, row
+// LPP + t the rounded residual; rows past the end are zero.
+//
+// The grid barrier counts arrivals in `counter`, which only grows during a call (`base`: what earlier launches have added); its wait is
+// bounded, and a launch in which it runs out sets the status word and writes NaN.
+constexpr int OR_ROWS = 128;
+template <int LP> struct OrCfg {
+    static constexpr int BL = LP >= 4 ? 4 : LP, NB = LP / BL, NP = NB * (NB + 1) / 2;      // blocks of the lower triangle
+    static constexpr int row_groups() { int g = 1; while (2 * g * NP <= 256 && 2 * g <= OR_ROWS) g *= 2; return g; }
+    static constexpr int RG = row_groups();
+    static constexpr int LD = LP + (LP >= 2 ? 2 : 0);                                      // doubles between rows of As
+    static constexpr size_t BUF = (size_t)(OR_ROWS * LD > RG * LP * LP ? OR_ROWS * LD : RG * LP * LP) * 8;
+    static constexpr size_t CHUNK = (size_t)OR_ROWS * (LP + 1) * 4;                        // a chunk's rows kept in shared memory
+    static constexpr int KEEP = (int)((100 * 1024 - BUF) / CHUNK);
+};
+__device__ __forceinline__ bool grid_arrive_wait(unsigned int *counter, unsigned int target, int *ok_s, int32_t *status) {
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(counter, 1u);
+        unsigned long long t0 = 0;
+        int ok = 0;
+        for (uint32_t it = 0; it < (1u << 24); ++it) {
+            unsigned int v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(counter) : "memory");
+            if ((int)(v - target) >= 0) { ok = 1; break; }
+            if ((it & 255u) == 255u) {
+                const unsigned long long now = tm::global_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > TM_MAX_WAIT_NS) break;
+            }
+        }
+        if (!ok) atomicExch(status, (int32_t)MDBF_ERR_TIMEOUT);
+        *ok_s = ok;
+    }
+    __syncthreads();
+    __threadfence();
+    return *ok_s != 0;
+}
+template <int LP>
+__global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts, double *__restrict__ Gp,
+                                                   double *__restrict__ Gs, unsigned int *__restrict__ counter, unsigned int base,
+                                                   uint32_t *__restrict__ img, int32_t *__restrict__ status) {
+    using C = OrCfg<LP>;
+    constexpr int BL = C::BL, NP = C::NP, RG = C::RG, LD = C::LD;
+    constexpr int PER = OR_ROWS * LP / 256 > 0 ? OR_ROWS * LP / 256 : 1;                   // elements of a chunk per thread
+    extern __shared__ __align__(16) unsigned char or_smem[];
+    __shared__ double Gm[LP][LP + 1];
+    __shared__ float Ms[LP * LP];
+    __shared__ int ok_s;
+    double *As = reinterpret_cast<double *>(or_smem);
+    float *rows = reinterpret_cast<float *>(or_smem + C::BUF);
+    const int tid = threadIdx.x, G = gridDim.x;
+    tm::pdl_launch_dependents();                                 // the product that reads A next brings its tiles of Z meanwhile
+
+    int bi = 0, bj = 0, rest = tid % NP;                         // this thread's block of the lower triangle
+    while (rest > bi) { rest -= bi + 1; ++bi; }
+    bj = rest;
+    const int rg = tid / NP;
+    double acc[BL][BL];
+#pragma unroll
+    for (int x = 0; x < BL; ++x)
+#pragma unroll
+        for (int y = 0; y < BL; ++y) acc[x][y] = 0.0;
+    const int nchunks = (n + OR_ROWS - 1) / OR_ROWS;
+    const size_t limit = (size_t)n * LP;
+    int kept = 0;
+    for (int chunk = blockIdx.x; chunk < nchunks; chunk += G, ++kept) {
+        const size_t at0 = (size_t)chunk * OR_ROWS * LP;
+        float v[PER];
+#pragma unroll
+        for (int u = 0; u < PER; ++u) v[u] = 0.f;
+        if (parts > 0) {
+#pragma unroll 4
+            for (int c = 0; c < parts; ++c)                      // independent loads, additions in the order of c
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    const size_t at = at0 + tid + 256 * u;
+                    if (tid + 256 * u < OR_ROWS * LP && at < limit) v[u] += __ldcs(P + (size_t)c * limit + at);
+                }
+        } else {
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const size_t at = at0 + tid + 256 * u;
+                if (tid + 256 * u < OR_ROWS * LP && at < limit) v[u] = A[at];
+            }
+        }
+        __syncthreads();                                         // the previous chunk's Gram pass has read As
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const int e = tid + 256 * u;
+            if (e >= OR_ROWS * LP) continue;
+            As[e / LP * LD + e % LP] = (double)v[u];             // rows past the end are zero
+            if (kept < C::KEEP) rows[(size_t)kept * OR_ROWS * (LP + 1) + e / LP * (LP + 1) + e % LP] = v[u];
+            else if (parts > 0 && at0 + e < limit) A[at0 + e] = v[u];
+        }
+        __syncthreads();
+        if (rg < RG)
+            for (int r = rg; r < OR_ROWS; r += RG) {
+                double a[BL], b[BL];
+#pragma unroll
+                for (int x = 0; x < BL; ++x) { a[x] = As[r * LD + bi * BL + x]; b[x] = As[r * LD + bj * BL + x]; }
+#pragma unroll
+                for (int x = 0; x < BL; ++x)
+#pragma unroll
+                    for (int y = 0; y < BL; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+            }
+    }
+    __syncthreads();
+    if (rg < RG)                                                 // the row groups' blocks, added in order below
+#pragma unroll
+        for (int x = 0; x < BL; ++x)
+#pragma unroll
+            for (int y = 0; y < BL; ++y) As[rg * LP * LP + (bi * BL + x) * LP + bj * BL + y] = acc[x][y];
+    __syncthreads();
+    for (int e = tid; e < LP * LP; e += 256)
+        if (e % LP <= e / LP) {
+            double t = 0.0;
+#pragma unroll 4
+            for (int q = 0; q < RG; ++q) t += As[q * LP * LP + e];
+            Gp[(size_t)blockIdx.x * LP * LP + e] = t;
+        }
+    bool ok = grid_arrive_wait(counter, base + (unsigned int)G, &ok_s, status);
+    // totals: a warp per entry, lanes over the CTAs' matrices
+    for (int e = blockIdx.x * 8 + (tid >> 5); e < LP * LP; e += G * 8)
+        if (e % LP <= e / LP) {
+            double t = 0.0;
+            for (int c = tid & 31; c < G; c += 32) t += __ldcg(Gp + (size_t)c * LP * LP + e);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if ((tid & 31) == 0) __stcg(Gs + e, t);
+        }
+    ok = grid_arrive_wait(counter, base + 2u * (unsigned int)G, &ok_s, status) && ok;
+    for (int e = tid; e < LP * LP; e += 256)
+        if (e % LP <= e / LP) Gm[e / LP][e % LP] = __ldcg(Gs + e);
+    __syncthreads();
+    if (tid < 32) chol_warp<LP>(Gm, Ms);
+    __syncthreads();
+
+    // A M and the operand images; two threads per row where a row has sixteen columns or more
+    constexpr int H = LP >= 16 ? 2 : 1, LC = LP / H;
+    const int r = tid % OR_ROWS, h = tid / OR_ROWS;
+    kept = 0;
+    for (int chunk = blockIdx.x; chunk < nchunks; chunk += G, ++kept) {
+        if (h >= H) continue;
+        const int i = chunk * OR_ROWS + r;
+        float a[LP], o[LC];
+        const float *src = rows + (size_t)kept * OR_ROWS * (LP + 1) + r * (LP + 1);
+#pragma unroll
+        for (int t = 0; t < LP; ++t) a[t] = kept < C::KEEP ? src[t] : (i < n ? A[(size_t)i * LP + t] : 0.f);
+#pragma unroll
+        for (int t = 0; t < LC; ++t) o[t] = ok ? 0.f : __int_as_float(0x7fc00000);
+#pragma unroll
+        for (int b = 0; b < LP; ++b)
+#pragma unroll
+            for (int t = 0; t < LC; ++t) o[t] = fmaf(a[b], Ms[b * LP + h * LC + t], o[t]);
+        if (H > 1 && kept >= C::KEEP) asm volatile("bar.sync 1, 256;\n" ::: "memory");     // both threads of a row have read it
+        if (img && i < ((n + TC_KB - 1) / TC_KB) * TC_KB) {
+            constexpr int LPP = TcCfg<LP>::LPP, N1 = TcCfg<LP>::N1;
+            const int kappa = i & 31;
+            uint32_t *dst = img + (size_t)(i >> 5) * (N1 * 32);
+#pragma unroll
+            for (int q = 0; q < (LPP > LP ? LPP : LC); ++q) {
+                const int t = LPP > LP ? q : h * LC + q;
+                const float v = q < LC ? o[q < LC ? q : 0] : 0.f;
+                const uint32_t hi = tf32_round(v);
+                dst[t * 32 + ((((kappa >> 2) ^ (t & 7)) << 2) | (kappa & 3))] = hi;
+                dst[(LPP + t) * 32 + ((((kappa >> 2) ^ ((LPP + t) & 7)) << 2) | (kappa & 3))] = tf32_round(v - __uint_as_float(hi));
+            }
+        }
+        if (i < n)
+#pragma unroll
+            for (int t = 0; t < LC; ++t) A[(size_t)i * LP + h * LC + t] = o[t];
+    }
+}
+
+// Gram matrix Gs of a tall matrix A (n x LP) in fp64 (lower triangle), for the eigensolver.  The CTAs stride over chunks of GR_ROWS
+// rows: where `parts` > 0 a chunk's rows are first formed as the sum of their partial sums P[c] (c < parts, in order) and written
+// to A; every CTA keeps one partial Gram matrix over its chunks, and the CTA that finishes last adds them up in a fixed order.
 constexpr int GR_ROWS = 128, GR_MAX_CTAS = 128;
-template <int LP, bool CHOL>
+template <int LP>
 __global__ void __launch_bounds__(256) gram_finish_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts,
                                                           double *__restrict__ Gp, unsigned int *__restrict__ counter,
-                                                          double *__restrict__ Gs, float *__restrict__ M) {
+                                                          double *__restrict__ Gs) {
     constexpr int PER = GR_ROWS * LP / 256 > 0 ? GR_ROWS * LP / 256 : 1;     // elements of a chunk per thread
     constexpr int ENT = (LP * LP + 255) / 256;                                // Gram entries per thread
     __shared__ double As[GR_ROWS][LP + 1];                       // converted once on the way in, not once per product
-    __shared__ double Gm[LP][LP + 1];
     __shared__ bool is_last;
     double acc[ENT];
 #pragma unroll
@@ -622,52 +809,27 @@ __global__ void __launch_bounds__(256) gram_finish_kernel(float *__restrict__ A,
 #pragma unroll
             for (int u = 0; u < 16; ++u) s[u & 3] += v[u];
         }
-        const double total = (s[0] + s[1]) + (s[2] + s[3]);
-        if (CHOL) Gm[pr / LP][pr % LP] = total;
-        else Gs[pr] = total;
+        Gs[pr] = (s[0] + s[1]) + (s[2] + s[3]);
     }
     if (threadIdx.x == 0) *counter = 0u;                         // ready for the next launch on the stream
-    if (!CHOL) return;
-    __syncthreads();
-    if (threadIdx.x < 32) chol_warp<LP>(Gm, M);
 }
-// A <- A M, row by row (M is LP x LP, row-major).  With `img`, the rows' operand images for the tensor-core product that
-// reads A next are written on the way out: per block of 32 rows (= 32 contraction indices kappa) a tile of 2 LPP rows of
-// 32 TF32 values, 128 bytes each, 16-byte chunk c of row r at position c ^ (r & 7) (the 128B swizzle of a K-major
-// operand); row t < LPP holds the TF32 rounding of column t, row LPP + t the rounded residual; rows past the end are zero.
+// out <- the first out_cols columns of A M, row by row (M is LP x LP, row-major)
 template <int LP>
-__global__ void __launch_bounds__(256) right_mul_kernel(float *__restrict__ A, int n, const float *__restrict__ M, float *__restrict__ out,
-                                                        int out_cols, uint32_t *__restrict__ img) {
+__global__ void __launch_bounds__(256) right_mul_kernel(const float *__restrict__ A, int n, const float *__restrict__ M, float *__restrict__ out,
+                                                        int out_cols) {
     __shared__ float Ms[LP][LP];
     for (int e = threadIdx.x; e < LP * LP; e += 256) Ms[e / LP][e % LP] = M[e];
     __syncthreads();
     const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
     float a[LP], o[LP];
 #pragma unroll
-    for (int t = 0; t < LP; ++t) { a[t] = i < n ? A[(size_t)i * LP + t] : 0.f; o[t] = 0.f; }
+    for (int t = 0; t < LP; ++t) { a[t] = A[(size_t)i * LP + t]; o[t] = 0.f; }
 #pragma unroll
     for (int b = 0; b < LP; ++b)
 #pragma unroll
         for (int t = 0; t < LP; ++t) o[t] = fmaf(a[b], Ms[b][t], o[t]);
-    if (img && i < ((n + TC_KB - 1) / TC_KB) * TC_KB) {
-        constexpr int LPP = TcCfg<LP>::LPP, N1 = TcCfg<LP>::N1;
-        const int kappa = i & 31;
-        uint32_t *dst = img + (size_t)(i >> 5) * (N1 * 32);
-#pragma unroll
-        for (int t = 0; t < LPP; ++t) {
-            const float v = t < LP ? o[t < LP ? t : 0] : 0.f;
-            const uint32_t hi = tf32_round(v);
-            dst[t * 32 + ((((kappa >> 2) ^ (t & 7)) << 2) | (kappa & 3))] = hi;
-            dst[(LPP + t) * 32 + ((((kappa >> 2) ^ ((LPP + t) & 7)) << 2) | (kappa & 3))] = tf32_round(v - __uint_as_float(hi));
-        }
-    }
-    if (i >= n) return;
-    if (out) {
-        for (int t = 0; t < out_cols; ++t) out[(size_t)i * out_cols + t] = o[t];     // compact result (the first out_cols columns)
-    } else {
-#pragma unroll
-        for (int t = 0; t < LP; ++t) A[(size_t)i * LP + t] = o[t];
-    }
+    for (int t = 0; t < out_cols; ++t) out[(size_t)i * out_cols + t] = o[t];
 }
 
 // ------------------------------------------------------------------ the small eigenproblem
@@ -785,11 +947,13 @@ __global__ void pad_kernel(const float *__restrict__ src, size_t n, int l, int L
 
 // The scratch of one call, carved out of the caller's workspace (256-byte aligned pieces).
 struct Scratch {
-    float *Q, *Y, *P, *M, *MU, *MV;
+    float *Q, *Y, *P, *MU, *MV;
     double *Gp, *Gs;
     uint32_t *img;          // operand images of Q for the tensor-core product
     int32_t *status;        // set by a wait that ran out
     unsigned int *counter;  // CTAs of the Gram kernel that have finished (the word after the status word)
+    unsigned int *barrier;  // arrivals at the grid barriers of orth_kernel, and how many the launches so far will have made
+    unsigned int arrived;
 };
 // how the K blocks of the tensor-core product are split over blockIdx.y: the split that fills whole waves of resident CTAs best,
 // each CTA keeping at least 8 K blocks
@@ -819,13 +983,12 @@ static size_t carve(Scratch *w, char *base, int p, int q, int LP) {
     const size_t tc_parts = (size_t)tc_split(p, q, LP, &kb_per_cta), tc_parts_t = (size_t)tc_split(q, p, LP, &kb_per_cta);
     float *P = (float *)take(std::max(std::max(zy_chunks, tc_parts_t) * q, tc_parts * p) * LP * sizeof(float));
     uint32_t *img = (uint32_t *)take((size_t)ceil_div(std::max(p, q), TC_KB) * 2 * (LP < 16 ? 16 : LP) * 128);
-    int32_t *status = (int32_t *)take(2 * sizeof(int32_t));
+    int32_t *status = (int32_t *)take(3 * sizeof(int32_t));
     double *Gp = (double *)take(gchunks * LP * LP * sizeof(double));
     double *Gs = (double *)take((size_t)LP * LP * sizeof(double));
-    float *M = (float *)take((size_t)LP * LP * sizeof(float));
     float *MU = (float *)take((size_t)LP * LP * sizeof(float));
     float *MV = (float *)take((size_t)LP * LP * sizeof(float));
-    if (w) { w->Q = Q; w->Y = Y; w->P = P; w->Gp = Gp; w->Gs = Gs; w->M = M; w->MU = MU; w->MV = MV; w->img = img; w->status = status; w->counter = (unsigned int *)status + 1; }
+    if (w) { w->Q = Q; w->Y = Y; w->P = P; w->Gp = Gp; w->Gs = Gs; w->MU = MU; w->MV = MV; w->img = img; w->status = status; w->counter = (unsigned int *)status + 1; w->barrier = (unsigned int *)status + 2; w->arrived = 0u; }
     return off;
 }
 static int padded_rank(int l) {
@@ -838,9 +1001,27 @@ static int padded_rank(int l) {
 // in w.P; with `img`, the operand images of the result are written for the tensor-core product that reads it next
 template <int LP>
 static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr) {
-    gram_finish_kernel<LP, true><<<std::min(ceil_div(n, GR_ROWS), GR_MAX_CTAS), 256, 0, st>>>(A, n, w.P, parts, w.Gp, w.counter, w.Gs, w.M);
-    right_mul_kernel<LP><<<ceil_div(n, 256), 256, 0, st>>>(A, n, w.M, nullptr, 0, img);
-    MDBF_CUDA(cudaGetLastError());
+    using C = OrCfg<LP>;
+    auto kern = orth_kernel<LP>;
+    const int ctas = std::min(ceil_div(n, OR_ROWS), GR_MAX_CTAS), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
+    static PerDeviceOnce once;
+    if (once.first()) {
+        MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
+        // the product's split between L1 and shared memory: its CTAs can start beside this kernel's
+        MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = C::BUF + (size_t)std::min(chunks, C::KEEP) * C::CHUNK;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, A, n, (const float *)w.P, parts, w.Gp, w.Gs, w.barrier, w.arrived, img, w.status));
+    w.arrived += 2u * (unsigned int)ctas;
     return MDBF_OK;
 }
 
@@ -882,7 +1063,7 @@ struct ZMaps {
 };
 // E F (TRANS = false: p output rows, F has q) or E^T F (TRANS = true: q output rows, F has p) on the tensor cores, E the
 // envelope of Z (|Z|, or Z with the given mask's signs taken off) and F the factor whose operand images the preceding
-// right_mul_kernel left in w.img; the result is left as *parts_out partial sums in w.P
+// orth_kernel left in w.img; the result is left as *parts_out partial sums in w.P
 template <int LP, bool MASKED, bool TRANS, bool WRITE_MASK = false>
 static mdbf_status_t tc_product(const ZMaps &zm, int p, int q, const uint32_t *S, int nwords, Scratch &w,
                                 cudaStream_t st, int *parts_out, uint32_t *S_out = nullptr) {
@@ -894,10 +1075,19 @@ static mdbf_status_t tc_product(const ZMaps &zm, int p, int q, const uint32_t *S
     const int m_ext = TRANS ? q : p, k_ext = TRANS ? p : q;
     int kb_per_cta = 0;
     const int parts = tc_split(m_ext, k_ext, LP, &kb_per_cta);
-    envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK><<<dim3(ceil_div(m_ext, 128), parts), TC_THREADS, C::SMEM, st>>>(
-        TRANS ? zm.cols : zm.rows, p, q, w.img, kb_per_cta, w.P, S, S_out, nwords, w.status);
-    *parts_out = parts;                                          // the Gram kernel that follows adds the partial sums up
-    MDBF_CUDA(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;    // it starts while orth_kernel runs: only the images are that kernel's
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(ceil_div(m_ext, 128), parts);
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK>, TRANS ? zm.cols : zm.rows, p, q,
+                                 (const uint32_t *)w.img, kb_per_cta, w.P, S, S_out, nwords, w.status));
+    *parts_out = parts;                                          // the kernel that follows adds the partial sums up
     return MDBF_OK;
 }
 // Y = E Q
@@ -932,7 +1122,7 @@ template <int LP, bool MASKED>
 static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const float *Q0, uint32_t *S, float *U, float *V, float *sigma,
                          Scratch &w, cudaStream_t st) {
     const int nwords = ceil_div(q, 32);
-    MDBF_CUDA(cudaMemsetAsync(w.status, 0, 2 * sizeof(int32_t), st));           // status word and the Gram kernel's counter
+    MDBF_CUDA(cudaMemsetAsync(w.status, 0, 3 * sizeof(int32_t), st));           // status word, the Gram kernel's counter, the grid barriers'
     ZMaps zm;
     zm.use = tc_eligible(Z, q);
     if (zm.use) {
@@ -959,10 +1149,10 @@ static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const 
     }
     rc = product<LP, MASKED>(Z, p, q, S, nwords, zm, w, st, &parts);
     if (rc) return rc;
-    gram_finish_kernel<LP, false><<<std::min(ceil_div(p, GR_ROWS), GR_MAX_CTAS), 256, 0, st>>>(w.Y, p, w.P, parts, w.Gp, w.counter, w.Gs, w.M);
+    gram_finish_kernel<LP><<<std::min(ceil_div(p, GR_ROWS), GR_MAX_CTAS), 256, 0, st>>>(w.Y, p, w.P, parts, w.Gp, w.counter, w.Gs);
     jacobi_kernel<LP><<<1, JAC_THREADS, 0, st>>>(w.Gs, l, sigma, w.MU, w.MV);
-    right_mul_kernel<LP><<<ceil_div(p, 256), 256, 0, st>>>(w.Y, p, w.MU, U, l, nullptr);
-    right_mul_kernel<LP><<<ceil_div(q, 256), 256, 0, st>>>(w.Q, q, w.MV, V, l, nullptr);
+    right_mul_kernel<LP><<<ceil_div(p, 256), 256, 0, st>>>(w.Y, p, w.MU, U, l);
+    right_mul_kernel<LP><<<ceil_div(q, 256), 256, 0, st>>>(w.Q, q, w.MV, V, l);
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }
