@@ -837,14 +837,17 @@ __global__ void __launch_bounds__(256) right_mul_kernel(const float *__restrict_
 // writes the singular values s_t = sqrt(lambda_t) and the two LP x LP matrices that turn (Y, Q) into the balanced
 // factors: MU[b][t] = W[b][t] s_t^-1/2, MV[b][t] = W[b][t] s_t^1/2 (zero columns beyond l and for vanished values).
 // Round-robin ordering: n - 1 rounds of n / 2 rotations on disjoint index pairs (n = l rounded up to even; a pair with
-// the dummy index is skipped).  Thread i < n / 2 works out the rotation of pair i; then thread (k, i) applies rotation
-// i to row k (columns p, q of G and of W), and after a barrier to column k (rows p, q of G).  The tangent is taken in
+// the dummy index is skipped).  What bounds it is the chain of a round: thread i < n / 2 works out the rotation of pair i; then
+// thread (i, j) turns the 2 x 2 block of G where the rows of pair i meet the columns of pair j from both sides, and thread
+// (k, i) row k of W by pair i.  The blocks do not overlap, so a round is two barriers (rows and columns one after the other: three;
+// EIGFIG.  Every thread working out its own two rotations, without the trip through shared memory, was slower: fp64).  The tangent is taken in
 // fp32 (any angle near the optimal one converges; fp64 division and square roots were most of a round), the cosine
 // and sine from it in fp64, so that every rotation is orthogonal to fp64 rounding.
-constexpr int JAC_THREADS = 256;
+constexpr int jac_threads(int LP) { return LP <= 16 ? 192 : 768; }       // LP^2 / 4 blocks of G and LP^2 / 2 pairs of W
 template <int LP>
-__global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double *__restrict__ Gs, int l, float *__restrict__ sigma,
+__global__ void __launch_bounds__(jac_threads(LP)) jacobi_kernel(const double *__restrict__ Gs, int l, float *__restrict__ sigma,
                                                              float *__restrict__ MU, float *__restrict__ MV) {
+    constexpr int JAC_THREADS = jac_threads(LP);
     __shared__ double G[LP][LP + 1], W[LP][LP + 1], rc[LP], rs[LP];
     __shared__ int order[LP], rp[LP], rq[LP];
     __shared__ int done;
@@ -875,7 +878,11 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double *__res
         if (done) break;
         for (int r = 0; r < n - 1; ++r) {
             if (tid < half) {
-                const int a = tid == 0 ? n - 1 : (r + tid) % (n - 1), b = tid == 0 ? r : (r - tid + (n - 1)) % (n - 1);
+                int a = n - 1, b = r;
+                if (tid > 0) {
+                    a = r + tid; if (a >= n - 1) a -= n - 1;
+                    b = r - tid; if (b < 0) b += n - 1;
+                }
                 const int pi = min(a, b), qi = max(a, b);
                 double c = 1.0, sn = 0.0;
                 if (qi < l) {
@@ -890,27 +897,24 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double *__res
                 rp[tid] = pi; rq[tid] = qi; rc[tid] = c; rs[tid] = sn;
             }
             __syncthreads();
-            for (int idx = tid; idx < l * half; idx += JAC_THREADS) {
-                const int k = idx / half, i = idx - k * half;
-                const double c = rc[i], sn = rs[i];
-                if (sn == 0.0) continue;
-                const int pi = rp[i], qi = rq[i];
-                const double gkp = G[k][pi], gkq = G[k][qi];
-                G[k][pi] = c * gkp - sn * gkq;
-                G[k][qi] = sn * gkp + c * gkq;
-                const double wkp = W[k][pi], wkq = W[k][qi];
-                W[k][pi] = c * wkp - sn * wkq;
-                W[k][qi] = sn * wkp + c * wkq;
-            }
-            __syncthreads();
-            for (int idx = tid; idx < l * half; idx += JAC_THREADS) {
-                const int k = idx / half, i = idx - k * half;
-                const double c = rc[i], sn = rs[i];
-                if (sn == 0.0) continue;
-                const int pi = rp[i], qi = rq[i];
-                const double gpk = G[pi][k], gqk = G[qi][k];
-                G[pi][k] = c * gpk - sn * gqk;
-                G[qi][k] = sn * gpk + c * gqk;
+            const int nb = half * half, wi = tid - nb;
+            if (tid < nb) {
+                const int i = tid / half, j = tid - i * half;
+                const int ip = rp[i], iq = rq[i], jp = rp[j], jq = rq[j];
+                const bool qi = iq < l, qj = jq < l;             // (a dummy index is always the larger of its pair)
+                const double ic = rc[i], is = rs[i], jc = rc[j], js = rs[j];
+                const double a = G[ip][jp], b = qj ? G[ip][jq] : 0.0, c = qi ? G[iq][jp] : 0.0, d = qi && qj ? G[iq][jq] : 0.0;
+                const double a1 = jc * a - js * b, b1 = js * a + jc * b, c1 = jc * c - js * d, d1 = js * c + jc * d;
+                G[ip][jp] = ic * a1 - is * c1;
+                if (qj) G[ip][jq] = ic * b1 - is * d1;
+                if (qi) G[iq][jp] = is * a1 + ic * c1;
+                if (qi && qj) G[iq][jq] = is * b1 + ic * d1;
+            } else if (wi < l * half) {
+                const int k = wi / half, i = wi - k * half;
+                const int ip = rp[i], iq = rq[i];
+                const double c = rc[i], sn = rs[i], a = W[k][ip], b = iq < l ? W[k][iq] : 0.0;
+                W[k][ip] = c * a - sn * b;
+                if (iq < l) W[k][iq] = sn * a + c * b;
             }
             __syncthreads();
         }
@@ -1150,7 +1154,7 @@ static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const 
     rc = product<LP, MASKED>(Z, p, q, S, nwords, zm, w, st, &parts);
     if (rc) return rc;
     gram_finish_kernel<LP><<<std::min(ceil_div(p, GR_ROWS), GR_MAX_CTAS), 256, 0, st>>>(w.Y, p, w.P, parts, w.Gp, w.counter, w.Gs);
-    jacobi_kernel<LP><<<1, JAC_THREADS, 0, st>>>(w.Gs, l, sigma, w.MU, w.MV);
+    jacobi_kernel<LP><<<1, jac_threads(LP), 0, st>>>(w.Gs, l, sigma, w.MU, w.MV);
     right_mul_kernel<LP><<<ceil_div(p, 256), 256, 0, st>>>(w.Y, p, w.MU, U, l);
     right_mul_kernel<LP><<<ceil_div(q, 256), 256, 0, st>>>(w.Q, q, w.MV, V, l);
     MDBF_CUDA(cudaGetLastError());
