@@ -500,42 +500,34 @@ __global__ void chunk_sum_kernel(const float *__restrict__ P, int nchunks, size_
 }
 
 // ------------------------------------------------------------------ orth(): Cholesky QR, Gram matrix in fp64
-// One warp, lane k = row k of G in registers: G = L L^T (G: the summed Gram matrix, lower triangle), then lane k = column k
-// of L^-1 by forward substitution; rows of L travel by shuffles.  M[b][a] = (L^-1)[a][b], so that A M has orthonormal
-// columns.  A zero (or numerically vanished) pivot - a padding column, or a block wider than the rank of the matrix -
+// One warp, lane k = row k of G in registers: G = L L^T (G: the summed Gram matrix, lower triangle); beside it lane k builds column k
+// of L^-1 by forward substitution, each column of L serving both as soon as it is known (one set of shuffles and one chain of
+// pivots: 4.5 us when the inverse followed the factor, 2.3 us now at l = 16).  M[b][a] = (L^-1)[a][b], so that A M has
+// orthonormal columns.  A zero (or numerically vanished) pivot - a padding column, or a block wider than the rank of the matrix -
 // leaves its column as it is instead of dividing by zero.
 template <int LP>
 __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], float *__restrict__ M) {
     const int k = threadIdx.x & 31;
-    double g[LP], invd[LP];
+    double g[LP], x[LP];                                         // row k of G, then of L; right-hand side, then column k of L^-1
     double scale = 0.0;
 #pragma unroll
     for (int j = 0; j < LP; ++j) {
-        g[j] = (k < LP && j <= k) ? Gm[k < LP ? k : 0][j] : 0.0;
+        g[j] = j <= k ? Gm[k < LP ? k : 0][j] : 0.0;             // (above the diagonal: never read by another lane)
+        x[j] = j == k ? 1.0 : 0.0;
         scale = fmax(scale, Gm[j][j]);
     }
 #pragma unroll
     for (int c = 0; c < LP; ++c) {
         const double dcc = __shfl_sync(0xffffffffu, g[c], c);
-        const double inv = (dcc > 1e-24 * scale && dcc > 0.0) ? rsqrt(dcc) : 0.0;
-        invd[c] = inv;                                           // 1 / L[c][c], the same in every lane
-        g[c] = k == c ? dcc * inv : g[c] * inv;                  // column c of L (zero above the diagonal)
+        const double inv = (dcc > 1e-24 * scale && dcc > 0.0) ? rsqrt(dcc) : 0.0;      // 1 / L[c][c], the same in every lane
+        g[c] *= inv;                                             // column c of L below the diagonal
+        x[c] = inv > 0.0 ? x[c] * inv : (c == k ? 1.0 : 0.0);    // (zero for c < k from the start)
 #pragma unroll
         for (int jj = c + 1; jj < LP; ++jj) {
             const double ljc = __shfl_sync(0xffffffffu, g[c], jj);
-            if (k >= jj) g[jj] -= g[c] * ljc;
+            g[jj] = fma(-g[c], ljc, g[jj]);
+            x[jj] = fma(-ljc, x[c], x[jj]);
         }
-    }
-    double x[LP];
-#pragma unroll
-    for (int i = 0; i < LP; ++i) {
-        double sum = i == k ? 1.0 : 0.0;
-#pragma unroll
-        for (int m = 0; m < i; ++m) {
-            const double lim = __shfl_sync(0xffffffffu, g[m], i);     // L[i][m]
-            if (m >= k) sum -= lim * x[m];
-        }
-        x[i] = i >= k ? (invd[i] > 0.0 ? sum * invd[i] : (i == k ? 1.0 : 0.0)) : 0.0;
     }
     if (k < LP) {
 #pragma unroll
@@ -550,7 +542,8 @@ __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], float *__r
 // matrix and the multiplication; every CTA adds some entries of the Gram matrix (a warp per entry) between two grid barriers and
 // factors the total itself, so no CTA does the others' work in series.  The Gram matrix is accumulated in 4 x 4 register
 // blocks (shared memory bound it: two 8-byte loads per multiply-add before).  Measured, whole mdbf_msvid calls (two launches and the last CTA in series -> this):
-// 28672 x 6016, l = 16, 4 iterations 1504 -> 1417 us; 8192 x 3712, 8 iterations 1030 -> 887; 2048 x 1024, 8 iterations 677 -> 565.
+// 28672 x 6016, l = 16, 4 iterations 1504 -> 1359 us; 8192 x 3712, 8 iterations 1030 -> 807; 2048 x 1024, 8 iterations 677 -> 486
+// (with the eigensolver below).
 //
 // Images: per block of 32 rows (= 32 contraction indices kappa) a tile of 2 LPP rows of 32 TF32 values, 128 bytes each, 16-byte chunk c
 // of row r at position c ^ (r & 7) (the 128B swizzle of a K-major operand); row t < LPP holds the TF32 rounding of column t, row
@@ -840,7 +833,8 @@ __global__ void __launch_bounds__(256) right_mul_kernel(const float *__restrict_
 // the dummy index is skipped).  What bounds it is the chain of a round: thread i < n / 2 works out the rotation of pair i; then
 // thread (i, j) turns the 2 x 2 block of G where the rows of pair i meet the columns of pair j from both sides, and thread
 // (k, i) row k of W by pair i.  The blocks do not overlap, so a round is two barriers (rows and columns one after the other: three;
-// EIGFIG.  Every thread working out its own two rotations, without the trip through shared memory, was slower: fp64).  The tangent is taken in
+// 83 us for the kernel at l = 16, 56 now.  Every thread working out its own two rotations, without the trip through shared memory, was
+// slower: fp64).  The tangent is taken in
 // fp32 (any angle near the optimal one converges; fp64 division and square roots were most of a round), the cosine
 // and sine from it in fp64, so that every rotation is orthogonal to fp64 rounding.
 constexpr int jac_threads(int LP) { return LP <= 16 ? 192 : 768; }       // LP^2 / 4 blocks of G and LP^2 / 2 pairs of W
