@@ -1,17 +1,24 @@
-// Dense fp32 product C = A B on the tensor cores at close to fp32 accuracy: tcgen05 kind::tf32 and the three-term split
-//     a b  ~  a_hi b_hi + a_hi b_lo + a_lo b_hi          (each part a TF32 number; the dropped a_lo b_lo is below 2^-24 a b)
+// Dense fp32 product C = A B on the tensor cores at close to fp32 accuracy: tcgen05 kind::f16 on a scaled two-part split
+//     a b  ~  a_hi b_hi + a_hi b_lo + a_lo b_hi          (the dropped a_lo b_lo is below 2^-24 a b)
 // with fp32 accumulation in tensor memory.  It serves the least-squares step of the ADMM refinement (W V and V^T V,
-// Eq. admm-U-tilde), where the FP32 pipe would need five times as long.
+// Eq. admm-U-tilde), where the FP32 pipe would need eight times as long.
 //
-// Two passes.  split_image_kernel turns an operand into "images": per tile of 128 rows (output rows for A, output
-// columns for B) and block of 32 contraction indices one 32 KB piece holding hi (128 rows of 32 TF32 values, 128 bytes
+// The split.  A row of an operand (a row of A, a column of B) is multiplied by the power of two that brings its largest entry into
+// [2^14, 2^15); hi = the scaled entry rounded to fp16, lo = the exact residual rounded to fp16: 11 + 11 significant bits, the same as
+// two TF32 parts, with an absolute floor 2^-39 below the row's largest entry where lo runs out of exponent.  The product is multiplied by
+// both inverse scales on the way out (exact).  fp16 operands issue at twice the TF32 rate and are half the bytes: 8192 x 3712 x 3712
+// 943 -> 566 us; 8192 x 3712 x 8192 on 124 SMs 2193 -> 1271; error of an ADMM iterate against fp64 2.0e-6 -> 1.4e-6.
+//
+// Two passes.  The split kernels turn an operand into "images": per tile of 128 rows (output rows for A, output
+// columns for B) and block of 64 contraction indices one 32 KB piece holding hi (128 rows of 64 fp16 values, 128 bytes
 // each) and lo (the same shape behind it), rows K-major with the 128B swizzle a shared-memory matrix descriptor expects
-// (16-byte chunk c of row r at position c ^ (r & 7)); tails are zero.  Either operand may be given transposed: an
+// (16-byte chunk c of row r at position c ^ (r & 7)); tails are zero.  Behind the pieces lie the rows' inverse scales, behind those the
+// bits of their largest magnitudes.  Either operand may be given transposed: an
 // element is read at src[i * stride_i + k * stride_k] with one of the strides equal to one.
 // gemm3x_kernel: one CTA per SM walks over 128 x 256 tiles of C (two column tiles of B side by side: the stream from L2
 // into shared memory, 96 KB per K block, is what bounds the kernel, and a wider tile spends less of it per flop); one
 // lane streams the pieces of each K block into a ring by bulk copies, one lane issues  D (+)= A_hi B_hi, D += A_hi B_lo,
-// D += A_lo B_hi  (N = 256, four K steps of 8 each), the eight epilogue warps read the accumulators and store.  Every wait is bounded; on expiry the status word is
+// D += A_lo B_hi  (N = 256, four K steps of 16 each), the eight epilogue warps read the accumulators and store.  Every wait is bounded; on expiry the status word is
 // set and the tiles still to be written come out as NaN.
 #include <algorithm>
 #include <cstdint>
@@ -22,78 +29,114 @@
 namespace mdbf {
 namespace g3x {
 
-constexpr int TILE = 128, KB = 32;
-constexpr int HALF = TILE * KB * 4;            // bytes of the hi (or lo) part of a piece
+constexpr int TILE = 128, KB = 64;
+constexpr int HALF = TILE * KB * 2;            // bytes of the hi (or lo) part of a piece
 constexpr int PIECE = 2 * HALF;                // 32 KB
 constexpr int STAGES = 2;
-constexpr int KCHUNK = 4;                      // K blocks accumulated in tensor memory before the sum moves to fp32 registers
+constexpr int KCHUNK = 2;                      // K blocks accumulated in tensor memory before the sum moves to fp32 registers
 constexpr int STAGE_BYTES = 3 * PIECE;         // A piece, then B_hi of two column tiles, then their B_lo
 constexpr int EPI_WARPS = 8;                   // two per quarter of the TMEM lanes, each with half of the tile's columns
 constexpr int THREADS = (EPI_WARPS + 2) * 32;  // epilogue warps, loader, issuer
 constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES;
 
-// hi = v rounded to the nearest TF32 number (half-ulp add on the bits; the top binade is truncated so that nothing rounds
-// up to infinity), lo = the exact residual rounded the same way
-__device__ __forceinline__ void split_tf32(float v, uint32_t &hi, uint32_t &lo) {
-    const uint32_t b = __float_as_uint(v);
-    hi = ((b & 0x7F000000u) == 0x7F000000u ? b : b + 0x1000u) & 0xFFFFE000u;
-    lo = (__float_as_uint(v - __uint_as_float(hi)) + 0x1000u) & 0xFFFFE000u;
+// scale and inverse scale of a row from the bits of its largest magnitude: powers of two, 2^14 <= max * scale < 2^15 (an all-zero or
+// denormal row is scaled up as far as the inverse stays normal, a row with an infinity or NaN not at all)
+__device__ __forceinline__ float row_scale(uint32_t maxbits, float *inverse) {
+    const int e = (int)(maxbits >> 23);
+    const int f = e == 255 ? 127 : min(253, 268 - e);
+    *inverse = __uint_as_float((uint32_t)(254 - f) << 23);
+    return __uint_as_float((uint32_t)f << 23);
 }
-// grid: (K blocks, tiles); block 256 = 128 rows x 2 halves of the 8 chunks
-template <bool K_CONTIGUOUS>
-__global__ void __launch_bounds__(256) split_image_kernel(const float *__restrict__ src, size_t stride_i, size_t stride_k, int ni, int nk,
-                                                          int nkb, uint32_t *__restrict__ img) {
-    const int kb = blockIdx.x, it = blockIdx.y;
-    unsigned char *piece = reinterpret_cast<unsigned char *>(img) + ((size_t)it * nkb + kb) * PIECE;
-    if (K_CONTIGUOUS) {
-        // a quarter warp = one row's 128 bytes: whole-line reads, 16-byte writes that cover a row
-        const int chunk = threadIdx.x & 7;
-        for (int r = threadIdx.x >> 3; r < TILE; r += 32) {
-            const int i = it * TILE + r, k0 = kb * KB + 4 * chunk;
-            uint32_t h[4], l[4];
+// eight entries -> 16 bytes of hi and 16 of lo
+__device__ __forceinline__ void split8(const float (&v)[8], float scale, uint4 &hi, uint4 &lo) {
+    uint32_t h[4], l[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float v = (i < ni && k0 + u < nk) ? src[(size_t)i * stride_i + (size_t)(k0 + u)] : 0.f;
-                split_tf32(v, h[u], l[u]);
-            }
-            const int off = r * 128 + ((chunk ^ (r & 7)) << 4);
-            *reinterpret_cast<uint4 *>(piece + off) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4 *>(piece + HALF + off) = make_uint4(l[0], l[1], l[2], l[3]);
+    for (int u = 0; u < 4; ++u) {
+        const float a = v[2 * u] * scale, b = v[2 * u + 1] * scale;
+        const __half2 hh = __floats2half2_rn(a, b);
+        const float2 back = __half22float2(hh);
+        const __half2 ll = __floats2half2_rn(a - back.x, b - back.y);
+        h[u] = *reinterpret_cast<const uint32_t *>(&hh);
+        l[u] = *reinterpret_cast<const uint32_t *>(&ll);
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+__device__ __forceinline__ void store_split(unsigned char *piece, int r, int chunk, const uint4 &hi, const uint4 &lo) {
+    const int off = r * 128 + ((chunk ^ (r & 7)) << 4);
+    *reinterpret_cast<uint4 *>(piece + off) = hi;
+    *reinterpret_cast<uint4 *>(piece + HALF + off) = lo;
+}
+// Contraction indices contiguous: a warp per row, once for the largest magnitude, once (out of L1 / L2) for the images; eight lanes write
+// a row's 128 bytes of a K block.
+__global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict__ src, size_t stride_i, int ni, int nk, int nkb,
+                                                         unsigned char *__restrict__ img, float *__restrict__ inv) {
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const float *a = src + (size_t)min(row, ni - 1) * stride_i;
+    const int n = row < ni ? nk : 0;                             // rows behind the matrix are zeros
+    const bool vec = (reinterpret_cast<uintptr_t>(a) & 15u) == 0;
+    float m = 0.f;
+    if (vec) {
+#pragma unroll 4
+        for (int k = lane * 4; k + 4 <= n; k += 128) {
+            const float4 v = *reinterpret_cast<const float4 *>(a + k);
+            m = fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
         }
+        for (int k = (n & ~3) + lane; k < n; k += 32) m = fmaxf(m, fabsf(a[k]));
     } else {
-        // thread = row (consecutive rows are consecutive in memory), two threads per row share its 8 chunks
-        const int r = threadIdx.x & 127, i = it * TILE + r;
-        for (int chunk = threadIdx.x >> 7; chunk < 8; chunk += 2) {
-            const int k0 = kb * KB + 4 * chunk;
-            uint32_t h[4], l[4];
+#pragma unroll 4
+        for (int k = lane; k < n; k += 32) m = fmaxf(m, fabsf(a[k]));
+    }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float v = (i < ni && k0 + u < nk) ? src[(size_t)i + (size_t)(k0 + u) * stride_k] : 0.f;
-                split_tf32(v, h[u], l[u]);
-            }
-            const int off = r * 128 + ((chunk ^ (r & 7)) << 4);
-            *reinterpret_cast<uint4 *>(piece + off) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4 *>(piece + HALF + off) = make_uint4(l[0], l[1], l[2], l[3]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float inverse;
+    const float scale = row_scale(__float_as_uint(m), &inverse);
+    if (lane == 0) inv[row] = inverse;
+    unsigned char *tile = img + (size_t)(row / TILE) * nkb * PIECE;
+    const int r = row % TILE;
+    for (int kb = lane >> 3; kb < nkb; kb += 4) {
+        const int k0 = kb * KB + 8 * (lane & 7);
+        float v[8];
+        if (vec && k0 + 8 <= n) {
+            const float4 x = *reinterpret_cast<const float4 *>(a + k0), y = *reinterpret_cast<const float4 *>(a + k0 + 4);
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = k0 + u < n ? a[k0 + u] : 0.f;
         }
+        uint4 hi, lo;
+        split8(v, scale, hi, lo);
+        store_split(tile + (size_t)kb * PIECE, r, lane & 7, hi, lo);
     }
 }
-
-__device__ __forceinline__ void umma_ss_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+// Rows contiguous (a transposed operand): largest magnitudes by a pass of their own, thread = row, 256 contraction indices per CTA ...
+__global__ void __launch_bounds__(256) column_max_kernel(const float *__restrict__ src, size_t stride_k, int ni, int nk, uint32_t *__restrict__ maxbits) {
+    const int i = blockIdx.x * 256 + threadIdx.x, k0 = blockIdx.y * 256, k1 = min(k0 + 256, nk);
+    if (i >= ni) return;
+    float m = 0.f;
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) m = fmaxf(m, fabsf(src[(size_t)k * stride_k + i]));
+    atomicMax(maxbits + i, __float_as_uint(m));                  // magnitudes order like their bits
 }
-// instruction descriptor: fp32 accumulator, A and B TF32, both K-major, M = 128
-__device__ __forceinline__ uint32_t idesc_tf32(int n) {
-    uint32_t d = 0;
-    d |= 1u << 4;                       // D: fp32
-    d |= 2u << 7;                       // A: tf32
-    d |= 2u << 10;                      // B: tf32
-    d |= (uint32_t)(n >> 3) << 17;      // N
-    d |= (uint32_t)(128 >> 4) << 24;    // M
-    return d;
+// ... then the images, thread = row (consecutive rows are consecutive in memory), two threads per row share its 8 chunks
+__global__ void __launch_bounds__(256) split_columns_kernel(const float *__restrict__ src, size_t stride_k, int ni, int nk, int nkb,
+                                                            unsigned char *__restrict__ img, float *__restrict__ inv, const uint32_t *__restrict__ maxbits) {
+    const int kb = blockIdx.x, it = blockIdx.y;
+    unsigned char *piece = img + ((size_t)it * nkb + kb) * PIECE;
+    const int r = threadIdx.x & 127, i = it * TILE + r;
+    float inverse;
+    const float scale = row_scale(maxbits[i], &inverse);         // (zero behind the matrix)
+    if (kb == 0 && threadIdx.x < TILE) inv[i] = inverse;
+#pragma unroll
+    for (int chunk = threadIdx.x >> 7; chunk < 8; chunk += 2) {
+        const int k0 = kb * KB + 8 * chunk;
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = (i < ni && k0 + u < nk) ? src[(size_t)i + (size_t)(k0 + u) * stride_k] : 0.f;
+        uint4 hi, lo;
+        split8(v, scale, hi, lo);
+        store_split(piece, r, chunk, hi, lo);
+    }
 }
 
 // Persistent: CTA c takes the tiles c, c + gridDim.x, ... (row tile = t / ntn2, so that CTAs running side by side share
@@ -105,7 +148,7 @@ __device__ __forceinline__ uint32_t idesc_tf32(int n) {
 // the number of 128-column tiles of B's images, ntn2 = ceil(ntn / 2) the number of tiles here; an odd last tile has no
 // second half: nothing is copied for it, the products read whatever the buffer holds, and nothing of it is stored.
 __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__restrict__ Aimg, const uint32_t *__restrict__ Bimg,
-                                                            float *__restrict__ C, int n, int r, int nkb, int ntn, int ntn2, int ntiles,
+                                                            const float *__restrict__ Ainv, const float *__restrict__ Binv, float *__restrict__ C, int n, int r, int nkb, int ntn, int ntn2, int ntiles,
                                                             int32_t *__restrict__ status) {
     using namespace tm;
     extern __shared__ unsigned char g3_smem_raw[];
@@ -175,13 +218,17 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
             }
             if (row < n && col0 < r) {
                 float *out = C + (size_t)row * r + col0;
+                const float ri = Ainv[row];
                 if (vec && col0 + TILE <= r) {
 #pragma unroll
-                    for (int e = 0; e < TILE; e += 4) *reinterpret_cast<float4 *>(out + e) = make_float4(sum[e], sum[e + 1], sum[e + 2], sum[e + 3]);
+                    for (int e = 0; e < TILE; e += 4) {
+                        const float4 ci = *reinterpret_cast<const float4 *>(Binv + col0 + e);
+                        *reinterpret_cast<float4 *>(out + e) = make_float4(sum[e] * ri * ci.x, sum[e + 1] * ri * ci.y, sum[e + 2] * ri * ci.z, sum[e + 3] * ri * ci.w);
+                    }
                 } else {
 #pragma unroll
                     for (int e = 0; e < TILE; ++e)
-                        if (col0 + e < r) out[e] = sum[e];
+                        if (col0 + e < r) out[e] = sum[e] * ri * Binv[col0 + e];
                 }
             }
         }
@@ -216,7 +263,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
     } else {
         // ====================================== issuer ======================================
         if (lane == 0) {
-            const uint32_t idesc = idesc_tf32(2 * TILE);
+            const uint32_t idesc = make_idesc_fmt(2 * TILE, 0u);
             bool alive = true;
             int g = 0, it = 0;
             const int nch = nkb > 0 ? (nkb + KCHUNK - 1) / KCHUNK : 1;
@@ -238,12 +285,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                         const uint64_t b_hi = make_smem_desc(stage + (uint32_t)PIECE), b_lo = make_smem_desc(stage + (uint32_t)(2 * PIECE));
                         const bool fresh = kb == ch * KCHUNK;    // the chunk starts on a cleared accumulator
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)           // 8 TF32 = 32 bytes per K step
-                            umma_ss_tf32(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, (!fresh || ks > 0) ? 1u : 0u);
+                        for (int ks = 0; ks < 4; ++ks)           // 16 fp16 = 32 bytes per K step
+                            umma_ss(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, (!fresh || ks > 0) ? 1u : 0u);
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) umma_ss_tf32(d, a_hi + (uint64_t)(2 * ks), b_lo + (uint64_t)(2 * ks), idesc, 1u);
+                        for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_hi + (uint64_t)(2 * ks), b_lo + (uint64_t)(2 * ks), idesc, 1u);
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) umma_ss_tf32(d, a_lo + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
+                        for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_lo + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
                         umma_commit(empty_bar + 8 * s);
                     }
                     if (alive && nkb > 0) umma_commit(acc_full + 8 * as);
@@ -261,16 +308,26 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
 
 }  // namespace g3x
 
+// pieces, then per tile row the inverse scale and the bits of the largest magnitude
+static size_t g3x_pieces(int rows, int depth) { return (size_t)ceil_div(rows, g3x::TILE) * (size_t)ceil_div(depth, g3x::KB) * g3x::PIECE; }
 size_t gemm3x_image_bytes(int64_t rows, int64_t depth) {
-    return (size_t)ceil_div((int)rows, g3x::TILE) * (size_t)ceil_div((int)depth, g3x::KB) * g3x::PIECE;
+    return g3x_pieces((int)rows, (int)depth) + (size_t)ceil_div((int)rows, g3x::TILE) * g3x::TILE * 8;
 }
+static float *g3x_inverse(uint32_t *img, int rows, int depth) { return reinterpret_cast<float *>(reinterpret_cast<char *>(img) + g3x_pieces(rows, depth)); }
 
 // images of an operand with `rows` tile rows and `depth` contraction indices; element (i, k) at src[i * stride_i + k * stride_k]
 mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, int rows, int depth, uint32_t *img, cudaStream_t st) {
-    const dim3 grid(ceil_div(depth, g3x::KB), ceil_div(rows, g3x::TILE));
-    if (stride_k == 1) g3x::split_image_kernel<true><<<grid, 256, 0, st>>>(src, stride_i, stride_k, rows, depth, (int)grid.x, img);
-    else if (stride_i == 1) g3x::split_image_kernel<false><<<grid, 256, 0, st>>>(src, stride_i, stride_k, rows, depth, (int)grid.x, img);
-    else { set_error("gemm3x_split: one of the strides must be 1"); return MDBF_ERR_INVALID_ARG; }
+    const int nkb = ceil_div(depth, g3x::KB), tiles = ceil_div(rows, g3x::TILE);
+    float *inv = g3x_inverse(img, rows, depth);
+    unsigned char *pieces = reinterpret_cast<unsigned char *>(img);
+    if (stride_k == 1) {
+        g3x::split_rows_kernel<<<tiles * (g3x::TILE / 8), 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
+    } else if (stride_i == 1) {
+        uint32_t *maxbits = reinterpret_cast<uint32_t *>(inv + (size_t)tiles * g3x::TILE);
+        MDBF_CUDA(cudaMemsetAsync(maxbits, 0, (size_t)tiles * g3x::TILE * 4, st));
+        g3x::column_max_kernel<<<dim3(ceil_div(rows, 256), ceil_div(depth, 256)), 256, 0, st>>>(src, stride_k, rows, depth, maxbits);
+        g3x::split_columns_kernel<<<dim3(nkb, tiles), 256, 0, st>>>(src, stride_k, rows, depth, nkb, pieces, inv, maxbits);
+    } else { set_error("gemm3x_split: one of the strides must be 1"); return MDBF_ERR_INVALID_ARG; }
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }
@@ -292,8 +349,9 @@ mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, i
         if (dev >= 0 && dev < 64) sms_of_device[dev] = sms;
     }
     const int ntn2 = ceil_div(ntn, 2), ntiles = ntm * ntn2;
-    g3x::gemm3x_kernel<<<std::min(ntiles, std::max(1, sms - spare_sms)), g3x::THREADS, g3x::SMEM, st>>>(Aimg, Bimg, C, n, r, ceil_div(depth, g3x::KB), ntn, ntn2,
-                                                                              ntiles, status);
+    g3x::gemm3x_kernel<<<std::min(ntiles, std::max(1, sms - spare_sms)), g3x::THREADS, g3x::SMEM, st>>>(
+        Aimg, Bimg, g3x_inverse(const_cast<uint32_t *>(Aimg), n, depth), g3x_inverse(const_cast<uint32_t *>(Bimg), r, depth), C, n, r,
+        ceil_div(depth, g3x::KB), ntn, ntn2, ntiles, status);
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }

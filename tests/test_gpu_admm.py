@@ -216,3 +216,25 @@ def test_bench_size_update_on_sampled_rows():
     np.testing.assert_allclose(g["U"][rows], Sg * (g["Ul"][rows] @ g["Vl"].T), atol=2e-5 * scale)
     np.testing.assert_allclose(g["Lam"][rows], Lam[rows].astype(np.float64) + g["tilde"][rows] - g["U"][rows], atol=2e-5 * scale)
     assert np.all(np.isfinite(g["sigma"])) and np.all(np.diff(g["sigma"]) <= 1e-6 * g["sigma"][0])
+
+
+@pytest.mark.parametrize("N,Mc,R,transpose", [(130, 200, 65, False), (257, 129, 128, True), (70, 320, 64, False)])
+def test_rows_of_very_different_scale(N, Mc, R, transpose):
+    """The products scale each operand row by a power of two: rows of W and columns of V across twenty orders of magnitude,
+    rows of zeros and tiny rows among them, against the definition in fp64, row by row."""
+    Wop, V, U, Lam = problem(N, Mc, R, seed=77)
+    rng = np.random.default_rng(3)
+    Wop = (Wop * 10.0 ** rng.uniform(-10, 10, (N, 1))).astype(np.float32)
+    Wop[3] = 0.0
+    Wop[5] *= np.float32(1e-24) / max(np.abs(Wop[5]).max(), 1e-30)
+    U, Lam = np.zeros_like(U), np.zeros_like(Lam)                             # U_tilde = W V (V^T V + rho I)^-1: each row keeps its scale
+    W = np.ascontiguousarray(Wop.T) if transpose else Wop
+    rho = 0.5 * float(np.sum(V.astype(np.float64) ** 2)) / R
+    g = run_update(W, V, U, Lam, rho, 4, 1, 2, transpose)
+    Vd, Wd = V.astype(np.float64), Wop.astype(np.float64)
+    ref = np.linalg.solve(Vd.T @ Vd + rho * np.eye(R), (Wd @ Vd).T).T
+    scale = np.abs(ref).max(axis=1)
+    err = np.abs(g["tilde"] - ref).max(axis=1)
+    # fp32-accurate products and an fp32 factorisation of a system of condition (sigma_max^2 + rho) / rho: the suite's 2e-4 of
+    # the largest entry, here of each row's own
+    assert np.all(err <= 2e-4 * scale + 1e-37), (err / np.maximum(scale, 1e-300)).max()
