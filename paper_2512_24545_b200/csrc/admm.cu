@@ -9,16 +9,14 @@
 //
 // The two dense products (W V and V^T V, once per call) run on the tensor cores at close to fp32 accuracy (gemm3x.cu: scaled
 // fp16 operands in a three-term split); V's operand images serve both, as the right operand of W V and as both operands of
-// V^T V.  The Cholesky factorisation of the R x R system (cuSOLVER) and one triangular solve for the factor's inverse
-// (cuBLAS) are library routines; the inverse of the system is formed and then applied, in every inner iteration, by the
-// same tensor-core product.  Everything
-// specific to the method is this library's own: the MSVID step (mdbf_msvid: sign mask + rank-l envelope on the tensor
+// V^T V.  The Cholesky factorisation of the R x R system (cuSOLVER) is the one library routine; its factor is inverted here by
+// doubling, the inverse of the system is formed and then applied, in every inner iteration, by the same tensor-core product.
+// Everything specific to the method is this library's own: the MSVID step (mdbf_msvid: sign mask + rank-l envelope on the tensor
 // cores), the elementwise passes around it, and the reconstruction of the dense factor from the compact one fused with
 // the dual update.
 //
 // The system is symmetric, so the column-major solver works on the row-major memory as it is; what it calls the lower
 // triangle are the rows above the diagonal here.
-#include <cublas_v2.h>
 #include <cusolverDn.h>
 
 #include <algorithm>
@@ -30,7 +28,6 @@ namespace mdbf {
 namespace admm {
 
 struct Libs {
-    cublasHandle_t blas = nullptr;
     cusolverDnHandle_t solver = nullptr;
     float *potrf_ws = nullptr;          // the factorisation's scratch, as large as the largest request so far
     int potrf_floats = 0;
@@ -43,26 +40,21 @@ static thread_local Libs g_libs;
 static mdbf_status_t get_libs(int device, cudaStream_t st, Libs **out) {
     Libs &L = g_libs;
     if (L.device != device) {
-        if (L.blas) cublasDestroy(L.blas);
         if (L.solver) cusolverDnDestroy(L.solver);
         if (L.potrf_ws) cudaFree(L.potrf_ws);
         if (L.side) cudaStreamDestroy(L.side);
         if (L.fork) cudaEventDestroy(L.fork);
         if (L.join) cudaEventDestroy(L.join);
         L = Libs();
-        if (cublasCreate(&L.blas) != CUBLAS_STATUS_SUCCESS) { L = Libs(); set_error("cublasCreate failed"); return MDBF_ERR_CUDA; }
         if (cusolverDnCreate(&L.solver) != CUSOLVER_STATUS_SUCCESS) {
-            cublasDestroy(L.blas);
             L = Libs();
             set_error("cusolverDnCreate failed");
             return MDBF_ERR_CUDA;
         }
-        cublasSetMathMode(L.blas, CUBLAS_PEDANTIC_MATH);          // plain fp32 products
         if (cudaStreamCreateWithFlags(&L.side, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&L.join, cudaEventDisableTiming) != cudaSuccess ||
-            cublasSetStream(L.blas, L.side) != CUBLAS_STATUS_SUCCESS || cusolverDnSetStream(L.solver, L.side) != CUSOLVER_STATUS_SUCCESS) {
-            cublasDestroy(L.blas);
+            cusolverDnSetStream(L.solver, L.side) != CUSOLVER_STATUS_SUCCESS) {
             cusolverDnDestroy(L.solver);
             if (L.side) cudaStreamDestroy(L.side);
             if (L.fork) cudaEventDestroy(L.fork);
@@ -97,9 +89,110 @@ __global__ void ridge_kernel(float *__restrict__ G, int r, float rho) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < r) G[(size_t)i * r + i] += rho;
 }
-__global__ void identity_kernel(float *__restrict__ X, int r) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x, a = blockIdx.y;
-    if (b < r) X[(size_t)a * r + b] = a == b ? 1.f : 0.f;
+
+// ------------------------------------------------------------------ Y = U^-1, U upper triangular (r x r, row-major)
+// By doubling: the diagonal blocks of TI_LEAF columns are inverted all at once, then neighbouring inverses Y11, Y22 are joined,
+//     [U11 U12]^-1   [Y11  -Y11 U12 Y22]
+//     [     U22]   = [          Y22    ],
+// all pairs of a size in two batched products: log2(r / TI_LEAF) levels instead of the r / 256 dependent steps of a triangular solve
+// with r right-hand sides (r = 3712: 2.6 ms of such steps in the library's solver, 0.5 ms here).  Pairs of blocks of
+// TI_DENSE columns and more go through the tensor-core product.
+constexpr int TI_LEAF = 128, TI_DENSE = 1024;
+constexpr int TI_SMEM = 2 * TI_LEAF * (TI_LEAF + 1) * 4;
+// CTA = one diagonal block, thread = column of the inverse, back substitution: the row of U is the same for the whole warp (a
+// broadcast), the column of Y is the thread's own.  The block's lower triangle is written as zeros.
+__global__ void __launch_bounds__(TI_LEAF) tri_leaf_kernel(const float *__restrict__ U, float *__restrict__ Y, int r) {
+    extern __shared__ float ti_smem[];
+    float (*us)[TI_LEAF + 1] = reinterpret_cast<float (*)[TI_LEAF + 1]>(ti_smem);
+    float (*ys)[TI_LEAF + 1] = us + TI_LEAF;
+    const int o = blockIdx.x * TI_LEAF, j = threadIdx.x, s = min(TI_LEAF, r - o);
+    for (int i = 0; i < TI_LEAF; ++i) us[i][j] = (i < s && j < s && j >= i) ? U[(size_t)(o + i) * r + o + j] : (i == j ? 1.f : 0.f);
+    __syncthreads();
+    for (int i = TI_LEAF - 1; i >= 0; --i) {
+        float a[4] = {i == j ? 1.f : 0.f, 0.f, 0.f, 0.f};
+        int k = i + 1;
+        for (; k + 4 <= TI_LEAF; k += 4)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a[u] = fmaf(-us[i][k + u], ys[k + u][j], a[u]);
+        for (; k < TI_LEAF; ++k) a[0] = fmaf(-us[i][k], ys[k][j], a[0]);
+        ys[i][j] = i <= j ? ((a[0] + a[1]) + (a[2] + a[3])) / us[i][i] : 0.f;
+    }
+    if (j < s)
+        for (int i = 0; i < s; ++i) Y[(size_t)(o + i) * r + o + j] = ys[i][j];
+}
+// One of the two products that join the pairs of blocks of s columns (blockIdx.z = pair): out = A B (FIRST: A = U12, B = Y22; P) or
+// -A B (A = Y11, B = P; Y12), fp32 on the CUDA cores: 64 x 64 tiles, 256 threads of 4 x 4, the triangular operand's zeros skipped.
+template <bool FIRST>
+__global__ void __launch_bounds__(256) tri_join_kernel(const float *__restrict__ A, const float *__restrict__ B, float *__restrict__ out, int r, int s) {
+    __shared__ __align__(16) float as[16][68], bs[16][68];       // [k][row], [k][column]
+    const int o = blockIdx.z * 2 * s, s2 = min(s, r - o - s);
+    const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+    if (j0 >= s2) return;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const float *a = A + (size_t)o * r + (FIRST ? o + s : o);                                // U12 (s x s2) or Y11 (s x s)
+    const float *b = FIRST ? B + (size_t)(o + s) * r + o + s : B + (size_t)o * r + o + s;    // Y22 (s2 x s2) or P (s x s2)
+    const int depth = FIRST ? s2 : s;
+    const int k_lo = FIRST ? 0 : i0, k_hi = FIRST ? min(depth, j0 + 64) : depth;             // Y22[k][j] = 0 for k > j, Y11[i][k] = 0 for k < i
+    float acc[4][4] = {};
+    for (int k0 = k_lo; k0 < k_hi; k0 += 16) {
+        {
+            const int kk = tid & 15;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int row = (tid >> 4) + 16 * u;
+                as[kk][row] = (i0 + row < s && k0 + kk < k_hi) ? a[(size_t)(i0 + row) * r + k0 + kk] : 0.f;
+                const int col = tid & 63, kb = (tid >> 6) + 4 * u;
+                bs[kb][col] = (k0 + kb < k_hi && j0 + col < s2) ? b[(size_t)(k0 + kb) * r + j0 + col] : 0.f;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const float4 x = *reinterpret_cast<const float4 *>(&as[k][4 * ty]), y = *reinterpret_cast<const float4 *>(&bs[k][4 * tx]);
+            const float xa[4] = {x.x, x.y, x.z, x.w}, yb[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xa[p], yb[q], acc[p][q]);
+        }
+        __syncthreads();
+    }
+    float *dst = out + (size_t)o * r + o + s;
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (i0 + 4 * ty + p < s && j0 + 4 * tx + q < s2) dst[(size_t)(i0 + 4 * ty + p) * r + j0 + 4 * tx + q] = FIRST ? acc[p][q] : -acc[p][q];
+}
+// U (upper triangle read) -> Y (r x r, written whole); P: r x r scratch, img: operand images of two r / 2 x r / 2 blocks
+static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *img, int r, int32_t *status, cudaStream_t st) {
+    static PerDeviceOnce once;
+    if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(tri_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TI_SMEM));
+    MDBF_CUDA(cudaMemsetAsync(Y, 0, (size_t)r * r * sizeof(float), st));
+    tri_leaf_kernel<<<ceil_div(r, TI_LEAF), TI_LEAF, TI_SMEM, st>>>(U, Y, r);
+    for (int s = TI_LEAF; s < r; s *= 2) {
+        const int pairs = ceil_div(r - s, 2 * s);                // pairs whose second block is not empty
+        if (s < TI_DENSE) {
+            const dim3 grid(ceil_div(s, 64), ceil_div(s, 64), pairs);
+            tri_join_kernel<true><<<grid, 256, 0, st>>>(U, Y, P, r, s);
+            tri_join_kernel<false><<<grid, 256, 0, st>>>(Y, P, Y, r, s);
+            continue;
+        }
+        for (int p = 0; p < pairs; ++p) {
+            const int o = p * 2 * s, s2 = std::min(s, r - o - s);
+            const size_t d11 = (size_t)o * r + o, d12 = d11 + s, d22 = (size_t)(o + s) * r + o + s;
+            uint32_t *a = img, *b = img + gemm3x_image_bytes(s, s) / 4;
+            mdbf_status_t rc = gemm3x_split(U + d12, (size_t)r, 1, s, s2, a, st);                      // P = U12 Y22
+            if (rc == MDBF_OK) rc = gemm3x_split(Y + d22, 1, (size_t)r, s2, s2, b, st);
+            if (rc == MDBF_OK) rc = gemm3x_run(a, b, G3xOut{P + d12, r, false, nullptr, nullptr}, s, s2, s2, status, st);
+            if (rc == MDBF_OK) rc = gemm3x_split(Y + d11, (size_t)r, 1, s, s, a, st);                  // Y12 = -Y11 P
+            if (rc == MDBF_OK) rc = gemm3x_split(P + d12, 1, (size_t)r, s2, s, b, st);
+            if (rc == MDBF_OK) rc = gemm3x_run(a, b, G3xOut{Y + d12, r, true, nullptr, nullptr}, s, s2, s, status, st);
+            if (rc) return rc;
+        }
+    }
+    MDBF_CUDA(cudaGetLastError());
+    return MDBF_OK;
 }
 // T = B0 + rho (U - Lam)
 __global__ void rhs_kernel(const float *__restrict__ B0, const float *__restrict__ U, const float *__restrict__ Lam, float rho,
@@ -252,8 +345,7 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     // images: op(W)[i][k] = W[i * w_cols + k], or W[k * w_cols + i] when transposed;  V^T[j][k] = V[k * r + j]
     rc = gemm3x_split(V, 1, (size_t)r, ri, mi, w.Vimg, st);
     if (rc) return rc;
-    // Fork.  Side stream: G = V^T V + rho I, its Cholesky factor, L X = I by one triangular solve (X = L^-1, column-major;
-    // read row-major it is Y = L^-T), G^-1 = Y Y^T as a product of Y's images with themselves - the inverse written out,
+    // Fork.  Side stream: G = V^T V + rho I, its Cholesky factor L, Y = L^-T, G^-1 = Y Y^T as a product of Y's images with themselves - the inverse written out,
     // as Eq. admm-U-tilde has it, so that every inner iteration's solve is one product on the tensor cores instead of two
     // triangular solves with N right-hand sides on the FP32 pipe.  Caller's stream meanwhile: W's images and B0 = op(W) V,
     // on all SMs but a few that are left to the solver's small kernels.  Z is free until the loop below.
@@ -270,11 +362,9 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     if (rc) return rc;
     ss = cusolverDnSpotrf(L->solver, CUBLAS_FILL_MODE_LOWER, ri, w.G, ri, L->potrf_ws, L->potrf_floats, w.info);
     if (ss != CUSOLVER_STATUS_SUCCESS) { set_error("%s: cusolverDnSpotrf returned %d", who, (int)ss); return MDBF_ERR_CUDA; }
-    admm::identity_kernel<<<dim3(ceil_div(ri, 256), ri), 256, 0, s2>>>(w.Z, ri);
-    const float one = 1.f;
-    cublasStatus_t bs = cublasStrsm(L->blas, CUBLAS_SIDE_LEFT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, ri, ri, &one,
-                                    w.G, ri, w.Z, ri);
-    if (bs != CUBLAS_STATUS_SUCCESS) { set_error("%s: cublasStrsm returned %d", who, (int)bs); return MDBF_ERR_CUDA; }
+    // the solver's lower triangle is, read row-major, U = L^T; Y = U^-1 = L^-T.  T is free until the loop, Y's images until Y is done
+    rc = admm::tri_inverse(w.G, w.Z, w.T, w.Yimg, ri, w.info + 2, s2);
+    if (rc) return rc;
     rc = gemm3x_split(w.Z, (size_t)r, 1, ri, ri, w.Yimg, s2);
     if (rc == MDBF_OK) rc = gemm3x_run(w.Yimg, w.Yimg, w.G, ri, ri, ri, w.info + 2, s2);
     if (rc) return rc;

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) split_columns_kernel(const float *__restr
 // the number of 128-column tiles of B's images, ntn2 = ceil(ntn / 2) the number of tiles here; an odd last tile has no
 // second half: nothing is copied for it, the products read whatever the buffer holds, and nothing of it is stored.
 __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__restrict__ Aimg, const uint32_t *__restrict__ Bimg,
-                                                            const float *__restrict__ Ainv, const float *__restrict__ Binv, float *__restrict__ C, int n, int r, int nkb, int ntn, int ntn2, int ntiles,
+                                                            const float *__restrict__ Ainv, const float *__restrict__ Binv, const G3xOut o, int n, int r, int nkb, int ntn, int ntn2, int ntiles,
                                                             int32_t *__restrict__ status) {
     using namespace tm;
     extern __shared__ unsigned char g3_smem_raw[];
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
         // thread = one row and one half (128 columns) of the tile; the chunks' sums are added in registers, in fp32
         const int half = warp >> 2;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const bool vec = (r & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0;
+        const bool vec = (o.ldc & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.C) | reinterpret_cast<uintptr_t>(o.add) | reinterpret_cast<uintptr_t>(o.sum)) & 15u) == 0;
         bool alive = true;
         int it = 0;
         const int nch = nkb > 0 ? (nkb + KCHUNK - 1) / KCHUNK : 1;
@@ -217,18 +217,28 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                 if (alive) mbar_arrive(acc_empty + 8 * as);       // the accumulator may be overwritten
             }
             if (row < n && col0 < r) {
-                float *out = C + (size_t)row * r + col0;
-                const float ri = Ainv[row];
+                const size_t at = (size_t)row * o.ldc + col0;
+                float *out = o.C + at;
+                const float ri = o.negate ? -Ainv[row] : Ainv[row];
                 if (vec && col0 + TILE <= r) {
 #pragma unroll
                     for (int e = 0; e < TILE; e += 4) {
                         const float4 ci = *reinterpret_cast<const float4 *>(Binv + col0 + e);
-                        *reinterpret_cast<float4 *>(out + e) = make_float4(sum[e] * ri * ci.x, sum[e + 1] * ri * ci.y, sum[e + 2] * ri * ci.z, sum[e + 3] * ri * ci.w);
+                        const float4 v = make_float4(sum[e] * ri * ci.x, sum[e + 1] * ri * ci.y, sum[e + 2] * ri * ci.z, sum[e + 3] * ri * ci.w);
+                        *reinterpret_cast<float4 *>(out + e) = v;
+                        if (o.sum) {
+                            const float4 a = *reinterpret_cast<const float4 *>(o.add + at + e);
+                            *reinterpret_cast<float4 *>(o.sum + at + e) = make_float4(v.x + a.x, v.y + a.y, v.z + a.z, v.w + a.w);
+                        }
                     }
                 } else {
 #pragma unroll
                     for (int e = 0; e < TILE; ++e)
-                        if (col0 + e < r) out[e] = sum[e] * ri * Binv[col0 + e];
+                        if (col0 + e < r) {
+                            const float v = sum[e] * ri * Binv[col0 + e];
+                            out[e] = v;
+                            if (o.sum) o.sum[at + e] = v + o.add[at + e];
+                        }
                 }
             }
         }
@@ -336,6 +346,11 @@ mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, i
 // to kernels of another stream
 mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, int n, int r, int depth, int32_t *status, cudaStream_t st,
                          int spare_sms) {
+    const G3xOut o = {C, r, false, nullptr, nullptr};
+    return gemm3x_run(Aimg, Bimg, o, n, r, depth, status, st, spare_sms);
+}
+mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, const G3xOut &o, int n, int r, int depth, int32_t *status, cudaStream_t st,
+                         int spare_sms) {
     static PerDeviceOnce once;
     if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(g3x::gemm3x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g3x::SMEM));
     const int ntm = ceil_div(n, g3x::TILE), ntn = ceil_div(r, g3x::TILE);
@@ -350,7 +365,7 @@ mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, i
     }
     const int ntn2 = ceil_div(ntn, 2), ntiles = ntm * ntn2;
     g3x::gemm3x_kernel<<<std::min(ntiles, std::max(1, sms - spare_sms)), g3x::THREADS, g3x::SMEM, st>>>(
-        Aimg, Bimg, g3x_inverse(const_cast<uint32_t *>(Aimg), n, depth), g3x_inverse(const_cast<uint32_t *>(Bimg), r, depth), C, n, r,
+        Aimg, Bimg, g3x_inverse(const_cast<uint32_t *>(Aimg), n, depth), g3x_inverse(const_cast<uint32_t *>(Bimg), r, depth), o, n, r,
         ceil_div(depth, g3x::KB), ntn, ntn2, ntiles, status);
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;

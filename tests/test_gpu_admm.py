@@ -238,3 +238,21 @@ def test_rows_of_very_different_scale(N, Mc, R, transpose):
     # fp32-accurate products and an fp32 factorisation of a system of condition (sigma_max^2 + rho) / rho: the suite's 2e-4 of
     # the largest entry, here of each row's own
     assert np.all(err <= 2e-4 * scale + 1e-37), (err / np.maximum(scale, 1e-300)).max()
+
+
+@pytest.mark.parametrize("R", [1, 127, 128, 129, 257, 384, 1025, 2180])
+def test_inverse_of_the_system_by_doubling(R):
+    """The triangular factor is inverted in diagonal blocks of 128 that are joined pair by pair: a lone ragged block, a pair whose
+    second block is one column, odd numbers of blocks, and pairs that go through the tensor-core product (from 1024 columns).
+    rho is the system's mean diagonal, so its condition number stays near 5 and fp32 rounding (2^-24) in factor, inverse and product,
+    each amplified by it, comes to about 1e-6 of the iterate; the bound is that of the ragged shapes above."""
+    n, m = R + 37, R + 11
+    g = torch.Generator(device="cuda").manual_seed(70 + R)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    W, V, U, Lam = rnd(n, m), rnd(m, R), rnd(n, R), 0.1 * rnd(n, R)
+    rho = float((V.double() ** 2).sum() / R)
+    V8 = V.double()
+    want = torch.linalg.solve(V8.T @ V8 + rho * torch.eye(R, device="cuda", dtype=torch.float64),
+                              (W.double() @ V8 + rho * (U.double() - Lam.double())).T).T
+    got = run_update(W.cpu().numpy(), V.cpu().numpy(), U.cpu().numpy(), Lam.cpu().numpy(), rho, 1, 1, 4)["tilde"]
+    assert np.max(np.abs(got - want.cpu().numpy())) <= 2e-5 * float(want.abs().max())
