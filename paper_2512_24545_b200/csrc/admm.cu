@@ -194,56 +194,60 @@ static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *i
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }
-// T = B0 + rho (U - Lam)
-__global__ void rhs_kernel(const float *__restrict__ B0, const float *__restrict__ U, const float *__restrict__ Lam, float rho,
-                           float *__restrict__ T, size_t count) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-        T[e] = B0[e] + rho * (U[e] - Lam[e]);
-}
-// Z = U_tilde + Lam
-__global__ void sum_kernel(const float *__restrict__ Ut, const float *__restrict__ Lam, float *__restrict__ Z, size_t count) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x) Z[e] = Ut[e] + Lam[e];
-}
-// U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam += U_tilde - U.
-// CTA = 32 rows x 256 columns; thread = column (its row of Vl in registers), the rows' Ul in shared memory.
-constexpr int RC_ROWS = 32, RC_COLS = 256, RC_MAXL = 32;
+// U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam = Z - U with Z = U_tilde + Lam.
+// Bound by memory (Z read, U and Lam written: 12 bytes per entry; 8192 x 3712, l = 16: 99 us against 180 with U_tilde and the old Lam
+// read instead of Z and the products over 32 terms for every l).  CTA = 32 rows x 256 columns; thread = column (its row of Vl in
+// registers), the rows' Ul in shared memory, eight rows' loads in flight together; L = l rounded up to 4, 8, 16 or 32.
+constexpr int RC_ROWS = 32, RC_COLS = 256, RC_BATCH = 8;
+template <int L>
 __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__restrict__ S, const float *__restrict__ Ul,
-                                                             const float *__restrict__ Vl, int l, const float *__restrict__ Ut,
+                                                             const float *__restrict__ Vl, int l, const float *__restrict__ Z,
                                                              float *__restrict__ U, float *__restrict__ Lam, int n, int r, int nwords) {
-    __shared__ float us[RC_ROWS][RC_MAXL];
+    __shared__ __align__(16) float us[RC_ROWS][L];
     const int i0 = blockIdx.y * RC_ROWS;
-    for (int e = threadIdx.x; e < RC_ROWS * RC_MAXL; e += RC_COLS) {
-        const int i = e / RC_MAXL, t = e - i * RC_MAXL;
+    for (int e = threadIdx.x; e < RC_ROWS * L; e += RC_COLS) {
+        const int i = e / L, t = e - i * L;
         us[i][t] = (i0 + i < n && t < l) ? Ul[(size_t)(i0 + i) * l + t] : 0.f;
     }
     __syncthreads();
     const int j = blockIdx.x * RC_COLS + threadIdx.x;
     if (j >= r) return;
-    float v[RC_MAXL];
+    float v[L];
 #pragma unroll
-    for (int t = 0; t < RC_MAXL; ++t) v[t] = t < l ? Vl[(size_t)j * l + t] : 0.f;
-    for (int ib = 0; ib < RC_ROWS && i0 + ib < n; ib += 4) {     // four rows at a time: their loads are in flight together
-        float ut[4], lm[4];
-        uint32_t word[4];
+    for (int t = 0; t < L; ++t) v[t] = t < l ? Vl[(size_t)j * l + t] : 0.f;
+    float z[RC_BATCH];
+    uint32_t word[RC_BATCH];
+    auto load = [&](int ib) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool in = i0 + ib + u < n;
-            const size_t at = (size_t)(i0 + ib + u) * r + j;
-            ut[u] = in ? Ut[at] : 0.f;
-            lm[u] = in ? Lam[at] : 0.f;
-            word[u] = in ? S[(size_t)(i0 + ib + u) * nwords + (j >> 5)] : 0u;
+        for (int u = 0; u < RC_BATCH; ++u) {
+            const int i = min(i0 + ib + u, n - 1);
+            z[u] = Z[(size_t)i * r + j];
+            word[u] = S[(size_t)i * nwords + (j >> 5)];
         }
+    };
+    load(0);
+#pragma unroll 1
+    for (int ib = 0; ib < RC_ROWS && i0 + ib < n; ib += RC_BATCH) {
+        float val[RC_BATCH], lam[RC_BATCH];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (i0 + ib + u >= n) break;
+        for (int u = 0; u < RC_BATCH; ++u) {
             float e = 0.f;
 #pragma unroll
-            for (int t = 0; t < RC_MAXL; ++t) e = fmaf(us[ib + u][t], v[t], e);
-            const float val = ((word[u] >> (j & 31)) & 1u) ? -e : e;
-            const size_t at = (size_t)(i0 + ib + u) * r + j;
-            U[at] = val;
-            Lam[at] = lm[u] + (ut[u] - val);
+            for (int t = 0; t < L; t += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(&us[ib + u][t]);
+                e = fmaf(a.x, v[t], fmaf(a.y, v[t + 1], fmaf(a.z, v[t + 2], fmaf(a.w, v[t + 3], e))));
+            }
+            val[u] = ((word[u] >> (j & 31)) & 1u) ? -e : e;
+            lam[u] = z[u] - val[u];
         }
+        load(ib + RC_BATCH);                                     // the next rows' loads run under these stores
+#pragma unroll
+        for (int u = 0; u < RC_BATCH; ++u)
+            if (i0 + ib + u < n) {
+                const size_t at = (size_t)(i0 + ib + u) * r + j;
+                U[at] = val[u];
+                Lam[at] = lam[u];
+            }
     }
 }
 // a failed factorisation (not expected: the system is positive definite for rho > 0) or an expired wait of the product
@@ -254,7 +258,7 @@ __global__ void flag_kernel(const int *__restrict__ info, float *__restrict__ si
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 struct Scratch {
-    float *B0, *T, *Z, *G;
+    float *B0, *T, *Z, *G;      // T: scratch of the triangular inverse
     uint32_t *Wimg, *Vimg;      // operand images of op(W) (N row tiles, M deep) and of V^T (R row tiles, M deep)
     uint32_t *Yimg;             // images of L^-T (R x R), formed on the side stream while W's are in use
     int *info;                  // [0], [1]: the solver's; [2]: status word of the product kernel
@@ -268,7 +272,7 @@ static mdbf_status_t carve(Scratch *w, char *base, int64_t n, int64_t m, int64_t
     size_t off = 0;
     auto take = [&](size_t bytes) { char *p = base ? base + off : nullptr; off += align256(bytes); return p; };
     float *B0 = (float *)take((size_t)n * r * sizeof(float));
-    float *T = (float *)take((size_t)n * r * sizeof(float));
+    float *T = (float *)take((size_t)r * r * sizeof(float));
     float *Z = (float *)take((size_t)n * r * sizeof(float));
     float *G = (float *)take((size_t)r * r * sizeof(float));
     uint32_t *Wimg = (uint32_t *)take(gemm3x_image_bytes(n, m));
@@ -362,7 +366,7 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     if (rc) return rc;
     ss = cusolverDnSpotrf(L->solver, CUBLAS_FILL_MODE_LOWER, ri, w.G, ri, L->potrf_ws, L->potrf_floats, w.info);
     if (ss != CUSOLVER_STATUS_SUCCESS) { set_error("%s: cusolverDnSpotrf returned %d", who, (int)ss); return MDBF_ERR_CUDA; }
-    // the solver's lower triangle is, read row-major, U = L^T; Y = U^-1 = L^-T.  T is free until the loop, Y's images until Y is done
+    // the solver's lower triangle is, read row-major, U = L^T; Y = U^-1 = L^-T.  Z is free until the loop, Y's images until Y is done
     rc = admm::tri_inverse(w.G, w.Z, w.T, w.Yimg, ri, w.info + 2, s2);
     if (rc) return rc;
     rc = gemm3x_split(w.Z, (size_t)r, 1, ri, ri, w.Yimg, s2);
@@ -376,22 +380,18 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     MDBF_CUDA(cudaStreamWaitEvent(st, L->join, 0));
     rc = gemm3x_split(w.G, (size_t)r, 1, ri, ri, w.Vimg, st);
     if (rc) return rc;
-    const size_t count = (size_t)n * r;
-    const int ew_grid = (int)std::min<size_t>((count + 255) / 256, 148u * 16);
     const int nwords = (int)((r + 31) / 32);
     for (int it = 0; it < n_inner; ++it) {
-        admm::rhs_kernel<<<ew_grid, 256, 0, st>>>(w.B0, U, Lambda, rho, w.T, count);
-        // U_tilde = T G^-1, over T's own memory (its images live where W's were)
-        rc = gemm3x_split(w.T, (size_t)r, 1, ni, ri, w.Wimg, st);
-        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, w.T, ni, ri, ri, w.info + 2, st);
+        // Z = U_tilde + Lam, U_tilde = (B0 + rho (U - Lam)) G^-1: the right-hand side goes straight into images (where W's were), Lam is
+        // added on the way out; U_tilde itself is written only where the caller wants the last one
+        rc = gemm3x_split_rhs(w.B0, U, Lambda, rho, ni, ri, w.Wimg, st);
+        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, G3xOut{it == n_inner - 1 ? U_tilde : nullptr, ri, false, Lambda, w.Z}, ni, ri, ri, w.info + 2, st);
         if (rc) return rc;
-        admm::sum_kernel<<<ew_grid, 256, 0, st>>>(w.T, Lambda, w.Z, count);
         rc = mdbf_msvid(w.Z, n, r, l, n_iter, Q0, S_packed, Ul, Vl, sigma, w.msvid, w.msvid_bytes, stream);
         if (rc) return rc;
-        admm::recon_dual_kernel<<<dim3(ceil_div(ri, admm::RC_COLS), ceil_div(ni, admm::RC_ROWS)), admm::RC_COLS, 0, st>>>(
-            S_packed, Ul, Vl, l, w.T, U, Lambda, ni, ri, nwords);
+        auto recon = l <= 4 ? admm::recon_dual_kernel<4> : l <= 8 ? admm::recon_dual_kernel<8> : l <= 16 ? admm::recon_dual_kernel<16> : admm::recon_dual_kernel<32>;
+        recon<<<dim3(ceil_div(ri, admm::RC_COLS), ceil_div(ni, admm::RC_ROWS)), admm::RC_COLS, 0, st>>>(S_packed, Ul, Vl, l, w.Z, U, Lambda, ni, ri, nwords);
     }
-    if (U_tilde) MDBF_CUDA(cudaMemcpyAsync(U_tilde, w.T, count * sizeof(float), cudaMemcpyDeviceToDevice, st));
     admm::flag_kernel<<<1, 32, 0, st>>>(w.info, sigma, l);                      // the factorisation's flag or an expired wait
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;

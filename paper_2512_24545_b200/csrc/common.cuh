@@ -109,8 +109,9 @@ mdbf_status_t require_device(int *dev_out);
 // fp32-accurate dense product on the tensor cores (gemm3x.cu): operand images, then C = A B
 size_t gemm3x_image_bytes(int64_t rows, int64_t depth);
 mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, int rows, int depth, uint32_t *img, cudaStream_t st);
+mdbf_status_t gemm3x_split_rhs(const float *B0, const float *U, const float *Lam, float rho, int rows, int depth, uint32_t *img, cudaStream_t st);
 struct G3xOut {
-    float *C;                     // row-major, ldc entries from row to row
+    float *C;                     // row-major, ldc entries from row to row; may be null where `sum` is all that is wanted
     int ldc;
     bool negate;                  // C = -A B
     const float *add;             // with `sum`: sum = C + add, both laid out as C

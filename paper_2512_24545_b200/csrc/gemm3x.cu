@@ -67,47 +67,93 @@ __device__ __forceinline__ void store_split(unsigned char *piece, int r, int chu
     *reinterpret_cast<uint4 *>(piece + off) = hi;
     *reinterpret_cast<uint4 *>(piece + HALF + off) = lo;
 }
-// Contraction indices contiguous: a warp per row, once for the largest magnitude, once (out of L1 / L2) for the images; eight lanes write
-// a row's 128 bytes of a K block.
-__global__ void __launch_bounds__(256) split_rows_kernel(const float *__restrict__ src, size_t stride_i, int ni, int nk, int nkb,
-                                                         unsigned char *__restrict__ img, float *__restrict__ inv) {
-    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    const float *a = src + (size_t)min(row, ni - 1) * stride_i;
-    const int n = row < ni ? nk : 0;                             // rows behind the matrix are zeros
-    const bool vec = (reinterpret_cast<uintptr_t>(a) & 15u) == 0;
-    float m = 0.f;
-    if (vec) {
-#pragma unroll 4
-        for (int k = lane * 4; k + 4 <= n; k += 128) {
-            const float4 v = *reinterpret_cast<const float4 *>(a + k);
-            m = fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
-        }
-        for (int k = (n & ~3) + lane; k < n; k += 32) m = fmaxf(m, fabsf(a[k]));
-    } else {
-#pragma unroll 4
-        for (int k = lane; k < n; k += 32) m = fmaxf(m, fabsf(a[k]));
+// What a row is read from: a matrix, or the right-hand side of the refinement's system, B0 + rho (U - Lam) (Eq. admm-U-tilde), which
+// this way is never written out.
+struct RowsOf {
+    const float *src;
+    __device__ __forceinline__ bool vec(size_t at) const { return (reinterpret_cast<uintptr_t>(src + at) & 15u) == 0; }
+    __device__ __forceinline__ float at(size_t e) const { return src[e]; }
+    __device__ __forceinline__ float4 at4(size_t e) const { return *reinterpret_cast<const float4 *>(src + e); }
+};
+struct RowsOfRhs {
+    const float *b0, *u, *lam;
+    float rho;
+    __device__ __forceinline__ bool vec(size_t at) const {
+        return ((reinterpret_cast<uintptr_t>(b0 + at) | reinterpret_cast<uintptr_t>(u + at) | reinterpret_cast<uintptr_t>(lam + at)) & 15u) == 0;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float inverse;
-    const float scale = row_scale(__float_as_uint(m), &inverse);
-    if (lane == 0) inv[row] = inverse;
-    unsigned char *tile = img + (size_t)(row / TILE) * nkb * PIECE;
-    const int r = row % TILE;
-    for (int kb = lane >> 3; kb < nkb; kb += 4) {
-        const int k0 = kb * KB + 8 * (lane & 7);
-        float v[8];
+    __device__ __forceinline__ float at(size_t e) const { return b0[e] + rho * (u[e] - lam[e]); }
+    __device__ __forceinline__ float4 at4(size_t e) const {
+        const float4 b = *reinterpret_cast<const float4 *>(b0 + e), x = *reinterpret_cast<const float4 *>(u + e), y = *reinterpret_cast<const float4 *>(lam + e);
+        return make_float4(b.x + rho * (x.x - y.x), b.y + rho * (x.y - y.y), b.z + rho * (x.z - y.z), b.w + rho * (x.w - y.w));
+    }
+};
+// Contraction indices contiguous: CTA = row, NV chunks of eight entries per thread stay in registers between the search for the largest
+// magnitude and the split, so that the source is read once (what a longer row has beyond them is read twice); eight lanes write a
+// row's 128 bytes of a K block.
+// Bound by memory: the right-hand side of 8192 x 3712 in 67 us (16 bytes per entry, 7.3 TB/s with what L2 still holds), 87 + 60 us as a
+// pass of its own and a split that read its row twice.
+template <class SRC, int NV>
+__global__ void __launch_bounds__(256) split_rows_kernel(const SRC src, size_t stride_i, int ni, int nk, int nkb,
+                                                         unsigned char *__restrict__ img, float *__restrict__ inv) {
+    __shared__ float warp_max[8];
+    const int row = blockIdx.x, tid = threadIdx.x;
+    const size_t base = (size_t)min(row, ni - 1) * stride_i;
+    const int n = row < ni ? nk : 0;                             // rows behind the matrix are zeros
+    const bool vec = src.vec(base);
+    auto load = [&](int chunk, float (&v)[8]) {
+        const int k0 = 8 * chunk;
         if (vec && k0 + 8 <= n) {
-            const float4 x = *reinterpret_cast<const float4 *>(a + k0), y = *reinterpret_cast<const float4 *>(a + k0 + 4);
+            const float4 x = src.at4(base + k0), y = src.at4(base + k0 + 4);
             v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
         } else {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = k0 + u < n ? a[k0 + u] : 0.f;
+            for (int u = 0; u < 8; ++u) v[u] = k0 + u < n ? src.at(base + k0 + u) : 0.f;
         }
-        uint4 hi, lo;
-        split8(v, scale, hi, lo);
-        store_split(tile + (size_t)kb * PIECE, r, lane & 7, hi, lo);
+    };
+    float v[NV][8], m = 0.f;
+#pragma unroll
+    for (int c = 0; c < NV; ++c) load(tid + 256 * c, v[c]);
+#pragma unroll
+    for (int c = 0; c < NV; ++c)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m = fmaxf(m, fabsf(v[c][u]));
+    for (int chunk = tid + 256 * NV; 8 * chunk < n; chunk += 256) {
+        float x[8];
+        load(chunk, x);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m = fmaxf(m, fabsf(x[u]));
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31) == 0) warp_max[tid >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) m = fmaxf(m, warp_max[w]);
+    float inverse;
+    const float scale = row_scale(__float_as_uint(m), &inverse);
+    if (tid == 0) inv[row] = inverse;
+    unsigned char *tile = img + (size_t)(row / TILE) * nkb * PIECE;
+    const int r = row % TILE;
+    auto store = [&](int chunk, const float (&x)[8]) {
+        uint4 hi, lo;
+        split8(x, scale, hi, lo);
+        store_split(tile + (size_t)(chunk >> 3) * PIECE, r, chunk & 7, hi, lo);
+    };
+#pragma unroll
+    for (int c = 0; c < NV; ++c)
+        if (tid + 256 * c < 8 * nkb) store(tid + 256 * c, v[c]);
+    for (int chunk = tid + 256 * NV; chunk < 8 * nkb; chunk += 256) {
+        float x[8];
+        load(chunk, x);
+        store(chunk, x);
+    }
+}
+template <class SRC>
+static void launch_split_rows(const SRC &src, size_t stride_i, int rows, int depth, int nkb, int tiles, unsigned char *pieces, float *inv, cudaStream_t st) {
+    const int grid = tiles * TILE;
+    if (nkb <= 32) split_rows_kernel<SRC, 1><<<grid, 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
+    else if (nkb <= 64) split_rows_kernel<SRC, 2><<<grid, 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
+    else split_rows_kernel<SRC, 4><<<grid, 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
 }
 // Rows contiguous (a transposed operand): largest magnitudes by a pass of their own, thread = row, 256 contraction indices per CTA ...
 __global__ void __launch_bounds__(256) column_max_kernel(const float *__restrict__ src, size_t stride_k, int ni, int nk, uint32_t *__restrict__ maxbits) {
@@ -218,17 +264,22 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
             }
             if (row < n && col0 < r) {
                 const size_t at = (size_t)row * o.ldc + col0;
-                float *out = o.C + at;
                 const float ri = o.negate ? -Ainv[row] : Ainv[row];
                 if (vec && col0 + TILE <= r) {
 #pragma unroll
-                    for (int e = 0; e < TILE; e += 4) {
-                        const float4 ci = *reinterpret_cast<const float4 *>(Binv + col0 + e);
-                        const float4 v = make_float4(sum[e] * ri * ci.x, sum[e + 1] * ri * ci.y, sum[e + 2] * ri * ci.z, sum[e + 3] * ri * ci.w);
-                        *reinterpret_cast<float4 *>(out + e) = v;
+                    for (int e0 = 0; e0 < TILE; e0 += 32) {      // eight loads of the addend in flight: 8192 x 3712, 566 us without it: +30, +85 one at a time
+                        float4 a[8];
                         if (o.sum) {
-                            const float4 a = *reinterpret_cast<const float4 *>(o.add + at + e);
-                            *reinterpret_cast<float4 *>(o.sum + at + e) = make_float4(v.x + a.x, v.y + a.y, v.z + a.z, v.w + a.w);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) a[q] = *reinterpret_cast<const float4 *>(o.add + at + e0 + 4 * q);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const int e = e0 + 4 * q;
+                            const float4 ci = *reinterpret_cast<const float4 *>(Binv + col0 + e);
+                            const float4 v = make_float4(sum[e] * ri * ci.x, sum[e + 1] * ri * ci.y, sum[e + 2] * ri * ci.z, sum[e + 3] * ri * ci.w);
+                            if (o.C) *reinterpret_cast<float4 *>(o.C + at + e) = v;
+                            if (o.sum) *reinterpret_cast<float4 *>(o.sum + at + e) = make_float4(v.x + a[q].x, v.y + a[q].y, v.z + a[q].z, v.w + a[q].w);
                         }
                     }
                 } else {
@@ -236,7 +287,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                     for (int e = 0; e < TILE; ++e)
                         if (col0 + e < r) {
                             const float v = sum[e] * ri * Binv[col0 + e];
-                            out[e] = v;
+                            if (o.C) o.C[at + e] = v;
                             if (o.sum) o.sum[at + e] = v + o.add[at + e];
                         }
                 }
@@ -331,13 +382,20 @@ mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, i
     float *inv = g3x_inverse(img, rows, depth);
     unsigned char *pieces = reinterpret_cast<unsigned char *>(img);
     if (stride_k == 1) {
-        g3x::split_rows_kernel<<<tiles * (g3x::TILE / 8), 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
+        g3x::launch_split_rows(g3x::RowsOf{src}, stride_i, rows, depth, nkb, tiles, pieces, inv, st);
     } else if (stride_i == 1) {
         uint32_t *maxbits = reinterpret_cast<uint32_t *>(inv + (size_t)tiles * g3x::TILE);
         MDBF_CUDA(cudaMemsetAsync(maxbits, 0, (size_t)tiles * g3x::TILE * 4, st));
         g3x::column_max_kernel<<<dim3(ceil_div(rows, 256), ceil_div(depth, 256)), 256, 0, st>>>(src, stride_k, rows, depth, maxbits);
         g3x::split_columns_kernel<<<dim3(nkb, tiles), 256, 0, st>>>(src, stride_k, rows, depth, nkb, pieces, inv, maxbits);
     } else { set_error("gemm3x_split: one of the strides must be 1"); return MDBF_ERR_INVALID_ARG; }
+    MDBF_CUDA(cudaGetLastError());
+    return MDBF_OK;
+}
+
+mdbf_status_t gemm3x_split_rhs(const float *B0, const float *U, const float *Lam, float rho, int rows, int depth, uint32_t *img, cudaStream_t st) {
+    g3x::launch_split_rows(g3x::RowsOfRhs{B0, U, Lam, rho}, (size_t)depth, rows, depth, ceil_div(depth, g3x::KB), ceil_div(rows, g3x::TILE),
+                           reinterpret_cast<unsigned char *>(img), g3x_inverse(img, rows, depth), st);
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }
