@@ -356,7 +356,8 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     cudaStream_t s2 = L->side;
     MDBF_CUDA(cudaEventRecord(L->fork, st));
     MDBF_CUDA(cudaStreamWaitEvent(s2, L->fork, 0));
-    rc = gemm3x_run(w.Vimg, w.Vimg, w.G, ri, ri, mi, w.info + 2, s2);
+    // the solver reads one triangle: half of V^T V; Y is triangular: a third of the products of Y Y^T
+    rc = gemm3x_run(w.Vimg, w.Vimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_UPPER}, ri, ri, mi, w.info + 2, s2);
     if (rc) return rc;
     admm::ridge_kernel<<<ceil_div(ri, 256), 256, 0, s2>>>(w.G, ri, rho);
     int lwork = 0;
@@ -370,7 +371,7 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     rc = admm::tri_inverse(w.G, w.Z, w.T, w.Yimg, ri, w.info + 2, s2);
     if (rc) return rc;
     rc = gemm3x_split(w.Z, (size_t)r, 1, ri, ri, w.Yimg, s2);
-    if (rc == MDBF_OK) rc = gemm3x_run(w.Yimg, w.Yimg, w.G, ri, ri, ri, w.info + 2, s2);
+    if (rc == MDBF_OK) rc = gemm3x_run(w.Yimg, w.Yimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_FACTORS}, ri, ri, ri, w.info + 2, s2);
     if (rc) return rc;
     MDBF_CUDA(cudaEventRecord(L->join, s2));
     rc = transpose_w ? gemm3x_split(W, 1, (size_t)w_cols, ni, mi, w.Wimg, st) : gemm3x_split(W, (size_t)w_cols, 1, ni, mi, w.Wimg, st);

@@ -110,12 +110,16 @@ mdbf_status_t require_device(int *dev_out);
 size_t gemm3x_image_bytes(int64_t rows, int64_t depth);
 mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, int rows, int depth, uint32_t *img, cudaStream_t st);
 mdbf_status_t gemm3x_split_rhs(const float *B0, const float *U, const float *Lam, float rho, int rows, int depth, uint32_t *img, cudaStream_t st);
+// G3X_UPPER: a symmetric result, only the tiles on and above the diagonal are formed.  G3X_FACTORS: both operands are upper triangular
+// (rows of A and columns of B zero before the diagonal), the products start at the diagonal.
+enum G3xPart { G3X_ALL, G3X_UPPER, G3X_FACTORS };
 struct G3xOut {
     float *C;                     // row-major, ldc entries from row to row; may be null where `sum` is all that is wanted
     int ldc;
     bool negate;                  // C = -A B
     const float *add;             // with `sum`: sum = C + add, both laid out as C
     float *sum;
+    int part = G3X_ALL;
 };
 mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, int n, int r, int depth, int32_t *status, cudaStream_t st,
                          int spare_sms = 0);

@@ -185,6 +185,22 @@ __global__ void __launch_bounds__(256) split_columns_kernel(const float *__restr
     }
 }
 
+// Tile t of the walk: row tile by row tile; of a symmetric result only the tiles that reach the diagonal or lie above it.
+__device__ __forceinline__ void tile_of(int t, int ntn2, int part, int &mt, int &nt2) {
+    if (part != G3X_UPPER) {
+        mt = t / ntn2;
+        nt2 = t - mt * ntn2;
+        return;
+    }
+    int p = 0;                                                   // row tiles 2p and 2p + 1 start at column tile p
+    while (t >= 2 * (ntn2 - p)) { t -= 2 * (ntn2 - p); ++p; }
+    const int second = t >= ntn2 - p;
+    mt = 2 * p + second;
+    nt2 = p + t - (second ? ntn2 - p : 0);
+}
+// first K block with anything in it: rows of upper triangular operands are zero before the diagonal
+__device__ __forceinline__ int first_kb(int part, int mt, int nt2) { return part == G3X_FACTORS ? max(mt * TILE, nt2 * 2 * TILE) / KB : 0; }
+
 // Persistent: CTA c takes the tiles c, c + gridDim.x, ... (row tile = t / ntn2, so that CTAs running side by side share
 // their pieces of A in L2).  Two accumulators of 256 tensor-memory columns alternate between tiles: the epilogue of
 // one tile runs under the products of the next.  All three terms of a tile accumulate into the same columns, for KCHUNK
@@ -235,9 +251,10 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
         const bool vec = (o.ldc & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.C) | reinterpret_cast<uintptr_t>(o.add) | reinterpret_cast<uintptr_t>(o.sum)) & 15u) == 0;
         bool alive = true;
         int it = 0;
-        const int nch = nkb > 0 ? (nkb + KCHUNK - 1) / KCHUNK : 1;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-            const int mt = t / ntn2, nt2 = t - mt * ntn2;
+            int mt, nt2;
+            tile_of(t, ntn2, o.part, mt, nt2);
+            const int nk = nkb - first_kb(o.part, mt, nt2), nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
             const int row = mt * TILE + (warp & 3) * 32 + lane;
             const int col0 = nt2 * 2 * TILE + half * TILE;
             float sum[TILE];
@@ -246,7 +263,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                 if (alive) alive = mbar_wait(acc_full + 8 * as, ((uint32_t)(it >> 1)) & 1u, abort_flag, status);
                 alive = __all_sync(0xffffffffu, alive);
                 tc_fence_after();
-                if (alive && nkb > 0) {
+                if (alive && nk > 0) {
 #pragma unroll
                     for (int j = 0; j < TILE / 16; ++j) {
                         uint32_t d[16];
@@ -299,11 +316,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
             bool alive = true;
             int g = 0;                                           // K blocks issued so far, over all of this CTA's tiles
             for (int t = blockIdx.x; t < ntiles && alive; t += gridDim.x) {
-                const int mt = t / ntn2, nt2 = t - mt * ntn2;
+                int mt, nt2;
+                tile_of(t, ntn2, o.part, mt, nt2);
                 const bool two = 2 * nt2 + 1 < ntn;              // the tile has a second column tile
                 const uint32_t *a_src = Aimg + (size_t)mt * nkb * (PIECE / 4);
                 const uint32_t *b0_src = Bimg + (size_t)(2 * nt2) * nkb * (PIECE / 4), *b1_src = b0_src + (size_t)nkb * (PIECE / 4);
-                for (int kb = 0; kb < nkb && alive; ++kb, ++g) {
+                for (int kb = first_kb(o.part, mt, nt2); kb < nkb && alive; ++kb, ++g) {
                     const int s = g % STAGES;
                     alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(g / STAGES)) & 1u) ^ 1u, abort_flag, status);
                     if (!alive) break;
@@ -327,16 +345,18 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
             const uint32_t idesc = make_idesc_fmt(2 * TILE, 0u);
             bool alive = true;
             int g = 0, it = 0;
-            const int nch = nkb > 0 ? (nkb + KCHUNK - 1) / KCHUNK : 1;
             for (int t = blockIdx.x; t < ntiles && alive; t += gridDim.x) {
+                int mt, nt2;
+                tile_of(t, ntn2, o.part, mt, nt2);
+                const int kb0 = first_kb(o.part, mt, nt2), nk = nkb - kb0, nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
                 for (int ch = 0; ch < nch && alive; ++ch, ++it) {
                     const int as = it & 1;
                     alive = mbar_wait(acc_empty + 8 * as, (((uint32_t)(it >> 1)) & 1u) ^ 1u, abort_flag, status);
                     if (!alive) break;
                     tc_fence_after();
                     const uint32_t d = tmem + (uint32_t)(as * 2 * TILE);
-                    const int kb_end = min(nkb, (ch + 1) * KCHUNK);
-                    for (int kb = ch * KCHUNK; kb < kb_end && alive; ++kb, ++g) {
+                    const int kb_begin = kb0 + ch * KCHUNK, kb_end = min(nkb, kb_begin + KCHUNK);
+                    for (int kb = kb_begin; kb < kb_end && alive; ++kb, ++g) {
                         const int s = g % STAGES;
                         alive = mbar_wait(full_bar + 8 * s, ((uint32_t)(g / STAGES)) & 1u, abort_flag, status);
                         if (!alive) break;
@@ -344,7 +364,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                         const uint32_t stage = smem_base + (uint32_t)(s * STAGE_BYTES);
                         const uint64_t a_hi = make_smem_desc(stage), a_lo = make_smem_desc(stage + (uint32_t)HALF);
                         const uint64_t b_hi = make_smem_desc(stage + (uint32_t)PIECE), b_lo = make_smem_desc(stage + (uint32_t)(2 * PIECE));
-                        const bool fresh = kb == ch * KCHUNK;    // the chunk starts on a cleared accumulator
+                        const bool fresh = kb == kb_begin;         // the chunk starts on a cleared accumulator
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)           // 16 fp16 = 32 bytes per K step
                             umma_ss(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, (!fresh || ks > 0) ? 1u : 0u);
@@ -354,7 +374,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                         for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_lo + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
                         umma_commit(empty_bar + 8 * s);
                     }
-                    if (alive && nkb > 0) umma_commit(acc_full + 8 * as);
+                    if (alive && nk > 0) umma_commit(acc_full + 8 * as);
                     else mbar_arrive(acc_full + 8 * as);
                 }
             }
@@ -404,7 +424,7 @@ mdbf_status_t gemm3x_split_rhs(const float *B0, const float *U, const float *Lam
 // to kernels of another stream
 mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, int n, int r, int depth, int32_t *status, cudaStream_t st,
                          int spare_sms) {
-    const G3xOut o = {C, r, false, nullptr, nullptr};
+    const G3xOut o = {C, r, false, nullptr, nullptr, G3X_ALL};
     return gemm3x_run(Aimg, Bimg, o, n, r, depth, status, st, spare_sms);
 }
 mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, const G3xOut &o, int n, int r, int depth, int32_t *status, cudaStream_t st,
@@ -421,7 +441,13 @@ mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, const G3xOu
         MDBF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (dev >= 0 && dev < 64) sms_of_device[dev] = sms;
     }
-    const int ntn2 = ceil_div(ntn, 2), ntiles = ntm * ntn2;
+    const int ntn2 = ceil_div(ntn, 2);
+    if (o.part != G3X_ALL && (n != r || (o.part == G3X_FACTORS && depth != n))) { set_error("gemm3x_run: a symmetric result is square"); return MDBF_ERR_INVALID_ARG; }
+    int ntiles = ntm * ntn2;
+    if (o.part == G3X_UPPER) {
+        ntiles = 0;
+        for (int mt = 0; mt < ntm; ++mt) ntiles += ntn2 - mt / 2;
+    }
     g3x::gemm3x_kernel<<<std::min(ntiles, std::max(1, sms - spare_sms)), g3x::THREADS, g3x::SMEM, st>>>(
         Aimg, Bimg, g3x_inverse(const_cast<uint32_t *>(Aimg), n, depth), g3x_inverse(const_cast<uint32_t *>(Bimg), r, depth), o, n, r,
         ceil_div(depth, g3x::KB), ntn, ntn2, ntiles, status);
