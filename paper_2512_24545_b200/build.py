@@ -1,4 +1,5 @@
-"""Build libmdbf.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Build libmdbf.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and mdbf_calls.so beside it: the forward calls as
+a CPython extension module.
 
     python -m paper_2512_24545_b200.build [--force] [--verbose] [--bounds-check]
 
@@ -12,11 +13,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmdbf.so")
+CALLS = os.path.join(HERE, "mdbf_calls.so")
 SOURCES = ["mdbf_api.cu", "pack.cu", "reconstruct.cu", "forward_alu.cu", "forward_prefill.cu", "forward_tmem_t1.cu", "forward_t1.cu", "forward_static.cu", "forward_mat.cu", "msvid.cu", "gemm3x.cu", "admm.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -38,7 +41,8 @@ def _newest_source() -> float:
 def build(force: bool = False, verbose: bool = False, bounds_check: bool | None = None) -> str:
     variant = "bounds-check" if _bounds_check_requested(bounds_check) else "default"
     on_disk = open(STAMP).read().strip() if os.path.exists(STAMP) else "default"
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source() and on_disk == variant:
+    newest = _newest_source()
+    if not force and on_disk == variant and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, CALLS)):
         return LIB
     flags = NVCC_FLAGS + (["-DMDBF_BOUNDS_CHECK"] if variant == "bounds-check" else [])
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -63,6 +67,8 @@ def build(force: bool = False, verbose: bool = False, bounds_check: bool | None 
         raise RuntimeError("nvcc failed")
     subprocess.check_call([nvcc, "-shared", "-o", LIB, *objs, "-lcudart", "-lcusolver",
                            "-Xlinker", "-rpath=/usr/local/cuda/lib64"])
+    subprocess.check_call(["gcc", "-shared", "-fPIC", "-O2", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+                           "-o", CALLS, os.path.join(CSRC, "pycalls.c"), "-L", HERE, "-l:libmdbf.so", "-Wl,-rpath,$ORIGIN"])
     with open(STAMP, "w") as f:
         f.write(variant + "\n")
     return LIB

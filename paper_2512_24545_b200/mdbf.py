@@ -1,5 +1,5 @@
-"""ctypes binding of libmdbf.so — same names as include/mdbf.h, argument
-marshalling only.  Every computation runs in the CUDA library; there is no
+"""Binding of libmdbf.so — same names as include/mdbf.h, argument marshalling
+only: by ctypes, and by an extension module (mdbf_calls.so) for the forward calls.  Every computation runs in the CUDA library; there is no
 fallback: if the library has not been built or no sm_100 device is present the
 calls raise.
 
@@ -10,6 +10,8 @@ host buffers as numpy arrays.  Streams are raw cudaStream_t integers
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from typing import Optional
 
@@ -17,6 +19,7 @@ import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmdbf.so")
+CALLS_PATH = os.path.join(_HERE, "mdbf_calls.so")
 
 F32, F16, BF16 = 0, 1, 2
 KERNEL_AUTO, KERNEL_ALU, KERNEL_PREFILL, KERNEL_TMEM, KERNEL_MAT, KERNEL_I8 = 0, 1, 3, 4, 5, 6
@@ -48,6 +51,7 @@ class Desc(ctypes.Structure):
 
 
 _lib: Optional[ctypes.CDLL] = None
+_calls = None
 
 
 def lib() -> ctypes.CDLL:
@@ -100,6 +104,21 @@ def lib() -> ctypes.CDLL:
     L.mdbf_debug_fail_alloc.restype = None
     _lib = L
     return L
+
+
+def calls():
+    """The forward calls' extension module, loaded with the library it links to."""
+    global _calls
+    if _calls is None:
+        lib()
+        if not os.path.exists(CALLS_PATH):
+            raise RuntimeError(f"{CALLS_PATH} is missing: build it with `python -m paper_2512_24545_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("mdbf_calls", CALLS_PATH)
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("mdbf_calls", loader))
+        loader.exec_module(module)
+        module.set_addr(_addr)
+        _calls = module
+    return _calls
 
 
 def last_error() -> str:
@@ -163,31 +182,30 @@ def mdbf_set_kernel(h: int, kernel: int) -> None:
 
 
 def mdbf_linear_forward(h: int, x, y, T: int, act_dtype: int, stream: int = 0) -> None:
-    _check(lib().mdbf_linear_forward(h, _addr(x), _addr(y), T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward(h, x, y, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 def mdbf_linear_forward_sum(handles, x, y, acc, T: int, act_dtype: int, stream: int = 0) -> None:
     """y = sum_p W_hat^(p) x over the given layer handles; acc is a device float32 T x d_out scratch."""
-    arr = (ctypes.c_void_p * len(handles))(*handles)
-    _check(lib().mdbf_linear_forward_sum(ctypes.cast(arr, ctypes.c_void_p), len(handles), _addr(x), _addr(y), _addr(acc),
-                                         T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward_sum(handles, x, y, acc, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 def mdbf_linear_forward_siblings(handles, x, ys, T: int, act_dtype: int, stream: int = 0) -> None:
     """ys[i] = W_hat_i x for layers that share the input x (q/k/v, gate/up); ys are device addresses."""
-    hs = (ctypes.c_void_p * len(handles))(*handles)
-    outs = (ctypes.c_void_p * len(ys))(*[_addr(y) for y in ys])
-    _check(lib().mdbf_linear_forward_siblings(ctypes.cast(hs, ctypes.c_void_p), len(handles), _addr(x),
-                                              ctypes.cast(outs, ctypes.c_void_p), T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward_siblings(handles, x, ys, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 def mdbf_linear_forward_group(handles, xs, ys, T: int, act_dtype: int, stream: int = 0) -> None:
     """ys[i] = W_hat_i xs[i] for independent layers (own inputs); xs, ys are device addresses."""
-    hs = (ctypes.c_void_p * len(handles))(*handles)
-    ins = (ctypes.c_void_p * len(xs))(*[_addr(x) for x in xs])
-    outs = (ctypes.c_void_p * len(ys))(*[_addr(y) for y in ys])
-    _check(lib().mdbf_linear_forward_group(ctypes.cast(hs, ctypes.c_void_p), len(handles), ctypes.cast(ins, ctypes.c_void_p),
-                                           ctypes.cast(outs, ctypes.c_void_p), T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward_group(handles, xs, ys, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 def mdbf_prepare_host_staging(h: int) -> None:
@@ -196,12 +214,16 @@ def mdbf_prepare_host_staging(h: int) -> None:
 
 
 def mdbf_linear_forward_host(h: int, x_host, y_host, T: int, act_dtype: int, stream: int = 0) -> None:
-    _check(lib().mdbf_linear_forward_host(h, _addr(x_host), _addr(y_host), T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward_host(h, x_host, y_host, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 def mdbf_linear_forward_host_async(h: int, x_host, y_host, T: int, act_dtype: int, stream: int = 0) -> None:
     """Host buffers, no synchronisation: y_host is valid once the caller has synchronised `stream`."""
-    _check(lib().mdbf_linear_forward_host_async(h, _addr(x_host), _addr(y_host), T, act_dtype, stream))
+    status = (_calls or calls()).linear_forward_host_async(h, x_host, y_host, T, act_dtype, stream)
+    if status:
+        _check(status)
 
 
 STATIC_MAX_KT = 262144
