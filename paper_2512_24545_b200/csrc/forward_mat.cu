@@ -127,6 +127,19 @@ __device__ __forceinline__ void mt_expand_half(const uint32_t (&v)[32], uint32_t
         }
     }
 }
+// the same for 16 columns, `half` their 16 sign bits
+__device__ __forceinline__ void mt_expand16(const uint32_t (&v)[16], uint32_t half, uint32_t (&o)[8]) {
+#pragma unroll
+    for (int c2 = 0; c2 < 2; ++c2) {
+        const uint32_t byte = (half >> (8 * c2)) & 0xFFu;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int col = c2 * 8 + 2 * i;
+            const uint32_t e = tm::pack_bf16x2(__uint_as_float(v[col]), __uint_as_float(v[col + 1]));
+            o[c2 * 4 + i] = e ^ ((byte * (0x40008000u >> (2 * i))) & 0x80008000u);
+        }
+    }
+}
 // Barriers tested together, so that the latencies of the tests overlap.
 __device__ __forceinline__ bool mt_wait2(uint32_t bar_a, uint32_t par_a, uint32_t bar_b, uint32_t par_b,
                                          volatile int *abort_flag, int32_t *status) {
@@ -477,18 +490,23 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
 }
 
 // ------------------------------------------------------------------ tiles of at most 64 tokens
-// With few tokens the tensor pipe is idle and the per-pair chains of the single-thread roles and of the
-// builders set the pace, so this variant runs TWO pipelines side by side: pairs of K blocks alternate
-// between two halves g = pair & 1, each with its own envelope buffer (128 TMEM columns), W_hat tile slot,
-// group of 8 builder warps (a warp: one block of the pair, 32 rows, all 64 columns), main-MMA issuer and
-// accumulator; the epilogue adds the two accumulators.  Loaders and the mini-MMA issuer are shared.
-// TMEM: D0 0..63, D1 64..127, W_hat slots 128 + 64 g, envelope buffers 256 + 128 g.
-constexpr int MS_W_TMA = MT_XWARPS;
-constexpr int MS_W_MMA0 = MT_XWARPS + 1;
-constexpr int MS_W_ENV = MT_XWARPS + 2;
-constexpr int MS_W_MINI = MT_XWARPS + 3;
-constexpr int MS_W_MMA1 = MT_XWARPS + 4;
-constexpr int MS_THREADS = (MS_W_MMA1 + 1) * 32;
+// With few tokens the tensor pipe is idle and the chain of a pair of K blocks - envelope mini-MMA, tile builders, main MMA - sets the
+// pace, so this variant keeps two or three pairs in flight: pair p works in buffer p % nb of tensor memory, which holds the pair's
+// envelope values (fp32, 128 columns) and then, over those that a builder warp has read, its part of the W_hat tile (a warp: one block of
+// the pair, 32 rows, 64 columns of values -> 32 packed ones).  A buffer has its own group of 8 builder warps, its own main-MMA
+// issuer and its own accumulator; the epilogue adds the accumulators.  Loaders and the mini-MMA issuer are shared; the issuing warps run
+// converged (see elect_one).
+// TMEM: accumulators 0..127 (three of 32 columns up to 32 tokens, two of 64 above: then three buffers no longer fit), buffers 128 + 128 g.
+// What bounds it: the issue slots of a busy SM and the mini-MMA issuer.  11008 x 3968, 16 tokens: 0.36 us a pair, 0.47 with
+// single-lane issuers; per forward 4096 -> 3968 -> 11008: 16 tokens 25.8 -> 20.6 us, 64 tokens 27.0 -> 24.4; 1723 x 2312, k = 877, 37 tokens
+// 13.2 -> 11.5.  (Two CTAs of one pipeline each per SM: 25.2 and 18.3, the second because a CTA's few pairs run one after the other.)
+constexpr int MS_BUFS = 3;
+constexpr int MS_XWARPS = 8 * MS_BUFS;
+constexpr int MS_W_TMA = MS_XWARPS;
+constexpr int MS_W_ENV = MS_XWARPS + 1;
+constexpr int MS_W_MINI = MS_XWARPS + 2;
+constexpr int MS_W_MMA0 = MS_XWARPS + 3;
+constexpr int MS_THREADS = (MS_W_MMA0 + MS_BUFS) * 32;
 constexpr int MS_BN = 64;
 
 template <bool STAGE_A, bool SPLIT>
@@ -496,12 +514,12 @@ __global__ void __launch_bounds__(MS_THREADS, 1)
 mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
     using namespace tm;
     extern __shared__ unsigned char mt_smem_raw[];
-    __shared__ __align__(8) uint64_t bars[MT_MAX_NS + MT_MAX_NS / 2 + 8 + 2 * MT_MAX_NV + 2];
+    __shared__ __align__(8) uint64_t bars[MT_MAX_NS + MT_MAX_NS / 2 + 3 * MS_BUFS + 2 * MT_MAX_NV + 2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t smem_base = (smem_u32(mt_smem_raw) + 1023u) & ~1023u;
     unsigned char *smem_gen = mt_smem_raw + (smem_base - smem_u32(mt_smem_raw));
     const int nbp = a.ns / 2, nv = a.nv;
@@ -511,11 +529,10 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
     const uint32_t v_smem = u_smem + img_bytes;
     const uint32_t bfull_bar = smem_u32(&bars[0]);                  // per activation tile
     const uint32_t bempty_bar = bfull_bar + 8 * MT_MAX_NS;          // per pair of activation tiles
-    const uint32_t afull_bar = bempty_bar + 8 * (MT_MAX_NS / 2);    // [2] per half
-    const uint32_t aempty_bar = afull_bar + 16;
-    const uint32_t efull_bar = aempty_bar + 16;
-    const uint32_t eempty_bar = efull_bar + 16;
-    const uint32_t vfull_bar = eempty_bar + 16;
+    const uint32_t efull_bar = bempty_bar + 8 * (MT_MAX_NS / 2);    // per buffer: envelope values written,
+    const uint32_t afull_bar = efull_bar + 8 * MS_BUFS;             // W_hat tile written,
+    const uint32_t free_bar = afull_bar + 8 * MS_BUFS;              // W_hat tile read by the main MMAs
+    const uint32_t vfull_bar = free_bar + 8 * MS_BUFS;
     const uint32_t vempty_bar = vfull_bar + 8 * MT_MAX_NV;
     const uint32_t accum_bar = vempty_bar + 8 * MT_MAX_NV;
     const uint32_t u_bar = accum_bar + 8;
@@ -528,21 +545,21 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
     const int kb0 = SPLIT ? (int)crank * 2 * a.ppc : 0;
     const int nkb = SPLIT ? max(0, min(2 * a.ppc, nkb_total - kb0)) : nkb_total;
     const int npr = (nkb + 1) / 2;
+    const int nb = a.bn <= 32 ? MS_BUFS : 2, d_cols = a.bn <= 32 ? 32 : 64;      // buffers in use, columns of an accumulator
 
     if (tid == 0) {
         for (int s = 0; s < MT_MAX_NS; ++s) mbar_init(bfull_bar + 8 * s, 1);
         for (int s = 0; s < MT_MAX_NS / 2; ++s) mbar_init(bempty_bar + 8 * s, 1);
-        for (int g = 0; g < 2; ++g) {
-            mbar_init(afull_bar + 8 * g, MT_XWARPS / 2);            // one arrival per builder warp of the half
-            mbar_init(aempty_bar + 8 * g, 1);
+        for (int g = 0; g < MS_BUFS; ++g) {
             mbar_init(efull_bar + 8 * g, 1);
-            mbar_init(eempty_bar + 8 * g, MT_XWARPS / 2);
+            mbar_init(afull_bar + 8 * g, 8);                        // one arrival per builder warp of the buffer
+            mbar_init(free_bar + 8 * g, 1);
         }
         for (int v = 0; v < MT_MAX_NV; ++v) {
             mbar_init(vfull_bar + 8 * v, 1);
             mbar_init(vempty_bar + 8 * v, 1);
         }
-        mbar_init(accum_bar, 2);                                    // both main-MMA issuers
+        mbar_init(accum_bar, (uint32_t)nb);                         // every main-MMA issuer
         mbar_init(u_bar, 1);
         abort_flag_s = 0;
         fence_barrier_init();
@@ -554,9 +571,9 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_slot;                   // + 64 g
-    const uint32_t tmem_a = tmem_base_slot + 2 * MS_BN;       // + 64 g
-    const uint32_t tmem_e = tmem_base_slot + 256;             // + 128 g
+    const uint32_t tmem_base = warp_uniform(tmem_base_slot);
+    const uint32_t tmem_d = tmem_base;                   // + 64 g
+    const uint32_t tmem_buf = tmem_base + 2 * MS_BN;     // + 128 g
     pdl_launch_dependents();
     if (SPLIT) cluster.barrier_arrive();                      // see mat_stage_kernel
 
@@ -566,40 +583,31 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
         const int arow = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint2 *wp = a.wk2 + ((size_t)rb * a.kb_pad + kb0) * MT_BM + arow;       // + kb * 128
+        const int step = 2 * nb;                                                       // K blocks from one pair of the group to its next
         const int kbf = 2 * g + blk;                                                   // this warp's first block
         uint2 w_next = kbf < nkb ? __ldg(wp + (size_t)kbf * MT_BM) : make_uint2(0u, 0u);
-        uint2 w_next2 = kbf + 4 < nkb ? __ldg(wp + (size_t)(kbf + 4) * MT_BM) : make_uint2(0u, 0u);
+        uint2 w_next2 = kbf + step < nkb ? __ldg(wp + (size_t)(kbf + step) * MT_BM) : make_uint2(0u, 0u);
+        const uint32_t col = tmem_buf + (uint32_t)(g * 128 + blk * 64) + lane_base;
         bool alive = true;
-        for (int i = 0; 2 * i + g < npr && alive; ++i) {
-            const int kb = 2 * (2 * i + g) + blk;
-            const uint32_t ph = (uint32_t)i & 1u;
+        for (int i = 0; g < nb && nb * i + g < npr && alive; ++i) {
+            const int kb = kbf + step * i;
             const uint2 w = w_next;
             w_next = w_next2;
-            w_next2 = kb + 8 < nkb ? __ldg(wp + (size_t)(kb + 8) * MT_BM) : make_uint2(0u, 0u);
-            alive = mbar_wait(efull_bar + 8 * g, ph, abort_flag, a.status);
+            w_next2 = kb + 2 * step < nkb ? __ldg(wp + (size_t)(kb + 2 * step) * MT_BM) : make_uint2(0u, 0u);
+            alive = mbar_wait(efull_bar + 8 * g, (uint32_t)i & 1u, abort_flag, a.status);
             if (!alive) break;
             tc_fence_after();
-            uint32_t o0[16], o1[16];
-            {
-                uint32_t v[32];
-                tmem_ld32(tmem_e + (uint32_t)(g * 128 + blk * 64) + lane_base, v);
-                tmem_ld_wait();
-                mt_expand_half(v, w.x, o0);
-                tmem_ld32(tmem_e + (uint32_t)(g * 128 + blk * 64 + 32) + lane_base, v);
-                tmem_ld_wait();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(eempty_bar + 8 * g);
-                mt_expand_half(v, w.y, o1);
+            // 16 values at a time: the next load runs under the expansion; the packed columns lie over values read before
+            uint32_t v[2][16], o[8];
+            tmem_ld16(col, v[0]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q < 3) tmem_ld16(col + 16u * (q + 1), v[(q + 1) & 1]);
+                mt_expand16(v[q & 1], (q & 2 ? w.y : w.x) >> (16 * (q & 1)), o);
+                if (q < 3) tmem_ld_wait();
+                tmem_st8(col + 8u * q, o);
             }
-            alive = mbar_wait(aempty_bar + 8 * g, ph ^ 1u, abort_flag, a.status);
-            if (!alive) break;
-            tc_fence_after();
-            const uint32_t a_col = tmem_a + (uint32_t)(g * 64 + blk * 32) + lane_base;
-            tmem_st8(a_col, *reinterpret_cast<const uint32_t (*)[8]>(&o0[0]));
-            tmem_st8(a_col + 8, *reinterpret_cast<const uint32_t (*)[8]>(&o0[8]));
-            tmem_st8(a_col + 16, *reinterpret_cast<const uint32_t (*)[8]>(&o1[0]));
-            tmem_st8(a_col + 24, *reinterpret_cast<const uint32_t (*)[8]>(&o1[8]));
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
@@ -607,7 +615,7 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
         }
 
         // ================================= epilogue ==================================
-        // the four warps of a lane quadrant take 16 tokens each; out = D0 + D1
+        // 16 tokens per warp of a lane quadrant; out = D0 + D1
         const int egrow = row0 + arow;
         const int chunk = warp >> 2;
         if (alive) alive = mbar_wait(accum_bar, 0u, abort_flag, a.status);
@@ -617,15 +625,9 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc[j] = 0.f;
         if (alive && chunk * 16 < a.bn) {
-            uint32_t v[16];
-            if (npr > 0) {
-                tmem_ld16(tmem_d + lane_base + (uint32_t)(chunk * 16), v);
-                tmem_ld_wait();
-#pragma unroll
-                for (int j = 0; j < 16; ++j) acc[j] = __uint_as_float(v[j]);
-            }
-            if (npr > 1) {
-                tmem_ld16(tmem_d + MS_BN + lane_base + (uint32_t)(chunk * 16), v);
+            for (int d = 0; d < nb && d < npr; ++d) {
+                uint32_t v[16];
+                tmem_ld16(tmem_d + (uint32_t)(d * d_cols) + lane_base + (uint32_t)(chunk * 16), v);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 16; ++j) acc[j] += __uint_as_float(v[j]);
@@ -662,7 +664,7 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
             cluster.sync();
             if (alive && !*abort_flag) {
                 const int nranks = (int)cluster.num_blocks();
-                for (int slot = chunk; slot < a.tpr; slot += 4) {
+                for (int slot = chunk; slot < a.tpr; slot += MS_XWARPS / 4) {
                     const int t = (int)crank * a.tpr + slot;
                     if (t >= a.bn || t >= a.T || egrow >= a.rows) continue;
                     float sum = 0.f;
@@ -716,55 +718,61 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
         }
         __syncwarp();
     } else if (warp == MS_W_MINI) {
-        // ======================= envelope mini-MMA issuer, buffers alternate =======================
-        if (lane == 0) {
-            const uint32_t idesc_mini = make_idesc_fmt(2 * MT_BK, a.env_fmt);
-            bool alive = mbar_wait(u_bar, 0u, abort_flag, a.status);
-            int vb = 0;
-            uint32_t vph = 0;
-            for (int p = 0; p < npr && alive; ++p) {
-                const int g = p & 1;
-                alive = mt_wait2(vfull_bar + 8 * vb, vph, eempty_bar + 8 * g, ((uint32_t)(p >> 1) & 1u) ^ 1u, abort_flag, a.status);
-                if (!alive) break;
-                tc_fence_after();
+        // ======================= envelope mini-MMA issuer =======================
+        const uint32_t idesc_mini = make_idesc_fmt(2 * MT_BK, a.env_fmt);
+        bool alive = __all_sync(0xffffffffu, mbar_wait(u_bar, 0u, abort_flag, a.status));
+        int vb = 0, g = 0;
+        uint32_t vph = 0, gph = 1;
+        for (int p = 0; p < npr && alive; ++p) {
+            alive = __all_sync(0xffffffffu, mt_wait2(vfull_bar + 8 * vb, vph, free_bar + 8 * g, gph, abort_flag, a.status));
+            if (!alive) break;
+            tc_fence_after();
+            if (elect_one()) {
                 for (int q = 0; q < a.kc / 2; ++q) {
                     const uint64_t ud = make_smem_desc_plain(u_smem + (uint32_t)q * 4096u, 2048u, 128u);
                     const uint64_t vd = make_smem_desc_plain(v_smem + (uint32_t)vb * img_bytes + (uint32_t)q * 4096u, 2048u, 128u);
-                    umma_ss(tmem_e + (uint32_t)(g * 128), ud, vd, idesc_mini, q > 0 ? 1u : 0u);
+                    umma_ss(tmem_buf + (uint32_t)(g * 128), ud, vd, idesc_mini, q > 0 ? 1u : 0u);
                 }
                 umma_commit(efull_bar + 8 * g);
                 umma_commit(vempty_bar + 8 * vb);
-                if (++vb == nv) { vb = 0; vph ^= 1u; }
             }
+            __syncwarp();
+            if (++vb == nv) { vb = 0; vph ^= 1u; }
+            if (++g == nb) { g = 0; gph ^= 1u; }
         }
-        __syncwarp();
     } else {
-        // ===================== main MMA issuers: issuer g takes the pairs p = g, g + 2, ... =====================
-        const int g = warp == MS_W_MMA0 ? 0 : 1;
-        if (lane == 0) {
-            const uint32_t idesc_main = make_idesc(a.bn);
-            bool alive = true;
-            int it = 0;
-            for (int p = g; p < npr && alive; p += 2, ++it) {
-                const int bp = p % nbp;
-                const uint32_t bph = (uint32_t)(p / nbp) & 1u, aph = (uint32_t)it & 1u;
-                const int s0 = 2 * bp;
-                const bool two = 2 * p + 1 < nkb;
-                alive = two ? mt_wait3(afull_bar + 8 * g, aph, bfull_bar + 8 * s0, bph, bfull_bar + 8 * (s0 + 1), bph, abort_flag, a.status)
-                            : mt_wait2(afull_bar + 8 * g, aph, bfull_bar + 8 * s0, bph, abort_flag, a.status);
-                if (!alive) break;
-                tc_fence_after();
-                for (int h = 0; h < (two ? 2 : 1); ++h) {
-                    const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(s0 + h) * b_bytes);
-                    const uint32_t a_t = tmem_a + (uint32_t)(g * 64 + h * 32);
+        // ===================== main MMA issuers: issuer g takes the pairs p = g, g + nb, ... =====================
+        const int g = warp - MS_W_MMA0;
+        const uint32_t idesc_main = make_idesc(a.bn);
+        const uint32_t d_t = tmem_d + (uint32_t)(g * d_cols), a_t = tmem_buf + (uint32_t)(g * 128);
+        bool alive = true;
+        int it = 0, bp = g;                                      // a ring of nbp pairs, a multiple of nb
+        uint32_t bph = 0;
+        for (int p = g; g < nb && p < npr && alive; p += nb, ++it) {
+            const int s0 = 2 * bp;
+            const bool two = 2 * p + 1 < nkb;
+            const uint32_t aph = (uint32_t)it & 1u;
+            alive = __all_sync(0xffffffffu, two ? mt_wait3(afull_bar + 8 * g, aph, bfull_bar + 8 * s0, bph, bfull_bar + 8 * (s0 + 1), bph, abort_flag, a.status)
+                                                : mt_wait2(afull_bar + 8 * g, aph, bfull_bar + 8 * s0, bph, abort_flag, a.status));
+            if (!alive) break;
+            tc_fence_after();
+            const uint64_t b0 = make_smem_desc(smem_base + (uint32_t)s0 * b_bytes), b1 = make_smem_desc(smem_base + (uint32_t)(s0 + 1) * b_bytes);
+            if (elect_one()) {
 #pragma unroll
-                    for (int k4 = 0; k4 < MT_BK / 16; ++k4)
-                        umma_ts(tmem_d + (uint32_t)(g * MS_BN), a_t + (uint32_t)(8 * k4), bdesc + (uint64_t)(2 * k4), idesc_main,
-                                (it > 0 || h > 0 || k4 > 0) ? 1u : 0u);
+                for (int k4 = 0; k4 < MT_BK / 16; ++k4)
+                    umma_ts(d_t, a_t + (uint32_t)(8 * k4), b0 + (uint64_t)(2 * k4), idesc_main, (it > 0 || k4 > 0) ? 1u : 0u);
+                if (two) {
+#pragma unroll
+                    for (int k4 = 0; k4 < MT_BK / 16; ++k4) umma_ts(d_t, a_t + (uint32_t)(64 + 8 * k4), b1 + (uint64_t)(2 * k4), idesc_main, 1u);
                 }
-                umma_commit(aempty_bar + 8 * g);
+                umma_commit(free_bar + 8 * g);
                 umma_commit(bempty_bar + 8 * bp);
             }
+            __syncwarp();
+            bp += nb;
+            if (bp >= nbp) { bp -= nbp; bph ^= 1u; }
+        }
+        if (g < nb && elect_one()) {
             if (alive && it > 0) umma_commit(accum_bar); else mbar_arrive(accum_bar);
         }
         __syncwarp();
@@ -935,6 +943,9 @@ static mdbf_status_t launch_mat(const MatArgs &a0, int large_ks, const CUtensorM
         if (small) part_bytes = (size_t)ks * a.tpr * MT_BM * sizeof(float);       // (the large tiles put them into the activation ring)
     }
     a.ns = mt_ring(a.kc, a.nv, a.bn, part_bytes);
+    // A parity test cannot tell phase n from phase n - 2, so an issuer has to have seen the last phase of every barrier it waits on: a ring
+    // slot must come back to the issuer that used it, whether two or three take turns.
+    if (small && a.ns != MT_MAX_NS) { set_error("materialised-envelope kernel: a ring of %d activation tiles instead of %d", a.ns, MT_MAX_NS); return MDBF_ERR_SHAPE; }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(rb, ceil_div(a.T, a.bn), ks);
     cfg.blockDim = dim3(small ? MS_THREADS : MT_THREADS);

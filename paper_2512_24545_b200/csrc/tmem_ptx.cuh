@@ -80,6 +80,17 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
 }
+// One lane of a converged warp, the same one every time.  The issuing roles run their loops with the whole warp and enter only the MMAs and
+// commits through this: the operands then stay in uniform registers, whereas in a loop that a single lane runs every operand of every
+// MMA is moved there first (about 105 cycles an MMA, 300 for the mini-MMA and its two commits; a pair of K blocks of the
+// small-tile kernel took 0.47 us that way and takes 0.36 this way).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t q;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(q));
+    return q != 0u;
+}
+// a value that is the same in every lane, so that the compiler knows
+template <class T> __device__ __forceinline__ T warp_uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
