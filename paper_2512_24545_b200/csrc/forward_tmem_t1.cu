@@ -117,7 +117,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
     const bool stage_a = a.stage_a != 0;
 
     cg::cluster_group cluster = cg::this_cluster();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t smem_base = (smem_u32(tx_smem_raw) + 1023u) & ~1023u;
     unsigned char *smem_gen = tx_smem_raw + (smem_base - smem_u32(tx_smem_raw));
     const int nas = a.nastages, nss = a.nsstages;
@@ -189,7 +189,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
     __syncthreads();
     tc_fence_after();
     pdl_launch_dependents();
-    const uint32_t tmem = tmem_base_slot;
+    const uint32_t tmem = warp_uniform(tmem_base_slot);
     const uint32_t tmem_a0 = tmem + (uint32_t)(TX_ISSUERS * NB);
 
     float outv = 0.f;
@@ -348,13 +348,13 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
             }
         for (int pr = w; pr < npr && alive; pr += TX_ISSUERS, ++it) {
             alive = tx_wait(v_full + 8 * as, as_ph, abort_flag, a.status);
-            if (!alive) break;
-            alive = tx_wait(a_full + 8 * as, as_ph, abort_flag, a.status);
+            if (alive) alive = tx_wait(a_full + 8 * as, as_ph, abort_flag, a.status);
+            alive = __all_sync(0xffffffffu, alive);
             if (!alive) break;
             tc_fence_after();
-            if (lane == 0) {
-                const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(as * VBYTES));
-                const uint32_t a_t = tmem_a0 + (uint32_t)(as * 64);
+            const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(as * VBYTES));
+            const uint32_t a_t = tmem_a0 + (uint32_t)(as * 64);
+            if (elect_one()) {
 #pragma unroll
                 for (int k8 = 0; k8 < 8; ++k8)               // K block k8 / 4 of the pair, 16 k per MMA
                     umma_ts(d_tmem, a_t + (uint32_t)(8 * k8), bdesc + (uint64_t)((k8 >> 2) * (NB * 128 / 16) + 2 * (k8 & 3)), idesc,
@@ -365,7 +365,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
             as += TX_ISSUERS;
             while (as >= nas) { as -= nas; as_ph ^= 1u; }
         }
-        if (lane == 0) {
+        if (elect_one()) {
             if (alive && it > 0) umma_commit(acc_bar);       // arrives when this issuer's MMAs have retired
             else mbar_arrive(acc_bar);
         }
