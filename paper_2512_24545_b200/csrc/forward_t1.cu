@@ -417,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) t1_stage_kernel(const __grid_cons
     __shared__ unsigned long long cs_s[32];
     volatile int *abort_flag = &abort_flag_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = tm::warp_uniform(tid >> 5), lane = tid & 31;
     const int cta = blockIdx.x;
     const uint32_t smem_base = (smem_u32(t1_smem_raw) + 1023u) & ~1023u;
     unsigned char *smem_gen = t1_smem_raw + (smem_base - smem_u32(t1_smem_raw));
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1) t1_stage_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_slot;
+    const uint32_t tmem = warp_uniform(tmem_base_slot);
     const uint32_t tmem_a0 = tmem + (uint32_t)(4 * NB);         // A stages: [row block j][NAG][32 columns]
 
     pdl_launch_dependents();
@@ -688,25 +688,25 @@ __global__ void __launch_bounds__(kThreads, 1) t1_stage_kernel(const __grid_cons
         Seg sg;
         while (alive && it.next(g, sg)) {
             const bool valid = k < sg.nrb;
-            alive = bwait(acc_empty, (uint32_t)nseg_done & 1u, abort_flag, status0);   // accumulators read and cleared
+            alive = __all_sync(0xffffffffu, bwait(acc_empty, (uint32_t)nseg_done & 1u, abort_flag, status0));   // accumulators read and cleared
             if (!alive) break;
             int issued = 0;
             for (int p = sg.p0; p < sg.p1 && alive; ++p, ++qn) {
                 if ((qn & 1) != par) continue;
                 const int is = qn % NIM;
-                alive = bwait(i_full + 8 * is, (uint32_t)(qn / NIM) & 1u, abort_flag, status0);
+                alive = __all_sync(0xffffffffu, bwait(i_full + 8 * is, (uint32_t)(qn / NIM) & 1u, abort_flag, status0));
                 if (!alive) break;
                 if (!valid) {                                    // no such row block: only release the image (after this issuer's earlier MMAs)
-                    if (lane == 0) umma_commit(i_empty + 8 * is);
+                    if (elect_one()) umma_commit(i_empty + 8 * is);
                     __syncwarp();
                     continue;
                 }
-                alive = bwait(a_full + 8 * (k * NAG + par), ause & 1u, abort_flag, status0);
+                alive = __all_sync(0xffffffffu, bwait(a_full + 8 * (k * NAG + par), ause & 1u, abort_flag, status0));
                 if (!alive) break;
                 tc_fence_after();
-                if (lane == 0) {
-                    const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(is * IMG));
-                    const uint32_t a_t = tmem_a0 + (uint32_t)((k * NAG + par) * 32);
+                const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(is * IMG));
+                const uint32_t a_t = tmem_a0 + (uint32_t)((k * NAG + par) * 32);
+                if (elect_one()) {
 #pragma unroll
                     for (int q = 0; q < 4; ++q)                  // 32 K positions (bytes) per MMA
                         umma_ts_i8(d_tmem, a_t + (uint32_t)(8 * q), bdesc + (uint64_t)(2 * q), idesc, 1u);
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kThreads, 1) t1_stage_kernel(const __grid_cons
                 ++issued;
                 ++ause;
             }
-            if (lane == 0) {
+            if (elect_one()) {
                 if (alive && issued > 0) umma_commit(acc_full);  // arrives when this issuer's MMAs have retired
                 else mbar_arrive(acc_full);
             }
