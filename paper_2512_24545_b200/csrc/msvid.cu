@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t smem_base = (smem_u32(tc_smem_raw) + 1023u) & ~1023u;
     unsigned char *smem_gen = tc_smem_raw + (smem_base - smem_u32(tc_smem_raw));
     const uint32_t img_base = smem_base + (uint32_t)(TC_RAW * TC_TILE);
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_slot;
+    const uint32_t tmem = warp_uniform(tmem_base_slot);
     const uint32_t tmem_a0 = tmem + (uint32_t)C::ACC_COLS;       // A stage s: columns [64 s, 64 s + 32) = E_hi, the next 32 = E_lo
 
     if (warp < TC_CONVERTERS / 32) {
@@ -388,22 +388,27 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
     } else if (warp == TC_W_ISSUE || warp == TC_W_ISSUE + 1) {
         // ================================== MMA issuers ===================================
         const bool first = warp == TC_W_ISSUE;                   // first: D1 = E_hi [q_hi | q_lo]; second: D2 = E_lo q_hi
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_tf32(first ? N1 : N2);
-            const uint32_t d_tmem = tmem + (first ? 0u : (uint32_t)N1);
-            bool alive = true;
-            for (int kb = 0; kb < nkb && alive; ++kb) {
-                const int s = kb % TC_STAGES;
-                alive = mbar_wait(full_bar + 8 * s, ((uint32_t)(kb / TC_STAGES)) & 1u, abort_flag, status);
-                if (!alive) break;
-                tc_fence_after();
-                const uint32_t a_t = tmem_a0 + (uint32_t)(s * 64) + (first ? 0u : 32u);
-                const uint64_t bdesc = make_smem_desc(img_base + (uint32_t)(s * C::IMG));
+        const uint32_t idesc = make_idesc_tf32(first ? N1 : N2);
+        const uint32_t d_tmem = tmem + (first ? 0u : (uint32_t)N1);
+        bool alive = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int kb = 0; kb < nkb && alive; ++kb) {
+            alive = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * s, ph, abort_flag, status));
+            if (!alive) break;
+            tc_fence_after();
+            const uint32_t a_t = tmem_a0 + (uint32_t)(s * 64) + (first ? 0u : 32u);
+            const uint64_t bdesc = make_smem_desc(img_base + (uint32_t)(s * C::IMG));
+            if (elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)                   // 8 TF32 per K step: 8 TMEM columns of A, 32 bytes of B
                     umma_ts_tf32(d_tmem, a_t + (uint32_t)(8 * ks), bdesc + (uint64_t)(2 * ks), idesc, (kb > 0 || ks > 0) ? 1u : 0u);
                 umma_commit(empty_bar + 8 * s);                  // frees the A stage and the image together
             }
+            __syncwarp();
+            if (++s == TC_STAGES) { s = 0; ph ^= 1u; }
+        }
+        if (elect_one()) {
             if (alive && nkb > 0) umma_commit(accum_bar);
             else mbar_arrive(accum_bar);
         }
