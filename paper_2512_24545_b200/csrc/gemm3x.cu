@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t smem_base = (smem_u32(g3_smem_raw) + 1023u) & ~1023u;
     const uint32_t full_bar = smem_u32(&bars[0]), empty_bar = smem_u32(&bars[STAGES]);
     const uint32_t acc_full = smem_u32(&bars[2 * STAGES]), acc_empty = smem_u32(&bars[2 * STAGES + 2]);
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base_slot;
+    const uint32_t tmem = warp_uniform(tmem_base_slot);
 
     if (warp < EPI_WARPS) {
         // ===================================== epilogue =====================================
@@ -341,30 +341,30 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
         __syncwarp();
     } else {
         // ====================================== issuer ======================================
-        if (lane == 0) {
-            const uint32_t idesc = make_idesc_fmt(2 * TILE, 0u);
-            bool alive = true;
-            int g = 0, it = 0;
-            for (int t = blockIdx.x; t < ntiles && alive; t += gridDim.x) {
-                int mt, nt2;
-                tile_of(t, ntn2, o.part, mt, nt2);
-                const int kb0 = first_kb(o.part, mt, nt2), nk = nkb - kb0, nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
-                for (int ch = 0; ch < nch && alive; ++ch, ++it) {
-                    const int as = it & 1;
-                    alive = mbar_wait(acc_empty + 8 * as, (((uint32_t)(it >> 1)) & 1u) ^ 1u, abort_flag, status);
+        const uint32_t idesc = make_idesc_fmt(2 * TILE, 0u);
+        bool alive = true;
+        int s = 0, it = 0;
+        uint32_t ph = 0;
+        for (int t = blockIdx.x; t < ntiles && alive; t += gridDim.x) {
+            int mt, nt2;
+            tile_of(t, ntn2, o.part, mt, nt2);
+            const int kb0 = first_kb(o.part, mt, nt2), nk = nkb - kb0, nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
+            for (int ch = 0; ch < nch && alive; ++ch, ++it) {
+                const int as = it & 1;
+                alive = __all_sync(0xffffffffu, mbar_wait(acc_empty + 8 * as, (((uint32_t)(it >> 1)) & 1u) ^ 1u, abort_flag, status));
+                if (!alive) break;
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(as * 2 * TILE);
+                const int kb_begin = kb0 + ch * KCHUNK, kb_end = min(nkb, kb_begin + KCHUNK);
+                for (int kb = kb_begin; kb < kb_end && alive; ++kb) {
+                    alive = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * s, ph, abort_flag, status));
                     if (!alive) break;
                     tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(as * 2 * TILE);
-                    const int kb_begin = kb0 + ch * KCHUNK, kb_end = min(nkb, kb_begin + KCHUNK);
-                    for (int kb = kb_begin; kb < kb_end && alive; ++kb, ++g) {
-                        const int s = g % STAGES;
-                        alive = mbar_wait(full_bar + 8 * s, ((uint32_t)(g / STAGES)) & 1u, abort_flag, status);
-                        if (!alive) break;
-                        tc_fence_after();
-                        const uint32_t stage = smem_base + (uint32_t)(s * STAGE_BYTES);
-                        const uint64_t a_hi = make_smem_desc(stage), a_lo = make_smem_desc(stage + (uint32_t)HALF);
-                        const uint64_t b_hi = make_smem_desc(stage + (uint32_t)PIECE), b_lo = make_smem_desc(stage + (uint32_t)(2 * PIECE));
-                        const bool fresh = kb == kb_begin;         // the chunk starts on a cleared accumulator
+                    const uint32_t stage = smem_base + (uint32_t)(s * STAGE_BYTES);
+                    const uint64_t a_hi = make_smem_desc(stage), a_lo = make_smem_desc(stage + (uint32_t)HALF);
+                    const uint64_t b_hi = make_smem_desc(stage + (uint32_t)PIECE), b_lo = make_smem_desc(stage + (uint32_t)(2 * PIECE));
+                    const bool fresh = kb == kb_begin;           // the chunk starts on a cleared accumulator
+                    if (elect_one()) {
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)           // 16 fp16 = 32 bytes per K step
                             umma_ss(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, (!fresh || ks > 0) ? 1u : 0u);
@@ -374,12 +374,16 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
                         for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_lo + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
                         umma_commit(empty_bar + 8 * s);
                     }
+                    __syncwarp();
+                    if (++s == STAGES) { s = 0; ph ^= 1u; }
+                }
+                if (elect_one()) {
                     if (alive && nk > 0) umma_commit(acc_full + 8 * as);
                     else mbar_arrive(acc_full + 8 * as);
                 }
+                __syncwarp();
             }
         }
-        __syncwarp();
     }
     tc_fence_before();
     __syncthreads();
