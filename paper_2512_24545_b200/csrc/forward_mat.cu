@@ -170,7 +170,7 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
     const uint32_t smem_base = (smem_u32(mt_smem_raw) + 1023u) & ~1023u;
     unsigned char *smem_gen = mt_smem_raw + (smem_base - smem_u32(mt_smem_raw));
     const int nbp = a.ns / 2, nv = a.nv;                            // activation-tile slots in pairs, V-image slots
@@ -224,8 +224,9 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_d = tmem_base_slot;                   // accumulator: columns 0 .. 255
-    const uint32_t tmem_e = tmem_base_slot + MT_BN;           // envelope values of a pair of K blocks: 128 columns
+    const uint32_t tmem_base = warp_uniform(tmem_base_slot);
+    const uint32_t tmem_d = tmem_base;                   // accumulator: columns 0 .. 255
+    const uint32_t tmem_e = tmem_base + MT_BN;           // envelope values of a pair of K blocks: 128 columns
     const uint32_t tmem_a = tmem_e + 2 * MT_BK;               // W_hat tiles: MT_NA pairs x (2 blocks x 32 columns of bf16 pairs)
     pdl_launch_dependents();
 
@@ -426,15 +427,15 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
         __syncwarp();
     } else if (warp == MT_W_MINI) {
         // ============ envelope mini-MMA issuer: E(pair p) = U image x V image(p)^T, 128 columns ============
-        if (lane == 0) {
-            const uint32_t idesc_mini = make_idesc_fmt(2 * MT_BK, a.env_fmt);
-            bool alive = mbar_wait(u_bar, 0u, abort_flag, a.status);
-            int vb = 0;
-            uint32_t vph = 0;
-            for (int p = 0; p < npr && alive; ++p) {
-                alive = mt_wait2(vfull_bar + 8 * vb, vph, eempty_bar, ((uint32_t)p & 1u) ^ 1u, abort_flag, a.status);
-                if (!alive) break;
-                tc_fence_after();
+        const uint32_t idesc_mini = make_idesc_fmt(2 * MT_BK, a.env_fmt);
+        bool alive = __all_sync(0xffffffffu, mbar_wait(u_bar, 0u, abort_flag, a.status));
+        int vb = 0;
+        uint32_t vph = 0;
+        for (int p = 0; p < npr && alive; ++p) {
+            alive = __all_sync(0xffffffffu, mt_wait2(vfull_bar + 8 * vb, vph, eempty_bar, ((uint32_t)p & 1u) ^ 1u, abort_flag, a.status));
+            if (!alive) break;
+            tc_fence_after();
+            if (elect_one()) {
                 for (int q = 0; q < a.kc / 2; ++q) {
                     const uint64_t ud = make_smem_desc_plain(u_smem + (uint32_t)q * 4096u, 2048u, 128u);
                     const uint64_t vd = make_smem_desc_plain(v_smem + (uint32_t)vb * img_bytes + (uint32_t)q * 4096u, 2048u, 128u);
@@ -442,39 +443,43 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
                 }
                 umma_commit(efull_bar);
                 umma_commit(vempty_bar + 8 * vb);
-                if (++vb == nv) { vb = 0; vph ^= 1u; }
             }
+            __syncwarp();
+            if (++vb == nv) { vb = 0; vph ^= 1u; }
         }
-        __syncwarp();
     } else {
         // ================================ main MMA issuer =================================
         // a pair of K blocks per step: W_hat tiles from TMEM, activation tiles from shared memory, 8 MMAs,
         // one commit frees the TMEM slot and one the pair of activation tiles
-        if (lane == 0) {
-            const uint32_t idesc_main = make_idesc(a.bn);
-            bool alive = true;
-            int bp = 0;
-            uint32_t ph = 0;
-            for (int p = 0; p < npr && alive; ++p) {
-                const int s0 = 2 * bp, as = p & (MT_NA - 1);
-                const uint32_t aph = (uint32_t)(p / MT_NA) & 1u;
-                const bool two = 2 * p + 1 < nkb;
-                alive = two ? mt_wait3(afull_bar + 8 * as, aph, bfull_bar + 8 * s0, ph, bfull_bar + 8 * (s0 + 1), ph, abort_flag, a.status)
-                            : mt_wait2(afull_bar + 8 * as, aph, bfull_bar + 8 * s0, ph, abort_flag, a.status);
-                if (!alive) break;
-                tc_fence_after();
-                for (int h = 0; h < (two ? 2 : 1); ++h) {
-                    const uint64_t bdesc = make_smem_desc(smem_base + (uint32_t)(s0 + h) * b_bytes);
-                    const uint32_t a_t = tmem_a + (uint32_t)(as * 64 + h * 32);
+        const uint32_t idesc_main = make_idesc(a.bn);
+        bool alive = true;
+        int bp = 0;
+        uint32_t ph = 0;
+        for (int p = 0; p < npr && alive; ++p) {
+            const int s0 = 2 * bp, as = p & (MT_NA - 1);
+            const uint32_t aph = (uint32_t)(p / MT_NA) & 1u;
+            const bool two = 2 * p + 1 < nkb;
+            alive = __all_sync(0xffffffffu, two ? mt_wait3(afull_bar + 8 * as, aph, bfull_bar + 8 * s0, ph, bfull_bar + 8 * (s0 + 1), ph, abort_flag, a.status)
+                                                : mt_wait2(afull_bar + 8 * as, aph, bfull_bar + 8 * s0, ph, abort_flag, a.status));
+            if (!alive) break;
+            tc_fence_after();
+            const uint64_t b0 = make_smem_desc(smem_base + (uint32_t)s0 * b_bytes), b1 = make_smem_desc(smem_base + (uint32_t)(s0 + 1) * b_bytes);
+            const uint32_t a_t = tmem_a + (uint32_t)(as * 64);
+            if (elect_one()) {
 #pragma unroll
-                    for (int k4 = 0; k4 < MT_BK / 16; ++k4)
-                        umma_ts(tmem_d, a_t + (uint32_t)(8 * k4), bdesc + (uint64_t)(2 * k4), idesc_main,
-                                (p > 0 || h > 0 || k4 > 0) ? 1u : 0u);
+                for (int k4 = 0; k4 < MT_BK / 16; ++k4)
+                    umma_ts(tmem_d, a_t + (uint32_t)(8 * k4), b0 + (uint64_t)(2 * k4), idesc_main, (p > 0 || k4 > 0) ? 1u : 0u);
+                if (two) {
+#pragma unroll
+                    for (int k4 = 0; k4 < MT_BK / 16; ++k4) umma_ts(tmem_d, a_t + (uint32_t)(32 + 8 * k4), b1 + (uint64_t)(2 * k4), idesc_main, 1u);
                 }
                 umma_commit(aempty_bar + 8 * as);
                 umma_commit(bempty_bar + 8 * bp);
-                if (++bp == nbp) { bp = 0; ph ^= 1u; }
             }
+            __syncwarp();
+            if (++bp == nbp) { bp = 0; ph ^= 1u; }
+        }
+        if (elect_one()) {
             if (alive) { if (nkb > 0) umma_commit(accum_bar); else mbar_arrive(accum_bar); }
         }
         __syncwarp();
