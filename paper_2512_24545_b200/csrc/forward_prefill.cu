@@ -617,8 +617,11 @@ mdbf_status_t ensure_prefill_scratch(Layer &L) {
     if (L.xsB) return MDBF_OK;
     L.xs_rows = ((size_t)L.d.max_T * L.LP + 255) / 256 * 256;
     __nv_bfloat16 *b = nullptr, *a = nullptr;
-    MDBF_CUDA(dev_malloc(&b, L.xs_rows * L.padB * 2));
-    cudaError_t e = dev_malloc(&a, L.xs_rows * L.padA * 2);
+    // in the allocator's whole blocks of 2 MB: taken on demand and large, they share none with a handle's small buffers, whatever was allocated
+    // and freed before
+    const size_t block = (size_t)2 << 20;
+    MDBF_CUDA(dev_malloc(&b, (L.xs_rows * L.padB * 2 + block - 1) / block * block));
+    cudaError_t e = dev_malloc(&a, (L.xs_rows * L.padA * 2 + block - 1) / block * block);
     if (e == cudaSuccess) e = cudaMemset(b, 0, L.xs_rows * L.padB * 2);
     if (e == cudaSuccess) e = cudaMemset(a, 0, L.xs_rows * L.padA * 2);
     if (e != cudaSuccess) { cudaFree(b); cudaFree(a); return cuda_fail(e, "scratch of the expanded order"); }
