@@ -499,12 +499,13 @@ mat_stage_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in, c
 // pace, so this variant keeps two or three pairs in flight: pair p works in buffer p % nb of tensor memory, which holds the pair's
 // envelope values (fp32, 128 columns) and then, over those that a builder warp has read, its part of the W_hat tile (a warp: one block of
 // the pair, 32 rows, 64 columns of values -> 32 packed ones).  A buffer has its own group of 8 builder warps, its own main-MMA
-// issuer and its own accumulator; the epilogue adds the accumulators.  Loaders and the mini-MMA issuer are shared; the issuing warps run
+// issuer and its own accumulator; the epilogue adds the accumulators.  Loaders and the mini-MMA issuer are shared; all of these warps run
 // converged (see elect_one).
 // TMEM: accumulators 0..127 (three of 32 columns up to 32 tokens, two of 64 above: then three buffers no longer fit), buffers 128 + 128 g.
 // What bounds it: the issue slots of a busy SM and the mini-MMA issuer.  11008 x 3968, 16 tokens: 0.36 us a pair, 0.47 with
-// single-lane issuers; per forward 4096 -> 3968 -> 11008: 16 tokens 25.8 -> 20.6 us, 64 tokens 27.0 -> 24.4; 1723 x 2312, k = 877, 37 tokens
-// 13.2 -> 11.5.  (Two CTAs of one pipeline each per SM: 25.2 and 18.3, the second because a CTA's few pairs run one after the other.)
+// single-lane issuers; per forward 4096 -> 3968 -> 11008: 16 tokens 25.5 us with single-lane roles, 20.5 with converged issuers, 17.6 with
+// converged loaders too (the large tiles' loaders stay single-lane: no difference there); 64 tokens 27.0, 24.7, 23.6; 1723 x 2312,
+// k = 877, 37 tokens 12.6, 11.1, 10.9.  (Two CTAs of one pipeline each per SM: 25.2 and 18.3, the second because a CTA's few pairs run one after the other.)
 constexpr int MS_BUFS = 3;
 constexpr int MS_XWARPS = 8 * MS_BUFS;
 constexpr int MS_W_TMA = MS_XWARPS;
@@ -685,43 +686,48 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
             }
         }
     } else if (warp == MS_W_TMA) {
-        // ============================ activation-tile loader ===========================
-        if (lane == 0) {
-            bool alive = true;
-            pdl_wait();
-            int bp = 0;
-            uint32_t ph = 0;
-            for (int p = 0; p < npr && alive; ++p) {
-                alive = mbar_wait(bempty_bar + 8 * bp, ph ^ 1u, abort_flag, a.status);
-                if (!alive) break;
-                for (int h = 0; h < 2 && 2 * p + h < nkb; ++h) {
-                    const int s = 2 * bp + h;
-                    mbar_arrive_expect_tx(bfull_bar + 8 * s, b_bytes);
-                    tma_load_2d(smem_base + (uint32_t)s * b_bytes, &tmap_in, (kb0 + 2 * p + h) * MT_BK, 0, bfull_bar + 8 * s);
+        // ============================ activation-tile loader (converged) ===========================
+        bool alive = true;
+        pdl_wait();                                   // the activations come from the previous kernel
+        int bp = 0;
+        uint32_t ph = 0;
+        for (int p = 0; p < npr && alive; ++p) {
+            alive = __all_sync(0xffffffffu, mbar_wait(bempty_bar + 8 * bp, ph ^ 1u, abort_flag, a.status));
+            if (!alive) break;
+            const int s = 2 * bp, x = (kb0 + 2 * p) * MT_BK;
+            const bool two = 2 * p + 1 < nkb;
+            if (elect_one()) {
+                mbar_arrive_expect_tx(bfull_bar + 8 * s, b_bytes);
+                tma_load_2d(smem_base + (uint32_t)s * b_bytes, &tmap_in, x, 0, bfull_bar + 8 * s);
+                if (two) {
+                    mbar_arrive_expect_tx(bfull_bar + 8 * s + 8, b_bytes);
+                    tma_load_2d(smem_base + (uint32_t)(s + 1) * b_bytes, &tmap_in, x + MT_BK, 0, bfull_bar + 8 * s + 8);
                 }
-                if (++bp == nbp) { bp = 0; ph ^= 1u; }
             }
-            if (!alive) drain_delay();
+            __syncwarp();
+            if (++bp == nbp) { bp = 0; ph ^= 1u; }
         }
-        __syncwarp();
+        if (!alive) drain_delay();
     } else if (warp == MS_W_ENV) {
-        // ============================= envelope-image loader ===========================
-        if (lane == 0) {
-            bool alive = true;
+        // ============================= envelope-image loader (converged) ===========================
+        bool alive = true;
+        if (elect_one()) {
             mbar_arrive_expect_tx(u_bar, img_bytes);
             bulk_load(u_smem, a.uimg + (size_t)rb * (img_bytes / 2), img_bytes, u_bar);
-            int vb = 0;
-            uint32_t vph = 0;
-            for (int p = 0; p < npr && alive; ++p) {
-                alive = mbar_wait(vempty_bar + 8 * vb, vph ^ 1u, abort_flag, a.status);
-                if (!alive) break;
+        }
+        int vb = 0;
+        uint32_t vph = 0;
+        for (int p = 0; p < npr && alive; ++p) {
+            alive = __all_sync(0xffffffffu, mbar_wait(vempty_bar + 8 * vb, vph ^ 1u, abort_flag, a.status));
+            if (!alive) break;
+            if (elect_one()) {
                 mbar_arrive_expect_tx(vfull_bar + 8 * vb, img_bytes);
                 bulk_load(v_smem + (uint32_t)vb * img_bytes, a.vimg + (size_t)(kb0 / 2 + p) * (img_bytes / 2), img_bytes, vfull_bar + 8 * vb);
-                if (++vb == nv) { vb = 0; vph ^= 1u; }
             }
-            if (!alive) drain_delay();
+            __syncwarp();
+            if (++vb == nv) { vb = 0; vph ^= 1u; }
         }
-        __syncwarp();
+        if (!alive) drain_delay();
     } else if (warp == MS_W_MINI) {
         // ======================= envelope mini-MMA issuer =======================
         const uint32_t idesc_mini = make_idesc_fmt(2 * MT_BK, a.env_fmt);
