@@ -46,8 +46,7 @@ NCU_TRAFFIC_BYTES_PER_LAUNCH = {
     ("msvid_28672x6016_l16", "envelope_product_tc_kernel"): 708300000,   # Z once per pass (689.9 MB) + operand images and partial sums,
                                                                            # scaled by rows x cols from the 8192 x 8192 capture
     ("msvid_8192x8192_l16", "envelope_product_tc_kernel"): 275523328,      # 269.6 MB read + 5.9 MB written for 268.4 MB of Z
-    ("admm_8192x8192_r3712_l16", "gemm3x_kernel"): 1156590808,            # its largest launch, W V: 1.038 GB read (images 0.78 GB; V's are re-read
-                                                                           # by every row tile, four fifths of that from L2) + 118.6 MB written
+    ("admm_8192x8192_r3712_l16", "gemm3x_kernel"): None,                   # images are half the bytes of the last capture's (1156590808 for W V)
     ("block70b_T2048", "mat_stage_kernel"): 197116928,             # its largest launch, down stage B (185.9 MB read: 117 MB of x, partly twice,
                                                                    # + signs; 11.3 MB written); gate / up stage A: 123.3 MB
 }
@@ -451,6 +450,22 @@ def measure(workload, kernel, steps, warmup, dist, world, local, no_graph=False,
 
 
 # ------------------------------------------------------------ quantizer, first step (MSVID)
+def msvid_launch_count(l, n_iter):
+    """As msvid.cu issues them on the tensor-core path: start block 1 + 2, per iteration two products and two orthogonalisations (+ 1 where
+    the narrow transposed product takes the scalar kernel and its partial-sum pass), last block 1, final product and factors 5."""
+    return 1 + 2 + n_iter * (4 + (1 if l <= 4 else 0)) + 1 + 5
+
+
+def tri_inverse_launch_count(r):
+    """As admm.cu issues them: the diagonal blocks of 64, two products per level below 1024 columns, from there per pair of blocks two
+    products and six passes that write operand images."""
+    n, size = 1, 64
+    while size < r:
+        n += 2 if size < 1024 else 8 * ((r - size + 2 * size - 1) // (2 * size))
+        size *= 2
+    return n
+
+
 def measure_msvid(workload, steps, warmup, dist, world, local, want_e2e=True, min_timed_ms=0.0):
     """msvid_<rows>x<cols>_l<l>[_it<n>]: one step = one mdbf_msvid call on a resident rows x cols fp32 matrix (sign mask +
     rank-l envelope, n subspace iterations).  Algorithmic bytes: the 2 n + 1 product passes each read Z once (rows * cols * 4
@@ -527,9 +542,7 @@ def measure_msvid(workload, steps, warmup, dist, world, local, want_e2e=True, mi
     value = replicas.aggregate_throughput(step_bytes * steps / 1e9, world, ms_max / 1e3)
     per_gpu = step_bytes * steps / 1e9 / (ms_max / 1e3)
     peak = peaks["hbm_gbs"]
-    # as msvid.cu issues them for these shapes: start block 1 + 2 x 2, per iteration 2 products + 2 x 2 (+ 1 where the narrow
-    # transposed product takes the scalar kernel and its partial-sum pass), last block once more 2, final product and factors 5
-    launches_per_call = 1 + 4 + n_iter * (6 + (1 if l <= 4 else 0)) + 2 + 5
+    launches_per_call = msvid_launch_count(l, n_iter)
     out = {
         "metric": "msvid_algorithmic_GBps", "value": value, "unit": "GB/s", "steps": steps, "warmup": max(3, warmup),
         "ms_per_step": ms_max / steps,
@@ -647,7 +660,7 @@ def measure_admm(workload, steps, warmup, dist, world, local, want_e2e=True):
     ms_max, e2e_ms_max = replicas.max_over_ranks([ms, e2e_s * 1e3], dist, device="cuda")
     value = replicas.aggregate_throughput(flops * steps / 1e12, world, ms_max / 1e3)
     per_gpu = flops * steps / 1e12 / (ms_max / 1e3)
-    msvid_launches = 1 + 4 + n_iter * (6 + (1 if l <= 4 else 0)) + 2 + 5
+    msvid_launches = msvid_launch_count(l, n_iter)
     out = {
         "metric": "admm_update_TFLOPs", "value": value, "unit": "TFLOP/s", "steps": steps, "warmup": max(3, warmup),
         "ms_per_step": ms_max / steps,
@@ -659,13 +672,13 @@ def measure_admm(workload, steps, warmup, dist, world, local, want_e2e=True):
         "e2e": ({"value": replicas.aggregate_throughput(flops * e2e_steps / 1e12, world, e2e_ms_max / 1e3), "unit": "TFLOP/s",
                  "h2d_bytes_per_step": (N * Mc + Mc * R + N * R) * 4, "d2h_bytes_per_step": 2 * N * R * 4 + N * nwords * 4}
                 if want_e2e else None),
-        # this library's kernels (the solver library's are not counted): 2 splits + 2 products + ridge + identity + split, product,
-        # split for the inverse + flag; per inner iteration rhs, split, product, sum, MSVID, reconstruction
-        "gpu_launches": (10 + n_inner * (5 + msvid_launches)) * steps,
+        # this library's kernels (the solver library's are not counted): images of V (2) and W (1), their two products, ridge, the
+        # triangular inverse, images and product for the system's inverse and its images (3), flag; per inner iteration images of the
+        # right-hand side, product, MSVID, reconstruction
+        "gpu_launches": (2 + 1 + 2 + 1 + tri_inverse_launch_count(R) + 3 + 1 + n_inner * (3 + msvid_launches)) * steps,
         "clocks": clocks,
         "roofline": {"bound": "tensor", "achieved": per_gpu, "peak": peak, "unit": "TFLOP/s", "frac": per_gpu / peak,
-                     "peak_source": f"of {peak_kind}: the sustained bf16 GEMM figure (kind::tf32 issues at the 16-bit rate on this part: 1.6 PFLOP/s "
-                                    "executed with the tensor pipe 75 % busy); the three-term split spends three tensor-core products per "
+                     "peak_source": f"of {peak_kind}: the sustained bf16 GEMM figure (the products run on fp16 parts); the three-term split spends three tensor-core products per "
                                     "product counted, so a third of the peak is this scheme's ceiling",
                      "kernel": "gemm3x_kernel", "traffic": NCU_TRAFFIC_BYTES_PER_LAUNCH.get((workload, "gemm3x_kernel"))},
     }

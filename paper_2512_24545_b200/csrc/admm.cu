@@ -97,7 +97,7 @@ __global__ void ridge_kernel(float *__restrict__ G, int r, float rho) {
 // all pairs of a size in two batched products: log2(r / TI_LEAF) levels instead of the r / 256 dependent steps of a triangular solve
 // with r right-hand sides (r = 3712: 2.6 ms of such steps in the library's solver, 0.5 ms here).  Pairs of blocks of
 // TI_DENSE columns and more go through the tensor-core product.
-constexpr int TI_LEAF = 128, TI_DENSE = 1024;
+constexpr int TI_LEAF = 64, TI_DENSE = 1024;                     // leaves of 128: 45 us longer at r = 3712, of 32: the same
 constexpr int TI_SMEM = 2 * TI_LEAF * (TI_LEAF + 1) * 4;
 // CTA = one diagonal block, thread = column of the inverse, back substitution: the row of U is the same for the whole warp (a
 // broadcast), the column of Y is the thread's own.  The block's lower triangle is written as zeros.

@@ -240,9 +240,9 @@ def test_rows_of_very_different_scale(N, Mc, R, transpose):
     assert np.all(err <= 2e-4 * scale + 1e-37), (err / np.maximum(scale, 1e-300)).max()
 
 
-@pytest.mark.parametrize("R", [1, 127, 128, 129, 257, 384, 1025, 2180])
+@pytest.mark.parametrize("R", [1, 63, 64, 65, 129, 192, 1025, 2180])
 def test_inverse_of_the_system_by_doubling(R):
-    """The triangular factor is inverted in diagonal blocks of 128 that are joined pair by pair: a lone ragged block, a pair whose
+    """The triangular factor is inverted in diagonal blocks of 64 that are joined pair by pair: a lone ragged block, a pair whose
     second block is one column, odd numbers of blocks, and pairs that go through the tensor-core product (from 1024 columns).
     rho is the system's mean diagonal, so its condition number stays near 5 and fp32 rounding (2^-24) in factor, inverse and product,
     each amplified by it, comes to about 1e-6 of the iterate; the bound is that of the ragged shapes above."""
