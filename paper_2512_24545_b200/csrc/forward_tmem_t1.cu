@@ -379,36 +379,38 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
         }
     } else if (warp == TX_W_ISSUER0 + TX_ISSUERS) {
         // ============================== sign-word loader ================================
-        if (lane == 0) {
-            bool alive = true;
-            int rs = 0;
-            uint32_t ph = 1;                                 // the first fill was requested above
-            for (int pr = nss; pr < npr; ++pr) {
-                alive = tx_wait(s_empty + 8 * rs, ph ^ 1u, abort_flag, a.status);
-                if (!alive) break;
+        bool alive = true;
+        int rs = 0;
+        uint32_t ph = 1;                                     // the first fill was requested above
+        for (int pr = nss; pr < npr; ++pr) {
+            alive = __all_sync(0xffffffffu, tx_wait(s_empty + 8 * rs, ph ^ 1u, abort_flag, a.status));
+            if (!alive) break;
+            if (elect_one()) {
                 mbar_arrive_expect_tx(s_full + 8 * rs, 2048u);
                 bulk_load(smem_base + off_s + (uint32_t)(rs * 2048), sign_src + (size_t)pr * 256, 2048u, s_full + 8 * rs);
-                if (++rs == nss) { rs = 0; ph ^= 1u; }
             }
-            if (!alive) drain_delay();
+            __syncwarp();
+            if (++rs == nss) { rs = 0; ph ^= 1u; }
         }
+        if (!alive) drain_delay();
         __syncwarp();
         cluster_wait();
     } else if (warp == TX_W_ISSUER0 + TX_ISSUERS + 1) {
         // ================================ V-tile loader ==================================
-        if (lane == 0) {
-            bool alive = true;
-            int vs = 0;
-            uint32_t ph = 1;
-            for (int pr = nas; pr < npr; ++pr) {
-                alive = tx_wait(a_empty + 8 * vs, ph ^ 1u, abort_flag, a.status);
-                if (!alive) break;
+        bool alive = true;
+        int vs = 0;
+        uint32_t ph = 1;
+        for (int pr = nas; pr < npr; ++pr) {
+            alive = __all_sync(0xffffffffu, tx_wait(a_empty + 8 * vs, ph ^ 1u, abort_flag, a.status));
+            if (!alive) break;
+            if (elect_one()) {
                 mbar_arrive_expect_tx(v_full + 8 * vs, (uint32_t)VBYTES);
                 bulk_load(smem_base + (uint32_t)(vs * VBYTES), v_src + (size_t)pr * 2 * NB * 64, (uint32_t)VBYTES, v_full + 8 * vs);
-                if (++vs == nas) { vs = 0; ph ^= 1u; }
             }
-            if (!alive) drain_delay();
+            __syncwarp();
+            if (++vs == nas) { vs = 0; ph ^= 1u; }
         }
+        if (!alive) drain_delay();
         __syncwarp();
         cluster_wait();
     }
