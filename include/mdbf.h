@@ -221,8 +221,8 @@ mdbf_status_t mdbf_linear_forward_host(mdbf_handle_t h, const void *x_host, void
  * `stream` and the call returns; y_host holds the result once the caller has synchronised the
  * stream (or an event recorded after the call).  x_host must stay unchanged and both buffers
  * allocated until then; pageable buffers make the copies synchronous, so use pinned memory.  Calls
- * on different handles pipeline on one stream: the next layer's input copy overlaps this layer's
- * kernels.  Two calls on the SAME handle share its staging buffers and are ordered by the stream. */
+ * on one stream run in order, reads of x_host included: x_host may be the buffer that an earlier call on the stream
+ * writes.  Two calls on the SAME handle share its staging buffers and must be on one stream. */
 mdbf_status_t mdbf_linear_forward_host_async(mdbf_handle_t h, const void *x_host, void *y_host, int32_t T,
                                              int32_t act_dtype, void *stream);
 

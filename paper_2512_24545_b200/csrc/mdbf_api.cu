@@ -152,16 +152,15 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
     return cudaMalloc(p, bytes);
 }
 
-// x from pinned host memory into the handle's staging buffer.  The reads of host memory start before the wait for the previous
-// kernel (which may still read the staging buffer), the launch's dependents before either has ended.
+// x from pinned host memory into the handle's staging buffer.  x is read, like any input on the stream, only when the previous kernel has
+// ended: that kernel may be the one that writes it (a layer that leaves its y in the same pinned buffer).  What runs early is the launch
+// itself, and the launch of this kernel's dependents.  (No __restrict__: a load marked read-only could be moved above the wait.)
 template <typename V>
-__global__ void __launch_bounds__(256) host_fetch_kernel(const V *__restrict__ src, V *__restrict__ dst, int n) {
+__global__ void __launch_bounds__(256) host_fetch_kernel(const V *src, V *dst, int n) {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int i = blockIdx.x * 256 + threadIdx.x;
-    V v = V();
-    if (i < n) v = src[i];
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    if (i < n) dst[i] = v;
+    if (i < n) dst[i] = src[i];
 }
 static mdbf_status_t launch_host_fetch(const void *src, void *dst, size_t bytes, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
@@ -192,8 +191,8 @@ static void *device_view(const void *host) {
 // Which buffers of a host-buffer forward the kernels move themselves (pinned ones only; the copy engine moves the others).  A copy
 // costs its stream hand-over, some 5 us on either side of kernels that take less than that; the kernels pay the
 // link's latency and reach less of its rate.  Per call, synchronised (us): y stored by the last stage instead of copied: 8 KB 35.9 ->
-// 29.4, 128 KB 50.7 -> 44.0, 256 KB 54.5 -> 50.4, 1 MB 104 -> 124.  x fetched by a kernel, on top of that: 8 KB 29.4 -> 32.5,
-// 16 KB 30.6 -> 30.3, 28 KB 30.2 -> 27.8, 128 KB 44.0 -> 40.7, 1 MB 104 -> 99.
+// 29.4, 128 KB 50.7 -> 44.0, 256 KB 54.5 -> 50.4, 1 MB 104 -> 124.  x copied -> fetched by a kernel, y stored by the last stage either way
+// (1024 rows, k = 384): 8 KB 20.6 -> 20.8, 16 KB 21.8 -> 22.0, 28 KB 25.5 -> 23.2, 128 KB 35.6 -> 29.5, 256 KB 37.0 -> 33.4, 1 MB 56.1 -> 53.1.
 constexpr size_t kHostFetchMin = 20u << 10, kHostFetchMax = 1u << 20, kHostStoreMax = 256u << 10;
 
 }  // namespace mdbf

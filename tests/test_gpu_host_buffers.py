@@ -50,3 +50,37 @@ def test_host_buffers(d_out, d_in, T, memory):
         torch.cuda.synchronize()
         assert torch.equal(yh.view(T, d_out), yd.cpu())
         assert M.mdbf_poll_status(g.h) == 0
+
+
+@pytest.mark.parametrize("mid,T", [(8192, 1), (11008, 1), (4096, 4), (2048, 64)])      # 16, 22, 32 and 256 KB between the layers
+@pytest.mark.parametrize("first", ["host_async", "device"])
+def test_a_layer_reads_what_the_one_before_it_leaves_in_pinned_memory(mid, T, first):
+    """Calls queued on one stream without a wait in between: the second layer's input is the buffer the first one's output goes into."""
+    one = inputs.scaled(inputs.qproj(1664), name="one", d_out=mid, d_in=8192, k=2048, l=16, seed=41)
+    two = inputs.scaled(inputs.qproj(1664), name="two", d_out=640, d_in=mid, k=256, l=4, seed=42)
+    st = torch.cuda.current_stream().cuda_stream
+    with GpuLayer(one, T) as a, GpuLayer(two, T) as b:
+        M.mdbf_prepare_host_staging(a.h)
+        M.mdbf_prepare_host_staging(b.h)
+        x = torch.from_numpy(inputs.make_activations(one, T)).to(torch.bfloat16)
+        xd, xh = x.cuda(), x.pin_memory()
+        buf = torch.zeros((T, mid), dtype=torch.bfloat16).pin_memory()
+        out, want = (torch.zeros((T, 640), dtype=torch.bfloat16).pin_memory() for _ in range(2))
+
+        def head():
+            if first == "device":
+                M.mdbf_linear_forward(a.h, xd.data_ptr(), buf.data_ptr(), T, M.BF16, st)
+            else:
+                M.mdbf_linear_forward_host_async(a.h, xh.data_ptr(), buf.data_ptr(), T, M.BF16, st)
+
+        head()
+        torch.cuda.synchronize()
+        M.mdbf_linear_forward_host(b.h, buf.data_ptr(), want.data_ptr(), T, M.BF16, st)
+        assert bool(torch.isfinite(want).all()) and float(want.float().abs().max()) > 0
+        for _ in range(5):
+            buf.zero_()
+            out.zero_()
+            head()
+            M.mdbf_linear_forward_host_async(b.h, buf.data_ptr(), out.data_ptr(), T, M.BF16, st)
+            torch.cuda.synchronize()
+            assert torch.equal(out, want)
