@@ -685,6 +685,8 @@ static mdbf_status_t forward_host_impl(mdbf_handle_t h, const void *x_host, void
     if (rc) return rc;
     if (!x_host || !y_host) { set_error("mdbf_linear_forward_host: NULL pointer"); return MDBF_ERR_INVALID_ARG; }
     Layer &L = h->L;
+    rc = check_device(L, "mdbf_linear_forward_host");            // before anything is queued: a kernel of another device cannot reach the staging buffer
+    if (rc) return rc;
     if (T < 1 || T > L.d.max_T) {
         set_error("mdbf_linear_forward_host: T=%d outside [1, max_T=%d]", T, L.d.max_T);
         return MDBF_ERR_SHAPE;
