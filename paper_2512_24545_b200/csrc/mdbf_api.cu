@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "plans.h"
 
 namespace mdbf {
 
@@ -182,11 +183,26 @@ static mdbf_status_t launch_host_fetch(const void *src, void *dst, size_t bytes,
     }
     return MDBF_OK;
 }
-// The device's address of a pinned host buffer, or null for memory the device cannot reach as it is.
-static void *device_view(const void *host) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+// The device's address of a pinned host buffer, or null for memory that the device cannot reach as it is, to its last byte.
+static void *device_view(const void *host, size_t bytes) {
+    typedef CUresult (*query_fn)(unsigned int, CUpointer_attribute *, void **, CUdeviceptr);
+    static const query_fn query = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return reinterpret_cast<query_fn>(p);
+    }();
+    unsigned int type = 0, managed = 0;                          // (an address the driver does not know leaves type 0)
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute attr[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *out[] = {&type, &managed, &device, &start, &size};
+    if (!query || query(5, attr, out, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return nullptr;
+    return (void *)(uintptr_t)host_view(HostRange{type == CU_MEMORYTYPE_HOST && !managed, device, start, size}, bytes);
 }
 // Which buffers of a host-buffer forward the kernels move themselves (pinned ones only; the copy engine moves the others).  A copy
 // costs its stream hand-over, some 5 us on either side of kernels that take less than that; the kernels pay the
@@ -699,14 +715,14 @@ static mdbf_status_t forward_host_impl(mdbf_handle_t h, const void *x_host, void
         return MDBF_ERR_INVALID_ARG;
     }
     const size_t xb = (size_t)T * L.d.d_in * es, yb = (size_t)T * L.d.d_out * es;
-    const void *xd = xb >= kHostFetchMin && xb <= kHostFetchMax ? device_view(x_host) : nullptr;
+    const void *xd = xb >= kHostFetchMin && xb <= kHostFetchMax ? device_view(x_host, xb) : nullptr;
     if (xd) {
         rc = launch_host_fetch(xd, L.xstage, xb, st);
         if (rc) return rc;
     } else {
         MDBF_CUDA(cudaMemcpyAsync(L.xstage, x_host, xb, cudaMemcpyHostToDevice, st));
     }
-    void *yd = yb <= kHostStoreMax ? device_view(y_host) : nullptr;
+    void *yd = yb <= kHostStoreMax ? device_view(y_host, yb) : nullptr;
     rc = forward_impl(h, L.xstage, yd ? yd : L.ystage, T, act_dtype, st);
     if (rc) return rc;
     if (!yd) MDBF_CUDA(cudaMemcpyAsync(y_host, L.ystage, yb, cudaMemcpyDeviceToHost, st));

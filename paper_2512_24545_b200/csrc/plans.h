@@ -1,0 +1,24 @@
+// Decisions of the host side that need no GPU, in plain C++ so that they can be checked on the CPU.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+
+namespace mdbf {
+
+// What the driver says about a host address: whether it lies in pinned memory, the device's address of it, and the one mapping
+// (allocation or registration) it belongs to.
+struct HostRange {
+    bool pinned;
+    uint64_t device, start;
+    size_t size;
+};
+// The device's address of `bytes` bytes of host memory from there on, or 0 where not all of them lie in that mapping (a registered part
+// of a larger array, say): what is behind it is not the device's to touch.
+inline uint64_t host_view(const HostRange &r, size_t bytes) {
+    if (!r.pinned || r.device == 0 || r.device < r.start) return 0;
+    const uint64_t off = r.device - r.start;
+    return off <= r.size && bytes <= r.size - off ? r.device : 0;
+}
+
+}  // namespace mdbf
