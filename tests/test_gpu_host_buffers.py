@@ -52,6 +52,22 @@ def test_host_buffers(d_out, d_in, T, memory):
         assert M.mdbf_poll_status(g.h) == 0
 
 
+@pytest.mark.parametrize("off", [1, 3])
+def test_output_off_its_element_boundary(off):
+    """y_host anywhere in a pinned byte arena: the copy takes it there."""
+    spec = inputs.scaled(inputs.qproj(1664), name="odd", d_out=1000, d_in=640, k=96, l=4, seed=32)
+    x = torch.from_numpy(inputs.make_activations(spec, 3)).to(torch.bfloat16)
+    st = torch.cuda.current_stream().cuda_stream
+    with GpuLayer(spec, 3) as g:
+        M.mdbf_prepare_host_staging(g.h)
+        xh, want = x.pin_memory(), torch.zeros((3, 1000), dtype=torch.bfloat16).pin_memory()
+        M.mdbf_linear_forward_host(g.h, xh.data_ptr(), want.data_ptr(), 3, M.BF16, st)
+        arena = torch.zeros(6000 + 16, dtype=torch.uint8).pin_memory()
+        M.mdbf_linear_forward_host(g.h, xh.data_ptr(), arena.data_ptr() + off, 3, M.BF16, st)
+        assert torch.equal(arena[off:off + 6000], want.view(torch.uint8).reshape(-1))
+        assert not bool(arena[:off].any()) and not bool(arena[off + 6000:].any())
+
+
 @pytest.mark.parametrize("mid,T", [(8192, 1), (11008, 1), (4096, 4), (2048, 64)])      # 16, 22, 32 and 256 KB between the layers
 @pytest.mark.parametrize("first", ["host_async", "device"])
 def test_a_layer_reads_what_the_one_before_it_leaves_in_pinned_memory(mid, T, first):

@@ -13,6 +13,7 @@ extern "C" {
 uint64_t t_host_view(int pinned, uint64_t device, uint64_t start, size_t size, size_t bytes) {
     return host_view(HostRange{pinned != 0, device, start, size}, bytes);
 }
+int t_host_store_direct(uint64_t device, size_t es) { return host_store_direct(device, es); }
 }
 """
 
@@ -25,6 +26,7 @@ def plans(tmp_path_factory):
     L = ctypes.CDLL(str(d / "plans.so"))
     u64, sz = ctypes.c_uint64, ctypes.c_size_t
     L.t_host_view.argtypes, L.t_host_view.restype = [ctypes.c_int, u64, u64, sz, sz], u64
+    L.t_host_store_direct.argtypes = [u64, sz]
     return L
 
 
@@ -38,3 +40,9 @@ def test_a_host_buffer_has_to_lie_in_one_pinned_mapping(plans, pinned, off, size
     assert plans.t_host_view(pinned, start + off, start, size, nbytes) == (start + off if ok else 0)
     assert plans.t_host_view(pinned, 0, 0, size, nbytes) == 0        # no device address
     assert plans.t_host_view(pinned, start - 1, start, size, 1) == 0
+
+
+@pytest.mark.parametrize("off,es,ok", [(0, 2, 1), (2, 2, 1), (1, 2, 0), (16, 4, 1), (4, 4, 1), (2, 4, 0), (3, 4, 0)])
+def test_kernels_store_y_on_element_boundaries_only(plans, off, es, ok):
+    assert plans.t_host_store_direct(0x7F0000000000 + off, es) == ok
+    assert plans.t_host_store_direct(0, es) == 0
