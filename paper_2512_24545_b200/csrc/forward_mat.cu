@@ -39,6 +39,7 @@
 // returns.  Every TMA and bulk copy targets the issuing CTA's own shared memory only.
 #include <cooperative_groups.h>
 
+#include "plans.h"
 #include "tmem_ptx.cuh"
 
 namespace cg = cooperative_groups;
@@ -514,6 +515,7 @@ constexpr int MS_W_MINI = MS_XWARPS + 2;
 constexpr int MS_W_MMA0 = MS_XWARPS + 3;
 constexpr int MS_THREADS = (MS_W_MMA0 + MS_BUFS) * 32;
 constexpr int MS_BN = 64;
+static_assert(kHostStoreMaxT <= MS_BN, "a y in host memory is stored by this kernel's plain stores");
 
 template <bool STAGE_A, bool SPLIT>
 __global__ void __launch_bounds__(MS_THREADS, 1)

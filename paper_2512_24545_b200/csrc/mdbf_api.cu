@@ -723,7 +723,7 @@ static mdbf_status_t forward_host_impl(mdbf_handle_t h, const void *x_host, void
         MDBF_CUDA(cudaMemcpyAsync(L.xstage, x_host, xb, cudaMemcpyHostToDevice, st));
     }
     void *yd = yb <= kHostStoreMax ? device_view(y_host, yb) : nullptr;
-    if (!host_store_direct((uint64_t)(uintptr_t)yd, es)) yd = nullptr;
+    if (!host_store_direct((uint64_t)(uintptr_t)yd, es, T)) yd = nullptr;
     rc = forward_impl(h, L.xstage, yd ? yd : L.ystage, T, act_dtype, st);
     if (rc) return rc;
     if (!yd) MDBF_CUDA(cudaMemcpyAsync(y_host, L.ystage, yb, cudaMemcpyDeviceToHost, st));

@@ -20,8 +20,10 @@ inline uint64_t host_view(const HostRange &r, size_t bytes) {
     const uint64_t off = r.device - r.start;
     return off <= r.size && bytes <= r.size - off ? r.device : 0;
 }
-// Whether a kernel may store y (bytes of `es`-byte elements) at this device address of host memory itself: whole elements on their
-// own boundary.  (A copy takes any address, so a slice of a byte arena is a valid y_host.)
-inline bool host_store_direct(uint64_t device, size_t es) { return device != 0 && device % es == 0; }
+// Whether a kernel may store y (bytes of `es`-byte elements, T tokens) at this device address of host memory itself: whole elements on
+// their own boundary (a copy takes any address, so a slice of a byte arena is a valid y_host), and at most as many tokens as the kernels
+// with plain stores take - beyond that y leaves through a tensor map, and those are made over device memory only.
+constexpr int kHostStoreMaxT = 64;
+inline bool host_store_direct(uint64_t device, size_t es, int T) { return device != 0 && device % es == 0 && T <= kHostStoreMaxT; }
 
 }  // namespace mdbf

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2512_24545_b200 import inputs, mdbf as M
-from helpers import GpuLayer
+from helpers import GpuLayer, TORCH_DT
 
 pytestmark = pytest.mark.gpu
 
@@ -18,35 +18,47 @@ def built():
 
 # bytes of x and of y (bf16): below, at and above 20 KB / 1 MB for x and 256 KB for y
 @pytest.mark.parametrize("d_out,d_in,T", [(64, 128, 1), (1000, 10240, 1), (1000, 10248, 1), (8192, 64, 16), (8200, 64, 16), (96, 8192, 64),
-                                          (96, 8200, 64), (70, 1001, 31)])
+                                          (96, 8200, 64), (70, 1001, 31),
+                                          (1024, 640, 100), (1280, 12800, 90), (200, 1001, 130)])      # more than 64 tokens: whole, split, expanded order
 @pytest.mark.parametrize("memory", ["pinned", "pageable", "pinned_odd"])
 def test_host_buffers(d_out, d_in, T, memory):
-    spec = inputs.scaled(inputs.qproj(1664), name="host", d_out=d_out, d_in=d_in, k=96, l=4, seed=31)
-    x = torch.from_numpy(inputs.make_activations(spec, T)).to(torch.bfloat16)
+    host_against_device(inputs.scaled(inputs.qproj(1664), name="host", d_out=d_out, d_in=d_in, k=96, l=4, seed=31), T, memory)
+
+
+@pytest.mark.parametrize("T", [3, 70])
+@pytest.mark.parametrize("memory", ["pinned", "pageable"])
+def test_host_buffers_fp32(T, memory):
+    host_against_device(inputs.tiny(), T, memory)
+
+
+def host_against_device(spec, T, memory):
+    d_out, d_in, dt = spec.d_out, spec.d_in, TORCH_DT[spec.act_dtype]
+    act = M.DTYPES[spec.act_dtype]
+    x = torch.from_numpy(inputs.make_activations(spec, T)).to(dt)
     st = torch.cuda.current_stream().cuda_stream
 
     def host(n):
         off = 1 if memory == "pinned_odd" else 0                  # two bytes past a 16-byte boundary
-        buf = torch.full((n + 16 + off,), 7.0, dtype=torch.bfloat16)
+        buf = torch.full((n + 16 + off,), 7.0, dtype=dt)
         buf = buf if memory == "pageable" else buf.pin_memory()
         return buf, buf[off:off + n]
 
     with GpuLayer(spec, T) as g:
-        xd, yd = x.cuda(), torch.zeros((T, d_out), dtype=torch.bfloat16, device="cuda")
-        M.mdbf_linear_forward(g.h, xd.data_ptr(), yd.data_ptr(), T, M.BF16, st)
+        xd, yd = x.cuda(), torch.zeros((T, d_out), dtype=dt, device="cuda")
+        M.mdbf_linear_forward(g.h, xd.data_ptr(), yd.data_ptr(), T, act, st)
         M.mdbf_prepare_host_staging(g.h)
         _, xh = host(T * d_in)
         xh.copy_(x.reshape(-1))
         whole, yh = host(T * d_out)
         for _ in range(2):
             yh.fill_(3.0)
-            M.mdbf_linear_forward_host(g.h, xh.data_ptr(), yh.data_ptr(), T, M.BF16, st)
+            M.mdbf_linear_forward_host(g.h, xh.data_ptr(), yh.data_ptr(), T, act, st)
             assert torch.equal(yh.view(T, d_out), yd.cpu())
         assert bool((whole[yh.storage_offset() + T * d_out:] == 7.0).all())
         xh.copy_((x * 2).reshape(-1))                             # other contents of the same buffer
         xd.mul_(2)
-        M.mdbf_linear_forward(g.h, xd.data_ptr(), yd.data_ptr(), T, M.BF16, st)
-        M.mdbf_linear_forward_host_async(g.h, xh.data_ptr(), yh.data_ptr(), T, M.BF16, st)
+        M.mdbf_linear_forward(g.h, xd.data_ptr(), yd.data_ptr(), T, act, st)
+        M.mdbf_linear_forward_host_async(g.h, xh.data_ptr(), yh.data_ptr(), T, act, st)
         torch.cuda.synchronize()
         assert torch.equal(yh.view(T, d_out), yd.cpu())
         assert M.mdbf_poll_status(g.h) == 0

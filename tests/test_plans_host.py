@@ -13,7 +13,7 @@ extern "C" {
 uint64_t t_host_view(int pinned, uint64_t device, uint64_t start, size_t size, size_t bytes) {
     return host_view(HostRange{pinned != 0, device, start, size}, bytes);
 }
-int t_host_store_direct(uint64_t device, size_t es) { return host_store_direct(device, es); }
+int t_host_store_direct(uint64_t device, size_t es, int T) { return host_store_direct(device, es, T); }
 }
 """
 
@@ -26,7 +26,7 @@ def plans(tmp_path_factory):
     L = ctypes.CDLL(str(d / "plans.so"))
     u64, sz = ctypes.c_uint64, ctypes.c_size_t
     L.t_host_view.argtypes, L.t_host_view.restype = [ctypes.c_int, u64, u64, sz, sz], u64
-    L.t_host_store_direct.argtypes = [u64, sz]
+    L.t_host_store_direct.argtypes = [u64, sz, ctypes.c_int]
     return L
 
 
@@ -42,7 +42,8 @@ def test_a_host_buffer_has_to_lie_in_one_pinned_mapping(plans, pinned, off, size
     assert plans.t_host_view(pinned, start - 1, start, size, 1) == 0
 
 
-@pytest.mark.parametrize("off,es,ok", [(0, 2, 1), (2, 2, 1), (1, 2, 0), (16, 4, 1), (4, 4, 1), (2, 4, 0), (3, 4, 0)])
-def test_kernels_store_y_on_element_boundaries_only(plans, off, es, ok):
-    assert plans.t_host_store_direct(0x7F0000000000 + off, es) == ok
-    assert plans.t_host_store_direct(0, es) == 0
+@pytest.mark.parametrize("off,es,T,ok", [(0, 2, 1, 1), (2, 2, 64, 1), (1, 2, 1, 0), (16, 4, 8, 1), (4, 4, 1, 1), (2, 4, 1, 0), (3, 4, 1, 0),
+                                         (0, 2, 65, 0), (0, 4, 2048, 0)])      # more than 64 tokens: stored through a tensor map
+def test_which_y_the_kernels_store_themselves(plans, off, es, T, ok):
+    assert plans.t_host_store_direct(0x7F0000000000 + off, es, T) == ok
+    assert plans.t_host_store_direct(0, es, T) == 0
