@@ -194,15 +194,17 @@ static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *i
     MDBF_CUDA(cudaGetLastError());
     return MDBF_OK;
 }
-// U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam = Z - U with Z = U_tilde + Lam.
-// Bound by memory (Z read, U and Lam written: 12 bytes per entry; 8192 x 3712, l = 16: 99 us against 180 with U_tilde and the old Lam
-// read instead of Z and the products over 32 terms for every l).  CTA = 32 rows x 256 columns; thread = column (its row of Vl in
-// registers), the rows' Ul in shared memory, eight rows' loads in flight together; L = l rounded up to 4, 8, 16 or 32.
+// U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam += U_tilde - U (Eq. admm-U-dual, rounded as written: near
+// convergence U_tilde - U and Lam are small beside Z = U_tilde + Lam, and Z - U would carry a rounding of Z into the dual in every
+// iteration; 8192 x 3712 at the end of a refinement, error of the dual step relative to the dual: 1.4e-6 with Z - U, below 6e-8 this way).
+// Bound by memory (U_tilde and Lam read, U and Lam written: 16 bytes per entry; 8192 x 3712, l = 16: 130 us, of which the traffic needs 74; four rows in flight and 64 registers: 121, spilling).  CTA = 32 rows x 256
+// columns; thread = column (its row of Vl in registers), the rows' Ul in shared memory, eight rows' loads in flight together; L = l
+// rounded up to 4, 8, 16 or 32.  Ut may be U itself: an entry is read by the thread that writes it.
 constexpr int RC_ROWS = 32, RC_COLS = 256, RC_BATCH = 8;
 template <int L>
 __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__restrict__ S, const float *__restrict__ Ul,
-                                                             const float *__restrict__ Vl, int l, const float *__restrict__ Z,
-                                                             float *__restrict__ U, float *__restrict__ Lam, int n, int r, int nwords) {
+                                                             const float *__restrict__ Vl, int l, const float *Ut, float *U,
+                                                             float *__restrict__ Lam, int n, int r, int nwords) {
     __shared__ __align__(16) float us[RC_ROWS][L];
     const int i0 = blockIdx.y * RC_ROWS;
     for (int e = threadIdx.x; e < RC_ROWS * L; e += RC_COLS) {
@@ -215,13 +217,14 @@ __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__r
     float v[L];
 #pragma unroll
     for (int t = 0; t < L; ++t) v[t] = t < l ? Vl[(size_t)j * l + t] : 0.f;
-    float z[RC_BATCH];
+    float ut[RC_BATCH], lm[RC_BATCH];
     uint32_t word[RC_BATCH];
     auto load = [&](int ib) {
 #pragma unroll
         for (int u = 0; u < RC_BATCH; ++u) {
             const int i = min(i0 + ib + u, n - 1);
-            z[u] = Z[(size_t)i * r + j];
+            ut[u] = Ut[(size_t)i * r + j];
+            lm[u] = Lam[(size_t)i * r + j];
             word[u] = S[(size_t)i * nwords + (j >> 5)];
         }
     };
@@ -238,9 +241,9 @@ __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__r
                 e = fmaf(a.x, v[t], fmaf(a.y, v[t + 1], fmaf(a.z, v[t + 2], fmaf(a.w, v[t + 3], e))));
             }
             val[u] = ((word[u] >> (j & 31)) & 1u) ? -e : e;
-            lam[u] = z[u] - val[u];
+            lam[u] = lm[u] + (ut[u] - val[u]);
         }
-        load(ib + RC_BATCH);                                     // the next rows' loads run under these stores
+        if (ib + RC_BATCH < RC_ROWS && i0 + ib + RC_BATCH < n) load(ib + RC_BATCH);      // the next rows' loads run under these stores
 #pragma unroll
         for (int u = 0; u < RC_BATCH; ++u)
             if (i0 + ib + u < n) {
@@ -383,15 +386,16 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     if (rc) return rc;
     const int nwords = (int)((r + 31) / 32);
     for (int it = 0; it < n_inner; ++it) {
-        // Z = U_tilde + Lam, U_tilde = (B0 + rho (U - Lam)) G^-1: the right-hand side goes straight into images (where W's were), Lam is
-        // added on the way out; U_tilde itself is written only where the caller wants the last one
+        // U_tilde = (B0 + rho (U - Lam)) G^-1 and Z = U_tilde + Lam: the right-hand side goes straight into images (where W's were) and U is
+        // free from there on, so it takes U_tilde; the last one goes where the caller wants it.  Lam is added on the way out.
         rc = gemm3x_split_rhs(w.B0, U, Lambda, rho, ni, ri, w.Wimg, st);
-        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, G3xOut{it == n_inner - 1 ? U_tilde : nullptr, ri, false, Lambda, w.Z}, ni, ri, ri, w.info + 2, st);
+        float *Ut = it == n_inner - 1 && U_tilde ? U_tilde : U;
+        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, G3xOut{Ut, ri, false, Lambda, w.Z}, ni, ri, ri, w.info + 2, st);
         if (rc) return rc;
         rc = mdbf_msvid(w.Z, n, r, l, n_iter, Q0, S_packed, Ul, Vl, sigma, w.msvid, w.msvid_bytes, stream);
         if (rc) return rc;
         auto recon = l <= 4 ? admm::recon_dual_kernel<4> : l <= 8 ? admm::recon_dual_kernel<8> : l <= 16 ? admm::recon_dual_kernel<16> : admm::recon_dual_kernel<32>;
-        recon<<<dim3(ceil_div(ri, admm::RC_COLS), ceil_div(ni, admm::RC_ROWS)), admm::RC_COLS, 0, st>>>(S_packed, Ul, Vl, l, w.Z, U, Lambda, ni, ri, nwords);
+        recon<<<dim3(ceil_div(ri, admm::RC_COLS), ceil_div(ni, admm::RC_ROWS)), admm::RC_COLS, 0, st>>>(S_packed, Ul, Vl, l, Ut, U, Lambda, ni, ri, nwords);
     }
     admm::flag_kernel<<<1, 32, 0, st>>>(w.info, sigma, l);                      // the factorisation's flag or an expired wait
     MDBF_CUDA(cudaGetLastError());

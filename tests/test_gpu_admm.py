@@ -256,3 +256,23 @@ def test_inverse_of_the_system_by_doubling(R):
                               (W.double() @ V8 + rho * (U.double() - Lam.double())).T).T
     got = run_update(W.cpu().numpy(), V.cpu().numpy(), U.cpu().numpy(), Lam.cpu().numpy(), rho, 1, 1, 4)["tilde"]
     assert np.max(np.abs(got - want.cpu().numpy())) <= 2e-5 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("N,Mc,R,l", [(200, 190, 64, 4), (515, 300, 129, 16), (130, 300, 36, 32)])
+def test_the_dual_is_rounded_at_its_own_size(N, Mc, R, l):
+    """Lam + (U_tilde - U) near convergence, where the dual and the difference are small beside the iterate: one rounding of the difference
+    and one of the sum, 2^-24 of either - and not one of the iterate, which is a hundred times as large."""
+    g = np.random.default_rng(8)
+    env = lambda rows: np.exp(0.25 * g.standard_normal((rows, l))) * 0.8 ** (0.5 * np.arange(l))
+    V = np.where(g.random((Mc, R)) < 0.5, -1.0, 1.0) * (env(Mc) @ env(R).T)
+    U = np.where(g.random((N, R)) < 0.5, -1.0, 1.0) * (env(N) @ env(R).T)
+    W = U @ V.T
+    Lam = 1e-4 * g.standard_normal((N, R)) * np.abs(U)
+    W, V, U, Lam = (a.astype(np.float32) for a in (W, V, U, Lam))
+    rho = 3.0 * float(np.sum(V.astype(np.float64) ** 2)) / R
+    out = run_update(W, V, U, Lam, rho, l, 1, 8)
+    step = out["tilde"] - out["U"]                                # exact in fp64, as is the sum
+    exact = Lam.astype(np.float64) + step
+    assert np.median(np.abs(exact)) < 0.02 * np.median(np.abs(out["tilde"]))
+    err = np.abs(out["Lam"] - exact)
+    assert np.all(err <= 2.0 ** -24 * (np.abs(step) + np.abs(exact)) * 1.001 + 1e-45), np.max(err / np.abs(exact))
