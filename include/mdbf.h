@@ -351,7 +351,7 @@ mdbf_status_t mdbf_msvid_workspace_bytes(int64_t rows, int64_t cols, int32_t l, 
  *   workspace  device, mdbf_admm_workspace_bytes(N, M, R, l) bytes on a 256-byte boundary (three N x R matrices, the R x R
  *              system, the operand images of op(W) and V - their size and a little more - and mdbf_msvid's workspace)
  * The dense products (W V, V^T V, the inverse of the system and its application) run on the tensor cores (fp16
- * operands, scaled per row, in a three-term split, fp32 accumulation in chunks of 128 contraction indices; U_tilde comes out within a few
+ * operands, scaled per row, in a three-term split, fp32 accumulation in chunks of 64 contraction indices; U_tilde comes out within a few
  * 1e-6 of its largest entry of the exact result); the Cholesky factorisation and the solves of the R x R system are cuSOLVER calls in
  * fp32; the MSVID step, the elementwise passes and the reconstruction of the dense factor fused with the dual update
  * are this library's kernels.  Asynchronous on `stream`; part of the work runs on a stream of the library's own that

@@ -1,13 +1,17 @@
 // Dense fp32 product C = A B on the tensor cores at close to fp32 accuracy: tcgen05 kind::f16 on a scaled two-part split
-//     a b  ~  a_hi b_hi + a_hi b_lo + a_lo b_hi          (the dropped a_lo b_lo is below 2^-24 a b)
+//     a b  ~  a_hi b_hi + 2^-11 (a_hi b_lo + a_lo b_hi)  (the dropped product of the low parts is below 2^-24 a b)
 // with fp32 accumulation in tensor memory.  It serves the least-squares step of the ADMM refinement (W V and V^T V,
 // Eq. admm-U-tilde), where the FP32 pipe would need eight times as long.
 //
 // The split.  A row of an operand (a row of A, a column of B) is multiplied by the power of two that brings its largest entry into
-// [2^14, 2^15); hi = the scaled entry rounded to fp16, lo = the exact residual rounded to fp16: 11 + 11 significant bits, the same as
-// two TF32 parts, with an absolute floor 2^-39 below the row's largest entry where lo runs out of exponent.  The product is multiplied by
+// [2^14, 2^15); hi = the scaled entry rounded to fp16, lo = 2^11 times the exact residual, rounded to fp16.  With the factor lo keeps the
+// exponent of hi, so entries down to 2^-29 of the row's largest have 11 + 11 significant bits, the same as two TF32 parts, and smaller ones
+// an absolute error of 2^-51 of it (without the factor: 2^-17 and 2^-40, which shows where small entries of W meet large ones of V; rows and
+// columns scaled against each other by 10^+-4: 6.0e-5 of the iterate without it, 7.9e-7 with it, 2.5e-6 with TF32 parts).  The cross terms
+// of a K block are formed first, and the first product of the high parts scales the accumulator by 2^-11 as it adds to it.  C is multiplied by
 // both inverse scales on the way out (exact).  fp16 operands issue at twice the TF32 rate and are half the bytes: 8192 x 3712 x 3712
-// 943 -> 566 us; 8192 x 3712 x 8192 on 124 SMs 2193 -> 1271; error of an ADMM iterate against fp64 2.0e-6 -> 1.4e-6.
+// 943 -> 566 us, 8192 x 3712 x 8192 on 124 SMs 2193 -> 1271, with single accumulations over two K blocks; the factor and one K block per
+// accumulation take 2.5 % more.  Error of an ADMM iterate against fp64 at that size: TF32 2.0e-6, without the factor 1.4e-6, now 5.8e-7.
 //
 // Two passes.  The split kernels turn an operand into "images": per tile of 128 rows (output rows for A, output
 // columns for B) and block of 64 contraction indices one 32 KB piece holding hi (128 rows of 64 fp16 values, 128 bytes
@@ -17,8 +21,8 @@
 // element is read at src[i * stride_i + k * stride_k] with one of the strides equal to one.
 // gemm3x_kernel: one CTA per SM walks over 128 x 256 tiles of C (two column tiles of B side by side: the stream from L2
 // into shared memory, 96 KB per K block, is what bounds the kernel, and a wider tile spends less of it per flop); one
-// lane streams the pieces of each K block into a ring by bulk copies, one lane issues  D (+)= A_hi B_hi, D += A_hi B_lo,
-// D += A_lo B_hi  (N = 256, four K steps of 16 each), the eight epilogue warps read the accumulators and store.  Every wait is bounded; on expiry the status word is
+// lane streams the pieces of each K block into a ring by bulk copies, one warp issues  D = A_hi B_lo, D += A_lo B_hi,
+// D = 2^-11 D + A_hi B_hi  (N = 256, four K steps of 16 each), the eight epilogue warps add the K blocks' accumulators up and store.  Every wait is bounded; on expiry the status word is
 // set and the tiles still to be written come out as NaN.
 #include <algorithm>
 #include <cstdint>
@@ -33,7 +37,7 @@ constexpr int TILE = 128, KB = 64;
 constexpr int HALF = TILE * KB * 2;            // bytes of the hi (or lo) part of a piece
 constexpr int PIECE = 2 * HALF;                // 32 KB
 constexpr int STAGES = 2;
-constexpr int KCHUNK = 2;                      // K blocks accumulated in tensor memory before the sum moves to fp32 registers
+constexpr int LO_SHIFT = 11;                   // lo is the residual times 2^11
 constexpr int STAGE_BYTES = 3 * PIECE;         // A piece, then B_hi of two column tiles, then their B_lo
 constexpr int EPI_WARPS = 8;                   // two per quarter of the TMEM lanes, each with half of the tile's columns
 constexpr int THREADS = (EPI_WARPS + 2) * 32;  // epilogue warps, loader, issuer
@@ -55,7 +59,7 @@ __device__ __forceinline__ void split8(const float (&v)[8], float scale, uint4 &
         const float a = v[2 * u] * scale, b = v[2 * u + 1] * scale;
         const __half2 hh = __floats2half2_rn(a, b);
         const float2 back = __half22float2(hh);
-        const __half2 ll = __floats2half2_rn(a - back.x, b - back.y);
+        const __half2 ll = __floats2half2_rn((a - back.x) * (float)(1 << LO_SHIFT), (b - back.y) * (float)(1 << LO_SHIFT));
         h[u] = *reinterpret_cast<const uint32_t *>(&hh);
         l[u] = *reinterpret_cast<const uint32_t *>(&ll);
     }
@@ -202,11 +206,10 @@ __device__ __forceinline__ void tile_of(int t, int ntn2, int part, int &mt, int 
 __device__ __forceinline__ int first_kb(int part, int mt, int nt2) { return part == G3X_FACTORS ? max(mt * TILE, nt2 * 2 * TILE) / KB : 0; }
 
 // Persistent: CTA c takes the tiles c, c + gridDim.x, ... (row tile = t / ntn2, so that CTAs running side by side share
-// their pieces of A in L2).  Two accumulators of 256 tensor-memory columns alternate between tiles: the epilogue of
-// one tile runs under the products of the next.  All three terms of a tile accumulate into the same columns, for KCHUNK
-// K blocks at a time: the tensor core's accumulation is not rounded to nearest, and its one-sided error grows with the
-// number of accumulations (6e-5 of the result over 8192 contraction indices, measured); the chunks' sums are added in
-// fp32 by the epilogue, in registers.  ntn is
+// their pieces of A in L2).  Two accumulators of 256 tensor-memory columns alternate: the epilogue of
+// one K block runs under the products of the next.  All three terms of a K block accumulate into the same columns, and the K blocks'
+// sums are added in fp32 by the epilogue, in registers: the tensor core's accumulation is not rounded to nearest, and its one-sided error
+// grows with the number of accumulations (6e-5 of the result over 8192 contraction indices, measured).  ntn is
 // the number of 128-column tiles of B's images, ntn2 = ceil(ntn / 2) the number of tiles here; an odd last tile has no
 // second half: nothing is copied for it, the products read whatever the buffer holds, and nothing of it is stored.
 __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__restrict__ Aimg, const uint32_t *__restrict__ Bimg,
@@ -245,7 +248,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
 
     if (warp < EPI_WARPS) {
         // ===================================== epilogue =====================================
-        // thread = one row and one half (128 columns) of the tile; the chunks' sums are added in registers, in fp32
+        // thread = one row and one half (128 columns) of the tile; the K blocks' sums are added in registers, in fp32
         const int half = warp >> 2;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const bool vec = (o.ldc & 3) == 0 && ((reinterpret_cast<uintptr_t>(o.C) | reinterpret_cast<uintptr_t>(o.add) | reinterpret_cast<uintptr_t>(o.sum)) & 15u) == 0;
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
             int mt, nt2;
             tile_of(t, ntn2, o.part, mt, nt2);
-            const int nk = nkb - first_kb(o.part, mt, nt2), nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
+            const int nk = nkb - first_kb(o.part, mt, nt2), nch = max(nk, 1);
             const int row = mt * TILE + (warp & 3) * 32 + lane;
             const int col0 = nt2 * 2 * TILE + half * TILE;
             float sum[TILE];
@@ -348,30 +351,28 @@ __global__ void __launch_bounds__(THREADS, 1) gemm3x_kernel(const uint32_t *__re
         for (int t = blockIdx.x; t < ntiles && alive; t += gridDim.x) {
             int mt, nt2;
             tile_of(t, ntn2, o.part, mt, nt2);
-            const int kb0 = first_kb(o.part, mt, nt2), nk = nkb - kb0, nch = nk > 0 ? (nk + KCHUNK - 1) / KCHUNK : 1;
+            const int nk = nkb - first_kb(o.part, mt, nt2), nch = max(nk, 1);
             for (int ch = 0; ch < nch && alive; ++ch, ++it) {
                 const int as = it & 1;
                 alive = __all_sync(0xffffffffu, mbar_wait(acc_empty + 8 * as, (((uint32_t)(it >> 1)) & 1u) ^ 1u, abort_flag, status));
                 if (!alive) break;
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(as * 2 * TILE);
-                const int kb_begin = kb0 + ch * KCHUNK, kb_end = min(nkb, kb_begin + KCHUNK);
-                for (int kb = kb_begin; kb < kb_end && alive; ++kb) {
+                if (nk > 0) {                                    // one K block
                     alive = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * s, ph, abort_flag, status));
-                    if (!alive) break;
                     tc_fence_after();
                     const uint32_t stage = smem_base + (uint32_t)(s * STAGE_BYTES);
                     const uint64_t a_hi = make_smem_desc(stage), a_lo = make_smem_desc(stage + (uint32_t)HALF);
                     const uint64_t b_hi = make_smem_desc(stage + (uint32_t)PIECE), b_lo = make_smem_desc(stage + (uint32_t)(2 * PIECE));
-                    const bool fresh = kb == kb_begin;           // the chunk starts on a cleared accumulator
-                    if (elect_one()) {
+                    if (alive && elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 4; ++ks)           // 16 fp16 = 32 bytes per K step
-                            umma_ss(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, (!fresh || ks > 0) ? 1u : 0u);
-#pragma unroll
-                        for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_hi + (uint64_t)(2 * ks), b_lo + (uint64_t)(2 * ks), idesc, 1u);
+                        for (int ks = 0; ks < 4; ++ks)           // 16 fp16 = 32 bytes per K step; the first one clears the accumulator
+                            umma_ss(d, a_hi + (uint64_t)(2 * ks), b_lo + (uint64_t)(2 * ks), idesc, ks > 0 ? 1u : 0u);
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) umma_ss(d, a_lo + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
+                        umma_ss_rescale<LO_SHIFT>(d, a_hi, b_hi, idesc);
+#pragma unroll
+                        for (int ks = 1; ks < 4; ++ks) umma_ss(d, a_hi + (uint64_t)(2 * ks), b_hi + (uint64_t)(2 * ks), idesc, 1u);
                         umma_commit(empty_bar + 8 * s);
                     }
                     __syncwarp();

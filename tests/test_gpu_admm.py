@@ -276,3 +276,21 @@ def test_the_dual_is_rounded_at_its_own_size(N, Mc, R, l):
     assert np.median(np.abs(exact)) < 0.02 * np.median(np.abs(out["tilde"]))
     err = np.abs(out["Lam"] - exact)
     assert np.all(err <= 2.0 ** -24 * (np.abs(step) + np.abs(exact)) * 1.001 + 1e-45), np.max(err / np.abs(exact))
+
+
+@pytest.mark.parametrize("N,Mc,R,transpose", [(150, 400, 64, False), (300, 700, 96, True)])
+def test_wide_range_inside_a_row(N, Mc, R, transpose):
+    """Rows of V across eight orders of magnitude and columns of W the other way: every term of W V matters, the smallest entries of a
+    row of W meet the largest of V.  Parts with 22 significant bits of each entry err by some 2^-22 of a term; parts whose error is
+    2^-40 of their row's largest entry err by 2^-40 * 10^4 * 10^4 = 1e-4 of one.  The bound is that of the well-conditioned systems above."""
+    W, V, U, Lam = problem(N, Mc, R, seed=91)
+    d = 10.0 ** np.random.default_rng(4).uniform(-4, 4, Mc)
+    Wop, V = (W / d).astype(np.float32), (V * d[:, None]).astype(np.float32)
+    U, Lam = np.zeros_like(U), np.zeros_like(Lam)
+    Vd, Wd = V.astype(np.float64), Wop.astype(np.float64)
+    rho = float(np.sum(Vd ** 2)) / R
+    g = run_update(np.ascontiguousarray(Wop.T) if transpose else Wop, V, U, Lam, rho, 4, 1, 2, transpose)
+    ref = np.linalg.solve(Vd.T @ Vd + rho * np.eye(R), (Wd @ Vd).T).T
+    err = np.max(np.abs(g["tilde"] - ref)) / np.max(np.abs(ref))
+    print("wide range:", err)
+    assert err <= 2e-5, err
