@@ -294,3 +294,19 @@ def test_wide_range_inside_a_row(N, Mc, R, transpose):
     err = np.max(np.abs(g["tilde"] - ref)) / np.max(np.abs(ref))
     print("wide range:", err)
     assert err <= 2e-5, err
+
+
+def test_rows_near_the_ends_of_fp32():
+    """Rows of W up to 10^34 against columns of V around 10^-1: each product and each sum is inside fp32, and so is what the row and
+    column scales make of them on the way out.  Bound per row as for the rows of very different scale."""
+    N, Mc, R = 140, 260, 64
+    Wop, V, U, Lam = problem(N, Mc, R, seed=78)
+    Wop = (Wop / np.abs(Wop).max(axis=1, keepdims=True) * 10.0 ** np.linspace(-28, 34, N)[:, None]).astype(np.float32)
+    V = (0.1 * V).astype(np.float32)
+    Vd, Wd = V.astype(np.float64), Wop.astype(np.float64)
+    rho = float(np.sum(Vd ** 2)) / R
+    g = run_update(Wop, V, np.zeros_like(U), np.zeros_like(Lam), rho, 4, 1, 2)
+    ref = np.linalg.solve(Vd.T @ Vd + rho * np.eye(R), (Wd @ Vd).T).T
+    assert np.abs(ref).max() < 1e37
+    err = np.abs(g["tilde"] - ref).max(axis=1) / np.abs(ref).max(axis=1)
+    assert np.all(err <= 2e-5), np.max(err)
