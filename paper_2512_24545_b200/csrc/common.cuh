@@ -200,7 +200,7 @@ bool t1_supports(const Layer &L);
 mdbf_status_t launch_forward_t1_group(Layer *const *Ls, int n, const void *const *xs, void *const *ys, cudaStream_t st, int stages = 3);
 constexpr int kMaxSiblings = 4;   // layers one launch of the one-token kernel can serve
 int last_t1_launch_count();
-mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, void *y, cudaStream_t st);
+mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, void *y, bool *fits, cudaStream_t st);
 mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st, int stages = 3, bool no_room = false);
 mdbf_status_t launch_wk2(const uint32_t *canon, int rows, int nwords, uint2 *out, int rblocks, int kb_pad,
                          cudaStream_t st);

@@ -678,10 +678,11 @@ static mdbf_status_t launch_stage(const TxMulti &full, const TxPlan &p, const in
 
 // Both stages of n layers that read the same x (n = 1: a single layer): one launch per stage.
 // sum_y != nullptr: the n layers are the terms of a sum; stage B of all terms shares one launch (they read the same x), stage A of
-// all terms another (tmem_t1_sum_kernel).
+// all terms another (tmem_t1_sum_kernel), whose ranks share a cluster: each term has fewer of them than on its own and a longer part
+// of its reduction per CTA.  Where that does not fit in shared memory *sum_fits is set to false and nothing is launched.
 template <int LP>
 static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const *ys, cudaStream_t st,
-                            void *sum_y = nullptr, int stages = 3, bool no_room = false) {
+                            void *sum_y = nullptr, int stages = 3, bool no_room = false, bool *sum_fits = nullptr) {
     int rowsB[TX_MAX_LAYERS], kbB[TX_MAX_LAYERS], rowsA[TX_MAX_LAYERS], kbA[TX_MAX_LAYERS];
     for (int i = 0; i < n; ++i) {
         rowsB[i] = Ls[i]->d.k; kbB[i] = Ls[i]->kbpB;
@@ -689,7 +690,12 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
     }
     g_t1_launches = 0;
     TxPlan pb, pa;
-    if (!plan_t1(n, rowsB, kbB, LP, &pb) || !plan_t1(n, rowsA, kbA, LP, &pa)) {
+    const bool fits = plan_t1(n, rowsB, kbB, LP, &pb) && plan_t1(n, rowsA, kbA, LP, &pa, sum_y ? n : 1);
+    if (sum_y) {
+        *sum_fits = fits;
+        if (!fits) return MDBF_OK;
+    }
+    if (!fits) {
         set_error("mdbf_linear_forward: the one-token TMEM kernel does not fit this shape");
         return MDBF_ERR_SHAPE;
     }
@@ -718,23 +724,13 @@ static mdbf_status_t run_t1(Layer *const *Ls, int n, const void *x, void *const 
     if (!(stages & 2)) return MDBF_OK;
     if (!sum_y) return launch_stage<LP>(ma, pa, kbA, &no_room, st);
     // the terms of a sum: one launch, all of them rounded into y together
-    TxMulti sum = ma;
-    TxPlan ps;
-    if (!plan_t1(n, rowsA, kbA, LP, &ps, n)) {
-        set_error("mdbf_linear_forward_sum: the one-token TMEM kernel does not fit this shape");
-        return MDBF_ERR_SHAPE;
-    }
-    sum.sum_ks = ps.ks / n;
-    sum.nlayers = n;
-    sum.rb_start[n] = ceil_div(rowsA[0], 128);
+    ma.sum_ks = pa.ks / n;
+    ma.rb_start[n] = ceil_div(rowsA[0], 128);
     for (int i = 0; i < n; ++i) {
-        TxArgs &s = sum.layer[i];
-        s.out = sum_y;
-        s.stage_a = 1;
-        s.pairs_per_cta = ps.pairs_per_cta[i];
-        s.nastages = ps.nastages; s.nsstages = ps.nsstages; s.tmem_cols = ps.tmem_cols;
+        ma.layer[i].out = sum_y;
+        ma.layer[i].stage_a = 1;
     }
-    return launch_t1<LP>(sum, ps, &no_room, st);
+    return launch_t1<LP>(ma, pa, &no_room, st);
 }
 
 // n <= TX_MAX_LAYERS layers with the same LP, all prepared for the one-token kernel.  no_room: the launch before this call leaves no
@@ -753,16 +749,16 @@ mdbf_status_t launch_forward_tmem_t1_multi(Layer *const *Ls, int n, const void *
     }
 }
 
-// The terms of a sum of layers (same LP, at most TX_MAX_LAYERS) at one token: y = bf16(sum of the terms' outputs).
-mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, void *y, cudaStream_t st) {
+// The terms of a sum of layers (same LP, at most TX_MAX_LAYERS) at one token: y = bf16(sum of the terms' outputs), or nothing and *fits = false.
+mdbf_status_t launch_forward_tmem_t1_sum(Layer *const *Ls, int n, const void *x, void *y, bool *fits, cudaStream_t st) {
     void *ys[TX_MAX_LAYERS] = {};
     switch (Ls[0]->LP) {
-        case 1: return run_t1<1>(Ls, n, x, ys, st, y);
-        case 2: return run_t1<2>(Ls, n, x, ys, st, y);
-        case 4: return run_t1<4>(Ls, n, x, ys, st, y);
-        case 8: return run_t1<8>(Ls, n, x, ys, st, y);
-        case 16: return run_t1<16>(Ls, n, x, ys, st, y);
-        case 32: return run_t1<32>(Ls, n, x, ys, st, y);
+        case 1: return run_t1<1>(Ls, n, x, ys, st, y, 3, false, fits);
+        case 2: return run_t1<2>(Ls, n, x, ys, st, y, 3, false, fits);
+        case 4: return run_t1<4>(Ls, n, x, ys, st, y, 3, false, fits);
+        case 8: return run_t1<8>(Ls, n, x, ys, st, y, 3, false, fits);
+        case 16: return run_t1<16>(Ls, n, x, ys, st, y, 3, false, fits);
+        case 32: return run_t1<32>(Ls, n, x, ys, st, y, 3, false, fits);
         default:
             set_error("mdbf_linear_forward_sum: the one-token TMEM kernel handles l <= 32 (got %d)", Ls[0]->d.l);
             return MDBF_ERR_SHAPE;

@@ -626,10 +626,13 @@ mdbf_status_t mdbf_linear_forward_sum(const mdbf_handle_t *terms, int32_t P, con
             terms[p]->last_kernel = MDBF_KERNEL_TMEM;
             terms[p]->last_launches = 0;
         }
-        mdbf_status_t rc = launch_forward_tmem_t1_sum(Ls, P, x, y, st);
+        bool fits = false;
+        mdbf_status_t rc = launch_forward_tmem_t1_sum(Ls, P, x, y, &fits, st);
         if (rc) return rc;
-        terms[0]->last_launches = last_t1_launch_count();
-        return MDBF_OK;
+        if (fits) {
+            terms[0]->last_launches = last_t1_launch_count();
+            return MDBF_OK;
+        }
     }
     // otherwise: term 0 stores its fp32 output into acc, the others add to it (stream order), a cast pass follows
     for (int p = 0; p < P; ++p) {

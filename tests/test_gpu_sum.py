@@ -88,6 +88,16 @@ def test_terms_share_the_cluster_of_a_row_block(ks, l):
     assert rel_err(y, ref) <= TOL["bf16"]
 
 
+@pytest.mark.parametrize("ks", [[100000, 64], [160000, 159000, 159500, 160000]])
+def test_terms_too_long_for_a_shared_cluster(ks):
+    """Each term fits the one-token kernel with up to eight ranks of its own, together they have too few: one after the other then."""
+    specs = term_specs(128, 128, ks, [1] * len(ks))
+    x = inputs.make_activations(specs[0], 1)
+    y, ref, _ = run_sum(specs, x)
+    assert np.all(np.isfinite(y))
+    assert rel_err(y, ref) <= TOL["bf16"]
+
+
 def test_fp32_terms_and_single_term():
     t = inputs.tiny()
     specs = [inputs.scaled(t, name="a", seed=1), inputs.scaled(t, name="b", seed=2, env_std=t.env_std * 0.5)]
