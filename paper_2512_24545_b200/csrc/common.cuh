@@ -106,6 +106,8 @@ void set_error(const char *fmt, ...);
 mdbf_status_t cuda_fail(cudaError_t e, const char *what);
 // MDBF_OK when the current device is one this library runs on (compute capability 10.x), MDBF_ERR_ARCH otherwise
 mdbf_status_t require_device(int *dev_out);
+// SMs of the current device (a part of a GPU has fewer than 148); asked of the runtime once per device
+mdbf_status_t device_sms(int *sms);
 // fp32-accurate dense product on the tensor cores (gemm3x.cu): operand images, then C = A B
 size_t gemm3x_image_bytes(int64_t rows, int64_t depth);
 mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, int rows, int depth, uint32_t *img, cudaStream_t st);

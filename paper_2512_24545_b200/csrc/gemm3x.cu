@@ -439,15 +439,9 @@ mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, const G3xOu
     static PerDeviceOnce once;
     if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(g3x::gemm3x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g3x::SMEM));
     const int ntm = ceil_div(n, g3x::TILE), ntn = ceil_div(r, g3x::TILE);
-    static int sms_of_device[64] = {};
-    int dev = 0, sms = 0;
-    MDBF_CUDA(cudaGetDevice(&dev));
-    if (dev >= 0 && dev < 64 && sms_of_device[dev]) {
-        sms = sms_of_device[dev];
-    } else {
-        MDBF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (dev >= 0 && dev < 64) sms_of_device[dev] = sms;
-    }
+    int sms = 0;
+    mdbf_status_t rc = device_sms(&sms);
+    if (rc) return rc;
     const int ntn2 = ceil_div(ntn, 2);
     if (o.part != G3X_ALL && (n != r || (o.part == G3X_FACTORS && depth != n))) { set_error("gemm3x_run: a symmetric result is square"); return MDBF_ERR_INVALID_ARG; }
     int ntiles = ntm * ntn2;

@@ -1,4 +1,5 @@
 // C-ABI entry points of libmdbf: argument checking, handle lifetime, dispatch.
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -54,6 +55,19 @@ static mdbf_status_t check_handle(mdbf_handle_t h, const char *fn) {
     if (h == nullptr || h->magic != kHandleMagic) {
         set_error("%s: invalid handle", fn);
         return MDBF_ERR_INVALID_ARG;
+    }
+    return MDBF_OK;
+}
+
+mdbf_status_t device_sms(int *sms) {
+    static std::atomic<int> known[64];
+    int dev = 0;
+    MDBF_CUDA(cudaGetDevice(&dev));
+    const bool slot = dev >= 0 && dev < 64;
+    *sms = slot ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (*sms == 0) {
+        MDBF_CUDA(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
+        if (slot) known[dev].store(*sms, std::memory_order_relaxed);
     }
     return MDBF_OK;
 }

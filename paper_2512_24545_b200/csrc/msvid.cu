@@ -26,6 +26,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "plans.h"
 #include "tmem_ptx.cuh"
 
 namespace mdbf {
@@ -1006,7 +1007,10 @@ template <int LP>
 static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr) {
     using C = OrCfg<LP>;
     auto kern = orth_kernel<LP>;
-    const int ctas = std::min(ceil_div(n, OR_ROWS), GR_MAX_CTAS), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
+    int sms = 0;
+    mdbf_status_t rc = device_sms(&sms);
+    if (rc) return rc;
+    const int ctas = orth_ctas(n, OR_ROWS, GR_MAX_CTAS, sms), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
     static PerDeviceOnce once;
     if (once.first()) {
         MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));

@@ -26,4 +26,11 @@ inline uint64_t host_view(const HostRange &r, size_t bytes) {
 constexpr int kHostStoreMaxT = 64;
 inline bool host_store_direct(uint64_t device, size_t es, int T) { return device != 0 && device % es == 0 && T <= kHostStoreMaxT; }
 
+// CTAs of the cooperative orthogonalisation of n rows in chunks of `chunk`: at most `most`, and one per SM, so that all of them run at once
+// on any device (a cooperative launch with more than that is refused).
+inline int orth_ctas(int n, int chunk, int most, int sms) {
+    const int chunks = (n + chunk - 1) / chunk, limit = sms < most ? sms : most;
+    return chunks < limit ? chunks : limit;
+}
+
 }  // namespace mdbf

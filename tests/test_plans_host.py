@@ -14,6 +14,7 @@ uint64_t t_host_view(int pinned, uint64_t device, uint64_t start, size_t size, s
     return host_view(HostRange{pinned != 0, device, start, size}, bytes);
 }
 int t_host_store_direct(uint64_t device, size_t es, int T) { return host_store_direct(device, es, T); }
+int t_orth_ctas(int n, int chunk, int most, int sms) { return orth_ctas(n, chunk, most, sms); }
 }
 """
 
@@ -47,3 +48,11 @@ def test_a_host_buffer_has_to_lie_in_one_pinned_mapping(plans, pinned, off, size
 def test_which_y_the_kernels_store_themselves(plans, off, es, T, ok):
     assert plans.t_host_store_direct(0x7F0000000000 + off, es, T) == ok
     assert plans.t_host_store_direct(0, es, T) == 0
+
+
+@pytest.mark.parametrize("sms", [1, 16, 32, 74, 128, 148])
+@pytest.mark.parametrize("n", [1, 128, 129, 5000, 28672, 1 << 21])
+def test_a_cooperative_launch_fits_on_the_device(plans, n, sms):
+    ctas, chunks = plans.t_orth_ctas(n, 128, 128, sms), -(-n // 128)
+    assert 1 <= ctas <= min(sms, 128, chunks)
+    assert ctas == chunks or ctas == min(sms, 128)
