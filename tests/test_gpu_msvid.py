@@ -47,7 +47,8 @@ def envelope_error(Z, U, V):
 # included), the others the scalar kernels; l = 8 and 32 take the remaining operand widths
 @pytest.mark.parametrize("shape,l", [(s, l) for s in [(300, 517), (1024, 768), (129, 33), (64, 2000), (2000, 64), (33, 40)]
                                      for l in (1, 4, 16)] + [((333, 516), 8), ((333, 516), 32), ((1000, 260), 8), ((1000, 260), 32),
-                                                             ((515, 1028), 16)])
+                                                             ((515, 1028), 16),
+                                                             ((140000, 48), 16), ((70000, 40), 32)])      # more rows than an orthogonalisation keeps in shared memory
 def test_sign_mask_exact_and_envelope_near_the_optimum(shape, l):
     rows, cols = shape
     Z = inputs.make_factor_matrix(rows, cols, seed=5)
