@@ -39,6 +39,8 @@
 // returns.  Every TMA and bulk copy targets the issuing CTA's own shared memory only.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "plans.h"
 #include "tmem_ptx.cuh"
 
@@ -837,11 +839,12 @@ static bool mt_split_fits(int kc, int nv, int bn, int ks) {
 // CTAs of the split kernel that run at once in clusters of `ks` (one CTA per SM; the SMs of a graphics processing cluster that a cluster size does
 // not divide stay idle: 148 at one rank, 128 or fewer at eight).  Asked of the runtime once per device and size.
 static int mt_resident(int ks) {
-    static int known[64][9] = {};
+    static std::atomic<int> known[64][9];
     int dev = 0;
     if (ks == 1) return 148;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 128 / ks * ks;
-    if (!known[dev][ks]) {
+    int resident = known[dev][ks].load(std::memory_order_relaxed);
+    if (resident == 0) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -859,9 +862,10 @@ static int mt_resident(int ks) {
             cudaGetLastError();
             n = 128 / ks;
         }
-        known[dev][ks] = n * ks;
+        resident = n * ks;
+        known[dev][ks].store(resident, std::memory_order_relaxed);
     }
-    return known[dev][ks];
+    return resident;
 }
 // Token tile and ranks along the reduction of one stage with more than 64 tokens: the least estimated time over waves of 148 CTAs.
 // A pair of K blocks costs 0.41 us + 0.16 us per 256 tokens (the issuing threads, then the tensor pipe), a CTA's set-up and
