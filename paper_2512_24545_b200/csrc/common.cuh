@@ -14,8 +14,10 @@ namespace mdbf {
 constexpr uint32_t kHandleMagic = 0x4D444246u;  // "MDBF"
 constexpr int kMaxL = 64;
 
-// tensor maps of the last materialised-order forward (they depend only on the pointers and T)
+// plan (token tile and ranks along the reduction of each stage: they depend on the layer and plan_T alone) and tensor maps (on the pointers
+// too) of the last materialised-order forward
 struct MatMaps {
+    int plan_T, bnB, ksB, bnA, ksA;
     bool valid;
     const void *x, *y;
     int T;
