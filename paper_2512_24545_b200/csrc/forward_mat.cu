@@ -48,16 +48,12 @@ namespace cg = cooperative_groups;
 
 namespace mdbf {
 
-constexpr int MT_BM = 128;
-constexpr int MT_BN = 256;
-constexpr int MT_BK = 64;
 constexpr int MT_XWARPS = 16;            // tile builders: (block of the pair) x (half of its 64 columns) x (32-row quadrant)
 constexpr int MT_W_TMA = MT_XWARPS;
 constexpr int MT_W_MMA = MT_W_TMA + 1;
 constexpr int MT_W_ENV = MT_W_TMA + 2;
 constexpr int MT_W_MINI = MT_W_TMA + 3;
 constexpr int MT_THREADS = (MT_W_MINI + 1) * 32;
-constexpr int MT_MAX_NS = 12;            // activation-tile ring depth: 6 tiles of 256 tokens, more with narrower tiles
 constexpr int MT_NA = 2;                 // W_hat tile slots in TMEM, a pair of K blocks (2 x 32 columns) each
 constexpr int MT_MAX_NV = 4;             // V-image ring depth in pairs of K blocks (4 with l <= 16, 3 with l <= 32)
 constexpr int MT_TMEM_COLS = 512;
@@ -516,7 +512,6 @@ constexpr int MS_W_ENV = MS_XWARPS + 1;
 constexpr int MS_W_MINI = MS_XWARPS + 2;
 constexpr int MS_W_MMA0 = MS_XWARPS + 3;
 constexpr int MS_THREADS = (MS_W_MMA0 + MS_BUFS) * 32;
-constexpr int MS_BN = 64;
 static_assert(kHostStoreMaxT <= MS_BN, "a y in host memory is stored by this kernel's plain stores");
 
 template <bool STAGE_A, bool SPLIT>
@@ -821,21 +816,6 @@ bool mat_path_supports(const Layer &L, const void *x, int T) {
     return L.uiA && L.zb && T >= 2 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && L.d.d_in % 8 == 0;
 }
 
-// shared memory: ring of activation tiles, U image, ring of V images, (split launches) partial sums, slack
-static int mt_ring(int kc, int nv, int bn, size_t part_bytes) {
-    const size_t avail = 227 * 1024 - 1024 - 1024 - (size_t)(1 + nv) * kc * 2048 - part_bytes;    // 1 KB static, 1 KB slack
-    const int n = (int)(avail / ((size_t)bn * MT_BK * 2)) / 2 * 2;
-    return n < MT_MAX_NS ? n : MT_MAX_NS;
-}
-static size_t mt_smem_bytes(int kc, int nv, int bn, size_t part_bytes) {
-    return (size_t)mt_ring(kc, nv, bn, part_bytes) * bn * MT_BK * 2 + (size_t)(1 + nv) * kc * 2048 + part_bytes + 1024;
-}
-// Tokens that a rank of a split large tile adds up (whole 32-column chunks), and whether the ranks' sums fit into the activation
-// ring they are pushed into: at 208 tokens, say, five ranks or more would run past it.
-static int mt_tpr(int bn, int ks) { return ceil_div(ceil_div(bn, ks), 32) * 32; }
-static bool mt_split_fits(int kc, int nv, int bn, int ks) {
-    return (size_t)ks * mt_tpr(bn, ks) * MT_BM * sizeof(float) <= (size_t)mt_ring(kc, nv, bn, 0) * bn * MT_BK * 2;
-}
 // CTAs of the split kernel that run at once in clusters of `ks` (one CTA per SM; the SMs of a graphics processing cluster that a cluster size does
 // not divide stay idle: 148 at one rank, 128 or fewer at eight).  Asked of the runtime once per device and size.
 static int mt_resident(int ks) {
@@ -866,31 +846,6 @@ static int mt_resident(int ks) {
         known[dev][ks].store(resident, std::memory_order_relaxed);
     }
     return resident;
-}
-// Token tile and ranks along the reduction of one stage with more than 64 tokens: the least estimated time over waves of 148 CTAs.
-// A pair of K blocks costs 0.41 us + 0.16 us per 256 tokens (the issuing threads, then the tensor pipe), a CTA's set-up and
-// epilogue 4 us + 2 us per 256 tokens, a split another 2.4 us per 256 tokens and 0.3 us per rank (fitted to a sweep; in units of 10 ns).  Several
-// token tiles are multiples of 64 tokens, the boxes of the output's tensor map.
-// Measured, us per forward, unsplit 256-token tiles -> the plan's: 4096 x 4096, k = 1664, T = 777: 41.4 -> 32.5 (stage B: 52 CTAs of
-// 32 pairs -> 130 of 16); 1024 x 8192, k = 512, T = 2048: 53.5 -> 28.4; 8192 x 8192, k = 3712, T = 100: 65.4 -> 33.2;
-// 8192 x 8192, T = 2048 (232 CTAs) stays whole: 197, two ranks 215.
-static void plan_mat(int rows, int cols, int T, int kc, int nv, int *bn_out, int *ks_out) {
-    const int rb = ceil_div(rows, MT_BM), npr = ceil_div(ceil_div(cols, MT_BK), 2);
-    const int one = ceil_div(T, 16) * 16;
-    const int cand[4] = {T <= MT_BN ? one : 256, T <= MT_BN ? 0 : 192, 128, 0};
-    long best = -1;
-    *bn_out = cand[0]; *ks_out = 1;
-    if (T <= MS_BN) return;                                // the small-tile kernel plans its own split
-    for (int bn : cand) {
-        if (bn == 0 || (bn < T && bn % 64 != 0) || (bn == 128 && T <= 128 && one != 128)) continue;
-        for (int ks = 1; ks <= 8; ++ks) {
-            const int per = ceil_div(npr, ks);
-            if (ks > 1 && (per * (ks - 1) >= npr || !mt_split_fits(kc, nv, bn, ks))) continue;
-            const long waves = ceil_div(rb * ceil_div(T, bn) * ks, mt_resident(ks));
-            const long cost = waves * ((long)per * (41 + bn / 16) + 400 + bn * 25 / 32 + (ks > 1 ? bn * 15 / 16 + 30 * ks : 0));
-            if (best < 0 || cost < best) { best = cost; *bn_out = bn; *ks_out = ks; }
-        }
-    }
 }
 // Tensor map of a bf16 output [T][rows] with rows `pitch` elements apart: box of 128 rows x 64 tokens, no swizzle.
 static mdbf_status_t make_out_tensor_map(CUtensorMap *out, const void *base, int T, int rows, int pitch) {
@@ -995,8 +950,8 @@ mdbf_status_t launch_forward_mat(Layer &L, const void *x, void *y, int T, cudaSt
     MatMaps &m = L.mat_maps;
     if (m.plan_T != T) {
         m.valid = false;
-        plan_mat(d.k, d.d_in, T, L.kcm, nv, &m.bnB, &m.ksB);
-        plan_mat(d.d_out, d.k, T, L.kcm, nv, &m.bnA, &m.ksA);
+        plan_mat(d.k, d.d_in, T, L.kcm, nv, mt_resident, &m.bnB, &m.ksB);
+        plan_mat(d.d_out, d.k, T, L.kcm, nv, mt_resident, &m.bnA, &m.ksA);
         m.plan_T = T;
     }
     // y goes out by TMA when its base and row pitch are 16-byte aligned and it is bf16; otherwise by plain stores.

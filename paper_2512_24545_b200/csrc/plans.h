@@ -33,4 +33,53 @@ inline int orth_ctas(int n, int chunk, int most, int sms) {
     return chunks < limit ? chunks : limit;
 }
 
+// ------------------------------------------------------------------ token tiles (forward_mat.cu)
+constexpr int MT_BM = 128;               // rows of a tile
+constexpr int MT_BN = 256;               // tokens of a large tile at most
+constexpr int MT_BK = 64;                // contraction indices of a K block
+constexpr int MT_MAX_NS = 12;            // activation-tile ring depth: 6 tiles of 256 tokens, more with narrower tiles
+constexpr int MS_BN = 64;                // tokens of a small tile at most
+inline int plan_ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+// shared memory: ring of activation tiles, U image, ring of V images, (split launches) partial sums, slack
+inline int mt_ring(int kc, int nv, int bn, size_t part_bytes) {
+    const size_t avail = 227 * 1024 - 1024 - 1024 - (size_t)(1 + nv) * kc * 2048 - part_bytes;    // 1 KB static, 1 KB slack
+    const int n = (int)(avail / ((size_t)bn * MT_BK * 2)) / 2 * 2;
+    return n < MT_MAX_NS ? n : MT_MAX_NS;
+}
+inline size_t mt_smem_bytes(int kc, int nv, int bn, size_t part_bytes) {
+    return (size_t)mt_ring(kc, nv, bn, part_bytes) * bn * MT_BK * 2 + (size_t)(1 + nv) * kc * 2048 + part_bytes + 1024;
+}
+// Tokens that a rank of a split large tile adds up (whole 32-column chunks), and whether the ranks' sums fit into the activation
+// ring they are pushed into: at 208 tokens, say, five ranks or more would run past it.
+inline int mt_tpr(int bn, int ks) { return plan_ceil_div(plan_ceil_div(bn, ks), 32) * 32; }
+inline bool mt_split_fits(int kc, int nv, int bn, int ks) {
+    return (size_t)ks * mt_tpr(bn, ks) * MT_BM * sizeof(float) <= (size_t)mt_ring(kc, nv, bn, 0) * bn * MT_BK * 2;
+}
+// Token tile and ranks along the reduction of one stage with more than 64 tokens: the least estimated time over waves of 148 CTAs.
+// A pair of K blocks costs 0.41 us + 0.16 us per 256 tokens (the issuing threads, then the tensor pipe), a CTA's set-up and
+// epilogue 4 us + 2 us per 256 tokens, a split another 2.4 us per 256 tokens and 0.3 us per rank (fitted to a sweep; in units of 10 ns).  Several
+// token tiles are multiples of 64 tokens, the boxes of the output's tensor map.
+// Measured, us per forward, unsplit 256-token tiles -> the plan's: 4096 x 4096, k = 1664, T = 777: 41.4 -> 32.5 (stage B: 52 CTAs of
+// 32 pairs -> 130 of 16); 1024 x 8192, k = 512, T = 2048: 53.5 -> 28.4; 8192 x 8192, k = 3712, T = 100: 65.4 -> 33.2;
+// 8192 x 8192, T = 2048 (232 CTAs) stays whole: 197, two ranks 215.
+// `resident(ks)`: CTAs that run at once in clusters of ks.
+inline void plan_mat(int rows, int cols, int T, int kc, int nv, int (*resident)(int), int *bn_out, int *ks_out) {
+    const int rb = plan_ceil_div(rows, MT_BM), npr = plan_ceil_div(plan_ceil_div(cols, MT_BK), 2);
+    const int one = plan_ceil_div(T, 16) * 16;
+    const int cand[4] = {T <= MT_BN ? one : 256, T <= MT_BN ? 0 : 192, 128, 0};
+    long best = -1;
+    *bn_out = cand[0]; *ks_out = 1;
+    if (T <= MS_BN) return;                                // the small-tile kernel plans its own split
+    for (int bn : cand) {
+        if (bn == 0 || (bn < T && bn % 64 != 0) || (bn == 128 && T <= 128 && one != 128)) continue;
+        for (int ks = 1; ks <= 8; ++ks) {
+            const int per = plan_ceil_div(npr, ks);
+            if (ks > 1 && (per * (ks - 1) >= npr || !mt_split_fits(kc, nv, bn, ks))) continue;
+            const long waves = plan_ceil_div(rb * plan_ceil_div(T, bn) * ks, resident(ks));
+            const long cost = waves * ((long)per * (41 + bn / 16) + 400 + bn * 25 / 32 + (ks > 1 ? bn * 15 / 16 + 30 * ks : 0));
+            if (best < 0 || cost < best) { best = cost; *bn_out = bn; *ks_out = ks; }
+        }
+    }
+}
 }  // namespace mdbf

@@ -1,6 +1,7 @@
 """The host side's decisions (csrc/plans.h), compiled for the CPU."""
 import ctypes
 import os
+import random
 import subprocess
 
 import pytest
@@ -15,6 +16,14 @@ uint64_t t_host_view(int pinned, uint64_t device, uint64_t start, size_t size, s
 }
 int t_host_store_direct(uint64_t device, size_t es, int T) { return host_store_direct(device, es, T); }
 int t_orth_ctas(int n, int chunk, int most, int sms) { return orth_ctas(n, chunk, most, sms); }
+static int resident_of(int ks) { return ks == 1 ? 148 : 148 / ks * ks - 8 % ks; }
+void t_plan_mat(int rows, int cols, int T, int kc, int nv, int *out) {
+    plan_mat(rows, cols, T, kc, nv, resident_of, out, out + 1);
+    out[2] = mt_tpr(out[0], out[1]);
+    out[3] = mt_ring(kc, nv, out[0], 0);
+    out[4] = (int)mt_smem_bytes(kc, nv, out[0], 0);
+}
+int t_small_ring(int kc, int nv, int bn, int ks) { return mt_ring(kc, nv, bn, (size_t)ks * plan_ceil_div(bn, ks) * MT_BM * 4); }
 }
 """
 
@@ -56,3 +65,39 @@ def test_a_cooperative_launch_fits_on_the_device(plans, n, sms):
     ctas, chunks = plans.t_orth_ctas(n, 128, 128, sms), -(-n // 128)
     assert 1 <= ctas <= min(sms, 128, chunks)
     assert ctas == chunks or ctas == min(sms, 128)
+
+
+KC_NV = ((2, 4), (4, 3))                                         # chunks of the mode axis and V-image slots: l <= 16, l <= 32
+
+
+@pytest.mark.parametrize("kc,nv", KC_NV)
+def test_plan_of_the_large_token_tiles(plans, kc, nv):
+    """Whatever the sizes: the ranks' sums of a split tile fit the activation ring they are pushed into, every rank has work, the tile is one
+    the kernel takes, and its shared memory is what a CTA may have."""
+    out = (ctypes.c_int * 5)()
+    rng = random.Random(kc)
+    log = lambda lo, hi: round(lo * (hi / lo) ** rng.random())
+    split = 0
+    for T in [*range(65, 1100), *(log(1100, 40000) for _ in range(200))]:
+        for _ in range(100):
+            rows, cols = log(1, 60000), log(1, 60000)
+            plans.t_plan_mat(rows, cols, T, kc, nv, out)
+            bn, ks, tpr, ring, smem = out
+            case = (rows, cols, T, bn, ks, tpr, ring)
+            assert 64 < bn <= 256 and bn % 16 == 0 and (bn >= T or bn % 64 == 0), case
+            assert 1 <= ks <= 8 and 4 <= ring <= 12 and ring % 2 == 0 and smem <= 226 * 1024, case
+            pairs = -(-(-(-cols // 64)) // 2)
+            if ks > 1:
+                split += 1
+                assert -(-pairs // ks) * (ks - 1) < pairs, case
+                assert tpr % 32 == 0 and tpr * ks >= bn, case
+                assert ks * tpr * 128 * 4 <= ring * bn * 64 * 2, case
+    assert split > 10000
+
+
+@pytest.mark.parametrize("kc,nv", KC_NV)
+def test_ring_of_the_small_token_tiles(plans, kc, nv):
+    """Two or three buffers take turns at the ring: it has its full depth, a multiple of both, for every tile and split."""
+    for bn in range(16, 65, 16):
+        for ks in range(1, 9):
+            assert plans.t_small_ring(kc, nv, bn, ks) == 12
