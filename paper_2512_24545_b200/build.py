@@ -1,5 +1,6 @@
-"""Build libmdbf.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and mdbf_calls.so beside it: the forward calls as
-a CPython extension module.
+"""Build libmdbf.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and beside it the forward calls as a CPython extension
+module, under a name that belongs to this interpreter.  Without a C compiler or Python's headers the module is left out and the
+binding makes those calls through ctypes.
 
     python -m paper_2512_24545_b200.build [--force] [--verbose] [--bounds-check]
 
@@ -19,7 +20,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmdbf.so")
-CALLS = os.path.join(HERE, "mdbf_calls.so")
+CALLS = os.path.join(HERE, "mdbf_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["mdbf_api.cu", "pack.cu", "reconstruct.cu", "forward_alu.cu", "forward_prefill.cu", "forward_tmem_t1.cu", "forward_t1.cu", "forward_static.cu", "forward_mat.cu", "msvid.cu", "gemm3x.cu", "admm.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -38,11 +39,28 @@ def _newest_source() -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def build_calls(force: bool = False, out: str = CALLS) -> bool:
+    """The extension module of the forward calls; False where this machine cannot make it."""
+    source, header = os.path.join(CSRC, "pycalls.c"), os.path.join(ROOT, "include", "mdbf.h")
+    if not force and os.path.exists(out) and os.path.getmtime(out) >= max(os.path.getmtime(source), os.path.getmtime(header)):
+        return True
+    cmd = [os.environ.get("CC", "gcc"), "-shared", "-fPIC", "-O2", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+           "-o", out, source]
+    try:
+        p = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        why = "" if p.returncode == 0 else p.stdout
+    except OSError as e:
+        why = str(e)
+    if why:
+        sys.stderr.write(f"mdbf: the forward calls stay with ctypes, {os.path.basename(out)} could not be built:\n{why}\n")
+    return not why
+
+
 def build(force: bool = False, verbose: bool = False, bounds_check: bool | None = None) -> str:
     variant = "bounds-check" if _bounds_check_requested(bounds_check) else "default"
     on_disk = open(STAMP).read().strip() if os.path.exists(STAMP) else "default"
-    newest = _newest_source()
-    if not force and on_disk == variant and all(os.path.exists(f) and os.path.getmtime(f) >= newest for f in (LIB, CALLS)):
+    build_calls(force)
+    if not force and on_disk == variant and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source():
         return LIB
     flags = NVCC_FLAGS + (["-DMDBF_BOUNDS_CHECK"] if variant == "bounds-check" else [])
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -67,8 +85,6 @@ def build(force: bool = False, verbose: bool = False, bounds_check: bool | None 
         raise RuntimeError("nvcc failed")
     subprocess.check_call([nvcc, "-shared", "-o", LIB, *objs, "-lcudart", "-lcusolver",
                            "-Xlinker", "-rpath=/usr/local/cuda/lib64"])
-    subprocess.check_call(["gcc", "-shared", "-fPIC", "-O2", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
-                           "-o", CALLS, os.path.join(CSRC, "pycalls.c"), "-L", HERE, "-l:libmdbf.so", "-Wl,-rpath,$ORIGIN"])
     with open(STAMP, "w") as f:
         f.write(variant + "\n")
     return LIB

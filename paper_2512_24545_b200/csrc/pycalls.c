@@ -2,7 +2,8 @@
  * 2 us), so the way from Python to the library counts: ctypes converts six arguments through their declared types and the marshalling
  * around it is interpreted, 0.9 us for mdbf_linear_forward; this way it is 0.2 us (4096 x 4096, k = 1664, one token, a layer called
  * over and over: 10.0 -> 8.9 us a call; a sum of two terms: 12.1 -> 9.5).  Only the calls of a forward pass are here, everything else
- * goes through ctypes.  The interpreter lock is released around each call, as ctypes does. */
+ * goes through ctypes.  The interpreter lock is released around each call, as ctypes does.  The module is not linked to the library: it is
+ * handed the functions of the one that ctypes has loaded. */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -10,6 +11,15 @@
 #include "mdbf.h"
 
 static PyObject *g_addr;                  /* mdbf._addr: the address of an array */
+
+/* the library's functions, in the order set_library takes their addresses in */
+typedef mdbf_status_t (*forward_fn)(mdbf_handle_t, const void *, void *, int32_t, int32_t, void *);
+static struct {
+    forward_fn forward, forward_host, forward_host_async;
+    mdbf_status_t (*sum)(const mdbf_handle_t *, int32_t, const void *, void *, float *, int32_t, int32_t, void *);
+    mdbf_status_t (*siblings)(const mdbf_handle_t *, int32_t, const void *, void *const *, int32_t, int32_t, void *);
+    mdbf_status_t (*group)(const mdbf_handle_t *, int32_t, const void *const *, void *const *, int32_t, int32_t, void *);
+} g_lib;
 
 /* integers as they are, None as NULL, a ctypes pointer by its value, anything else through _addr */
 static int pointer_arg(PyObject *o, void **out) {
@@ -41,12 +51,12 @@ static int pointer_list(PyObject *o, void **out, Py_ssize_t at_least, int32_t *n
     return ok;
 }
 static int count_is(Py_ssize_t n, Py_ssize_t want) {
+    if (!g_addr) { PyErr_SetString(PyExc_RuntimeError, "set_library has not been called"); return 0; }
     if (n == want) return 1;
     PyErr_Format(PyExc_TypeError, "%zd arguments instead of %zd", n, want);
     return 0;
 }
 
-typedef mdbf_status_t (*forward_fn)(mdbf_handle_t, const void *, void *, int32_t, int32_t, void *);
 static PyObject *forward(forward_fn f, PyObject *const *a, Py_ssize_t n) {
     void *h, *x, *y, *stream;
     int32_t T, act;
@@ -59,9 +69,9 @@ static PyObject *forward(forward_fn f, PyObject *const *a, Py_ssize_t n) {
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
-static PyObject *linear_forward(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(mdbf_linear_forward, a, n); }
-static PyObject *linear_forward_host(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(mdbf_linear_forward_host, a, n); }
-static PyObject *linear_forward_host_async(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(mdbf_linear_forward_host_async, a, n); }
+static PyObject *linear_forward(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(g_lib.forward, a, n); }
+static PyObject *linear_forward_host(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(g_lib.forward_host, a, n); }
+static PyObject *linear_forward_host_async(PyObject *m, PyObject *const *a, Py_ssize_t n) { (void)m; return forward(g_lib.forward_host_async, a, n); }
 
 static PyObject *linear_forward_sum(PyObject *m, PyObject *const *a, Py_ssize_t n) {
     void *hs[MAX_LAYERS], *x, *y, *acc, *stream;
@@ -72,7 +82,7 @@ static PyObject *linear_forward_sum(PyObject *m, PyObject *const *a, Py_ssize_t 
         return NULL;
     mdbf_status_t rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = mdbf_linear_forward_sum((const mdbf_handle_t *)hs, P, x, y, (float *)acc, T, act, stream);
+    rc = g_lib.sum((const mdbf_handle_t *)hs, P, x, y, (float *)acc, T, act, stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
@@ -85,7 +95,7 @@ static PyObject *linear_forward_siblings(PyObject *m, PyObject *const *a, Py_ssi
         return NULL;
     mdbf_status_t rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = mdbf_linear_forward_siblings((const mdbf_handle_t *)hs, L, x, ys, T, act, stream);
+    rc = g_lib.siblings((const mdbf_handle_t *)hs, L, x, ys, T, act, stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
@@ -98,18 +108,30 @@ static PyObject *linear_forward_group(PyObject *m, PyObject *const *a, Py_ssize_
         return NULL;
     mdbf_status_t rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = mdbf_linear_forward_group((const mdbf_handle_t *)hs, L, (const void *const *)xs, ys, T, act, stream);
+    rc = g_lib.group((const mdbf_handle_t *)hs, L, (const void *const *)xs, ys, T, act, stream);
     Py_END_ALLOW_THREADS
     return PyLong_FromLong(rc);
 }
-static PyObject *set_addr(PyObject *m, PyObject *f) {
+/* set_library(_addr, (six addresses)) */
+static PyObject *set_library(PyObject *m, PyObject *args) {
+    PyObject *f;
+    unsigned long long p[6];
     (void)m;
+    if (!PyArg_ParseTuple(args, "O(KKKKKK)", &f, &p[0], &p[1], &p[2], &p[3], &p[4], &p[5])) return NULL;
+    for (int i = 0; i < 6; ++i)
+        if (!p[i]) { PyErr_SetString(PyExc_ValueError, "a function's address is missing"); return NULL; }
+    g_lib.forward = (forward_fn)(uintptr_t)p[0];
+    g_lib.forward_host = (forward_fn)(uintptr_t)p[1];
+    g_lib.forward_host_async = (forward_fn)(uintptr_t)p[2];
+    *(void **)&g_lib.sum = (void *)(uintptr_t)p[3];
+    *(void **)&g_lib.siblings = (void *)(uintptr_t)p[4];
+    *(void **)&g_lib.group = (void *)(uintptr_t)p[5];
     Py_XSETREF(g_addr, Py_NewRef(f));
     Py_RETURN_NONE;
 }
 
 #define FAST(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, NULL}
 static PyMethodDef methods[] = {FAST(linear_forward), FAST(linear_forward_host), FAST(linear_forward_host_async), FAST(linear_forward_sum),
-                                FAST(linear_forward_siblings), FAST(linear_forward_group), {"set_addr", set_addr, METH_O, NULL}, {NULL, NULL, 0, NULL}};
+                                FAST(linear_forward_siblings), FAST(linear_forward_group), {"set_library", set_library, METH_VARARGS, NULL}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "mdbf_calls", NULL, -1, methods, NULL, NULL, NULL, NULL};
 PyMODINIT_FUNC PyInit_mdbf_calls(void) { return PyModule_Create(&module); }
