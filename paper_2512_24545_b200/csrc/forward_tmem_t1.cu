@@ -30,8 +30,9 @@
 // forward.  A CTA with two expander groups therefore takes half of an SM's registers and of its shared memory, so that the next
 // launch's CTA starts, sets up and requests its first operands while this one works; it gets the tensor memory as soon as
 // this one has read its accumulators.  Graph replay, us per forward, before -> after: 4096 x 4096, k = 1664, l = 16: 9.31 -> 7.64;
-// 8192 x 8192, k = 3712: 15.2 -> 14.1; q/k/v of 4096 x 4096: 15.0 -> 13.4; 11008 x 4096 gate and up: 22.0 -> 20.0.  Layers so small
-// that every launch had idle SMs to start on gained nothing and pay the extra barriers (640 x 640: 5.8 -> 6.0).
+// 8192 x 8192, k = 3712: 15.2 -> 14.1; q/k/v of 4096 x 4096: 15.0 -> 13.4; 11008 x 4096 gate and up: 22.0 -> 20.0.  With the roles
+// converged besides (elect_one), a whole MB less or more makes no exception: 640 x 640, k = 256: 6.3 -> 5.6, 4096 x 4096: 9.0 -> 7.1, 8192 x
+// 8192: 14.8 -> 12.3, 28672 x 8192, k = 6016: 34.4 -> 31.8.
 //
 // CTA = 128 sign rows x a slice of the reduction; the KS CTAs of a row block form a cluster and
 // reduce their partial outputs through distributed shared memory (deterministic, no atomics).

@@ -520,8 +520,10 @@ static mdbf_status_t forward_t1_auto(Layer *const *Ls, int n, const void *x, voi
         for (int s = 0; s < 2; ++s) {
             mdbf_status_t rc;
             if (i8_stages >> s & 1) { rc = launch_forward_t1_group(Ls, n, xs, ys, st, 1 << s); nl += 2; }
-            // beside an integer kernel: behind this forward's other stage, or in front of it and then, in a loop over such layers, behind the
-            // previous forward's (28672 x 8192, k = 6016 over and over: 39.3 us with this for the second stage only, 32.3 for either)
+            // beside an integer kernel, an SM per CTA: behind this forward's other stage it matters always (8192 x 28672, k = 6016: 38.3 us
+            // without, 32.2 with), in front of it only where an integer kernel came before, which a call cannot know.  28672 x 8192,
+            // k = 6016 over and over: 39.0 without, 32.1 with; behind an 8192-, a 640-square layer or an idle stream: 48.4, 39.3, 37.5
+            // without and 48.7, 39.3, 37.7 with, the same to the runs' scatter of 0.3.
             else { rc = launch_forward_tmem_t1_multi(Ls, n, x, ys, st, 1 << s, true); nl += last_t1_launch_count(); }
             if (rc) return rc;
         }
