@@ -310,3 +310,22 @@ def test_rows_near_the_ends_of_fp32():
     assert np.abs(ref).max() < 1e37
     err = np.abs(g["tilde"] - ref).max(axis=1) / np.abs(ref).max(axis=1)
     assert np.all(err <= 2e-5), np.max(err)
+
+
+@pytest.mark.parametrize("R", [129, 1100, 2180])
+def test_inverse_of_a_badly_conditioned_system(R):
+    """V nearly square and rho a hundredth of the system's mean diagonal: condition near 4 M / rho' = 400.  fp32 rounding of the factor,
+    the inverse (from 1024 columns joined on the tensor cores) and the product, 2^-24 each and amplified by it: 4 * 400 * 6e-8 = 1e-4 of the
+    iterate's largest entry, an order above what is seen."""
+    n, m = R + 37, R + 11
+    g = torch.Generator(device="cuda").manual_seed(170 + R)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    W, V, U, Lam = rnd(n, m), rnd(m, R), rnd(n, R), 0.1 * rnd(n, R)
+    rho = 0.01 * float((V.double() ** 2).sum() / R)
+    V8 = V.double()
+    want = torch.linalg.solve(V8.T @ V8 + rho * torch.eye(R, device="cuda", dtype=torch.float64),
+                              (W.double() @ V8 + rho * (U.double() - Lam.double())).T).T
+    got = run_update(W.cpu().numpy(), V.cpu().numpy(), U.cpu().numpy(), Lam.cpu().numpy(), rho, 1, 1, 4)["tilde"]
+    err = np.max(np.abs(got - want.cpu().numpy())) / float(want.abs().max())
+    print("condition:", R, err)
+    assert err <= 1e-4
