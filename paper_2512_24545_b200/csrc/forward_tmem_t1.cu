@@ -15,8 +15,8 @@
 // programmatic-dependent-launch wait.
 //
 // What the measurements on this GPU say the kernel has to respect:
-//   * tcgen05.mma with N = 16 lasts ~8 clocks but one thread issues at most one per ~50 clocks,
-//     and with A in shared memory every MMA re-reads 4 KB: A lives in TMEM and four issuer warps
+//   * tcgen05.mma with N = 16 lasts ~8 clocks but one warp issues at most one per ~50 clocks,
+//     and with A in shared memory every MMA re-reads 4 KB: A lives in TMEM and three issuer warps
 //     work round-robin, each on its own accumulator (summed in the epilogue).
 //   * The bit -> bf16 step costs one shift and one logic op per two bits, and logic ops issue at
 //     half rate: this, not HBM, bounds the big layers (<= 128 sign bits per clock and SM).
@@ -50,11 +50,17 @@ namespace mdbf {
 
 // expander groups of 4 warps (template parameter G of the kernel; group g takes the pairs g, g + G, ...): 2 for
 // CTAs with few pairs (all latency; two such CTAs fit on an SM), 3 for long CTAs (4: worse)
-constexpr int TX_ISSUERS = 4;                          // MMA issuer warps, one accumulator each (a thread issues ~1 MMA / 100+ clk here)
+constexpr int TX_ISSUERS = 3;                          // MMA issuer warps, one accumulator each (issuer w takes the pairs w, w + 3, ...)
 constexpr int tx_threads(int groups) { return groups * 128 + TX_ISSUERS * 32 + 64; }   // + sign loader warp + V loader warp
 constexpr int tx_ctas(int groups) { return groups <= 2 ? 2 : 1; }      // CTAs per SM the registers are held to (72 a thread with two groups)
-constexpr int TX_MAX_SSTAGES = 16;                     // sign ring: 2 KB per stage (one pair of K blocks)
-constexpr int TX_MAX_ASTAGES = 7;                      // A / V stages: 64 TMEM columns + two V tiles each
+constexpr int TX_SSTAGES = 8, TX_MAX_SSTAGES = 12;     // sign ring: 2 KB per stage (one pair of K blocks); the longer one from TX_LONG on
+constexpr int TX_ASTAGES = 6;                          // A / V stages: 64 TMEM columns + two V tiles each
+// A parity test cannot tell phase n of a barrier from phase n - 2, so whoever waits on a ring slot has to have seen its last phase: the slot
+// must come back to the same expander group and to the same issuer.  (With 7 stages, two groups and four issuers it came back to others, and
+// a group or an issuer that ran a ring ahead of another would have taken a slot that was still in use.)  It costs nothing: 4096 x 4096 7.15 ->
+// 6.97 us, 8192 x 8192 12.3 -> 12.0, 70B-class block 118.7 -> 117.4; with 2 issuers the block takes 3 % longer, with one 10 %.
+static_assert(TX_ASTAGES % TX_ISSUERS == 0 && TX_ASTAGES % 2 == 0 && TX_ASTAGES % 3 == 0, "slots belong to one issuer and one expander group");
+static_assert(TX_SSTAGES % 2 == 0 && TX_MAX_SSTAGES % 2 == 0 && TX_MAX_SSTAGES % 3 == 0, "slots belong to one expander group");
 constexpr int TX_MAX_DYN = 220 * 1024;                 // dynamic shared memory
 constexpr int TX_LONG = 48;                            // pairs of K blocks per CTA from which on a CTA has three expander groups
 
@@ -111,7 +117,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
     constexpr int NB = LP < 16 ? 16 : LP;                    // MMA N
     constexpr int VBYTES = 2 * NB * 128;                     // two tiles
     extern __shared__ unsigned char tx_smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * TX_MAX_SSTAGES + 3 * TX_MAX_ASTAGES + 1];
+    __shared__ __align__(8) uint64_t bars[2 * TX_MAX_SSTAGES + 3 * TX_ASTAGES + 1];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
@@ -128,8 +134,8 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
     uint32_t *xp = reinterpret_cast<uint32_t *>(smem_gen + off_x);
     float *part = reinterpret_cast<float *>(smem_gen + off_p);
 
-    constexpr int NB0 = TX_MAX_SSTAGES, NB1 = 2 * TX_MAX_SSTAGES, NB2 = NB1 + TX_MAX_ASTAGES,
-                  NB3 = NB2 + TX_MAX_ASTAGES, NB4 = NB3 + TX_MAX_ASTAGES;
+    constexpr int NB0 = TX_MAX_SSTAGES, NB1 = 2 * TX_MAX_SSTAGES, NB2 = NB1 + TX_ASTAGES,
+                  NB3 = NB2 + TX_ASTAGES, NB4 = NB3 + TX_ASTAGES;
     const uint32_t s_full = smem_u32(&bars[0]), s_empty = smem_u32(&bars[NB0]), v_full = smem_u32(&bars[NB1]),
                    a_full = smem_u32(&bars[NB2]), a_empty = smem_u32(&bars[NB3]), acc_bar = smem_u32(&bars[NB4]);
 
@@ -250,8 +256,8 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
 
         // One pair of K blocks per iteration: 2 x 64 sign bits of this row -> 64 TMEM columns.
         bool alive = true;
-        int rs = grp % nss, as = grp % nas;
-        uint32_t rs_ph = (uint32_t)(grp / nss) & 1u, as_ph = (uint32_t)(grp / nas) & 1u;
+        int rs = grp % nss, as = grp;
+        uint32_t rs_ph = (uint32_t)(grp / nss) & 1u, as_ph = 0u;
         int prev_as = -1;
         for (int pr = grp; pr < npr; pr += TX_GROUPS) {
             alive = tx_wait(s_full + 8 * rs, rs_ph, abort_flag, a.status);
@@ -338,15 +344,8 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
         const uint32_t d_tmem = tmem + (uint32_t)(w * NB);
         bool alive = true;
         int it = 0;
-        int as = w % nas;
-        uint32_t as_ph = (uint32_t)(w / nas) & 1u;
-        // An issuer whose first pair already reuses a stage (w >= nas) has to see the earlier phases of
-        // that stage complete first: a parity test alone cannot tell phase n from phase n - 2.
-        if (w < npr)
-            for (int k = 0; k < w / nas && alive; ++k) {
-                alive = tx_wait(v_full + 8 * as, (uint32_t)k & 1u, abort_flag, a.status);
-                if (alive) alive = tx_wait(a_full + 8 * as, (uint32_t)k & 1u, abort_flag, a.status);
-            }
+        int as = w;
+        uint32_t as_ph = 0u;
         for (int pr = w; pr < npr && alive; pr += TX_ISSUERS, ++it) {
             alive = tx_wait(v_full + 8 * as, as_ph, abort_flag, a.status);
             if (alive) alive = tx_wait(a_full + 8 * as, as_ph, abort_flag, a.status);
@@ -558,8 +557,6 @@ constexpr int TX_CARVEOUT = 58;
 // terms > 1: the n layers are the terms of a sum, whose ranks share the cluster of a row block (p->ks: all of them).
 static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p, int terms = 1) {
     const int NB = LP < 16 ? 16 : LP;
-    int nas = (512 - TX_ISSUERS * NB) / 64;
-    if (nas > TX_MAX_ASTAGES) nas = TX_MAX_ASTAGES;
     const int max_ks = 8 / terms;                             // portable cluster size
     int rb = 0, max_pairs = 0, min_pairs = 1 << 30;
     for (int i = 0; i < n; ++i) {
@@ -582,11 +579,11 @@ static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p
         p->pairs_per_cta[i] = ceil_div(kb_pad[i] / 2, best_ks);
         max_per = max(max_per, p->pairs_per_cta[i]);
     }
-    p->nastages = nas;
-    p->nsstages = min(max_per, max_per >= TX_LONG ? TX_MAX_SSTAGES : 8);
+    p->nastages = TX_ASTAGES;
+    p->nsstages = min(max_per, max_per >= TX_LONG ? TX_MAX_SSTAGES : TX_SSTAGES);
     p->tmem_cols = 512;
-    p->smem = 1024 + (size_t)nas * 2 * NB * 128 + (size_t)p->nsstages * 2048 + (size_t)max_per * 256 + 4096;
-    return nas >= 2 && p->smem <= TX_MAX_DYN;
+    p->smem = 1024 + (size_t)TX_ASTAGES * 2 * NB * 128 + (size_t)p->nsstages * 2048 + (size_t)max_per * 256 + 4096;
+    return p->smem <= TX_MAX_DYN;
 }
 
 static thread_local int g_t1_launches = 0;      // kernels the last one-token forward of this thread launched
