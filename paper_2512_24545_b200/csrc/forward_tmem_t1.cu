@@ -300,6 +300,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
         __syncwarp();
         if (alive && prev_as >= 0 && lane == 0) mbar_arrive(a_full + 8 * prev_as);
         if (grp != 0) alive = false;                         // only the first group runs the epilogue
+        __syncwarp();                                        // the cluster barrier wants the warp converged
         cluster_wait();
         if (alive) alive = mbar_wait(acc_bar, 0u, abort_flag, a.status);
         tc_fence_after();
@@ -422,6 +423,7 @@ __device__ __forceinline__ void tmem_t1_body(const TxArgs &a, const int rb, cons
     tc_fence_before();
     const unsigned crank = cluster.block_rank();
     if (warp < 4 && crank != 0) cluster.map_shared_rank(part, 0)[crank * 128 + row_l] = outv;
+    __syncwarp();
     cluster_arrive();
     if (freed) tmem_dealloc(tmem_base_slot, (uint32_t)a.tmem_cols);      // issuer warp 0, off the other ranks' critical path
     cluster_wait();
