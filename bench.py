@@ -46,7 +46,8 @@ NCU_TRAFFIC_BYTES_PER_LAUNCH = {
     ("msvid_28672x6016_l16", "envelope_product_tc_kernel"): 708300000,   # Z once per pass (689.9 MB) + operand images and partial sums,
                                                                            # scaled by rows x cols from the 8192 x 8192 capture
     ("msvid_8192x8192_l16", "envelope_product_tc_kernel"): 275523328,      # 269.6 MB read + 5.9 MB written for 268.4 MB of Z
-    ("admm_8192x8192_r3712_l16", "gemm3x_kernel"): None,                   # images are half the bytes of the last capture's (1156590808 for W V)
+    ("admm_8192x8192_r3712_l16", "gemm3x_kernel"): 1384669424,             # its largest launch, W V: 1.270 GB read (images 0.39 GB; V's are re-read
+                                                                           # by every row tile, most of it from L2) + 114.7 MB written
     ("block70b_T2048", "mat_stage_kernel"): 197116928,             # its largest launch, down stage B (185.9 MB read: 117 MB of x, partly twice,
                                                                    # + signs; 11.3 MB written); gate / up stage A: 123.3 MB
 }

@@ -348,12 +348,13 @@ mdbf_status_t mdbf_msvid_workspace_bytes(int64_t rows, int64_t cols, int32_t l, 
  *   S_packed (N x ceil(R / 32)), Ul (N x l), Vl (R x l), sigma (l)   device, written: the compact form of the new U,
  *              U = S (.) (Ul Vl^T), as mdbf_msvid returns it in the last inner iteration
  *   U_tilde    device, N x R fp32, written with the last inner iteration's least-squares iterate; may be NULL
- *   workspace  device, mdbf_admm_workspace_bytes(N, M, R, l) bytes on a 256-byte boundary (three N x R matrices, the R x R
- *              system, the operand images of op(W) and V - their size and a little more - and mdbf_msvid's workspace)
+ *   workspace  device, mdbf_admm_workspace_bytes(N, M, R, l) bytes on a 256-byte boundary (two N x R matrices, the R x R
+ *              system and a scratch of its size, the operand images of op(W), V and the R x R triangular inverse - their size and
+ *              a little more - and mdbf_msvid's workspace)
  * The dense products (W V, V^T V, the inverse of the system and its application) run on the tensor cores (fp16
  * operands, scaled per row, in a three-term split, fp32 accumulation in chunks of 64 contraction indices; U_tilde comes out within a few
- * 1e-6 of its largest entry of the exact result); the Cholesky factorisation and the solves of the R x R system are cuSOLVER calls in
- * fp32; the MSVID step, the elementwise passes and the reconstruction of the dense factor fused with the dual update
+ * 1e-6 of its largest entry of the exact result); the Cholesky factorisation of the R x R system is a cuSOLVER call in
+ * fp32; the inversion of its factor, the MSVID step, the elementwise passes and the reconstruction of the dense factor fused with the dual update
  * are this library's kernels.  Asynchronous on `stream`; part of the work runs on a stream of the library's own that
  * is forked from `stream` and joined to it by events inside the call.  The first call on a host thread creates the
  * solver's handles, that stream and its events, and allocates the scratch the factorisation asks for (kept for later calls; a larger request synchronises

@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(256) tri_join_kernel(const float *__restrict__
         for (int q = 0; q < 4; ++q)
             if (i0 + 4 * ty + p < s && j0 + 4 * tx + q < s2) dst[(size_t)(i0 + 4 * ty + p) * r + j0 + 4 * tx + q] = FIRST ? acc[p][q] : -acc[p][q];
 }
-// U (upper triangle read) -> Y (r x r, written whole); P: r x r scratch, img: operand images of two r / 2 x r / 2 blocks
+// U (upper triangle read) -> Y (r x r, written whole); P: r x r scratch, img: operand images of the two blocks of a
+// product, s and at most s rows by s at most (s the largest power of two times TI_LEAF below r: 2048 and 1664 at r = 3712), which r x r images hold
 static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *img, int r, int32_t *status, cudaStream_t st) {
     static PerDeviceOnce once;
     if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(tri_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TI_SMEM));
@@ -197,9 +198,10 @@ static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *i
 // U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam += U_tilde - U (Eq. admm-U-dual, rounded as written: near
 // convergence U_tilde - U and Lam are small beside Z = U_tilde + Lam, and Z - U would carry a rounding of Z into the dual in every
 // iteration; 8192 x 3712 at the end of a refinement, error of the dual step relative to the dual: 1.4e-6 with Z - U, below 6e-8 this way).
-// Bound by memory (U_tilde and Lam read, U and Lam written: 16 bytes per entry; 8192 x 3712, l = 16: 130 us, of which the traffic needs 74; four rows in flight and 64 registers: 121, spilling).  CTA = 32 rows x 256
-// columns; thread = column (its row of Vl in registers), the rows' Ul in shared memory, eight rows' loads in flight together; L = l
-// rounded up to 4, 8, 16 or 32.  Ut may be U itself: an entry is read by the thread that writes it.
+// Bound by memory (U_tilde and Lam read, U and Lam written: 16 bytes per entry; 8192 x 3712, l = 16: 130 us, of which the traffic needs
+// 74; four rows in flight and 64 registers: 121, but it spills).  CTA = 32 rows x 256 columns; thread = column (its row of Vl in
+// registers), the rows' Ul in shared memory, eight rows' loads in flight together; L = l rounded up to 4, 8, 16 or 32.  Ut may be U itself:
+// an entry is read by the thread that writes it.
 constexpr int RC_ROWS = 32, RC_COLS = 256, RC_BATCH = 8;
 template <int L>
 __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__restrict__ S, const float *__restrict__ Ul,

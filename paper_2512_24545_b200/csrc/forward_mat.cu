@@ -24,10 +24,10 @@
 //              columns of the W_hat tile with tcgen05.st (the A operand of the main MMA lives in TMEM:
 //              no shared-memory round trip, no proxy fence).  Afterwards they run the epilogue.
 //   warp 16    one lane issues the TMA loads of the activation tiles [tokens x 64] of a pair
-//   warp 17    one lane issues the 8 main MMAs of a pair (A from TMEM, B from shared memory); one commit
+//   warp 17    issues the 8 main MMAs of a pair (A from TMEM, B from shared memory), converged, by an elected lane; one commit
 //              frees the TMEM slot, one the pair of activation tiles
 //   warp 18    one lane bulk-copies the envelope images (U once, V per pair, ring of 3 or 4)
-//   warp 19    one lane issues the mini-MMA of a pair (U image x V image, 128 columns, no swizzle)
+//   warp 19    issues the mini-MMA of a pair (U image x V image, 128 columns, no swizzle), converged as well
 // Few row blocks and tokens leave SMs idle: then the reduction of a tile is split over a cluster of up to eight CTAs (SPLIT), each
 // running the same pipeline over its pairs, and the accumulators are added by token through distributed shared memory.
 // Shared memory holds only activation tiles (ring of 6 at 256 tokens per tile: the L2 latency of a
@@ -580,7 +580,7 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
     const uint32_t tmem_d = tmem_base;                   // + 64 g
     const uint32_t tmem_buf = tmem_base + 2 * MS_BN;     // + 128 g
     pdl_launch_dependents();
-    if (SPLIT) cluster.barrier_arrive();                      // see mat_stage_kernel
+    if (SPLIT) cluster.barrier_arrive();                      // this CTA runs: awaited before the first store into another one's shared memory
 
     if (warp < MS_W_TMA) {
         // ============================ W_hat tile builders ============================
@@ -620,7 +620,7 @@ mat_small_kernel(const MatArgs a, const __grid_constant__ CUtensorMap tmap_in) {
         }
 
         // ================================= epilogue ==================================
-        // 16 tokens per warp of a lane quadrant; out = D0 + D1
+        // 16 tokens per warp of a lane quadrant; out = the sum of the buffers' accumulators
         const int egrow = row0 + arow;
         const int chunk = warp >> 2;
         if (alive) alive = mbar_wait(accum_bar, 0u, abort_flag, a.status);
