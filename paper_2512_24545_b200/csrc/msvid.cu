@@ -509,25 +509,30 @@ __global__ void chunk_sum_kernel(const float *__restrict__ P, int nchunks, size_
 // One warp, lane k = row k of G in registers: G = L L^T (G: the summed Gram matrix, lower triangle); beside it lane k builds column k
 // of L^-1 by forward substitution, each column of L serving both as soon as it is known (one set of shuffles and one chain of
 // pivots: 4.5 us when the inverse followed the factor, 2.3 us now at l = 16).  M[b][a] = (L^-1)[a][b], so that A M has
-// orthonormal columns.  A zero (or numerically vanished) pivot - a padding column, or a block wider than the rank of the matrix -
-// leaves its column as it is instead of dividing by zero.
+// orthonormal columns.  A column that is in the span of those before it to 1e-6 of its length (a padding column, or a block wider than the
+// rank of the matrix: 1e-6 is what the products leave of a difference) becomes zero: normalising what is left of it would turn
+// rounding into a column that is not orthogonal to the others, and the result's singular values with it (|Z| constant or one entry, l = 16:
+// 10^3 times too large).  In a start block (`start`) it is normalised all the same, as a random restart, and kept as it is where
+// nothing at all is left.  An infinity or NaN turns all of it into NaN.
 template <int LP>
-__device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], float *__restrict__ M) {
+__device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], bool start, float *__restrict__ M) {
     const int k = threadIdx.x & 31;
     double g[LP], x[LP];                                         // row k of G, then of L; right-hand side, then column k of L^-1
-    double scale = 0.0;
+    double scale = 0.0, trace = 0.0;
 #pragma unroll
     for (int j = 0; j < LP; ++j) {
         g[j] = j <= k ? Gm[k < LP ? k : 0][j] : 0.0;             // (above the diagonal: never read by another lane)
         x[j] = j == k ? 1.0 : 0.0;
         scale = fmax(scale, Gm[j][j]);
+        trace += Gm[j][j];
     }
 #pragma unroll
     for (int c = 0; c < LP; ++c) {
         const double dcc = __shfl_sync(0xffffffffu, g[c], c);
-        const double inv = (dcc > 1e-24 * scale && dcc > 0.0) ? rsqrt(dcc) : 0.0;      // 1 / L[c][c], the same in every lane
+        const double inv = dcc > (start ? 1e-24 * scale : 1e-12 * Gm[c][c]) ? rsqrt(dcc) : 0.0;      // 1 / L[c][c], the same in every lane
         g[c] *= inv;                                             // column c of L below the diagonal
-        x[c] = inv > 0.0 ? x[c] * inv : (c == k ? 1.0 : 0.0);    // (zero for c < k from the start)
+        x[c] *= inv;                                             // (zero for c < k from the start)
+        if (start && inv == 0.0 && c == k) x[c] = 1.0;
 #pragma unroll
         for (int jj = c + 1; jj < LP; ++jj) {
             const double ljc = __shfl_sync(0xffffffffu, g[c], jj);
@@ -537,7 +542,7 @@ __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], float *__r
     }
     if (k < LP) {
 #pragma unroll
-        for (int a = 0; a < LP; ++a) M[k * LP + a] = (float)x[a];
+        for (int a = 0; a < LP; ++a) M[k * LP + a] = trace < 1e300 ? (float)x[a] : __int_as_float(0x7fc00000);
     }
 }
 // A <- an orthonormal basis of its columns (Cholesky QR), in one cooperative launch: sum of the partial products (parts > 0), Gram matrix
@@ -594,7 +599,7 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned int *counter, unsigned
 template <int LP>
 __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts, double *__restrict__ Gp,
                                                    double *__restrict__ Gs, unsigned int *__restrict__ counter, unsigned int base,
-                                                   uint32_t *__restrict__ img, int32_t *__restrict__ status) {
+                                                   uint32_t *__restrict__ img, bool start, int32_t *__restrict__ status) {
     using C = OrCfg<LP>;
     constexpr int BL = C::BL, NP = C::NP, RG = C::RG, LD = C::LD;
     constexpr int PER = OR_ROWS * LP / 256 > 0 ? OR_ROWS * LP / 256 : 1;                   // elements of a chunk per thread
@@ -688,7 +693,7 @@ __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n,
     for (int e = tid; e < LP * LP; e += 256)
         if (e % LP <= e / LP) Gm[e / LP][e % LP] = __ldcg(Gs + e);
     __syncthreads();
-    if (tid < 32) chol_warp<LP>(Gm, Ms);
+    if (tid < 32) chol_warp<LP>(Gm, start, Ms);
     __syncthreads();
 
     // A M and the operand images; two threads per row where a row has sixteen columns or more
@@ -1004,7 +1009,7 @@ static int padded_rank(int l) {
 // A <- an orthonormal basis of its columns (Cholesky QR); with `parts` > 0, A is first formed as the sum of the partial sums
 // in w.P; with `img`, the operand images of the result are written for the tensor-core product that reads it next
 template <int LP>
-static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr) {
+static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr, bool start = false) {
     using C = OrCfg<LP>;
     auto kern = orth_kernel<LP>;
     int sms = 0;
@@ -1027,7 +1032,7 @@ static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int part
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, A, n, (const float *)w.P, parts, w.Gp, w.Gs, w.barrier, w.arrived, img, w.status));
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, A, n, (const float *)w.P, parts, w.Gp, w.Gs, w.barrier, w.arrived, img, start, w.status));
     w.arrived += 2u * (unsigned int)ctas;
     return MDBF_OK;
 }
@@ -1141,9 +1146,9 @@ static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const 
     if (!MASKED && !zm.use) sign_pack_kernel<<<dim3(p, ceil_div(nwords, 8 * SP_WORDS)), 256, 0, st>>>(Z, q, nwords, S);
     pad_kernel<<<(int)std::min<size_t>(((size_t)q * LP + 255) / 256, 148u * 8), 256, 0, st>>>(Q0, (size_t)q, l, LP, w.Q);
     MDBF_CUDA(cudaGetLastError());
-    mdbf_status_t rc = orth<LP>(w.Q, q, w, st);                        // twice: the start block may be badly conditioned
+    mdbf_status_t rc = orth<LP>(w.Q, q, w, st, 0, nullptr, true);      // twice: the start block may be badly conditioned
     uint32_t *img_q = zm.use ? w.img : nullptr, *img_y = (zm.use && LP >= 8) ? w.img : nullptr;   // which products run on the tensor cores
-    if (rc == MDBF_OK) rc = orth<LP>(w.Q, q, w, st, 0, img_q);
+    if (rc == MDBF_OK) rc = orth<LP>(w.Q, q, w, st, 0, img_q, true);
     if (rc) return rc;
     int parts = 0;
     for (int it = 0; it < n_iter; ++it) {

@@ -206,6 +206,46 @@ def test_envelope_of_exact_low_rank_is_reproduced():
     assert np.linalg.norm(Z - Sm * (U @ V.T)) <= 2e-5 * np.linalg.norm(Z)
 
 
+@pytest.mark.parametrize("shape", [(200, 300), (129, 517), (1000, 64), (64, 2048)])
+@pytest.mark.parametrize("kind,l", [(kind, l) for kind in ("constant", "one entry", "outer product") for l in (2, 4, 16, 32)]
+                         + [(kind, l) for kind in ("three rows", "rank 3 and tiny noise") for l in (4, 16, 32)])
+def test_block_wider_than_the_rank(shape, kind, l):
+    """Columns of the block beyond the rank of |Z| carry nothing but rounding: they must not disturb the others.  Theorem 1's error to a few
+    fp32 roundings of the norm, singular values beyond the rank at rounding size."""
+    rng = np.random.default_rng(l)
+    if kind == "constant":
+        E, rank = np.full(shape, 0.37), 1
+    elif kind == "one entry":
+        E, rank = np.zeros(shape), 1
+        E[3, 5] = 2.0
+    elif kind == "outer product":
+        E, rank = np.abs(rng.standard_normal((shape[0], 1))) @ np.abs(rng.standard_normal((1, shape[1]))), 1
+    elif kind == "three rows":
+        E, rank = np.zeros(shape), 3
+        E[[1, 7, 30]] = np.abs(rng.standard_normal((3, shape[1])))
+    else:
+        E, rank = np.abs(rng.standard_normal((shape[0], 3))) @ np.abs(rng.standard_normal((3, shape[1]))), 3
+        E = E * (1 + 1e-7 * rng.standard_normal(shape))
+    Z = (np.where(rng.random(shape) < 0.5, -1.0, 1.0) * E).astype(np.float32)
+    Sp, U, V, s = run_msvid(Z, l, n_iter=6)
+    sv = np.linalg.svd(np.abs(Z.astype(np.float64)), compute_uv=False)
+    tail = np.sqrt(np.sum(sv[l:] ** 2))
+    assert np.all(np.isfinite(U)) and np.all(np.isfinite(V))
+    np.testing.assert_allclose(s[:rank], sv[:rank], rtol=2e-5, atol=1e-5 * sv[0])
+    assert np.all(s[rank:] <= 1e-4 * sv[0]), s / sv[0]
+    assert envelope_error(Z, U, V) <= 1.01 * tail + 2e-5 * np.linalg.norm(Z)
+
+
+def test_a_start_block_of_one_direction():
+    """All columns of Q0 equal: the block finds the leading singular directions all the same, or as many as it can - never more than there is."""
+    Z = inputs.make_factor_matrix(300, 400, seed=12)
+    sv = np.linalg.svd(np.abs(Z.astype(np.float64)), compute_uv=False)
+    Q0 = np.repeat(np.random.default_rng(1).standard_normal((400, 1)), 4, axis=1).astype(np.float32)
+    _, U, V, s = run_msvid(Z, 4, n_iter=8, Q0=Q0)
+    assert abs(s[0] - sv[0]) <= 2e-5 * sv[0] and np.all(s <= sv[:4] * (1 + 2e-5))
+    assert envelope_error(Z, U, V) <= np.sqrt(np.sum(sv[1:] ** 2)) * (1 + 1e-5)
+
+
 def test_full_size_factor():
     """4096 x 4096, l = 16: the mask against the oracle on every row, the singular values against the full SVD, the
     envelope error through ||A - A Q Q^T||^2 = ||A||^2 - sum s_t^2 (Q orthonormal) against Theorem 1's tail."""
