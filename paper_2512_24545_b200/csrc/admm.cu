@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(256) tri_join_kernel(const float *__restrict__
 // product, s and at most s rows by s at most (s the largest power of two times TI_LEAF below r: 2048 and 1664 at r = 3712), which r x r images hold
 static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *img, int r, int32_t *status, cudaStream_t st) {
     static PerDeviceOnce once;
-    if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(tri_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TI_SMEM));
+    if (auto first = once.first()) MDBF_CUDA(cudaFuncSetAttribute(tri_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TI_SMEM));
     MDBF_CUDA(cudaMemsetAsync(Y, 0, (size_t)r * r * sizeof(float), st));
     tri_leaf_kernel<<<ceil_div(r, TI_LEAF), TI_LEAF, TI_SMEM, st>>>(U, Y, r);
     for (int s = TI_LEAF; s < r; s *= 2) {

@@ -7,6 +7,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "mdbf.h"
 
 namespace mdbf {
@@ -160,16 +162,21 @@ template <> __device__ __forceinline__ void act_store<__nv_bfloat16>(__nv_bfloat
 
 __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
-// cudaFuncSetAttribute is per device: one flag per (call site, device).  Returns true the first time it is asked
-// about the current device (the caller then sets its attributes), false afterwards or when the device is unknown.
+// cudaFuncSetAttribute is per device: one flag per (call site, device).  `if (auto first = once.first()) { set attributes }`: the body runs
+// until it has been run to its end on the current device, so a second thread cannot launch before the attributes are set (two
+// threads that come first together both set them, which is harmless); always where the device is unknown.
 struct PerDeviceOnce {
-    bool done[64] = {};
-    bool first() {
+    std::atomic<bool> done[64] = {};
+    struct First {
+        std::atomic<bool> *slot;
+        bool run;
+        explicit operator bool() const { return run; }
+        ~First() { if (run && slot) slot->store(true, std::memory_order_release); }
+    };
+    First first() {
         int dev = -1;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;     // unknown device: set again, it is cheap
-        if (done[dev]) return false;
-        done[dev] = true;
-        return true;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return First{nullptr, true};
+        return First{&done[dev], !done[dev].load(std::memory_order_acquire)};
     }
 };
 inline size_t dtype_size(int dt) { return dt == MDBF_F32 ? 4 : 2; }

@@ -165,7 +165,7 @@ static mdbf_status_t alu_launch(const AluArgs &a0, cudaStream_t st) {
     a.part_off = (int)(base / 4);
     auto kern = alu_stage_kernel<TT, LB, InT, OutT>;
     static PerDeviceOnce once;
-    if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
+    if (auto first = once.first()) MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(tiles, ranks);
     cfg.blockDim = dim3(nw * 32);

@@ -880,7 +880,7 @@ static mdbf_status_t make_out_tensor_map(CUtensorMap *out, const void *base, int
 template <bool STAGE_A>
 static mdbf_status_t launch_mat(const MatArgs &a0, int large_ks, const CUtensorMap &tm, const CUtensorMap &tmo, cudaStream_t st) {
     static PerDeviceOnce once;
-    if (once.first()) {
+    if (auto first = once.first()) {
         const int max_smem = (int)mt_smem_bytes(4, 3, MT_BN, 0);
         MDBF_CUDA(cudaFuncSetAttribute(mat_stage_kernel<STAGE_A, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
         MDBF_CUDA(cudaFuncSetAttribute(mat_stage_kernel<STAGE_A, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));

@@ -528,7 +528,7 @@ mdbf_status_t make_xs_tensor_map(CUtensorMap *out, const void *base, size_t rows
 template <int LP, bool STAGE_A>
 static mdbf_status_t launch_gemm(const GemmArgs &a, const CUtensorMap &tm, cudaStream_t st) {
     static PerDeviceOnce once;
-    if (once.first()) {
+    if (auto first = once.first()) {
         MDBF_CUDA(cudaFuncSetAttribute(gemm_stage_kernel<LP, STAGE_A, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_BYTES));
         MDBF_CUDA(cudaFuncSetAttribute(gemm_stage_kernel<LP, STAGE_A, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, PF_SMEM_BYTES));
     }

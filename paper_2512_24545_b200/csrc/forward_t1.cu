@@ -878,7 +878,7 @@ static mdbf_status_t t1_launch(const t1::Group &grp, int ctas, cudaStream_t st, 
     auto image_kern = t1::t1_image_kernel<LP>;
     const size_t smem = t1::Cfg<LP>::SMEM;
     static PerDeviceOnce once;
-    if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(stage_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (auto first = once.first()) MDBF_CUDA(cudaFuncSetAttribute(stage_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     for (int s = 0; s < 2; ++s) {
         if (!(stages >> s & 1)) continue;
         // stage A right after this file's stage B: max |z| is already there

@@ -594,7 +594,7 @@ int last_t1_launch_count() { return g_t1_launches; }
 template <int LP, int G>
 static mdbf_status_t launch_t1g(const TxMulti &m, const TxPlan &p, bool alone, cudaStream_t st) {
     static PerDeviceOnce once;
-    if (once.first()) {
+    if (auto first = once.first()) {
         MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));
         if (G == 2) MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_kernel<LP, G>, cudaFuncAttributePreferredSharedMemoryCarveout, TX_CARVEOUT));
         MDBF_CUDA(cudaFuncSetAttribute(tmem_t1_multi_kernel<LP, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, TX_MAX_DYN));

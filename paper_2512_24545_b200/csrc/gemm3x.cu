@@ -437,7 +437,7 @@ mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, float *C, i
 mdbf_status_t gemm3x_run(const uint32_t *Aimg, const uint32_t *Bimg, const G3xOut &o, int n, int r, int depth, int32_t *status, cudaStream_t st,
                          int spare_sms) {
     static PerDeviceOnce once;
-    if (once.first()) MDBF_CUDA(cudaFuncSetAttribute(g3x::gemm3x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g3x::SMEM));
+    if (auto first = once.first()) MDBF_CUDA(cudaFuncSetAttribute(g3x::gemm3x_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g3x::SMEM));
     const int ntm = ceil_div(n, g3x::TILE), ntn = ceil_div(r, g3x::TILE);
     int sms = 0;
     mdbf_status_t rc = device_sms(&sms);

@@ -1017,7 +1017,7 @@ static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int part
     if (rc) return rc;
     const int ctas = orth_ctas(n, OR_ROWS, GR_MAX_CTAS, sms), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
     static PerDeviceOnce once;
-    if (once.first()) {
+    if (auto first = once.first()) {
         MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
         // the product's split between L1 and shared memory: its CTAs can start beside this kernel's
         MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
@@ -1081,7 +1081,7 @@ static mdbf_status_t tc_product(const ZMaps &zm, int p, int q, const uint32_t *S
                                 cudaStream_t st, int *parts_out, uint32_t *S_out = nullptr) {
     using C = TcCfg<LP>;
     static PerDeviceOnce once;
-    if (once.first())
+    if (auto first = once.first())
         MDBF_CUDA(cudaFuncSetAttribute(envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)C::SMEM));
     const int m_ext = TRANS ? q : p, k_ext = TRANS ? p : q;
