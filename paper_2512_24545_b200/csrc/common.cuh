@@ -112,6 +112,9 @@ mdbf_status_t cuda_fail(cudaError_t e, const char *what);
 mdbf_status_t require_device(int *dev_out);
 // SMs of the current device (a part of a GPU has fewer than 148); asked of the runtime once per device
 mdbf_status_t device_sms(int *sms);
+// Tensor map of a row-major matrix rows x cols with rows `pitch` bytes apart; box: columns x rows.
+mdbf_status_t encode_tensor_map(CUtensorMap *out, CUtensorMapDataType type, const void *base, size_t rows, size_t cols, size_t pitch, int box_cols,
+                                int box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion l2);
 // fp32-accurate dense product on the tensor cores (gemm3x.cu): operand images, then C = A B
 size_t gemm3x_image_bytes(int64_t rows, int64_t depth);
 mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, int rows, int depth, uint32_t *img, cudaStream_t st);

@@ -849,32 +849,8 @@ static int mt_resident(int ks) {
 }
 // Tensor map of a bf16 output [T][rows] with rows `pitch` elements apart: box of 128 rows x 64 tokens, no swizzle.
 static mdbf_status_t make_out_tensor_map(CUtensorMap *out, const void *base, int T, int rows, int pitch) {
-    typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static encode_fn fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        MDBF_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q));
-        if (!p || q != cudaDriverEntryPointSuccess) {
-            set_error("cuTensorMapEncodeTiled is not available from the driver");
-            return MDBF_ERR_CUDA;
-        }
-        fn = reinterpret_cast<encode_fn>(p);
-    }
-    const cuuint64_t gdim[2] = {(cuuint64_t)rows, (cuuint64_t)T};
-    const cuuint64_t gstride[1] = {(cuuint64_t)pitch * 2};
-    const cuuint32_t box[2] = {MT_BM, 64};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), gdim, gstride, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled (output) failed with CUresult %d", (int)r);
-        return MDBF_ERR_CUDA;
-    }
-    return MDBF_OK;
+    return encode_tensor_map(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, T, rows, (size_t)pitch * 2, MT_BM, 64, CU_TENSOR_MAP_SWIZZLE_NONE,
+                             CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
 
 template <bool STAGE_A>

@@ -72,6 +72,44 @@ mdbf_status_t device_sms(int *sms) {
     return MDBF_OK;
 }
 
+mdbf_status_t encode_tensor_map(CUtensorMap *out, CUtensorMapDataType type, const void *base, size_t rows, size_t cols, size_t pitch, int box_cols,
+                                int box_rows, CUtensorMapSwizzle swizzle, CUtensorMapL2promotion l2) {
+    typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static std::atomic<encode_fn> known{nullptr};
+    encode_fn fn = known.load(std::memory_order_relaxed);
+    if (!fn) {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        MDBF_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q));
+        if (!p || q != cudaDriverEntryPointSuccess) {
+            set_error("cuTensorMapEncodeTiled is not available from the driver");
+            return MDBF_ERR_CUDA;
+        }
+        fn = reinterpret_cast<encode_fn>(p);
+        known.store(fn, std::memory_order_relaxed);
+    }
+    const cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t gstride[1] = {(cuuint64_t)pitch};
+    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+    const cuuint32_t estr[2] = {1, 1};
+    CUresult r = CUDA_SUCCESS;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        r = fn(out, type, 2, const_cast<void *>(base), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, l2, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_ERROR_INVALID_CONTEXT) break;
+        // the driver's call wants the device's context current, which a thread has after its first call of the runtime that needs one
+        int dev = 0;
+        MDBF_CUDA(cudaGetDevice(&dev));
+        MDBF_CUDA(cudaSetDevice(dev));
+    }
+    if (r != CUDA_SUCCESS) {
+        set_error("cuTensorMapEncodeTiled failed with CUresult %d", (int)r);
+        return MDBF_ERR_CUDA;
+    }
+    return MDBF_OK;
+}
+
 // A layer lives on the device it was packed on; its kernels must be launched there.
 static mdbf_status_t check_device(const Layer &L, const char *fn) {
     int dev = -1;

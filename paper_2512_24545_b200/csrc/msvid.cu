@@ -1039,32 +1039,8 @@ static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int part
 
 // Tensor map of the fp32 matrix Z [p][q]: box of box_cols columns x box_rows rows, zero fill outside the matrix.
 static mdbf_status_t make_z_tensor_map(CUtensorMap *out, const float *Z, int p, int q, int box_cols, int box_rows, bool swizzle128) {
-    typedef CUresult (*encode_fn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static encode_fn fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult res;
-        MDBF_CUDA(cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &res));
-        if (!ptr || res != cudaDriverEntryPointSuccess) {
-            set_error("cuTensorMapEncodeTiled is not available from the driver");
-            return MDBF_ERR_CUDA;
-        }
-        fn = reinterpret_cast<encode_fn>(ptr);
-    }
-    const cuuint64_t gdim[2] = {(cuuint64_t)q, (cuuint64_t)p};
-    const cuuint64_t gstride[1] = {(cuuint64_t)q * sizeof(float)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    const CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(Z), gdim, gstride, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        set_error("cuTensorMapEncodeTiled (Z) failed with CUresult %d", (int)r);
-        return MDBF_ERR_CUDA;
-    }
-    return MDBF_OK;
+    return encode_tensor_map(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Z, p, q, (size_t)q * sizeof(float), box_cols, box_rows,
+                             swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 static bool tc_eligible(const float *Z, int q) { return (q & 3) == 0 && (reinterpret_cast<uintptr_t>(Z) & 15u) == 0; }
 
