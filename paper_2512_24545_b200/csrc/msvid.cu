@@ -518,21 +518,25 @@ template <int LP>
 __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], bool start, float *__restrict__ M) {
     const int k = threadIdx.x & 31;
     double g[LP], x[LP];                                         // row k of G, then of L; right-hand side, then column k of L^-1
-    double scale = 0.0, trace = 0.0;
 #pragma unroll
     for (int j = 0; j < LP; ++j) {
         g[j] = j <= k ? Gm[k < LP ? k : 0][j] : 0.0;             // (above the diagonal: never read by another lane)
         x[j] = j == k ? 1.0 : 0.0;
-        scale = fmax(scale, Gm[j][j]);
-        trace += Gm[j][j];
     }
+    // the limits are compared by the upper halves of the numbers (sign, exponent, 20 bits), off the chain of pivots: 2^-40 of the own
+    // length squared, in a start block 2^-80 of the largest, and what is not a normal number in any case
+    const int own = k < LP ? __double2hiint(Gm[k < LP ? k : 0][k < LP ? k : 0]) : 0;
+    const bool bad = __any_sync(0xffffffffu, (own & 0x7fffffff) >= 0x7e000000);
+    const int limit = max(start ? (int)__reduce_max_sync(0xffffffffu, own) - (80 << 20) : own - (40 << 20), 0x00100000);
 #pragma unroll
     for (int c = 0; c < LP; ++c) {
+        const int limit_c = __shfl_sync(0xffffffffu, limit, c);
         const double dcc = __shfl_sync(0xffffffffu, g[c], c);
-        const double inv = dcc > (start ? 1e-24 * scale : 1e-12 * Gm[c][c]) ? rsqrt(dcc) : 0.0;      // 1 / L[c][c], the same in every lane
+        const bool gone = __double2hiint(dcc) <= limit_c;
+        const double inv = gone ? 0.0 : rsqrt(dcc);              // 1 / L[c][c], the same in every lane
         g[c] *= inv;                                             // column c of L below the diagonal
         x[c] *= inv;                                             // (zero for c < k from the start)
-        if (start && inv == 0.0 && c == k) x[c] = 1.0;
+        if (start && gone && c == k) x[c] = 1.0;
 #pragma unroll
         for (int jj = c + 1; jj < LP; ++jj) {
             const double ljc = __shfl_sync(0xffffffffu, g[c], jj);
@@ -542,7 +546,7 @@ __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], bool start
     }
     if (k < LP) {
 #pragma unroll
-        for (int a = 0; a < LP; ++a) M[k * LP + a] = trace < 1e300 ? (float)x[a] : __int_as_float(0x7fc00000);
+        for (int a = 0; a < LP; ++a) M[k * LP + a] = bad ? __int_as_float(0x7fc00000) : (float)x[a];
     }
 }
 // A <- an orthonormal basis of its columns (Cholesky QR), in one cooperative launch: sum of the partial products (parts > 0), Gram matrix
