@@ -452,9 +452,9 @@ def measure(workload, kernel, steps, warmup, dist, world, local, no_graph=False,
 
 # ------------------------------------------------------------ quantizer, first step (MSVID)
 def msvid_launch_count(l, n_iter):
-    """As msvid.cu issues them on the tensor-core path: start block 1 + 2, per iteration two products and two orthogonalisations (+ 1 where
-    the narrow transposed product takes the scalar kernel and its partial-sum pass), last block 1, final product and factors 5."""
-    return 1 + 2 + n_iter * (4 + (1 if l <= 4 else 0)) + 1 + 5
+    """As msvid.cu issues them on the tensor-core path: start block 1 + 2, per iteration two products and what follows them (+ 1 where
+    the narrow transposed product takes the scalar kernel and its partial-sum pass), last block 1, final product and factors 4."""
+    return 1 + 2 + n_iter * (4 + (1 if l <= 4 else 0)) + 1 + 4
 
 
 def tri_inverse_launch_count(r):

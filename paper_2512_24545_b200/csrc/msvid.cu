@@ -8,7 +8,7 @@
 // takes the absolute value on the fly) is computed by block subspace iteration on a block of l columns:
 //
 //     Q  <- orth(Q0)                                 M x l start block, passed in by the caller
-//     repeat n_iter times:   Y <- orth(|Z| Q);   Q <- orth(|Z|^T Y)
+//     repeat n_iter times:   Y <- |Z| Q (the first two orthonormalised);   Q <- orth(|Z|^T Y)
 //     Y  <- |Z| Q;   Y^T Y = W diag(s^2) W^T        (l x l symmetric eigenproblem, Jacobi)
 //     U  <- Y W diag(s^-1/2),   V <- Q W diag(s^1/2)      balanced factors:  U V^T = Y Q^T ~ TSVD_l(|Z|)
 //
@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(AQ_WARPS * 32) absz_q_kernel(const float *__re
 // The two products of the subspace iteration with tcgen05 (kind::tf32, fp32 accumulators in tensor memory) and a
 // three-term split of the fp32 operands:  e = e_hi + e_lo,  q = q_hi + q_lo  (each part a TF32 number),
 //     e q  ~  e_hi q_hi + e_hi q_lo + e_lo q_hi                      (the dropped e_lo q_lo is below 2^-24 e q).
-// CTA = 128 output rows x a range of K blocks of 32 (split over blockIdx.y, partial sums per range).  Per K block:
+// Unit of work = 128 output rows x a share of the K blocks of 32 (partial sums per share); two CTAs per SM walk over the units, with
+// their rings running on from one unit to the next.  Per K block:
 //   one lane brings the raw 128 x 32 tile of Z into a ring of buffers by TMA (zero fill outside the matrix), so the
 //     bytes in flight do not depend on how many threads wait for them;
 //   8 converter warps (two groups on alternate K blocks, thread = output row = TMEM lane) read their row of the tile,
@@ -188,16 +189,26 @@ __global__ void __launch_bounds__(AQ_WARPS * 32) absz_q_kernel(const float *__re
 //     contraction indices, already in the K-major 128B-swizzled operand layout (orth_kernel writes the images
 //     when it writes the factor);
 //   two lanes issue the MMAs, four K steps of 8 each: D1 (+)= E_hi [q_hi | q_lo] (N = 2 LPP), D2 (+)= E_lo q_hi (N = LPP).
-// Epilogue: y[t] = D1[t] + D1[LPP + t] + D2[t] into the range's partial sums.
+// Epilogue (four warps of its own, so that the converters go on): y[t] = D1[t] + D1[LPP + t] + D2[t] into the share's partial sums.  Y = E Q takes the
+// accumulators out every TC_RUN K blocks and adds the runs up in registers: the tensor core's accumulation is not rounded to nearest, and
+// its one-sided error grows with the number of accumulations.
+//
+// What bounds it: memory.  Order of the units over Z: W = E^T Y walks the row ranges from the top down, Y = E Q then the row blocks from the
+// bottom up, all shares of a row block together.
+// Y = E Q of 28672 x 6016, l = 16, images to sums: 130 us with a launch of ten waves of CTAs, each with its own set-up, over 13 shares; 112 now,
+// 5 shares; W = E^T Y 105.  Whole mdbf_msvid calls (with Y not orthonormalised, see combine_kernel), before -> after: 28672 x 6016, 4
+// iterations 1345 -> 1275 us (1390 -> 1310 on another card); 5376 x 4688, 8 iterations 668 -> 540.
 // TRANS = false: Y = E Q    (output rows = rows of Z, contraction over its columns; TMA box of 32 columns x 128 rows,
 //                            128B-swizzled so that a thread's 16-byte reads of its own row spread over the banks)
 // TRANS = true:  W = E^T Y  (output rows = columns of Z, contraction over its rows; box of 128 columns x 32 rows)
 // Needs cols % 4 == 0 and Z on a 16-byte boundary (the tensor map's rules); other inputs take the scalar kernels.
 // Every wait is bounded; on expiry the status word of the workspace is set and the call's outputs are NaN.
 constexpr int TC_KB = 32, TC_CONVERTERS = 256;
-constexpr int TC_W_ISSUE = 8, TC_W_RAW = 10, TC_W_IMG = 11, TC_THREADS = 12 * 32;
+constexpr int TC_W_ISSUE = 8, TC_W_RAW = 10, TC_W_IMG = 11, TC_W_EPI = 12, TC_THREADS = 16 * 32;
 constexpr int TC_TILE = 128 * TC_KB * 4;                        // bytes of a raw tile
+constexpr int TC_RUN = 16;                                      // K blocks to an accumulation of Y = E Q
 constexpr int TC_RAW = 5;                                       // raw tiles in flight per CTA
+constexpr int TC_SLOTS = 148 * 2;                               // CTAs of a launch at most: two per SM
 template <int LP> struct TcCfg {
     static constexpr int LPP = LP < 16 ? 16 : LP;              // MMA N is a multiple of 16
     static constexpr int N1 = 2 * LPP, N2 = LPP;
@@ -242,17 +253,53 @@ __device__ __forceinline__ uint32_t make_idesc_tf32(int n) {
 // WRITE_MASK (plain product of |Z| only): the converters also pack the signs of what they read into S_out, the mask of
 // Eq. msvid-def (bit = 1 where the entry is below zero; zeros of either sign count as +1), so that the first pass over Z
 // yields it for free.
+// How a product is cut into units: `parts` shares of the K blocks of every 128 output rows.
+struct TcSplit {
+    int row_blocks, nkb, parts, per;                             // per: K blocks of a share, a range of them (the last one may be shorter)
+};
+// A CTA's way through its units, K block by K block.
+template <bool TRANS>
+struct TcWalk {
+    int unit, row0, part, kb, nkb;                               // kb of nkb within the unit
+    bool more;
+    __device__ __forceinline__ void load(const TcSplit &sp) {
+        more = unit < sp.row_blocks * sp.parts;
+        if (TRANS) {
+            part = unit / sp.row_blocks;
+            row0 = (unit - part * sp.row_blocks) * 128;
+        } else {
+            const int up = unit / sp.parts;
+            part = unit - up * sp.parts;
+            row0 = (sp.row_blocks - 1 - up) * 128;
+        }
+        nkb = min(sp.per, sp.nkb - part * sp.per);
+    }
+    __device__ __forceinline__ TcWalk(const TcSplit &sp, int ahead) : unit((int)blockIdx.x), kb(0) {
+        load(sp);
+        advance(sp, ahead);
+    }
+    __device__ __forceinline__ void advance(const TcSplit &sp, int by) {
+        kb += by;
+        while (more && kb >= nkb) {
+            kb -= nkb;
+            unit += (int)gridDim.x;
+            load(sp);
+        }
+    }
+    __device__ __forceinline__ int index(const TcSplit &sp) const { return part * sp.per + kb; }
+};
 template <int LP, bool MASKED, bool TRANS, bool WRITE_MASK>
 __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(const __grid_constant__ CUtensorMap tmap_z, int p, int q,
-                                                                  const uint32_t *__restrict__ img, int kb_per_cta, float *__restrict__ P,
+                                                                  const uint32_t *__restrict__ img, const TcSplit sp, float *__restrict__ P,
                                                                   const uint32_t *__restrict__ S, uint32_t *__restrict__ S_out, int nwords,
                                                                   int32_t *__restrict__ status) {
     static_assert(!WRITE_MASK || (!MASKED && !TRANS), "the mask is written by the plain product of |Z|");
+    static_assert(TC_W_EPI % 4 == 0, "an epilogue warp reads its own quarter of the TMEM lanes");
     using namespace tm;
     using C = TcCfg<LP>;
-    constexpr int LPP = C::LPP, N1 = C::N1, N2 = C::N2, TC_STAGES = C::STAGES;
+    constexpr int LPP = C::LPP, N1 = C::N1, N2 = C::N2, TC_STAGES = C::STAGES, RUN = TRANS ? 1 << 30 : TC_RUN;
     extern __shared__ unsigned char tc_smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * TC_STAGES + 2 * TC_RAW + 1];
+    __shared__ __align__(8) uint64_t bars[2 * TC_STAGES + 2 * TC_RAW + 2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag_s;
     volatile int *abort_flag = &abort_flag_s;
@@ -262,21 +309,9 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
     const uint32_t img_base = smem_base + (uint32_t)(TC_RAW * TC_TILE);
     const uint32_t full_bar = smem_u32(&bars[0]), empty_bar = smem_u32(&bars[TC_STAGES]);
     const uint32_t raw_full = smem_u32(&bars[2 * TC_STAGES]), raw_empty = smem_u32(&bars[2 * TC_STAGES + TC_RAW]);
-    const uint32_t accum_bar = smem_u32(&bars[2 * TC_STAGES + 2 * TC_RAW]);
-    const int m_ext = TRANS ? q : p, k_ext = TRANS ? p : q;
-    // Order of the CTAs over Z, so that a pass starts on what the pass before it read last and finds part of it in L2:
-    // W = E^T Y walks the row ranges from the top down (x = column block fastest, y = row range); Y = E Q then walks the
-    // row blocks from the bottom up, all column ranges of a row block together.
-    int bx = blockIdx.x, by = blockIdx.y;
-    if (!TRANS) {
-        const int lin = blockIdx.x + gridDim.x * blockIdx.y;
-        by = lin % gridDim.y;
-        bx = gridDim.x - 1 - lin / gridDim.y;
-    }
-    const int row0 = bx * 128;                                   // first output row (a row of Z, or a column when TRANS)
-    const int nkb_total = (k_ext + TC_KB - 1) / TC_KB;
-    const int kb0 = by * kb_per_cta;
-    const int nkb = max(0, min(kb_per_cta, nkb_total - kb0));
+    const uint32_t acc_full = smem_u32(&bars[2 * TC_STAGES + 2 * TC_RAW]), acc_empty = acc_full + 8;
+    const int m_ext = TRANS ? q : p;
+    pdl_launch_dependents();
     if (tid == 0) {
         for (int s = 0; s < TC_STAGES; ++s) {
             mbar_init(full_bar + 8 * s, 4 + 1);                  // the four warps of a converter group + the image's expect_tx
@@ -286,7 +321,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
             mbar_init(raw_full + 8 * s, 1);                      // the tile's expect_tx
             mbar_init(raw_empty + 8 * s, 4);                     // the four warps of the group that read it
         }
-        mbar_init(accum_bar, 2);
+        mbar_init(acc_full, 2);                                  // the two issuers, after a run's last K block
+        mbar_init(acc_empty, 4);                                 // the epilogue warps, once they have read the accumulators
         abort_flag_s = 0;
         fence_barrier_init();
     }
@@ -301,27 +337,33 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
     const uint32_t tmem_a0 = tmem + (uint32_t)C::ACC_COLS;       // A stage s: columns [64 s, 64 s + 32) = E_hi, the next 32 = E_lo
 
     if (warp < TC_CONVERTERS / 32) {
-        // ============================ converters, then epilogue ============================
-        const int grp = warp >> 2;                               // K blocks grp, grp + 2, ...
+        // =================================== converters ===================================
+        const int grp = warp >> 2;                               // K blocks grp, grp + 2, ... of this CTA
         const int r = (warp & 3) * 32 + lane;                    // output row within the tile = TMEM lane
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const int wcol = (row0 >> 5) + (warp & 3);               // TRANS: the warp's 32 columns are one packed word per row of Z
-        // mask word(s) of K block kb: a thread's own row and the block's word (plain), or lane i = the block's row i (TRANS)
-        auto mask_word = [&](int kb) -> uint32_t {
-            if (!MASKED || kb >= nkb) return 0u;
+        // mask word(s) of a K block: a thread's own row and the block's word (plain), or lane i = the block's row i (TRANS: the warp's 32
+        // columns are one packed word per row of Z)
+        auto mask_word = [&](const TcWalk<TRANS> &at) -> uint32_t {
+            if (!MASKED || !at.more) return 0u;
             if (TRANS) {
-                const int gr = (kb0 + kb) * TC_KB + lane;
+                const int gr = at.index(sp) * TC_KB + lane, wcol = (at.row0 >> 5) + (warp & 3);
                 return (gr < p && wcol < nwords) ? S[(size_t)gr * nwords + wcol] : 0u;
             }
-            return row0 + r < p ? S[(size_t)(row0 + r) * nwords + kb0 + kb] : 0u;
+            return at.row0 + r < p ? S[(size_t)(at.row0 + r) * nwords + at.index(sp)] : 0u;
         };
         bool alive = true;
-        uint32_t word = mask_word(grp);
-        for (int kb = grp; kb < nkb && alive; kb += 2) {
-            const int s = kb % TC_STAGES, rs = kb % TC_RAW;
-            const uint32_t word_next = mask_word(kb + 2);        // travels while this block is converted
-            alive = mbar_wait(raw_full + 8 * rs, ((uint32_t)(kb / TC_RAW)) & 1u, abort_flag, status);
-            if (alive) alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(kb / TC_STAGES)) & 1u) ^ 1u, abort_flag, status);
+        TcWalk<TRANS> at(sp, grp);
+        uint32_t word = mask_word(at);
+        for (int g = grp; at.more && alive; g += 2) {
+            const int s = g % TC_STAGES, rs = g % TC_RAW;
+            TcWalk<TRANS> next = at;
+            uint32_t word_next = 0u;
+            if (MASKED) {                                        // travels while this block is converted
+                next.advance(sp, 2);
+                word_next = mask_word(next);
+            }
+            alive = mbar_wait(raw_full + 8 * rs, ((uint32_t)(g / TC_RAW)) & 1u, abort_flag, status);
+            if (alive) alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(g / TC_STAGES)) & 1u) ^ 1u, abort_flag, status);
             alive = __all_sync(0xffffffffu, alive);
             if (!alive) break;
             tc_fence_after();
@@ -352,7 +394,7 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
                 tmem_st8(a_col + (uint32_t)(8 * c8), h);
                 tmem_st8(a_col + (uint32_t)(32 + 8 * c8), l);
             }
-            if (WRITE_MASK && row0 + r < p) S_out[(size_t)(row0 + r) * nwords + kb0 + kb] = signs;
+            if (WRITE_MASK && at.row0 + r < p) S_out[(size_t)(at.row0 + r) * nwords + at.index(sp)] = signs;
             __syncwarp();
             if (lane == 0) mbar_arrive(raw_empty + 8 * rs);
             tmem_st_wait();
@@ -360,31 +402,8 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
             __syncwarp();
             if (lane == 0) mbar_arrive(full_bar + 8 * s);
             word = word_next;
-        }
-        if (warp < 4) {
-            const int grow = row0 + r;
-            if (alive) alive = mbar_wait(accum_bar, 0u, abort_flag, status);
-            alive = __all_sync(0xffffffffu, alive);
-            tc_fence_after();
-            float y[LPP];
-#pragma unroll
-            for (int t = 0; t < LPP; ++t) y[t] = 0.f;
-            if (alive && nkb > 0) {
-#pragma unroll
-                for (int c16 = 0; c16 < (N1 + N2) / 16; ++c16) {
-                    uint32_t d[16];
-                    tmem_ld16(tmem + lane_base + (uint32_t)(c16 * 16), d);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) y[(c16 * 16 + e) % LPP] += __uint_as_float(d[e]);      // columns t, LPP + t and N1 + t belong to mode t
-                }
-            }
-            pdl_wait();                                          // the previous kernel reads the partial sums that are overwritten here
-            if (grow < m_ext) {
-                float *out = P + ((size_t)by * m_ext + grow) * LP;
-#pragma unroll
-                for (int t = 0; t < LP; ++t) out[t] = alive ? y[t] : __int_as_float(0x7fc00000);
-            }
+            if (MASKED) at = next;
+            else at.advance(sp, 2);
         }
     } else if (warp == TC_W_ISSUE || warp == TC_W_ISSUE + 1) {
         // ================================== MMA issuers ===================================
@@ -393,8 +412,14 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
         const uint32_t d_tmem = tmem + (first ? 0u : (uint32_t)N1);
         bool alive = true;
         int s = 0;
-        uint32_t ph = 0;
-        for (int kb = 0; kb < nkb && alive; ++kb) {
+        uint32_t ph = 0, run_ph = 0;
+        for (TcWalk<TRANS> at(sp, 0); at.more && alive; at.advance(sp, 1)) {
+            const int run = at.kb % RUN;
+            if (run == 0) {                                      // the epilogue has read the run before this one
+                alive = __all_sync(0xffffffffu, mbar_wait(acc_empty, run_ph ^ 1u, abort_flag, status));
+                run_ph ^= 1u;
+                if (!alive) break;
+            }
             alive = __all_sync(0xffffffffu, mbar_wait(full_bar + 8 * s, ph, abort_flag, status));
             if (!alive) break;
             tc_fence_after();
@@ -403,28 +428,25 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
             if (elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)                   // 8 TF32 per K step: 8 TMEM columns of A, 32 bytes of B
-                    umma_ts_tf32(d_tmem, a_t + (uint32_t)(8 * ks), bdesc + (uint64_t)(2 * ks), idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                    umma_ts_tf32(d_tmem, a_t + (uint32_t)(8 * ks), bdesc + (uint64_t)(2 * ks), idesc, (run > 0 || ks > 0) ? 1u : 0u);
                 umma_commit(empty_bar + 8 * s);                  // frees the A stage and the image together
+                if (run == RUN - 1 || at.kb == at.nkb - 1) umma_commit(acc_full);
             }
             __syncwarp();
             if (++s == TC_STAGES) { s = 0; ph ^= 1u; }
         }
-        if (elect_one()) {
-            if (alive && nkb > 0) umma_commit(accum_bar);
-            else mbar_arrive(accum_bar);
-        }
-        __syncwarp();
     } else if (warp == TC_W_RAW) {
         // ================================ raw tile loader ================================
         if (lane == 0) {
             bool alive = true;
-            for (int kb = 0; kb < nkb && alive; ++kb) {
-                const int rs = kb % TC_RAW;
-                alive = mbar_wait(raw_empty + 8 * rs, (((uint32_t)(kb / TC_RAW)) & 1u) ^ 1u, abort_flag, status);
+            int g = 0;
+            for (TcWalk<TRANS> at(sp, 0); at.more && alive; at.advance(sp, 1), ++g) {
+                const int rs = g % TC_RAW;
+                alive = mbar_wait(raw_empty + 8 * rs, (((uint32_t)(g / TC_RAW)) & 1u) ^ 1u, abort_flag, status);
                 if (!alive) break;
                 mbar_arrive_expect_tx(raw_full + 8 * rs, (uint32_t)TC_TILE);
-                if (TRANS) tma_load_2d(smem_base + (uint32_t)(rs * TC_TILE), &tmap_z, row0, (kb0 + kb) * TC_KB, raw_full + 8 * rs);
-                else tma_load_2d(smem_base + (uint32_t)(rs * TC_TILE), &tmap_z, (kb0 + kb) * TC_KB, row0, raw_full + 8 * rs);
+                const int k0 = at.index(sp) * TC_KB;
+                tma_load_2d(smem_base + (uint32_t)(rs * TC_TILE), &tmap_z, TRANS ? at.row0 : k0, TRANS ? k0 : at.row0, raw_full + 8 * rs);
             }
         }
         __syncwarp();
@@ -434,15 +456,50 @@ __global__ void __launch_bounds__(TC_THREADS, 2) envelope_product_tc_kernel(cons
             bool alive = true;
             pdl_wait();                                          // the images are the previous kernel's output; Z and the mask are older
             asm volatile("fence.proxy.async;\n" ::: "memory");   // written through the generic proxy, read by bulk copies
-            for (int kb = 0; kb < nkb && alive; ++kb) {
-                const int s = kb % TC_STAGES;
-                alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(kb / TC_STAGES)) & 1u) ^ 1u, abort_flag, status);
+            int g = 0;
+            for (TcWalk<TRANS> at(sp, 0); at.more && alive; at.advance(sp, 1), ++g) {
+                const int s = g % TC_STAGES;
+                alive = mbar_wait(empty_bar + 8 * s, (((uint32_t)(g / TC_STAGES)) & 1u) ^ 1u, abort_flag, status);
                 if (!alive) break;
                 mbar_arrive_expect_tx(full_bar + 8 * s, (uint32_t)C::IMG);
-                bulk_load(img_base + (uint32_t)(s * C::IMG), img + (size_t)(kb0 + kb) * (C::IMG / 4), (uint32_t)C::IMG, full_bar + 8 * s);
+                bulk_load(img_base + (uint32_t)(s * C::IMG), img + (size_t)at.index(sp) * (C::IMG / 4), (uint32_t)C::IMG, full_bar + 8 * s);
             }
         }
         __syncwarp();
+    } else {
+        // =================================== epilogue ====================================
+        const int r = (warp - TC_W_EPI) * 32 + lane;
+        const uint32_t lane_base = (uint32_t)((warp - TC_W_EPI) * 32) << 16;
+        bool alive = true;
+        uint32_t ph = 0;
+        pdl_wait();                                              // the previous kernel reads the partial sums that are overwritten here
+        for (TcWalk<TRANS> at(sp, 0); at.more; at.advance(sp, at.nkb)) {
+            float y[LPP];
+#pragma unroll
+            for (int t = 0; t < LPP; ++t) y[t] = 0.f;
+            for (int kb = 0; kb < at.nkb && alive; kb += RUN, ph ^= 1u) {
+                alive = mbar_wait(acc_full, ph, abort_flag, status);
+                alive = __all_sync(0xffffffffu, alive);
+                if (!alive) break;
+                tc_fence_after();
+#pragma unroll
+                for (int c16 = 0; c16 < (N1 + N2) / 16; ++c16) {
+                    uint32_t d[16];
+                    tmem_ld16(tmem + lane_base + (uint32_t)(c16 * 16), d);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) y[(c16 * 16 + e) % LPP] += __uint_as_float(d[e]);      // columns t, LPP + t and N1 + t belong to mode t
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty);
+            }
+            if (at.row0 + r < m_ext) {
+                float *out = P + ((size_t)at.part * m_ext + at.row0 + r) * LP;
+#pragma unroll
+                for (int t = 0; t < LP; ++t) out[t] = alive ? y[t] : __int_as_float(0x7fc00000);
+            }
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -566,7 +623,7 @@ __device__ __forceinline__ void chol_warp(const double (*Gm)[LP + 1], bool start
 //
 // The grid barrier counts arrivals in `counter`, which only grows during a call (`base`: what earlier launches have added); its wait is
 // bounded, and a launch in which it runs out sets the status word and writes NaN.
-constexpr int OR_ROWS = 128;
+constexpr int OR_ROWS = 128, OR_MAX_CTAS = 128;
 template <int LP> struct OrCfg {
     static constexpr int BL = LP >= 4 ? 4 : LP, NB = LP / BL, NP = NB * (NB + 1) / 2;      // blocks of the lower triangle
     static constexpr int row_groups() { int g = 1; while (2 * g * NP <= 256 && 2 * g <= OR_ROWS) g *= 2; return g; }
@@ -600,10 +657,14 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned int *counter, unsigned
     __threadfence();
     return *ok_s != 0;
 }
+//
+// Modes: OR_START (see chol_warp), OR_BLOCK, and OR_GRAM, which ends with the sum of the partial products in A and the Gram matrix in Gs, for
+// the eigensolver.  `scale`: where the powers of two go that bring the columns' lengths into (1/2, 1] (combine_kernel).
+enum OrthMode { OR_START, OR_BLOCK, OR_GRAM };
 template <int LP>
 __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts, double *__restrict__ Gp,
                                                    double *__restrict__ Gs, unsigned int *__restrict__ counter, unsigned int base,
-                                                   uint32_t *__restrict__ img, bool start, int32_t *__restrict__ status) {
+                                                   uint32_t *__restrict__ img, OrthMode mode, float *__restrict__ scale, int32_t *__restrict__ status) {
     using C = OrCfg<LP>;
     constexpr int BL = C::BL, NP = C::NP, RG = C::RG, LD = C::LD;
     constexpr int PER = OR_ROWS * LP / 256 > 0 ? OR_ROWS * LP / 256 : 1;                   // elements of a chunk per thread
@@ -655,7 +716,7 @@ __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n,
             if (e >= OR_ROWS * LP) continue;
             As[e / LP * LD + e % LP] = (double)v[u];             // rows past the end are zero
             if (kept < C::KEEP) rows[(size_t)kept * OR_ROWS * (LP + 1) + e / LP * (LP + 1) + e % LP] = v[u];
-            else if (parts > 0 && at0 + e < limit) A[at0 + e] = v[u];
+            if ((kept >= C::KEEP || mode == OR_GRAM) && parts > 0 && at0 + e < limit) A[at0 + e] = v[u];
         }
         __syncthreads();
         if (rg < RG)
@@ -691,14 +752,21 @@ __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n,
             for (int c = tid & 31; c < G; c += 32) t += __ldcg(Gp + (size_t)c * LP * LP + e);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if ((tid & 31) == 0) __stcg(Gs + e, t);
+            if ((tid & 31) == 0) __stcg(Gs + e, ok ? t : __longlong_as_double(0x7ff8000000000000ll));
         }
+    if (mode == OR_GRAM) return;
     ok = grid_arrive_wait(counter, base + 2u * (unsigned int)G, &ok_s, status) && ok;
     for (int e = tid; e < LP * LP; e += 256)
         if (e % LP <= e / LP) Gm[e / LP][e % LP] = __ldcg(Gs + e);
     __syncthreads();
-    if (tid < 32) chol_warp<LP>(Gm, start, Ms);
+    if (tid < 32) chol_warp<LP>(Gm, mode == OR_START, Ms);
     __syncthreads();
+    if (blockIdx.x == 0 && tid < LP) {                           // M's diagonal: the inverse lengths of what the columns before leave of a column
+        const float d = Ms[tid * LP + tid];
+        int e = 1;
+        if (d > 0.f && d <= 3.4028235e38f) frexpf(d, &e);
+        scale[tid] = scalbnf(1.f, e - 1);
+    }
 
     // A M and the operand images; two threads per row where a row has sixteen columns or more
     constexpr int H = LP >= 16 ? 2 : 1, LC = LP / H;
@@ -737,107 +805,88 @@ __global__ void __launch_bounds__(256) orth_kernel(float *__restrict__ A, int n,
     }
 }
 
-// Gram matrix Gs of a tall matrix A (n x LP) in fp64 (lower triangle), for the eigensolver.  The CTAs stride over chunks of GR_ROWS
-// rows: where `parts` > 0 a chunk's rows are first formed as the sum of their partial sums P[c] (c < parts, in order) and written
-// to A; every CTA keeps one partial Gram matrix over its chunks, and the CTA that finishes last adds them up in a fixed order.
-constexpr int GR_ROWS = 128, GR_MAX_CTAS = 128;
+// From the third iteration on Y is not orthonormalised before W = |Z|^T Y: the partial sums of Y = |Z| Q are added up, column t multiplied by
+// scale[t], and the operand images written.  Q is orthonormal and, after two iterations, its column t is close to the t-th singular vector:
+// the columns of |Z| Q are about as long as the singular values (which the scale takes off: the last orth()'s lengths, so W comes out
+// as long as it would from an orthonormal block), and what a column of W holds of the vectors before it is of its own size, so the
+// Cholesky QR of W finds a well-conditioned block.  The rounding errors that a column carries along the vectors before it grow by
+// another factor of their ratio until orth() takes them off; those across them, which stay, do not.  The first block, a product with a
+// random one, is dominated by the first vector in every column, and after it an unlucky start can still leave a column of Q that holds many times
+// its own size of them: with the second block left as it is too, two of sixteen matrices of 28672 x 6016 came out five to ten times
+// further from the same iteration in fp64 (2.3e-4 and 6.6e-5 of U instead of 1.8e-5 and 5e-6); from the third on none does.
+// Bound by latency: a pass over `parts` blocks in L2.  28672 x 16, 5 parts: 7 us, against 17 for orth_kernel.
+constexpr int CB_THREADS = 256;
 template <int LP>
-__global__ void __launch_bounds__(256) gram_finish_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts,
-                                                          double *__restrict__ Gp, unsigned int *__restrict__ counter,
-                                                          double *__restrict__ Gs) {
-    constexpr int PER = GR_ROWS * LP / 256 > 0 ? GR_ROWS * LP / 256 : 1;     // elements of a chunk per thread
-    constexpr int ENT = (LP * LP + 255) / 256;                                // Gram entries per thread
-    __shared__ double As[GR_ROWS][LP + 1];                       // converted once on the way in, not once per product
-    __shared__ bool is_last;
-    double acc[ENT];
+__global__ void __launch_bounds__(CB_THREADS) combine_kernel(float *__restrict__ A, int n, const float *__restrict__ P, int parts,
+                                                             const float *__restrict__ scale, uint32_t *__restrict__ img) {
+    constexpr int LPP = TcCfg<LP>::LPP, N1 = TcCfg<LP>::N1;
+    constexpr int TC = LP < 8 ? LP : 8, GROUPS = LP / TC;        // columns of a thread: 32 bytes of a row
+    tm::pdl_launch_dependents();                                 // the product that reads the images brings its tiles of Z meanwhile
+    const int rows = ceil_div(n, TC_KB) * TC_KB;                 // rows past the end are zero in the images
+    const int i = (int)(blockIdx.x * (CB_THREADS / GROUPS) + threadIdx.x % (CB_THREADS / GROUPS)), t0 = (int)threadIdx.x / (CB_THREADS / GROUPS) * TC;
+    tm::pdl_wait();
+    if (i >= rows) return;
+    float v[TC];
 #pragma unroll
-    for (int u = 0; u < ENT; ++u) acc[u] = 0.0;
-    const int nchunks = (n + GR_ROWS - 1) / GR_ROWS;
-    for (int chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-        const int i0 = chunk * GR_ROWS;
-        const size_t base = (size_t)i0 * LP, limit = (size_t)n * LP;
-        float v[PER];
-#pragma unroll
-        for (int u = 0; u < PER; ++u) v[u] = 0.f;
-        if (parts > 0) {
+    for (int t = 0; t < TC; ++t) v[t] = 0.f;
+    if (i < n) {
+        const size_t at = (size_t)i * LP + t0, part = (size_t)n * LP;
+        if constexpr (TC % 4 == 0) {
 #pragma unroll 4
-            for (int c = 0; c < parts; ++c)                       // independent loads, additions in the order of c
+            for (int c = 0; c < parts; ++c)                      // independent loads, additions in the order of c
 #pragma unroll
-                for (int u = 0; u < PER; ++u) {
-                    const size_t at = base + threadIdx.x + 256 * u;
-                    if (threadIdx.x + 256 * u < GR_ROWS * LP && at < limit) v[u] += __ldcs(P + (size_t)c * limit + at);
+                for (int t = 0; t < TC; t += 4) {
+                    const float4 x = __ldcs(reinterpret_cast<const float4 *>(P + c * part + at + t));
+                    v[t] += x.x; v[t + 1] += x.y; v[t + 2] += x.z; v[t + 3] += x.w;
                 }
         } else {
+            for (int c = 0; c < parts; ++c)
 #pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const size_t at = base + threadIdx.x + 256 * u;
-                if (threadIdx.x + 256 * u < GR_ROWS * LP && at < limit) v[u] = A[at];
-            }
+                for (int t = 0; t < TC; ++t) v[t] += __ldcs(P + c * part + at + t);
         }
-        __syncthreads();                                         // the previous chunk's Gram pass has read As
+        if (parts == 0)
 #pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int e = threadIdx.x + 256 * u;
-            if (e < GR_ROWS * LP) {
-                const size_t at = base + e;
-                if (parts > 0 && at < limit) A[at] = v[u];
-                As[e / LP][e % LP] = (double)v[u];               // rows past the end are zero
-            }
-        }
-        __syncthreads();
+            for (int t = 0; t < TC; ++t) v[t] = A[at + t];
 #pragma unroll
-        for (int u = 0; u < ENT; ++u) {
-            const int pr = threadIdx.x + 256 * u;
-            const int a = pr / LP, b = pr - a * LP;
-            if (pr < LP * LP && b <= a) {
-                double s0 = 0.0, s1 = 0.0;
-                for (int i = 0; i < GR_ROWS; i += 2) {
-                    s0 += As[i][a] * As[i][b];
-                    s1 += As[i + 1][a] * As[i + 1][b];
-                }
-                acc[u] += s0 + s1;
-            }
-        }
+        for (int t = 0; t < TC; ++t) v[t] *= scale[t0 + t];
+        if (!img)
+#pragma unroll
+            for (int t = 0; t < TC; ++t) A[at + t] = v[t];
     }
+    if (!img) return;
+    const int kappa = i & 31;
+    uint32_t *dst = img + (size_t)(i >> 5) * (N1 * 32);
 #pragma unroll
-    for (int u = 0; u < ENT; ++u)
-        if (threadIdx.x + 256 * u < LP * LP) Gp[(size_t)blockIdx.x * LP * LP + threadIdx.x + 256 * u] = acc[u];
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    for (int pr = threadIdx.x; pr < LP * LP; pr += 256) {
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int c = 0; c < (int)gridDim.x; c += 16) {           // sixteen loads in flight, added in the order of c
-            double v[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = c + u < (int)gridDim.x ? __ldcg(Gp + (size_t)(c + u) * LP * LP + pr) : 0.0;
-#pragma unroll
-            for (int u = 0; u < 16; ++u) s[u & 3] += v[u];
-        }
-        Gs[pr] = (s[0] + s[1]) + (s[2] + s[3]);
+    for (int u = 0; u < (LPP > LP ? LPP : TC); ++u) {            // (a narrow block's images are filled up with zeros, by its only group)
+        const int t = LPP > LP ? u : t0 + u;
+        const float x = u < TC ? v[u < TC ? u : 0] : 0.f;
+        const uint32_t hi = tf32_round(x);
+        dst[t * 32 + ((((kappa >> 2) ^ (t & 7)) << 2) | (kappa & 3))] = hi;
+        dst[(LPP + t) * 32 + ((((kappa >> 2) ^ ((LPP + t) & 7)) << 2) | (kappa & 3))] = tf32_round(x - __uint_as_float(hi));
     }
-    if (threadIdx.x == 0) *counter = 0u;                         // ready for the next launch on the stream
 }
-// out <- the first out_cols columns of A M, row by row (M is LP x LP, row-major)
+// U <- the first l columns of Y MU, V <- those of Q MV, row by row (MU, MV: LP x LP, row-major)
 template <int LP>
-__global__ void __launch_bounds__(256) right_mul_kernel(const float *__restrict__ A, int n, const float *__restrict__ M, float *__restrict__ out,
-                                                        int out_cols) {
+__global__ void __launch_bounds__(256) right_mul_kernel(const float *__restrict__ Y, int p, const float *__restrict__ MU, float *__restrict__ U,
+                                                        const float *__restrict__ Q, int q, const float *__restrict__ MV, float *__restrict__ V, int l) {
     __shared__ float Ms[LP][LP];
-    for (int e = threadIdx.x; e < LP * LP; e += 256) Ms[e / LP][e % LP] = M[e];
-    __syncthreads();
-    const int i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= n) return;
+    const int blocks_u = (p + 255) / 256;
+    const bool first = (int)blockIdx.x < blocks_u;
+    const int i = ((int)blockIdx.x - (first ? 0 : blocks_u)) * 256 + threadIdx.x, n = first ? p : q;
+    const float *A = first ? Y : Q, *M = first ? MU : MV;
+    float *out = first ? U : V;
     float a[LP], o[LP];
 #pragma unroll
-    for (int t = 0; t < LP; ++t) { a[t] = A[(size_t)i * LP + t]; o[t] = 0.f; }
+    for (int t = 0; t < LP; ++t) { a[t] = i < n ? A[(size_t)i * LP + t] : 0.f; o[t] = 0.f; }
+    tm::pdl_wait();                                              // M is the eigensolver's; Y and Q are older (and complete: it has waited for them)
+    for (int e = threadIdx.x; e < LP * LP; e += 256) Ms[e / LP][e % LP] = M[e];
+    __syncthreads();
+    if (i >= n) return;
 #pragma unroll
     for (int b = 0; b < LP; ++b)
 #pragma unroll
         for (int t = 0; t < LP; ++t) o[t] = fmaf(a[b], Ms[b][t], o[t]);
-    for (int t = 0; t < out_cols; ++t) out[(size_t)i * out_cols + t] = o[t];
+    for (int t = 0; t < l; ++t) out[(size_t)i * l + t] = o[t];
 }
 
 // ------------------------------------------------------------------ the small eigenproblem
@@ -861,6 +910,7 @@ __global__ void __launch_bounds__(jac_threads(LP)) jacobi_kernel(const double *_
     __shared__ int order[LP], rp[LP], rq[LP];
     __shared__ int done;
     const int tid = threadIdx.x;
+    tm::pdl_launch_dependents();
     for (int e = tid; e < LP * LP; e += JAC_THREADS) {
         const int a = e / LP, b = e - a * LP;
         G[a][b] = Gs[b <= a ? a * LP + b : b * LP + a];
@@ -960,48 +1010,47 @@ __global__ void pad_kernel(const float *__restrict__ src, size_t n, int l, int L
 
 // The scratch of one call, carved out of the caller's workspace (256-byte aligned pieces).
 struct Scratch {
-    float *Q, *Y, *P, *MU, *MV;
+    float *Q, *Y, *P, *MU, *MV, *scale;
     double *Gp, *Gs;
     uint32_t *img;          // operand images of Q for the tensor-core product
     int32_t *status;        // set by a wait that ran out
-    unsigned int *counter;  // CTAs of the Gram kernel that have finished (the word after the status word)
     unsigned int *barrier;  // arrivals at the grid barriers of orth_kernel, and how many the launches so far will have made
     unsigned int arrived;
 };
-// how the K blocks of the tensor-core product are split over blockIdx.y: the split that fills whole waves of resident CTAs best,
-// each CTA keeping at least 8 K blocks
-static int tc_split(int p, int q, int LP, int *kb_per_cta) {
-    const int slots = 148 * 2;                                   // two CTAs per SM
-    (void)LP;
+// The shares of the K blocks of p output rows over q contraction indices, at least 8 K blocks to a share.  W = E^T Y (`trans`): the split that fills
+// whole waves of resident CTAs best.  Y = E Q: every share costs 2 LP floats per row beside the row's q, written here and read by the kernel
+// that follows; what the longest CTA has above the average counts by less than half, for the others leave it their part of the
+// memory rate.  28672 x 6016, l = 16, us per mdbf_msvid of 4 iterations: Y in 2 shares 1288, 5 (taken) 1226, 6 1258, 9 1240, 13 (which fill the
+// CTAs best) 1269; W in 3 shares 1450, 6 (taken) 1242, 7 1366, 12 1268.
+static TcSplit tc_split(int p, int q, int LP, bool trans) {
     const int rb = ceil_div(p, 128), nkb = ceil_div(q, TC_KB);
-    int best = 1;
-    double best_eff = -1.0;
-    for (int ns = 1; ns <= 16 && nkb / ns >= 8; ++ns) {
+    TcSplit best = {rb, nkb, 1, nkb};
+    double best_cost = 1e30;
+    for (int ns = 1; ns <= 16 && (ns == 1 || nkb / ns >= 8); ++ns) {
         const int per = ceil_div(nkb, ns), parts = ceil_div(nkb, per);
-        const int ctas = rb * parts, waves = ceil_div(ctas, slots);
-        const double eff = (double)rb * nkb / ((double)waves * slots * per);
-        if (eff > best_eff + 1e-9) { best_eff = eff; best = ns; }
+        const double longest = (double)ceil_div(rb * parts, TC_SLOTS) * per * TC_SLOTS / ((double)rb * nkb);      // of the average CTA's K blocks
+        const double cost = trans ? longest : 1.0 + 0.4 * (longest - 1.0) + 2.0 * LP * parts / q;
+        if (cost < best_cost - 1e-9) { best_cost = cost; best.parts = parts; best.per = per; }
     }
-    *kb_per_cta = ceil_div(nkb, best);
-    return ceil_div(nkb, *kb_per_cta);
+    return best;
 }
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 static size_t carve(Scratch *w, char *base, int p, int q, int LP) {
-    const size_t zy_chunks = ceil_div(p, ZY_ROWS), gchunks = GR_MAX_CTAS;
+    const size_t zy_chunks = ceil_div(p, ZY_ROWS), gchunks = OR_MAX_CTAS;
     size_t off = 0;
     auto take = [&](size_t bytes) { char *ptr = base ? base + off : nullptr; off += align256(bytes); return ptr; };
     float *Q = (float *)take((size_t)q * LP * sizeof(float));
     float *Y = (float *)take((size_t)p * LP * sizeof(float));
-    int kb_per_cta = 0;
-    const size_t tc_parts = (size_t)tc_split(p, q, LP, &kb_per_cta), tc_parts_t = (size_t)tc_split(q, p, LP, &kb_per_cta);
+    const size_t tc_parts = (size_t)tc_split(p, q, LP, false).parts, tc_parts_t = (size_t)tc_split(q, p, LP, true).parts;
     float *P = (float *)take(std::max(std::max(zy_chunks, tc_parts_t) * q, tc_parts * p) * LP * sizeof(float));
     uint32_t *img = (uint32_t *)take((size_t)ceil_div(std::max(p, q), TC_KB) * 2 * (LP < 16 ? 16 : LP) * 128);
-    int32_t *status = (int32_t *)take(3 * sizeof(int32_t));
+    int32_t *status = (int32_t *)take(2 * sizeof(int32_t));
     double *Gp = (double *)take(gchunks * LP * LP * sizeof(double));
     double *Gs = (double *)take((size_t)LP * LP * sizeof(double));
     float *MU = (float *)take((size_t)LP * LP * sizeof(float));
     float *MV = (float *)take((size_t)LP * LP * sizeof(float));
-    if (w) { w->Q = Q; w->Y = Y; w->P = P; w->Gp = Gp; w->Gs = Gs; w->MU = MU; w->MV = MV; w->img = img; w->status = status; w->counter = (unsigned int *)status + 1; w->barrier = (unsigned int *)status + 2; w->arrived = 0u; }
+    float *scale = (float *)take((size_t)LP * sizeof(float));
+    if (w) { w->Q = Q; w->Y = Y; w->P = P; w->Gp = Gp; w->Gs = Gs; w->MU = MU; w->MV = MV; w->img = img; w->scale = scale; w->status = status; w->barrier = (unsigned int *)status + 1; w->arrived = 0u; }
     return off;
 }
 static int padded_rank(int l) {
@@ -1013,13 +1062,13 @@ static int padded_rank(int l) {
 // A <- an orthonormal basis of its columns (Cholesky QR); with `parts` > 0, A is first formed as the sum of the partial sums
 // in w.P; with `img`, the operand images of the result are written for the tensor-core product that reads it next
 template <int LP>
-static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr, bool start = false) {
+static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int parts = 0, uint32_t *img = nullptr, OrthMode mode = OR_BLOCK) {
     using C = OrCfg<LP>;
     auto kern = orth_kernel<LP>;
     int sms = 0;
     mdbf_status_t rc = device_sms(&sms);
     if (rc) return rc;
-    const int ctas = orth_ctas(n, OR_ROWS, GR_MAX_CTAS, sms), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
+    const int ctas = orth_ctas(n, OR_ROWS, OR_MAX_CTAS, sms), chunks = ceil_div(ceil_div(n, OR_ROWS), ctas);
     static PerDeviceOnce once;
     if (auto first = once.first()) {
         MDBF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024));
@@ -1036,9 +1085,34 @@ static mdbf_status_t orth(float *A, int n, Scratch &w, cudaStream_t st, int part
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, A, n, (const float *)w.P, parts, w.Gp, w.Gs, w.barrier, w.arrived, img, start, w.status));
-    w.arrived += 2u * (unsigned int)ctas;
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, A, n, (const float *)w.P, parts, w.Gp, w.Gs, w.barrier, w.arrived, img, mode, w.scale, w.status));
+    w.arrived += (mode == OR_GRAM ? 1u : 2u) * (unsigned int)ctas;
     return MDBF_OK;
+}
+
+// what a kernel launched beside the one before it is launched with (it waits for that one itself)
+template <class K, class... Args>
+static mdbf_status_t launch_beside(K kern, int ctas, int threads, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+    return MDBF_OK;
+}
+
+// the operand images of Y, or Y itself where img is null, from its partial sums
+template <int LP>
+static mdbf_status_t combine(float *A, int n, Scratch &w, cudaStream_t st, int parts, uint32_t *img) {
+    constexpr int per_cta = CB_THREADS / (LP < 8 ? 1 : LP / 8);
+    return launch_beside(combine_kernel<LP>, ceil_div(ceil_div(n, TC_KB) * TC_KB, per_cta), CB_THREADS, 0, st, A, n, (const float *)w.P, parts,
+                         (const float *)w.scale, img);
 }
 
 // Tensor map of the fp32 matrix Z [p][q]: box of box_cols columns x box_rows rows, zero fill outside the matrix.
@@ -1064,22 +1138,12 @@ static mdbf_status_t tc_product(const ZMaps &zm, int p, int q, const uint32_t *S
     if (auto first = once.first())
         MDBF_CUDA(cudaFuncSetAttribute(envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)C::SMEM));
-    const int m_ext = TRANS ? q : p, k_ext = TRANS ? p : q;
-    int kb_per_cta = 0;
-    const int parts = tc_split(m_ext, k_ext, LP, &kb_per_cta);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;    // it starts while orth_kernel runs: only the images are that kernel's
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(ceil_div(m_ext, 128), parts);
-    cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    MDBF_CUDA(cudaLaunchKernelEx(&cfg, envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK>, TRANS ? zm.cols : zm.rows, p, q,
-                                 (const uint32_t *)w.img, kb_per_cta, w.P, S, S_out, nwords, w.status));
-    *parts_out = parts;                                          // the kernel that follows adds the partial sums up
+    const TcSplit sp = TRANS ? tc_split(q, p, LP, true) : tc_split(p, q, LP, false);
+    // it starts while the kernel that writes the images runs: only they are that kernel's
+    mdbf_status_t rc = launch_beside(envelope_product_tc_kernel<LP, MASKED, TRANS, WRITE_MASK>, std::min(sp.row_blocks * sp.parts, TC_SLOTS), TC_THREADS, C::SMEM,
+                                     st, TRANS ? zm.cols : zm.rows, p, q, (const uint32_t *)w.img, sp, w.P, S, S_out, nwords, w.status);
+    if (rc) return rc;
+    *parts_out = sp.parts;                                       // the kernel that follows adds the partial sums up
     return MDBF_OK;
 }
 // Y = E Q
@@ -1114,7 +1178,7 @@ template <int LP, bool MASKED>
 static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const float *Q0, uint32_t *S, float *U, float *V, float *sigma,
                          Scratch &w, cudaStream_t st) {
     const int nwords = ceil_div(q, 32);
-    MDBF_CUDA(cudaMemsetAsync(w.status, 0, 3 * sizeof(int32_t), st));           // status word, the Gram kernel's counter, the grid barriers'
+    MDBF_CUDA(cudaMemsetAsync(w.status, 0, 2 * sizeof(int32_t), st));           // status word, the grid barriers' counter
     ZMaps zm;
     zm.use = tc_eligible(Z, q);
     if (zm.use) {
@@ -1126,14 +1190,14 @@ static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const 
     if (!MASKED && !zm.use) sign_pack_kernel<<<dim3(p, ceil_div(nwords, 8 * SP_WORDS)), 256, 0, st>>>(Z, q, nwords, S);
     pad_kernel<<<(int)std::min<size_t>(((size_t)q * LP + 255) / 256, 148u * 8), 256, 0, st>>>(Q0, (size_t)q, l, LP, w.Q);
     MDBF_CUDA(cudaGetLastError());
-    mdbf_status_t rc = orth<LP>(w.Q, q, w, st, 0, nullptr, true);      // twice: the start block may be badly conditioned
+    mdbf_status_t rc = orth<LP>(w.Q, q, w, st, 0, nullptr, OR_START);      // twice: the start block may be badly conditioned
     uint32_t *img_q = zm.use ? w.img : nullptr, *img_y = (zm.use && LP >= 8) ? w.img : nullptr;   // which products run on the tensor cores
-    if (rc == MDBF_OK) rc = orth<LP>(w.Q, q, w, st, 0, img_q, true);
+    if (rc == MDBF_OK) rc = orth<LP>(w.Q, q, w, st, 0, img_q, OR_START);
     if (rc) return rc;
     int parts = 0;
     for (int it = 0; it < n_iter; ++it) {
         rc = product<LP, MASKED>(Z, p, q, S, nwords, zm, w, st, &parts, (!MASKED && it == 0) ? S : nullptr);
-        if (rc == MDBF_OK) rc = orth<LP>(w.Y, p, w, st, parts, img_y);
+        if (rc == MDBF_OK) rc = it <= 1 ? orth<LP>(w.Y, p, w, st, parts, img_y) : combine<LP>(w.Y, p, w, st, parts, img_y);
         if (rc == MDBF_OK) rc = product_t<LP, MASKED>(Z, p, q, S, nwords, zm, w, st, &parts);
         if (rc == MDBF_OK) rc = orth<LP>(w.Q, q, w, st, parts, it == n_iter - 1 ? nullptr : img_q);
         if (rc == MDBF_OK && it == n_iter - 1) rc = orth<LP>(w.Q, q, w, st, 0, img_q);   // the last block carries the result: orthonormal to fp32
@@ -1141,12 +1205,12 @@ static mdbf_status_t run(const float *Z, int p, int q, int l, int n_iter, const 
     }
     rc = product<LP, MASKED>(Z, p, q, S, nwords, zm, w, st, &parts);
     if (rc) return rc;
-    gram_finish_kernel<LP><<<std::min(ceil_div(p, GR_ROWS), GR_MAX_CTAS), 256, 0, st>>>(w.Y, p, w.P, parts, w.Gp, w.counter, w.Gs);
+    rc = orth<LP>(w.Y, p, w, st, parts, nullptr, OR_GRAM);
+    if (rc) return rc;
     jacobi_kernel<LP><<<1, jac_threads(LP), 0, st>>>(w.Gs, l, sigma, w.MU, w.MV);
-    right_mul_kernel<LP><<<ceil_div(p, 256), 256, 0, st>>>(w.Y, p, w.MU, U, l);
-    right_mul_kernel<LP><<<ceil_div(q, 256), 256, 0, st>>>(w.Q, q, w.MV, V, l);
     MDBF_CUDA(cudaGetLastError());
-    return MDBF_OK;
+    return launch_beside(right_mul_kernel<LP>, ceil_div(p, 256) + ceil_div(q, 256), 256, 0, st, (const float *)w.Y, p, (const float *)w.MU, U,
+                         (const float *)w.Q, q, (const float *)w.MV, V, l);
 }
 
 static mdbf_status_t check_shape(const char *who, int64_t rows, int64_t cols, int32_t l) {

@@ -307,6 +307,32 @@ def test_projection_with_the_matrix_own_mask_is_msvid():
     np.testing.assert_array_equal(V1, V2)
 
 
+@pytest.mark.parametrize("shape,l", [((40000, 132), 16), ((516, 40000), 16), ((9000, 1500), 8), ((128, 544), 16), ((257, 516), 32)])
+def test_products_of_several_units_per_cta(shape, l):
+    """The tensor-core products walk over units of 128 output rows and a share of the contraction, Y's accumulated 16 K blocks at a time: more
+    units than CTAs in either product, shares that end in the middle of a run and exactly with one (544 columns: 17 K blocks in two shares), a
+    single row block.  Against the same iteration in fp64: W_hat is unique where the factors are not.  The envelope is a positive outer
+    product of rank 3 with a tenth of noise, whose leading vectors have converged after six iterations; the products' three-term
+    split leaves 2^-24 of a term, fp32 sums of up to 40 000 of them 2^-24 times their root: 1e-5 of the result."""
+    rows, cols = shape
+    rng = np.random.default_rng(rows + l)
+    E = np.exp(0.3 * rng.standard_normal((rows, 3))) @ (np.exp(0.3 * rng.standard_normal((3, cols))) * [[1.0], [0.5], [0.25]])
+    Z = (E * (1.0 + 0.1 * rng.standard_normal(shape)) * rng.choice([-1.0, 1.0], shape)).astype(np.float32)
+    Q0 = inputs.make_start_block(cols, l, 7)
+    Sp, U, V, _ = run_msvid(Z, l, 6, Q0)
+    np.testing.assert_array_equal(Sp, orc.pack_signs(np.where(Z >= 0, 1, -1).astype(np.int8)))
+    A = torch.from_numpy(np.abs(Z)).cuda().double()
+    Q = torch.linalg.qr(torch.from_numpy(Q0).cuda().double())[0]
+    for _ in range(6):
+        Q = torch.linalg.qr(A.T @ torch.linalg.qr(A @ Q)[0])[0]
+    want = ((A @ Q) @ Q.T).cpu().numpy()
+    got = U @ V.T
+    assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want), np.linalg.norm(got - want) / np.linalg.norm(want)
+    U2, V2, _ = run_projection(Z, np.where(Z >= 0, 1, -1).astype(np.int8), l, 6, seed=7)
+    np.testing.assert_array_equal(U2, U)                     # the kernels that take a mask
+    np.testing.assert_array_equal(V2, V)
+
+
 def test_msvid_of_both_factors_makes_a_layer():
     """Eq. mesvid-init-compact from given balanced factors: MSVID_l of U0 (d_out x k) and of V0^T (k x d_in) on the GPU,
     the two masks and envelopes packed into a layer, and that layer's dense reconstruction and forward compared with
