@@ -353,12 +353,10 @@ mdbf_status_t mdbf_msvid_workspace_bytes(int64_t rows, int64_t cols, int32_t l, 
  *              a little more - and mdbf_msvid's workspace)
  * The dense products (W V, V^T V, the inverse of the system and its application) run on the tensor cores (fp16
  * operands, scaled per row, in a three-term split, fp32 accumulation in chunks of 64 contraction indices; U_tilde comes out within a few
- * 1e-6 of its largest entry of the exact result); the Cholesky factorisation of the R x R system is a cuSOLVER call in
- * fp32; the inversion of its factor, the MSVID step, the elementwise passes and the reconstruction of the dense factor fused with the dual update
- * are this library's kernels.  Asynchronous on `stream`; part of the work runs on a stream of the library's own that
- * is forked from `stream` and joined to it by events inside the call.  The first call on a host thread creates the
- * solver's handles, that stream and its events, and allocates the scratch the factorisation asks for (kept for later calls; a larger request synchronises
- * the stream and reallocates).  A failed factorisation (not expected for rho > 0) or an expired wait of a kernel turns
+ * 1e-6 of its largest entry of the exact result); the R x R system is factored, and its factor inverted, in fp32 blocks that are joined
+ * by the same products.  Asynchronous on `stream`; part of the work runs on a stream of the library's own that is forked from
+ * `stream` and joined to it by events inside the call.  The first call on a host thread creates that stream and its events and
+ * allocates the factorisation's scratch (64 KB), which are kept for later calls.  A failed factorisation (not expected for rho > 0) or an expired wait of a kernel turns
  * sigma into NaN.
  * Errors: INVALID_ARG (NULL pointer, rho <= 0, counts out of range, workspace too small or misaligned), SHAPE, ARCH, CUDA. */
 mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows, int64_t w_cols, int32_t transpose_w, const float *V, int64_t r,

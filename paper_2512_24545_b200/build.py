@@ -83,7 +83,7 @@ def build(force: bool = False, verbose: bool = False, bounds_check: bool | None 
         failed |= p.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")
-    subprocess.check_call([nvcc, "-shared", "-o", LIB, *objs, "-lcudart", "-lcusolver",
+    subprocess.check_call([nvcc, "-shared", "-o", LIB, *objs, "-lcudart",
                            "-Xlinker", "-rpath=/usr/local/cuda/lib64"])
     with open(STAMP, "w") as f:
         f.write(variant + "\n")

@@ -9,79 +9,54 @@
 //
 // The two dense products (W V and V^T V, once per call) run on the tensor cores at close to fp32 accuracy (gemm3x.cu: scaled
 // fp16 operands in a three-term split); V's operand images serve both, as the right operand of W V and as both operands of
-// V^T V.  The Cholesky factorisation of the R x R system (cuSOLVER) is the one library routine; its factor is inverted here by
-// doubling, the inverse of the system is formed and then applied, in every inner iteration, by the same tensor-core product.
-// Everything specific to the method is this library's own: the MSVID step (mdbf_msvid: sign mask + rank-l envelope on the tensor
+// V^T V.  The R x R system is factored and its factor inverted together (factor_inverse), the inverse of the system is formed and then
+// applied, in every inner iteration, by the same tensor-core product.  Beside these: the MSVID step (mdbf_msvid: sign mask + rank-l envelope on the tensor
 // cores), the elementwise passes around it, and the reconstruction of the dense factor from the compact one fused with
 // the dual update.
-//
-// The system is symmetric, so the column-major solver works on the row-major memory as it is; what it calls the lower
-// triangle are the rows above the diagonal here.
-#include <cusolverDn.h>
-
 #include <algorithm>
 #include <cstdint>
 
 #include "common.cuh"
+#include "tmem_ptx.cuh"
 
 namespace mdbf {
 namespace admm {
 
-struct Libs {
-    cusolverDnHandle_t solver = nullptr;
-    float *potrf_ws = nullptr;          // the factorisation's scratch, as large as the largest request so far
-    int potrf_floats = 0;
+// What a host thread keeps between calls, all of it used on the side stream.
+struct Side {
+    float *diag = nullptr;              // the inverse of a step's diagonal block (CH_NB x CH_NB)
     int device = -1;
-    cudaStream_t side = nullptr;        // the R x R system is factored and inverted here while W V runs on the caller's stream
+    cudaStream_t stream = nullptr;      // the R x R system is factored and inverted here while W V runs on the caller's stream
     cudaEvent_t fork = nullptr, join = nullptr;
 };
-static thread_local Libs g_libs;
+static thread_local Side g_side;
 
-static mdbf_status_t get_libs(int device, cudaStream_t st, Libs **out) {
-    Libs &L = g_libs;
-    if (L.device != device) {
-        if (L.solver) cusolverDnDestroy(L.solver);
-        if (L.potrf_ws) cudaFree(L.potrf_ws);
-        if (L.side) cudaStreamDestroy(L.side);
-        if (L.fork) cudaEventDestroy(L.fork);
-        if (L.join) cudaEventDestroy(L.join);
-        L = Libs();
-        if (cusolverDnCreate(&L.solver) != CUSOLVER_STATUS_SUCCESS) {
-            L = Libs();
-            set_error("cusolverDnCreate failed");
+static void give_back(Side &S) {
+    if (S.diag) cudaFree(S.diag);
+    if (S.stream) cudaStreamDestroy(S.stream);
+    if (S.fork) cudaEventDestroy(S.fork);
+    if (S.join) cudaEventDestroy(S.join);
+    S = Side();
+}
+static mdbf_status_t get_side(int device, size_t floats, const char *who, Side **out) {
+    Side &S = g_side;
+    if (S.device != device) {
+        give_back(S);
+        if (dev_malloc((void **)&S.diag, floats * sizeof(float)) != cudaSuccess) {
+            S = Side();
+            set_error("%s: out of device memory for the factorisation's scratch (%zu bytes)", who, floats * sizeof(float));
             return MDBF_ERR_CUDA;
         }
-        if (cudaStreamCreateWithFlags(&L.side, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&L.join, cudaEventDisableTiming) != cudaSuccess ||
-            cusolverDnSetStream(L.solver, L.side) != CUSOLVER_STATUS_SUCCESS) {
-            cusolverDnDestroy(L.solver);
-            if (L.side) cudaStreamDestroy(L.side);
-            if (L.fork) cudaEventDestroy(L.fork);
-            if (L.join) cudaEventDestroy(L.join);
-            L = Libs();
+        if (cudaStreamCreateWithFlags(&S.stream, cudaStreamNonBlocking) != cudaSuccess ||
+            cudaEventCreateWithFlags(&S.fork, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&S.join, cudaEventDisableTiming) != cudaSuccess) {
+            give_back(S);
             set_error("could not create the side stream of the refinement step");
             return MDBF_ERR_CUDA;
         }
-        L.device = device;
+        S.device = device;
     }
-    (void)st;
-    *out = &L;
-    return MDBF_OK;
-}
-
-// the solver's scratch, as large as the largest request so far
-static mdbf_status_t grow_scratch(Libs *L, int floats, cudaStream_t st, const char *who) {
-    if (floats <= L->potrf_floats) return MDBF_OK;
-    MDBF_CUDA(cudaStreamSynchronize(st));                         // the stream that uses it: the old scratch may still be in use
-    if (L->potrf_ws) cudaFree(L->potrf_ws);
-    L->potrf_ws = nullptr;
-    L->potrf_floats = 0;
-    if (dev_malloc(&L->potrf_ws, (size_t)floats * sizeof(float)) != cudaSuccess) {
-        set_error("%s: out of device memory for the solver's scratch (%zu bytes)", who, (size_t)floats * sizeof(float));
-        return MDBF_ERR_CUDA;
-    }
-    L->potrf_floats = floats;
+    *out = &S;
     return MDBF_OK;
 }
 
@@ -90,110 +65,329 @@ __global__ void ridge_kernel(float *__restrict__ G, int r, float rho) {
     if (i < r) G[(size_t)i * r + i] += rho;
 }
 
-// ------------------------------------------------------------------ Y = U^-1, U upper triangular (r x r, row-major)
-// By doubling: the diagonal blocks of TI_LEAF columns are inverted all at once, then neighbouring inverses Y11, Y22 are joined,
-//     [U11 U12]^-1   [Y11  -Y11 U12 Y22]
-//     [     U22]   = [          Y22    ],
-// all pairs of a size in two batched products: log2(r / TI_LEAF) levels instead of the r / 256 dependent steps of a triangular solve
-// with r right-hand sides (r = 3712: 2.6 ms of such steps in the library's solver, 0.5 ms here).  Pairs of blocks of
-// TI_DENSE columns and more go through the tensor-core product.
-constexpr int TI_LEAF = 64, TI_DENSE = 1024;                     // leaves of 128: 45 us longer at r = 3712, of 32: the same
-constexpr int TI_SMEM = 2 * TI_LEAF * (TI_LEAF + 1) * 4;
-// CTA = one diagonal block, thread = column of the inverse, back substitution: the row of U is the same for the whole warp (a
-// broadcast), the column of Y is the thread's own.  The block's lower triangle is written as zeros.
-__global__ void __launch_bounds__(TI_LEAF) tri_leaf_kernel(const float *__restrict__ U, float *__restrict__ Y, int r) {
-    extern __shared__ float ti_smem[];
-    float (*us)[TI_LEAF + 1] = reinterpret_cast<float (*)[TI_LEAF + 1]>(ti_smem);
-    float (*ys)[TI_LEAF + 1] = us + TI_LEAF;
-    const int o = blockIdx.x * TI_LEAF, j = threadIdx.x, s = min(TI_LEAF, r - o);
-    for (int i = 0; i < TI_LEAF; ++i) us[i][j] = (i < s && j < s && j >= i) ? U[(size_t)(o + i) * r + o + j] : (i == j ? 1.f : 0.f);
-    __syncthreads();
-    for (int i = TI_LEAF - 1; i >= 0; --i) {
-        float a[4] = {i == j ? 1.f : 0.f, 0.f, 0.f, 0.f};
-        int k = i + 1;
-        for (; k + 4 <= TI_LEAF; k += 4)
+// ------------------------------------------------------------------ X = L^-1, L L^T = G (r x r, row-major, the triangle above the diagonal read)
+// With U = L^T, which takes G's place.  By halves, factorisation and inverse together:
+//
+//     [G11 G12]   U12 = X11 G12,  T = U12^T X11,  G22 - U12^T U12 = L22 L22^T,  X = [  X11        ]
+//     [    G22]                                                                     [-X22 T   X22 ]
+//
+// four products on the tensor cores (gemm3x_kernel) around the two diagonal halves, down to blocks of CH_LEAF columns.  Those go by steps of CH_NB
+// rows: one CTA factors and inverts the diagonal block (chol_diag_kernel), a launch multiplies the step's rows by that inverse
+// (chol_panel_kernel), another takes their outer product off the rows below (chol_update_kernel).  The rows are those of [G | I], so what
+// the elimination leaves in the place of I is X: the inverse costs no further steps.
+//
+// What bounds it is the chain of the steps, and in a step the chain of pivots.  The library's factorisation, one kernel of 0.33 us per column
+// whatever the size (1.2 ms at r = 3712, 2.1 beside W V), left the factor still to be inverted (0.5 ms); a step of 128 columns here takes 42 us,
+// 24 of them the diagonal block, and leaves the inverse.  Blocks of 512 columns: 0.5 ms longer at r = 3712, of 2048: the same, one of
+// 4096: 0.75 ms longer.  Whole mdbf_admm_factor_update, 8192 x 8192, r = 3712, l = 16, three inner iterations: 8247 -> 7725 us, of which 0.2 ms
+// are the MSVID steps' own.
+constexpr int CH_NB = 128, CH_LEAF = 1024;
+constexpr int CH_LD = CH_NB + 4;                                 // floats between rows of the diagonal block in shared memory
+constexpr int CD_P = 16, CD_SMEM = CH_NB * CH_LD * 4;            // columns of a panel of the diagonal block
+// One CTA: the m x m block at G (m <= CH_NB, filled up with the identity) -> the lower triangle of X, and D, the same CH_NB x CH_NB with zeros
+// elsewhere.  In place, by panels of CD_P columns: columns before the panel hold X's rows so far, those from it on what is left of the
+// block.  A warp factors the panel's own block and inverts it (lane k < 16: row k of the block, lane 16 + k: column k of its inverse; one
+// update serves both, each step's column of L comes from the lower lanes).  Then a thread per row below multiplies its part of the
+// panel by that inverse, a thread per column of X the panel's rows of X, and both go into `rb` (16 x CH_NB: the rows of X, the inverse, the
+// columns of L below it), whose products with its own part below the panel come off all rows below: 4 x 4 entries to a thread, the next
+// panel's own block by the factoring warp, which goes on with that block while the others do the rest (rb and the inverse are
+// doubled for it).  A pivot that is not positive sets info.
+__global__ void __launch_bounds__(256, 1) chol_diag_kernel(const float *__restrict__ G, float *__restrict__ X, float *__restrict__ D, int m, int ld, int *__restrict__ info) {
+    extern __shared__ __align__(16) float ch_smem[];
+    float *S = ch_smem;
+    __shared__ __align__(16) float rb2[2][CD_P][CH_NB];
+    __shared__ __align__(16) float inv2[2][CD_P][CD_P];          // the panel's inverse
+    const int tid = threadIdx.x, lane = tid & 31;
+    tm::pdl_launch_dependents();
+    tm::pdl_wait();
+    {
+        const int i = tid & (CH_NB - 1), k0 = tid >> 7;          // entry (i, k) is read above the diagonal
+        float v[CH_NB / 2];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) a[u] = fmaf(-us[i][k + u], ys[k + u][j], a[u]);
-        for (; k < TI_LEAF; ++k) a[0] = fmaf(-us[i][k], ys[k][j], a[0]);
-        ys[i][j] = i <= j ? ((a[0] + a[1]) + (a[2] + a[3])) / us[i][i] : 0.f;
-    }
-    if (j < s)
-        for (int i = 0; i < s; ++i) Y[(size_t)(o + i) * r + o + j] = ys[i][j];
-}
-// One of the two products that join the pairs of blocks of s columns (blockIdx.z = pair): out = A B (FIRST: A = U12, B = Y22; P) or
-// -A B (A = Y11, B = P; Y12), fp32 on the CUDA cores: 64 x 64 tiles, 256 threads of 4 x 4, the triangular operand's zeros skipped.
-template <bool FIRST>
-__global__ void __launch_bounds__(256) tri_join_kernel(const float *__restrict__ A, const float *__restrict__ B, float *__restrict__ out, int r, int s) {
-    __shared__ __align__(16) float as[16][68], bs[16][68];       // [k][row], [k][column]
-    const int o = blockIdx.z * 2 * s, s2 = min(s, r - o - s);
-    const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
-    if (j0 >= s2) return;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const float *a = A + (size_t)o * r + (FIRST ? o + s : o);                                // U12 (s x s2) or Y11 (s x s)
-    const float *b = FIRST ? B + (size_t)(o + s) * r + o + s : B + (size_t)o * r + o + s;    // Y22 (s2 x s2) or P (s x s2)
-    const int depth = FIRST ? s2 : s;
-    const int k_lo = FIRST ? 0 : i0, k_hi = FIRST ? min(depth, j0 + 64) : depth;             // Y22[k][j] = 0 for k > j, Y11[i][k] = 0 for k < i
-    float acc[4][4] = {};
-    for (int k0 = k_lo; k0 < k_hi; k0 += 16) {
-        {
-            const int kk = tid & 15;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int row = (tid >> 4) + 16 * u;
-                as[kk][row] = (i0 + row < s && k0 + kk < k_hi) ? a[(size_t)(i0 + row) * r + k0 + kk] : 0.f;
-                const int col = tid & 63, kb = (tid >> 6) + 4 * u;
-                bs[kb][col] = (k0 + kb < k_hi && j0 + col < s2) ? b[(size_t)(k0 + kb) * r + j0 + col] : 0.f;
-            }
+        for (int u = 0; u < CH_NB / 2; ++u) {
+            const int k = 2 * u + k0;
+            v[u] = k <= i && i < m ? G[(size_t)k * ld + i] : (i == k ? 1.f : 0.f);
         }
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            const float4 x = *reinterpret_cast<const float4 *>(&as[k][4 * ty]), y = *reinterpret_cast<const float4 *>(&bs[k][4 * tx]);
-            const float xa[4] = {x.x, x.y, x.z, x.w}, yb[4] = {y.x, y.y, y.z, y.w};
+        for (int u = 0; u < CH_NB / 2; ++u) S[i * CH_LD + 2 * u + k0] = v[u];
+    }
+    __syncthreads();
+    bool bad = false;
+    // the panel's own block at b, by one warp
+    auto factor = [&](int b, float (&inv_s)[CD_P][CD_P], float (&rb)[CD_P][CH_NB]) {
+        const int k = lane & (CD_P - 1);
+        const bool lower = lane < CD_P;
+        float v[CD_P];
+#pragma unroll
+        for (int j = 0; j < CD_P; j += 4) {
+            const float4 x = *reinterpret_cast<const float4 *>(S + (b + k) * CH_LD + b + j);
+            v[j] = lower ? x.x : (j == k ? 1.f : 0.f);
+            v[j + 1] = lower ? x.y : (j + 1 == k ? 1.f : 0.f);
+            v[j + 2] = lower ? x.z : (j + 2 == k ? 1.f : 0.f);
+            v[j + 3] = lower ? x.w : (j + 3 == k ? 1.f : 0.f);
+        }
+        float d = __shfl_sync(0xffffffffu, v[0], 0);
+#pragma unroll
+        for (int c = 0; c < CD_P; ++c) {
+            bad |= !(d > 0.f);
+            float inv = rsqrtf(d);
+            inv = fmaf(0.5f * inv, fmaf(-d * inv, inv, 1.f), inv);
+            v[c] *= inv;
+            if (c + 1 < CD_P) d = __shfl_sync(0xffffffffu, fmaf(-v[c], v[c], v[c + 1]), c + 1);      // the next pivot needs its own lane only
+#pragma unroll
+            for (int j = c + 1; j < CD_P; ++j) v[j] = fmaf(-v[c], __shfl_sync(0xffffffffu, v[c], j), v[j]);
+        }
+        if (!lower)
+#pragma unroll
+            for (int j = 0; j < CD_P; ++j) {
+                const float x = j >= k ? v[j] : 0.f;
+                inv_s[j][k] = x;
+                rb[j][b + k] = x;
+            }
+    };
+    // rows 4 rq .., columns 4 cq .. (cq <= rq), minus the panel's products
+    auto quad = [&](int b, int rq, int cq, const float (&rb)[CD_P][CH_NB]) {
+        float acc[4][4] = {};
+        float4 ls[CD_P], ys[CD_P];
+#pragma unroll
+        for (int c = 0; c < CD_P; ++c) {
+            ls[c] = *reinterpret_cast<const float4 *>(&rb[c][4 * rq]);
+            ys[c] = *reinterpret_cast<const float4 *>(&rb[c][4 * cq]);
+        }
+#pragma unroll
+        for (int c = 0; c < CD_P; ++c) {
+            const float la[4] = {ls[c].x, ls[c].y, ls[c].z, ls[c].w}, ya[4] = {ys[c].x, ys[c].y, ys[c].z, ys[c].w};
 #pragma unroll
             for (int p = 0; p < 4; ++p)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xa[p], yb[q], acc[p][q]);
+                for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(la[p], ya[q], acc[p][q]);
+        }
+        const bool panel = 4 * cq >= b && 4 * cq < b + CD_P;     // its columns start as columns of X here
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            float4 *at = reinterpret_cast<float4 *>(S + (4 * rq + p) * CH_LD + 4 * cq);
+            float4 o = panel ? make_float4(0.f, 0.f, 0.f, 0.f) : *at;
+            o.x -= acc[p][0]; o.y -= acc[p][1]; o.z -= acc[p][2]; o.w -= acc[p][3];
+            *at = o;
+        }
+    };
+    if (tid < 32) factor(0, inv2[0], rb2[0]);
+    __syncthreads();
+    for (int b = 0, buf = 0; b < m; b += CD_P, buf ^= 1) {
+        float (&rb)[CD_P][CH_NB] = rb2[buf];
+        const float (&inv_s)[CD_P][CD_P] = inv2[buf];
+        {
+            // index x behind the panel: row x of L21 = A21 L11^-T; before it: column x of the panel's rows of X; two threads, each with every other c
+            const int x = tid & (CH_NB - 1), half = tid >> 7;
+            if (x < b || x >= b + CD_P) {
+                const float *src = x < b ? S + b * CH_LD + x : S + x * CH_LD + b;
+                const int step = x < b ? CH_LD : 1;
+                float a[CD_P];
+#pragma unroll
+                for (int k = 0; k < CD_P; ++k) a[k] = src[k * step];
+#pragma unroll
+                for (int c2 = 0; c2 < CD_P; c2 += 2) {
+                    const float *row = inv_s[c2 + half];         // (zero behind its diagonal)
+                    float t[4] = {};
+#pragma unroll
+                    for (int k = 0; k < c2 + 2; ++k) t[k & 3] = fmaf(a[k], row[k], t[k & 3]);
+                    rb[c2 + half][x] = (t[0] + t[1]) + (t[2] + t[3]);
+                }
+            }
+        }
+        __syncthreads();
+        const int first = (b + CD_P) / 4;                        // first row quad below the panel
+        if (tid < 32) {
+            if (b + CD_P < m) {
+                if (lane < 10) {                                 // the next panel's own block
+                    const int p = lane < 1 ? 0 : lane < 3 ? 1 : lane < 6 ? 2 : 3;
+                    quad(b, first + p, first + lane - p * (p + 1) / 2, rb);
+                }
+                __syncwarp();
+                factor(b + CD_P, inv2[buf ^ 1], rb2[buf ^ 1]);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < 3; ++u) {                        // the panel's rows of X are done
+                const int e = tid - 32 + 224 * u, c = e / (CH_NB / 4), j = 4 * (e - c * (CH_NB / 4));
+                if (c < CD_P && j < b + CD_P) *reinterpret_cast<float4 *>(S + (b + c) * CH_LD + j) = *reinterpret_cast<const float4 *>(&rb[c][j]);
+            }
+            const int quads = CH_NB / 4 * (CH_NB / 4 + 1) / 2;
+            for (int t = tid - 32 + first * (first + 1) / 2; t < quads; t += 224) {      // t = rq (rq + 1) / 2 + cq
+                int rq = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+                if (rq * (rq + 1) / 2 > t) --rq;
+                if ((rq + 1) * (rq + 2) / 2 <= t) ++rq;
+                const int cq = t - rq * (rq + 1) / 2;
+                if (rq >= first + 4 || cq < first) quad(b, rq, cq, rb);
+            }
         }
         __syncthreads();
     }
-    float *dst = out + (size_t)o * r + o + s;
+    if (bad) *info = 1;
+#pragma unroll 32
+    for (int e = tid; e < CH_NB * CH_NB; e += 256) {
+        const int i = e / CH_NB, j = e - i * CH_NB;
+        const bool in = i < m && j <= i;
+        const float v = in ? S[i * CH_LD + j] : 0.f;
+        D[e] = v;
+        if (in) X[(size_t)i * ld + j] = v;
+    }
+}
+// Rows [b, b + m) of [X | G] times the inverse D of their diagonal block, in place: columns [0, b) of X, [b + CH_NB, n) of G; CTA = 32 columns.
+// Thread: rows ty, ty + 32, ty + 64, ty + 96 and four columns; the inverse's zeros are skipped by 32 rows.
+constexpr int CP_COLS = 32, CP_LDA = CH_NB + 4, CP_SMEM = (CH_NB * CP_LDA + CH_NB * CP_COLS) * 4;
+__global__ void __launch_bounds__(256) chol_panel_kernel(float *__restrict__ G, float *__restrict__ X, const float *__restrict__ D, int b, int m, int n, int ld) {
+    extern __shared__ __align__(16) float ch_smem[];
+    float *as = ch_smem, *bs = ch_smem + CH_NB * CP_LDA;         // [row][k], [k][column]
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int j0 = (int)blockIdx.x * CP_COLS < b ? (int)blockIdx.x * CP_COLS : (int)blockIdx.x * CP_COLS + CH_NB;
+    float *M = (j0 < b ? X : G) + (size_t)b * ld + j0;
+    const int cols = min(CP_COLS, (j0 < b ? b : n) - j0);
+    tm::pdl_launch_dependents();
+    tm::pdl_wait();
+#pragma unroll 16
+    for (int e = 4 * tid; e < CH_NB * CH_NB; e += 4 * 256)
+        *reinterpret_cast<float4 *>(as + e / CH_NB * CP_LDA + e % CH_NB) = *reinterpret_cast<const float4 *>(D + e);
+#pragma unroll 16
+    for (int e = tid; e < CH_NB * CP_COLS; e += 256) {
+        const int k = e / CP_COLS, j = e - k * CP_COLS;
+        bs[e] = k < m && j < cols ? M[(size_t)k * ld + j] : 0.f;
+    }
+    __syncthreads();
+    float acc[4][4] = {};
+#pragma unroll
+    for (int kq = 0; kq < 4; ++kq)                               // k in [32 kq, 32 kq + 32): rows from 32 kq on
+#pragma unroll 2
+        for (int k = 32 * kq; k < 32 * kq + 32; k += 4) {
+            float y[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 v = *reinterpret_cast<const float4 *>(bs + (k + u) * CP_COLS + 4 * tx);
+                y[u][0] = v.x; y[u][1] = v.y; y[u][2] = v.z; y[u][3] = v.w;
+            }
+#pragma unroll
+            for (int p = kq; p < 4; ++p) {
+                const float4 v = *reinterpret_cast<const float4 *>(as + (ty + 32 * p) * CP_LDA + k);
+                const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(x[u], y[u][q], acc[p][q]);
+            }
+        }
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (i0 + 4 * ty + p < s && j0 + 4 * tx + q < s2) dst[(size_t)(i0 + 4 * ty + p) * r + j0 + 4 * tx + q] = FIRST ? acc[p][q] : -acc[p][q];
+            if (ty + 32 * p < m && 4 * tx + q < cols) M[(size_t)(ty + 32 * p) * ld + 4 * tx + q] = acc[p][q];
 }
-// U (upper triangle read) -> Y (r x r, written whole); P: r x r scratch, img: operand images of the two blocks of a
-// product, s and at most s rows by s at most (s the largest power of two times TI_LEAF below r: 2048 and 1664 at r = 3712), which r x r images hold
-static mdbf_status_t tri_inverse(const float *U, float *Y, float *P, uint32_t *img, int r, int32_t *status, cudaStream_t st) {
-    static PerDeviceOnce once;
-    if (auto first = once.first()) MDBF_CUDA(cudaFuncSetAttribute(tri_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TI_SMEM));
-    MDBF_CUDA(cudaMemsetAsync(Y, 0, (size_t)r * r * sizeof(float), st));
-    tri_leaf_kernel<<<ceil_div(r, TI_LEAF), TI_LEAF, TI_SMEM, st>>>(U, Y, r);
-    for (int s = TI_LEAF; s < r; s *= 2) {
-        const int pairs = ceil_div(r - s, 2 * s);                // pairs whose second block is not empty
-        if (s < TI_DENSE) {
-            const dim3 grid(ceil_div(s, 64), ceil_div(s, 64), pairs);
-            tri_join_kernel<true><<<grid, 256, 0, st>>>(U, Y, P, r, s);
-            tri_join_kernel<false><<<grid, 256, 0, st>>>(Y, P, Y, r, s);
-            continue;
-        }
-        for (int p = 0; p < pairs; ++p) {
-            const int o = p * 2 * s, s2 = std::min(s, r - o - s);
-            const size_t d11 = (size_t)o * r + o, d12 = d11 + s, d22 = (size_t)(o + s) * r + o + s;
-            uint32_t *a = img, *b = img + gemm3x_image_bytes(s, s) / 4;
-            mdbf_status_t rc = gemm3x_split(U + d12, (size_t)r, 1, s, s2, a, st);                      // P = U12 Y22
-            if (rc == MDBF_OK) rc = gemm3x_split(Y + d22, 1, (size_t)r, s2, s2, b, st);
-            if (rc == MDBF_OK) rc = gemm3x_run(a, b, G3xOut{P + d12, r, false, nullptr, nullptr}, s, s2, s2, status, st);
-            if (rc == MDBF_OK) rc = gemm3x_split(Y + d11, (size_t)r, 1, s, s, a, st);                  // Y12 = -Y11 P
-            if (rc == MDBF_OK) rc = gemm3x_split(P + d12, 1, (size_t)r, s2, s, b, st);
-            if (rc == MDBF_OK) rc = gemm3x_run(a, b, G3xOut{Y + d12, r, true, nullptr, nullptr}, s, s2, s, status, st);
-            if (rc) return rc;
-        }
+// Rows below the step's CH_NB rows at b, tiles of 64 x 64: minus (U's columns of that row)^T times the step's rows, in X for columns [0, b + CH_NB)
+// and in G from the diagonal on.  blockIdx.y: row tile, blockIdx.x: the tiles of X, then those of G (the ones before the diagonal have no work).
+constexpr int CU_T = 64, CU_SMEM = 2 * CH_NB * CU_T * 4;
+__global__ void __launch_bounds__(256) chol_update_kernel(float *__restrict__ G, float *__restrict__ X, int b, int n, int ld) {
+    extern __shared__ __align__(16) float ch_smem[];
+    float *us = ch_smem, *bs = ch_smem + CH_NB * CU_T;           // [k][row], [k][column]
+    const int below = b + CH_NB, xt = below / CU_T;
+    const int i0 = below + (int)blockIdx.y * CU_T;
+    const bool in_x = (int)blockIdx.x < xt;
+    const int j0 = in_x ? (int)blockIdx.x * CU_T : below + ((int)blockIdx.x - xt) * CU_T;
+    tm::pdl_launch_dependents();
+    tm::pdl_wait();
+    if (!in_x && j0 < i0) return;
+    float *M = in_x ? X : G;
+    const int rows = min(CU_T, n - i0), cols = in_x ? CU_T : min(CU_T, n - j0);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+#pragma unroll 16
+    for (int e = tid; e < CH_NB * CU_T; e += 256) {
+        const int k = e / CU_T, c = e - k * CU_T;
+        us[e] = c < rows ? G[(size_t)(b + k) * ld + i0 + c] : 0.f;
+        bs[e] = c < cols ? M[(size_t)(b + k) * ld + j0 + c] : 0.f;
     }
-    MDBF_CUDA(cudaGetLastError());
+    float old[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) old[p][q] = 4 * ty + p < rows && 4 * tx + q < cols ? M[(size_t)(i0 + 4 * ty + p) * ld + j0 + 4 * tx + q] : 0.f;
+    __syncthreads();
+    float acc[4][4] = {};
+#pragma unroll 8
+    for (int k = 0; k < CH_NB; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(us + k * CU_T + 4 * ty), y = *reinterpret_cast<const float4 *>(bs + k * CU_T + 4 * tx);
+        const float xa[4] = {x.x, x.y, x.z, x.w}, yb[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xa[p], yb[q], acc[p][q]);
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (4 * ty + p < rows && 4 * tx + q < cols) M[(size_t)(i0 + 4 * ty + p) * ld + j0 + 4 * tx + q] = old[p][q] - acc[p][q];
+}
+template <class K, class... Args>
+static mdbf_status_t launch_step(K kern, dim3 grid, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;    // every kernel of a step waits for the one before it itself
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    MDBF_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
     return MDBF_OK;
+}
+static mdbf_status_t factor_leaf(float *G, float *X, float *D, int n, int ld, int *info, cudaStream_t st) {
+    static PerDeviceOnce once;
+    if (auto first = once.first()) {
+        MDBF_CUDA(cudaFuncSetAttribute(chol_diag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CD_SMEM));
+        MDBF_CUDA(cudaFuncSetAttribute(chol_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CP_SMEM));
+        MDBF_CUDA(cudaFuncSetAttribute(chol_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CU_SMEM));
+    }
+    mdbf_status_t rc = MDBF_OK;
+    for (int b = 0; b < n && rc == MDBF_OK; b += CH_NB) {
+        const int m = std::min(CH_NB, n - b);
+        const size_t at = (size_t)b * ld + b;
+        rc = launch_step(chol_diag_kernel, dim3(1), CD_SMEM, st, (const float *)(G + at), X + at, D, m, ld, info);
+        const int cols = n - m;                                  // without the diagonal block
+        if (rc == MDBF_OK && cols > 0) rc = launch_step(chol_panel_kernel, dim3(ceil_div(cols, CP_COLS)), CP_SMEM, st, G, X, (const float *)D, b, m, n, ld);
+        const int tiles = ceil_div(n - b - m, CU_T);
+        if (rc == MDBF_OK && tiles > 0) rc = launch_step(chol_update_kernel, dim3((b + CH_NB) / CU_T + tiles, tiles), CU_SMEM, st, G, X, b, n, ld);
+    }
+    return rc;
+}
+struct System {
+    float *G, *X, *P;           // the system (overwritten), the inverse factor (zeroed beforehand), scratch; all r x r
+    float *D;                   // CH_NB x CH_NB
+    uint32_t *img;              // operand images of two blocks of a product: s x s and s2 x s, or s x s2 and s2 x s2 (r x r images hold them)
+    int r;
+    int32_t *status;            // of the product kernel
+    int *info;                  // set by a pivot that is not positive
+};
+static mdbf_status_t factor_inverse(const System &f, int o, int n, cudaStream_t st) {
+    const size_t ld = (size_t)f.r, d11 = (size_t)o * ld + o;
+    if (n <= CH_LEAF) return factor_leaf(f.G + d11, f.X + d11, f.D, n, f.r, f.info, st);
+    int s = CH_LEAF;
+    while (2 * s < n) s *= 2;
+    const int s2 = n - s;
+    const size_t d12 = d11 + s, d21 = d11 + (size_t)s * ld, d22 = d21 + s;
+    mdbf_status_t rc = factor_inverse(f, o, s, st);
+    uint32_t *a = f.img, *b = f.img + gemm3x_image_bytes(s, s) / 4;
+    if (rc == MDBF_OK) rc = gemm3x_split(f.X + d11, ld, 1, s, s, a, st);                          // U12 = X11 G12
+    if (rc == MDBF_OK) rc = gemm3x_split(f.G + d12, 1, ld, s2, s, b, st);
+    if (rc == MDBF_OK) rc = gemm3x_run(a, b, G3xOut{f.G + d12, f.r, false, nullptr, nullptr}, s, s2, s, f.status, st);
+    if (rc == MDBF_OK) rc = gemm3x_split(f.G + d12, 1, ld, s2, s, b, st);                         // G22 - U12^T U12
+    if (rc == MDBF_OK) rc = gemm3x_run(b, b, G3xOut{nullptr, f.r, true, f.G + d22, f.G + d22, G3X_UPPER}, s2, s2, s, f.status, st);
+    if (rc == MDBF_OK) rc = gemm3x_split(f.X + d11, 1, ld, s, s, a, st);                          // T = U12^T X11
+    if (rc == MDBF_OK) rc = gemm3x_run(b, a, G3xOut{f.P + d21, f.r, false, nullptr, nullptr}, s2, s, s, f.status, st);
+    if (rc == MDBF_OK) rc = factor_inverse(f, o + s, s2, st);
+    if (rc == MDBF_OK) rc = gemm3x_split(f.P + d21, 1, ld, s, s2, a, st);                         // X21 = -X22 T
+    if (rc == MDBF_OK) rc = gemm3x_split(f.X + d22, ld, 1, s2, s2, b, st);
+    if (rc == MDBF_OK) rc = gemm3x_run(b, a, G3xOut{f.X + d21, f.r, true, nullptr, nullptr}, s2, s, s2, f.status, st);
+    return rc;
 }
 // U = S (.) (Ul Vl^T) entry by entry from the compact MSVID result, and Lam += U_tilde - U (Eq. admm-U-dual, rounded as written: near
 // convergence U_tilde - U and Lam are small beside Z = U_tilde + Lam, and Z - U would carry a rounding of Z into the dual in every
@@ -258,15 +452,15 @@ __global__ void __launch_bounds__(RC_COLS) recon_dual_kernel(const uint32_t *__r
 // a failed factorisation (not expected: the system is positive definite for rho > 0) or an expired wait of the product
 // kernel turns the singular values into NaN
 __global__ void flag_kernel(const int *__restrict__ info, float *__restrict__ sigma, int l) {
-    if ((info[0] != 0 || info[2] != 0) && threadIdx.x < l) sigma[threadIdx.x] = __int_as_float(0x7fc00000);
+    if ((info[0] != 0 || info[1] != 0) && threadIdx.x < l) sigma[threadIdx.x] = __int_as_float(0x7fc00000);
 }
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 struct Scratch {
-    float *B0, *T, *Z, *G;      // T: scratch of the triangular inverse
+    float *B0, *T, *Z, *G;      // T: scratch of the factorisation
     uint32_t *Wimg, *Vimg;      // operand images of op(W) (N row tiles, M deep) and of V^T (R row tiles, M deep)
-    uint32_t *Yimg;             // images of L^-T (R x R), formed on the side stream while W's are in use
-    int *info;                  // [0], [1]: the solver's; [2]: status word of the product kernel
+    uint32_t *Yimg;             // images of the factorisation's products and of L^-T (R x R), formed on the side stream while W's are in use
+    int *info;                  // [0]: the factorisation's; [1]: status word of the product kernel
     char *msvid;
     size_t msvid_bytes;
 };
@@ -283,7 +477,7 @@ static mdbf_status_t carve(Scratch *w, char *base, int64_t n, int64_t m, int64_t
     uint32_t *Wimg = (uint32_t *)take(gemm3x_image_bytes(n, m));
     uint32_t *Vimg = (uint32_t *)take(gemm3x_image_bytes(r, m));
     uint32_t *Yimg = (uint32_t *)take(gemm3x_image_bytes(r, r));
-    int *info = (int *)take(4 * sizeof(int));
+    int *info = (int *)take(2 * sizeof(int));
     char *mw = take(msv);
     if (w) { w->B0 = B0; w->T = T; w->Z = Z; w->G = G; w->Wimg = Wimg; w->Vimg = Vimg; w->Yimg = Yimg; w->info = info; w->msvid = mw; w->msvid_bytes = msv; }
     *total = off;
@@ -346,44 +540,37 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
     rc = require_device(&device);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    admm::Libs *L = nullptr;
-    rc = admm::get_libs(device, st, &L);
+    admm::Side *side = nullptr;
+    rc = admm::get_side(device, (size_t)admm::CH_NB * admm::CH_NB, who, &side);
     if (rc) return rc;
     const int ni = (int)n, mi = (int)m, ri = (int)r;
-    MDBF_CUDA(cudaMemsetAsync(w.info, 0, 4 * sizeof(int), st));
+    MDBF_CUDA(cudaMemsetAsync(w.info, 0, 2 * sizeof(int), st));
     // images: op(W)[i][k] = W[i * w_cols + k], or W[k * w_cols + i] when transposed;  V^T[j][k] = V[k * r + j]
     rc = gemm3x_split(V, 1, (size_t)r, ri, mi, w.Vimg, st);
     if (rc) return rc;
-    // Fork.  Side stream: G = V^T V + rho I, its Cholesky factor L, Y = L^-T, G^-1 = Y Y^T as a product of Y's images with themselves - the inverse written out,
-    // as Eq. admm-U-tilde has it, so that every inner iteration's solve is one product on the tensor cores instead of two
-    // triangular solves with N right-hand sides on the FP32 pipe.  Caller's stream meanwhile: W's images and B0 = op(W) V,
-    // on all SMs but a few that are left to the solver's small kernels.  Z is free until the loop below.
-    cudaStream_t s2 = L->side;
-    MDBF_CUDA(cudaEventRecord(L->fork, st));
-    MDBF_CUDA(cudaStreamWaitEvent(s2, L->fork, 0));
-    // the solver reads one triangle: half of V^T V; Y is triangular: a third of the products of Y Y^T
-    rc = gemm3x_run(w.Vimg, w.Vimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_UPPER}, ri, ri, mi, w.info + 2, s2);
+    // Fork.  Side stream: G = V^T V + rho I, X = L^-1 of its Cholesky factor L, G^-1 = X^T X as a product of X's images with themselves - the
+    // inverse written out, as Eq. admm-U-tilde has it, so that every inner iteration's solve is one product on the tensor cores instead
+    // of two triangular solves with N right-hand sides on the FP32 pipe.  Caller's stream meanwhile: W's images and B0 = op(W) V,
+    // on all SMs but those that are left to the factorisation's kernels.  Z is free until the loop below.
+    cudaStream_t s2 = side->stream;
+    MDBF_CUDA(cudaEventRecord(side->fork, st));
+    MDBF_CUDA(cudaStreamWaitEvent(s2, side->fork, 0));
+    // the factorisation reads one triangle: half of V^T V; X is triangular: a third of the products of X^T X
+    rc = gemm3x_run(w.Vimg, w.Vimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_UPPER}, ri, ri, mi, w.info + 1, s2);
+    if (rc) return rc;
+    // (queued before the factorisation's launches: behind them it began 0.7 ms later, when the host was through with those)
+    rc = transpose_w ? gemm3x_split(W, 1, (size_t)w_cols, ni, mi, w.Wimg, st) : gemm3x_split(W, (size_t)w_cols, 1, ni, mi, w.Wimg, st);
+    if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, w.B0, ni, ri, mi, w.info + 1, st, 48);
     if (rc) return rc;
     admm::ridge_kernel<<<ceil_div(ri, 256), 256, 0, s2>>>(w.G, ri, rho);
-    int lwork = 0;
-    cusolverStatus_t ss = cusolverDnSpotrf_bufferSize(L->solver, CUBLAS_FILL_MODE_LOWER, ri, w.G, ri, &lwork);
-    if (ss != CUSOLVER_STATUS_SUCCESS) { set_error("%s: cusolverDnSpotrf_bufferSize returned %d", who, (int)ss); return MDBF_ERR_CUDA; }
-    rc = admm::grow_scratch(L, lwork, s2, who);
+    MDBF_CUDA(cudaMemsetAsync(w.Z, 0, (size_t)r * r * sizeof(float), s2));
+    rc = admm::factor_inverse(admm::System{w.G, w.Z, w.T, side->diag, w.Yimg, ri, w.info + 1, w.info}, 0, ri, s2);
+    if (rc == MDBF_OK) rc = gemm3x_split(w.Z, 1, (size_t)r, ri, ri, w.Yimg, s2);
+    if (rc == MDBF_OK) rc = gemm3x_run(w.Yimg, w.Yimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_FACTORS}, ri, ri, ri, w.info + 1, s2);
     if (rc) return rc;
-    ss = cusolverDnSpotrf(L->solver, CUBLAS_FILL_MODE_LOWER, ri, w.G, ri, L->potrf_ws, L->potrf_floats, w.info);
-    if (ss != CUSOLVER_STATUS_SUCCESS) { set_error("%s: cusolverDnSpotrf returned %d", who, (int)ss); return MDBF_ERR_CUDA; }
-    // the solver's lower triangle is, read row-major, U = L^T; Y = U^-1 = L^-T.  Z is free until the loop, Y's images until Y is done
-    rc = admm::tri_inverse(w.G, w.Z, w.T, w.Yimg, ri, w.info + 2, s2);
-    if (rc) return rc;
-    rc = gemm3x_split(w.Z, (size_t)r, 1, ri, ri, w.Yimg, s2);
-    if (rc == MDBF_OK) rc = gemm3x_run(w.Yimg, w.Yimg, G3xOut{w.G, ri, false, nullptr, nullptr, G3X_FACTORS}, ri, ri, ri, w.info + 2, s2);
-    if (rc) return rc;
-    MDBF_CUDA(cudaEventRecord(L->join, s2));
-    rc = transpose_w ? gemm3x_split(W, 1, (size_t)w_cols, ni, mi, w.Wimg, st) : gemm3x_split(W, (size_t)w_cols, 1, ni, mi, w.Wimg, st);
-    if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, w.B0, ni, ri, mi, w.info + 2, st, 24);
-    if (rc) return rc;
+    MDBF_CUDA(cudaEventRecord(side->join, s2));
     // Join; the inverse's images go where V's were (symmetric: rows serve as columns)
-    MDBF_CUDA(cudaStreamWaitEvent(st, L->join, 0));
+    MDBF_CUDA(cudaStreamWaitEvent(st, side->join, 0));
     rc = gemm3x_split(w.G, (size_t)r, 1, ri, ri, w.Vimg, st);
     if (rc) return rc;
     const int nwords = (int)((r + 31) / 32);
@@ -392,7 +579,7 @@ extern "C" mdbf_status_t mdbf_admm_factor_update(const float *W, int64_t w_rows,
         // free from there on, so it takes U_tilde; the last one goes where the caller wants it.  Lam is added on the way out.
         rc = gemm3x_split_rhs(w.B0, U, Lambda, rho, ni, ri, w.Wimg, st);
         float *Ut = it == n_inner - 1 && U_tilde ? U_tilde : U;
-        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, G3xOut{Ut, ri, false, Lambda, w.Z}, ni, ri, ri, w.info + 2, st);
+        if (rc == MDBF_OK) rc = gemm3x_run(w.Wimg, w.Vimg, G3xOut{Ut, ri, false, Lambda, w.Z}, ni, ri, ri, w.info + 1, st);
         if (rc) return rc;
         rc = mdbf_msvid(w.Z, n, r, l, n_iter, Q0, S_packed, Ul, Vl, sigma, w.msvid, w.msvid_bytes, stream);
         if (rc) return rc;

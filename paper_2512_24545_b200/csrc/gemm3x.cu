@@ -159,13 +159,15 @@ static void launch_split_rows(const SRC &src, size_t stride_i, int rows, int dep
     else if (nkb <= 64) split_rows_kernel<SRC, 2><<<grid, 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
     else split_rows_kernel<SRC, 4><<<grid, 256, 0, st>>>(src, stride_i, rows, depth, nkb, pieces, inv);
 }
-// Rows contiguous (a transposed operand): largest magnitudes by a pass of their own, thread = row, 256 contraction indices per CTA ...
+// Rows contiguous (a transposed operand): largest magnitudes by a pass of their own, thread = row, CM_DEPTH contraction indices per CTA, all of
+// its loads in flight (1024 x 1024: 22 us with 256 indices per CTA, sixteen CTAs, eight loads at a time) ...
+constexpr int CM_DEPTH = 32;
 __global__ void __launch_bounds__(256) column_max_kernel(const float *__restrict__ src, size_t stride_k, int ni, int nk, uint32_t *__restrict__ maxbits) {
-    const int i = blockIdx.x * 256 + threadIdx.x, k0 = blockIdx.y * 256, k1 = min(k0 + 256, nk);
+    const int i = blockIdx.y * 256 + threadIdx.x, k0 = blockIdx.x * CM_DEPTH;
     if (i >= ni) return;
     float m = 0.f;
-#pragma unroll 8
-    for (int k = k0; k < k1; ++k) m = fmaxf(m, fabsf(src[(size_t)k * stride_k + i]));
+#pragma unroll
+    for (int u = 0; u < CM_DEPTH; ++u) m = fmaxf(m, fabsf(src[(size_t)min(k0 + u, nk - 1) * stride_k + i]));
     atomicMax(maxbits + i, __float_as_uint(m));                  // magnitudes order like their bits
 }
 // ... then the images, thread = row (consecutive rows are consecutive in memory), two threads per row share its 8 chunks
@@ -413,7 +415,7 @@ mdbf_status_t gemm3x_split(const float *src, size_t stride_i, size_t stride_k, i
     } else if (stride_i == 1) {
         uint32_t *maxbits = reinterpret_cast<uint32_t *>(inv + (size_t)tiles * g3x::TILE);
         MDBF_CUDA(cudaMemsetAsync(maxbits, 0, (size_t)tiles * g3x::TILE * 4, st));
-        g3x::column_max_kernel<<<dim3(ceil_div(rows, 256), ceil_div(depth, 256)), 256, 0, st>>>(src, stride_k, rows, depth, maxbits);
+        g3x::column_max_kernel<<<dim3(ceil_div(depth, g3x::CM_DEPTH), ceil_div(rows, 256)), 256, 0, st>>>(src, stride_k, rows, depth, maxbits);
         g3x::split_columns_kernel<<<dim3(nkb, tiles), 256, 0, st>>>(src, stride_k, rows, depth, nkb, pieces, inv, maxbits);
     } else { set_error("gemm3x_split: one of the strides must be 1"); return MDBF_ERR_INVALID_ARG; }
     MDBF_CUDA(cudaGetLastError());

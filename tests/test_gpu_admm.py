@@ -329,3 +329,19 @@ def test_inverse_of_a_badly_conditioned_system(R):
     err = np.max(np.abs(got - want.cpu().numpy())) / float(want.abs().max())
     print("condition:", R, err)
     assert err <= 1e-4
+
+
+@pytest.mark.parametrize("R", [15, 16, 17, 127, 128, 255, 257, 400, 1023, 1024, 1151, 2049, 3100])
+def test_factorisation_at_the_edges_of_its_steps(R):
+    """The system is factored and inverted in panels of 16, steps of 128 and blocks of 1024 columns that are joined on the tensor cores: a last
+    panel, step or block of one column and of one less than all, and three blocks.  Condition and bound as for the inverse by doubling."""
+    n, m = R + 5, R + 3
+    g = torch.Generator(device="cuda").manual_seed(270 + R)
+    rnd = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    W, V, U, Lam = rnd(n, m), rnd(m, R), rnd(n, R), 0.1 * rnd(n, R)
+    rho = float((V.double() ** 2).sum() / R)
+    V8 = V.double()
+    want = torch.linalg.solve(V8.T @ V8 + rho * torch.eye(R, device="cuda", dtype=torch.float64),
+                              (W.double() @ V8 + rho * (U.double() - Lam.double())).T).T
+    got = run_update(W.cpu().numpy(), V.cpu().numpy(), U.cpu().numpy(), Lam.cpu().numpy(), rho, 1, 1, 4)["tilde"]
+    assert np.max(np.abs(got - want.cpu().numpy())) <= 2e-5 * float(want.abs().max())
