@@ -42,6 +42,7 @@
 #include <cooperative_groups.h>
 #include <cstdlib>
 
+#include "plans.h"
 #include "tmem_ptx.cuh"
 
 namespace cg = cooperative_groups;
@@ -538,10 +539,6 @@ struct TxPlan {
     size_t smem;
 };
 
-// Fixed part of a CTA's time (set-up, cluster reduction) in units of one K block of streaming (swept on the
-// 7B- and 70B-class shapes).
-static int fixed_cost() { return 48; }
-
 // Two CTAs of a launch that share an SM take turns at its tensor memory, which costs a launch twice its time.  CTAs that start while
 // the previous launch still holds the other SMs are put there by the hardware, two on every idle SM: a launch that follows one
 // whose CTAs leave no room beside them (three expander groups, the integer kernel) asks for more than half of an SM's
@@ -554,27 +551,17 @@ constexpr size_t TX_ALONE_DYN = 114 * 1024;
 // footprints did not share an SM (11008 x 4096: 20.2 instead of 13.2 us).
 constexpr int TX_CARVEOUT = 58;
 
-// One plan for all the layers of a launch.  Cluster size along the reduction: one CTA per SM (all of
-// TMEM), as few waves as possible, the per-CTA fixed part weighed against its share of the reduction.
-// terms > 1: the n layers are the terms of a sum, whose ranks share the cluster of a row block (p->ks: all of them).
+// One plan for all the layers of a launch (plan_t1_ranks).  terms > 1: the n layers are the terms of a sum, whose ranks share the cluster of
+// a row block (p->ks: all of them).
 static bool plan_t1(int n, const int *rows, const int *kb_pad, int LP, TxPlan *p, int terms = 1) {
     const int NB = LP < 16 ? 16 : LP;
     const int max_ks = 8 / terms;                             // portable cluster size
-    int rb = 0, max_pairs = 0, min_pairs = 1 << 30;
+    int row_blocks[TX_MAX_LAYERS], pairs[TX_MAX_LAYERS];
     for (int i = 0; i < n; ++i) {
-        rb += ceil_div(rows[i], 128);
-        max_pairs = max(max_pairs, kb_pad[i] / 2);
-        min_pairs = min(min_pairs, kb_pad[i] / 2);
+        row_blocks[i] = ceil_div(rows[i], 128);
+        pairs[i] = kb_pad[i] / 2;
     }
-    if (terms > 1) rb = ceil_div(rows[0], 128) * terms;
-    long best_cost = -1;
-    int best_ks = 1;
-    for (int ks = 1; ks <= max_ks; ks *= 2) {
-        if (ks > 1 && ceil_div(min_pairs, ks) * (ks - 1) >= min_pairs) continue;     // an empty rank in some layer
-        const long waves = ceil_div(rb * ks, 148);
-        const long cost = waves * (2 * ceil_div(max_pairs, ks) + fixed_cost());
-        if (best_cost < 0 || cost < best_cost) { best_cost = cost; best_ks = ks; }
-    }
+    const int best_ks = plan_t1_ranks(n, row_blocks, pairs, max_ks, terms);
     p->ks = best_ks * terms;
     int max_per = 1;
     for (int i = 0; i < n; ++i) {

@@ -65,6 +65,20 @@ def test_tmem_kernel_edge_shapes(shape):
         check_parity(g, x, y, averaging=k >= 8)                 # a layer with a few terms: the per-element bound
 
 
+@pytest.mark.parametrize("d_out,d_in,k", [(128, 768, 130), (1100, 3 * 128 * 5, 7 * 128), (2304, 11 * 128 + 8, 2500), (4700, 86 * 128, 2400),
+                                          (300, 5 * 128, 6 * 128)])
+def test_clusters_of_any_size(d_out, d_in, k):
+    """The reduction is split over one to eight ranks, whatever divides: three to seven of them in one stage or the other, a last rank with fewer
+    pairs of K blocks than the others, rows behind the last whole row block."""
+    spec = spec_of(d_out, d_in, k, 16)
+    x = inputs.make_activations(spec, 1)
+    with GpuLayer(spec, 1) as g:
+        y = g.forward(x, kernel=M.KERNEL_TMEM)
+        assert M.mdbf_poll_status(g.h) == 0
+        check_parity(g, x, y)
+        np.testing.assert_array_equal(y, g.forward(x, kernel=M.KERNEL_TMEM))
+
+
 def test_tmem_kernel_takes_one_token_only():
     spec = spec_of(128, 128, 128, 16)
     x = inputs.make_activations(spec, 2)
